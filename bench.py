@@ -165,13 +165,13 @@ class ClockSampler:
 
 
 def step_kernels(w):
-    """Names of the Born and migration step kernels the workload runs: the
-    TMA-staged 2D kernels (no aperture windows), the per-thread-copy ones
-    (windows), or the fused 3D ones."""
+    """Names of the Born and migration step kernels the workload runs: the 2D
+    kernels of shots spanning the model, those of shots with aperture windows,
+    or the fused 3D ones."""
     if w.ndim == 3:
         return {"born": "k3f_born", "adjoint": "k3f_adj"}
     if getattr(w.geom, "win_nx", None) is not None:
-        return {"born": "k_fwd2d<BORN>", "adjoint": "k_adj2d"}
+        return {"born": "k_fwd2w", "adjoint": "k_adj2d"}
     return {"born": "k_fwd2t", "adjoint": "k_adj2t"}
 
 

@@ -49,9 +49,9 @@ lsrtm_status fail(lsrtm_status st, const std::string &msg)
 
 // Planes per wavefield slot: 10 ping-pong planes (Born: (p, dp) (vx, dvx)
 // (vz, dvz) (psi_px, dpsi_px) (psi_pz, dpsi_pz) as float2 pairs; background
-// only: p vx vz psi_px psi_pz; adjoint: (p, lambda_p) (vx, lambda_vx)
-// (vz, lambda_vz) pairs and four lambda CPML memories), 4 in-place node CPML
-// planes (forward).
+// only: p vx vz psi_px psi_pz; adjoint: (p, dt kappa lambda_p) (vx,
+// lambda_vx) (vz, lambda_vz) pairs and four lambda CPML memories), 4 in-place
+// node CPML planes (forward).
 constexpr int kStatePlanes2D = 10;
 constexpr int kPsivPlanes2D = 4;
 constexpr int kStatePlanes3D = 20;
@@ -104,8 +104,8 @@ struct lsrtm_handle {
     long long sstride1 = 0;      // slot stride of st[1] (3D: the fused kernels' pong buffer)
     Step3F f3born[2];            // fused 3D Born step arguments reading st[0] / st[1]
     Adj3F f3adj[2];              // fused 3D adjoint step arguments reading st[0] / st[1]
-    Maps2D m2d[2];             // 2D TMA row maps reading st[0] / st[1]
-    bool tma2d = false;          // the 2D Born and migration kernels stage rows by TMA (no aperture windows)
+    Maps2D m2d[2];               // 2D TMA row maps reading st[0] / st[1]
+    Maps2D m2rec[2];             // ... reading rec[0] / rec[1]
     int *kerr = nullptr;         // device error words: [0] fused-kernel tile copies, [1] non-finite guard
     int guard_K = 0;             // time steps between non-finite guard checks (0: off)
     long long guard_count = 0;   // guard launches queued or captured so far
@@ -501,9 +501,6 @@ lsrtm_status guard_step(lsrtm_handle *h, int kind, int i, int n, const float *st
     return LSRTM_OK;
 }
 
-// TMA row maps of the 2D migration reading state buffer j, or null.
-const Maps2D *maps2_of(const lsrtm_handle *h, int j) { return h->tma2d ? &h->m2d[j] : nullptr; }
-
 // Slot stride of state buffer j (3D: the fused kernels' ping and pong differ).
 long long slot_stride(const lsrtm_handle *h, int j) { return j ? h->sstride1 : h->sstride; }
 
@@ -562,7 +559,7 @@ lsrtm_status bg_forward(lsrtm_handle *h, bool hess)
                     a.n = n;
                     a.in = h->st[n & 1];
                     a.out = h->st[(n + 1) & 1];
-                    CU(launch_fwd2d(a, bs, false, true, hess, h->work));
+                    CU(launch_fwd2d(a, h->m2d[n & 1], bs, false, true, hess, h->work));
                     if (h->bands.fmt != BAND_F32) CU(launch_band_pack(h->bands, bs, s0, n, h->work));
                     CHECK(guard_step(h, GK_BACKGROUND, n, n, a.out, h->sstride, 1, bs));
                 }
@@ -621,7 +618,7 @@ lsrtm_status born_core(lsrtm_handle *h)
                 a.n = n;
                 a.in = h->st[n & 1];
                 a.out = h->st[(n + 1) & 1];
-                CU(launch_fwd2d(a, bs, true, false, false, h->work, maps2_of(h, n & 1)));
+                CU(launch_fwd2d(a, h->m2d[n & 1], bs, true, false, false, h->work));
                 CHECK(guard_step(h, GK_BORN, n, n, a.out, h->sstride, 2, bs));
             }
             return LSRTM_OK;
@@ -656,7 +653,7 @@ lsrtm_status model_core(lsrtm_handle *h)
                 a.n = n;
                 a.in = h->st[n & 1];
                 a.out = h->st[(n + 1) & 1];
-                CU(launch_fwd2d(a, bs, false, false, false, h->work));
+                CU(launch_fwd2d(a, h->m2d[n & 1], bs, false, false, false, h->work));
                 CHECK(guard_step(h, GK_MODELLING, n, n, a.out, h->sstride, 1, bs));
             }
             return LSRTM_OK;
@@ -757,7 +754,7 @@ lsrtm_status ck_forward(lsrtm_handle *h, int s0, int bs, bool hess)
                     CHECK(ck_copy(h, n / K, h->st[n & 1], h->sstride, 5, 0, bs, true));
                     CHECK(ck_copy(h, n / K, h->psiv, h->vstride, 2, 5, bs, true));
                 }
-                CU(launch_fwd2d(a, bs, false, false, hess, h->work));
+                CU(launch_fwd2d(a, h->m2d[n & 1], bs, false, false, hess, h->work));
                 CHECK(guard_step(h, GK_BACKGROUND, n, n, a.out, h->sstride, 1, bs));
             }
             return LSRTM_OK;
@@ -826,7 +823,7 @@ lsrtm_status ck_recompute(lsrtm_handle *h, int s0, int bs, int j)
             a.n = n;
             a.in = h->rec[n & 1];
             a.out = h->rec[(n + 1) & 1];
-            CU(launch_fwd2d(a, bs, false, true, false, h->work));
+            CU(launch_fwd2d(a, h->m2rec[n & 1], bs, false, true, false, h->work));
             if (pack) CU(launch_band_pack(sb, bs, s0, n, h->work));
             CHECK(guard_step(h, GK_RECOMPUTE, n, n, a.out, a.sstride, 1, bs));
         }
@@ -861,7 +858,7 @@ lsrtm_status ck_reverse(lsrtm_handle *h, int s0, int bs, int j)
             a.n = n;
             a.in = h->st[i & 1];
             a.out = h->st[(i + 1) & 1];
-            CU(launch_adj2d(a, maps2_of(h, i & 1), bs, h->work));
+            CU(launch_adj2d(a, h->m2d[i & 1], bs, h->work));
             CHECK(guard_step(h, GK_MIGRATION, nt - 1 - n, n, a.out, h->sstride, 2, bs));
         }
         return LSRTM_OK;
@@ -895,8 +892,9 @@ lsrtm_status adjoint_core_ckpt(lsrtm_handle *h, float *gout, bool want_hess)
             CHECK(adj3f_start(h, 0, s0, bs));
         } else {
             CU(launch_pack_adjoint(h->g, h->final_state, 0, bs, h->st[0], h->sstride, h->work));
-            CU(launch_inject_residual(h->g, h->trv, bs, s0, h->dstage, nt - 1,
-                                      reinterpret_cast<float2 *>(h->st[0]), h->sstride / 2, h->work));
+            CU(launch_inject_residual(h->gm, h->g, h->trv, bs, s0, h->dstage, nt - 1, h->kdt,
+                                      h->win ? h->win_x0_d : nullptr, reinterpret_cast<float2 *>(h->st[0]),
+                                      h->sstride / 2, h->work));
             h->launches += 2;
         }
         for (int j = h->ck_nseg - 1; j >= 0; --j) {
@@ -947,8 +945,9 @@ lsrtm_status adjoint_core(lsrtm_handle *h, float *gout, bool want_hess)
             h->launches++;
         } else {
             CU(launch_pack_adjoint(h->g, h->final_state, s0, bs, h->st[0], h->sstride, h->work));
-            CU(launch_inject_residual(h->g, h->trv, bs, s0, h->dstage, nt - 1,
-                                      reinterpret_cast<float2 *>(h->st[0]), h->sstride / 2, h->work));
+            CU(launch_inject_residual(h->gm, h->g, h->trv, bs, s0, h->dstage, nt - 1, h->kdt,
+                                      h->win ? h->win_x0_d : nullptr, reinterpret_cast<float2 *>(h->st[0]),
+                                      h->sstride / 2, h->work));
             h->launches += 2;
             CHECK(run_loop(h, G_ADJ, s0, bs, [&]() -> lsrtm_status {
                 CHECK(gather_model(h, s0, bs, false));
@@ -957,7 +956,7 @@ lsrtm_status adjoint_core(lsrtm_handle *h, float *gout, bool want_hess)
                     a.n = nt - 1 - i;
                     a.in = h->st[i & 1];
                     a.out = h->st[(i + 1) & 1];
-                    CU(launch_adj2d(a, maps2_of(h, i & 1), bs, h->work));
+                    CU(launch_adj2d(a, h->m2d[i & 1], bs, h->work));
                     CHECK(guard_step(h, GK_MIGRATION, i, nt - 1 - i, a.out, h->sstride, 2, bs));
                 }
                 return LSRTM_OK;
@@ -1266,8 +1265,8 @@ lsrtm_status adj3f_step(lsrtm_handle *h, int i, int n, int s0, const Bands &band
 lsrtm_status adj3f_start(lsrtm_handle *h, int fs0, int s0, int bs)
 {
     CU(launch_pack3f(h->g, h->final_state, fs0, bs, h->st[0], h->sstride, h->work));
-    CU(launch_inject_residual(h->g, h->trv, bs, s0, h->dstage, h->g.nt - 1, reinterpret_cast<float2 *>(h->st[0]),
-                              h->sstride / 2, h->work));
+    CU(launch_inject_residual(h->gm, h->g, h->trv, bs, s0, h->dstage, h->g.nt - 1, nullptr, nullptr,
+                              reinterpret_cast<float2 *>(h->st[0]), h->sstride / 2, h->work));
     h->launches += 2;
     return LSRTM_OK;
 }
@@ -1284,8 +1283,8 @@ lsrtm_status check_kernel_error(lsrtm_handle *h)
     CU(cudaMemsetAsync(h->kerr, 0, sizeof(e), h->work));
     CU(cudaStreamSynchronize(h->work));
     if (e[0])
-        return fail(LSRTM_ERR_CUDA, (e[0] & 2) ? "a fused 3D kernel refused a misaligned tile copy"
-                                               : "a fused 3D kernel gave up waiting for its tile copies");
+        return fail(LSRTM_ERR_CUDA, (e[0] & 2) ? "a time-step kernel refused a misaligned tile copy"
+                                               : "a time-step kernel gave up waiting for its tile copies");
     const int kind = e[1] >> 24, n = (e[1] & 0xFFFFFF) - 1;
     if (kind == GK_CG)
         return fail(LSRTM_ERR_NONFINITE, "non-finite CG scalar (<q,q>, gamma or <r,r>) at iteration " +
@@ -1585,13 +1584,15 @@ lsrtm_status create_impl(const lsrtm_config *cfg, const float *vp, const float *
     CU(cudaMallocHost(reinterpret_cast<void **>(&h->poll_h), 4 * sizeof(int)));
     for (cudaEvent_t &e : h->poll_ev) CU(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     if (d3) CHECK(setup_fused3d(h));
-    else if (!h->win) {
+    else {
         for (int b = 0; b < 2; ++b) {
-            cudaError_t e = maps2d(&h->m2d[b], h->g, h->st[b], h->sstride, h->kdt, h->binv, h->kd2, h->br2, h->img,
-                                   batch);
+            cudaError_t e = maps2d(&h->m2d[b], h->gm, h->g, h->st[b], h->sstride, h->kdt, h->binv, h->kd2, h->br2, h->img,
+                                   h->psiv, h->vstride, batch);
+            if (e == cudaSuccess && ckpt)
+                e = maps2d(&h->m2rec[b], h->gm, h->g, h->rec[b], 5 * g.plane, h->kdt, h->binv, h->kd2, h->br2, nullptr,
+                           h->rec_psiv, 2 * g.plane, batch);
             if (e != cudaSuccess) return fail(LSRTM_ERR_CUDA, std::string("tensor maps: ") + cudaGetErrorString(e));
         }
-        h->tma2d = true;
     }
     CU(cudaStreamSynchronize(h->work));
     return LSRTM_OK;
@@ -2280,9 +2281,9 @@ lsrtm_status lsrtm_autotune(lsrtm_handle *h, int steps, int *tzc_out, double *ms
                 a.n = i;
                 a.in = h->st[i & 1];
                 a.out = h->st[(i + 1) & 1];
-                launch_fwd2d(a, bs, true, false, false, h->work, maps2_of(h, i & 1));
+                launch_fwd2d(a, h->m2d[i & 1], bs, true, false, false, h->work);
                 a.n = steps - i;
-                launch_adj2d(a, maps2_of(h, i & 1), bs, h->work);
+                launch_adj2d(a, h->m2d[i & 1], bs, h->work);
             }
             cudaEventRecord(e1, h->work);
             cudaError_t e = cudaEventSynchronize(e1);

@@ -4,21 +4,29 @@
 // One launch advances every shot of a batch by one time step. A CTA of 256
 // threads owns one x-column per thread (240 output columns plus 2M halo
 // columns on each side for M = 4) and marches down a z-chunk of the padded
-// grid:
-//   * along z the stencil operands live in per-thread register rings of
-//     length 2M plus a group of look-ahead entries (the march is unrolled by
-//     one group of rows and the rings shift after every group);
-//   * along x each row passes through one shared-memory row per field;
-//   * the global loads of row z + PD - 1 are issued as asynchronous copies
-//     (cp.async, zero-filled out of range) into a PD-deep shared-memory stage
-//     ring while row z is computed;
+// grid, two rows (one group) at a time:
+//   * along z the stencil operands live in per-thread register rings (the
+//     march is unrolled by a few rows and the rings shift after every pass);
+//   * along x each group passes through two shared-memory rows per field;
+//   * the rows a group needs arrive by TMA: one thread issues each field's
+//     two rows as one 256 x 2 tile copy on the mbarrier of the group's stage
+//     while the previous group is computed. The tensor maps read zeros
+//     outside the padded grid, which is the operators' boundary convention;
 //   * a background field and its partner (the scattered field in Born
 //     modelling, the adjoint field in migration) are interleaved as float2 in
 //     HBM, so one 8-byte access and one packed FP32x2 FMA (FFMA2) serve both.
-// For every row the velocity stage (half nodes) is computed on the output
+// For every group the velocity stage (half nodes) is computed on the output
 // columns and the x halo, then the pressure stage (integer nodes), so a time
 // step needs no grid-wide barrier. Inputs and outputs are separate (ping-pong)
 // buffers; each state field is read once and written once per step from HBM.
+//
+// A stage is refilled only after a CTA barrier that follows every read of it:
+// the first barrier of the next group (a warm-up group, which fills the z
+// rings only, has one barrier of its own for this).
+//
+// Shots with aperture windows (WIN) have their own width, model planes (in
+// their slot) and x CPML profiles; CTAs past a shot's width exit at once.
+// Every state and model plane of a slot is zero past the shot's width.
 #include <algorithm>
 #include <mutex>
 #include <type_traits>
@@ -30,18 +38,11 @@ namespace lsrtm {
 namespace {
 
 constexpr int NTH = kThreads2D;
-constexpr int PDF = 4;   // depth of the asynchronous row pipeline (forward)
-constexpr int PDA = 3;   // depth of the asynchronous row pipeline (adjoint; 3 CTAs per SM fit)
-constexpr int kFwdMinBlocks = 2;   // resident CTAs per SM the register budget targets
-constexpr int kFwdTMinBlocks = 3;  // the TMA-staged Born kernel: three CTAs per SM (measured +25%)
-constexpr int kFwdPlainMinBlocks = 3;   // the background step without bands or pseudo-Hessian (modelling)
+constexpr int NS = 2;                    // stages: the group in use and the one in flight
+constexpr int kBornMinBlocks = 3;        // resident CTAs per SM the register budgets target
+constexpr int kPlainMinBlocks = 4;       // background step without bands or pseudo-Hessian (modelling)
+constexpr int kBandsMinBlocks = 3;
 constexpr int kAdjMinBlocks = 3;
-constexpr int kAdjMinBlocksFS = 2;   // the free-surface variant needs more registers
-// The z-marches are unrolled by 2M / k*GroupDiv rows and shift their register
-// rings after every group: a full 2M-row unroll made the migration loop body
-// large enough to miss in the instruction cache.
-constexpr int kAdjGroupDiv = 4;
-constexpr int kFwdGroupDiv = 2;
 
 // State layouts, as offsets in float planes within a shot slot.
 // Born: float2 pairs (background, scattered).
@@ -50,7 +51,8 @@ enum { B_PVX = 0, B_PVZ = 2 };                 // in-place node CPML memories
 // Background only (band saving, pseudo-Hessian): float.
 enum { G_P = 0, G_VX = 1, G_VZ = 2, G_PPX = 3, G_PPZ = 4 };
 enum { G_PVX = 0, G_PVZ = 1 };
-// Adjoint: float2 pairs (background, lambda) and float lambda CPML memories.
+// Adjoint: float2 pairs (p, dt kappa lambda_p), (v, lambda_v) and float
+// lambda CPML memories.
 enum { A_PL = 0, A_VX = 2, A_VZ = 4, A_LPPX = 6, A_LPPZ = 7, A_LPVX = 8, A_LPVZ = 9 };
 // Slots of aperture-windowed shots carry the window's own model after the
 // state: dt kappa and 1/rho (float planes), and the Born pairs (float2).
@@ -126,160 +128,163 @@ __device__ __forceinline__ long long pband_index(int iz, int ix, int M, int nz, 
 }
 
 
-// ---- asynchronous copies (pred = false zero-fills the destination)
-template <class T>
-__device__ __forceinline__ void cpa(T *dst, const T *src, bool pred)
-{
-    static_assert(sizeof(T) == 4 || sizeof(T) == 8, "4- or 8-byte copies");
-    unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
-    int n = pred ? (int)sizeof(T) : 0;
-    if (sizeof(T) == 4)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
-}
-
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-
-// Copy only where the field is used (the forward kernel's CPML memories): the
-// stage slot keeps stale data elsewhere, which no consumer reads (every
-// consumer tests the same condition), and warps outside the strips issue
-// nothing. (In the migration kernel the extra branches cost more registers
-// than the skipped copies save.)
-template <class T>
-__device__ __forceinline__ void cpa_if(T *dst, const T *src, bool pred)
-{
-    if (pred) cpa(dst, src, true);
-}
-
-// Waits until at most PDN-1 of this thread's copy groups are pending.
-template <int PDN>
-__device__ __forceinline__ void cp_wait_row() { asm volatile("cp.async.wait_group %0;\n" ::"n"(PDN - 1) : "memory"); }
-
 template <int M>
 struct Cols {
     static constexpr int W = 2 * M;            // ring length along z
     static constexpr int HXP = 2 * M;          // halo columns per side
     static constexpr int TXO = NTH - 2 * HXP;  // output columns per CTA
+    // every tile copy starts on a 16-byte boundary, for 4- and 8-byte elements
+    static_assert(TXO % 4 == 0 && HXP % 4 == 0, "CTA column starts must be multiples of 4 elements");
 };
 
-// Stage ring of the forward kernel: 8 fields of 8-byte slots per thread.
-constexpr int kFwdSlots = 8;
-constexpr size_t kFwdStageSlotBytes = (size_t)kFwdSlots * NTH * 8;
-constexpr size_t kFwdStageBytes = PDF * kFwdStageSlotBytes;
-// Stage ring of the adjoint kernel: 5 float2 fields then 9 float fields.
-constexpr int kAdjF2 = 5, kAdjF1 = 9;
-constexpr size_t kAdjStageFloats = (size_t)(2 * kAdjF2 + kAdjF1) * NTH;
-constexpr size_t kAdjStageBytes = PDA * kAdjStageFloats * sizeof(float);
+// A launch's arguments: the step and the row maps of its input state.
+struct Arg2D {
+    Step2D a;
+    Maps2D m;
+};
+
+// Copies field rows r0 and r1 (FR bytes each) of map plane q to dst and dst +
+// FR: one 2-row tile when they are adjacent, else (mirror rows of a free
+// surface, rows of different fields) one row each.
+template <bool PAIR>
+__device__ __forceinline__ void copy_rows(char *dst, unsigned FR, const CUtensorMap (&m)[2], int xs, int r0, int r1, int q,
+                                          uint64_t *b)
+{
+    if (PAIR || r1 == r0 + 1) {
+        tma::load3(dst, m[1], xs, r0, q, b);
+    } else {
+        tma::load3(dst, m[0], xs, r0, q, b);
+        tma::load3(dst + FR, m[0], xs, r1, q, b);
+    }
+}
+
+// Brings the line of *p into L1 ahead of its use by the same thread.
+__device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];\n" ::"l"(p)); }
+
+// Asynchronous copies of 4 bytes.
+__device__ __forceinline__ void cp_async4(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(tma::su32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
+// Half-node z CPML rows, node z CPML rows.
+__device__ __forceinline__ bool zpml_half(const GridDev &g, int k)
+{
+    return k >= 0 && k < g.Nz && (k <= g.z0 - 2 || k >= g.z0 + g.nz);
+}
+__device__ __forceinline__ bool zpml_node(const GridDev &g, int r)
+{
+    return r >= 0 && r < g.Nz && (r <= g.z0 - 1 || r >= g.z0 + g.nz);
+}
 
 // ---------------------------------------------------------------------------
 // Forward step from n to n+1. BORN: the background and the scattered field as
 // float2 pairs (Eq. scattereqln driven by the background). Otherwise the
 // background alone as float, with BANDS saving the boundary bands of p^n and
 // v^{n+1/2} and HESS accumulating the pseudo-Hessian diagonal of App. B.
+//
+// What bounds it: the Born step moves 64 B a cell, 57.9 from DRAM (the shots
+// of a batch share the model), and is held back by latencies between its
+// barriers (54% of the issue slots used). A group of two rows halves the
+// barriers; every warp issues one field's copy (one thread that issued all of
+// a row's was waited for 600 to 1000 cycles); interior rows and warps run
+// straight-line code, and what the strips need in the last stage comes with
+// the copies (their warps took twice the others' time and set the CTA's pace).
+// 96 shots of 424 x 1192 padded cells, order 8: 80.9 G cell-updates/s = 0.77
+// of the measured copy rate (a row at a time, one issuing thread: 67.6); the
+// background step with recording, 48 shots: 110.7 G (with per-thread copies:
+// 70.8). Windowed shots: with k_adj2d 1.27x over per-thread copies.
 // ---------------------------------------------------------------------------
-template <bool BORN>
-struct FwdT {
-    using T = typename std::conditional<BORN, float2, float>::type;   // state (pair)
-    using R = typename std::conditional<BORN, float2, float>::type;   // (1/rho, rr) or 1/rho
-    using K = typename std::conditional<BORN, float2, float>::type;   // (dt kappa, dt kappa dlnk) or dt kappa
+template <int M, bool BORN, bool HESS>
+struct FwdLay {
+    using T = typename std::conditional<BORN, float2, float>::type;   // state (pair), (1/rho, rr), (dt kappa, dt kappa dlnk)
+    static constexpr unsigned FR = NTH * sizeof(T);   // one field row
+    static constexpr unsigned F = 2 * FR;             // a field's rows of a group
+    // stage: p (rows z + 2M - 1), vz and psi_pz (half rows z + M - 1), vx, dt kappa and psi_px (rows z)
+    static constexpr unsigned P = 0, VZ = F, VX = 2 * F, KD = 3 * F, PZ = 4 * F, PX = 5 * F, STAGE = 6 * F;
+    // 1/rho: rows z + M of group j in slot j % NB; the x stage of group j reads group j - M/2's
+    static constexpr int NB = M / 2 + NS;
+    static constexpr unsigned BR = NS * STAGE;
+    static constexpr unsigned SP = BR + NB * F;       // [2][NTH] p of the group's rows
+    static constexpr unsigned SV = SP + F;            // [2][NTH] vx
+    static constexpr unsigned SH = SV + F;            // [2][NTH] (b G_x)^2 (HESS)
+    static constexpr unsigned BAR = SH + (HESS ? 2 * NTH * 4 : 0) + 128;
+    static constexpr unsigned SMEM = BAR + 64 + 128;  // + alignment slack
+    static_assert(STAGE % 128 == 0 && F % 128 == 0, "copy destinations stay 128-byte aligned");
 };
 
-template <bool BORN>
-struct FwdRow {
-    using T = typename FwdT<BORN>::T;
-    using R = typename FwdT<BORN>::R;
-    using K = typename FwdT<BORN>::K;
-    T p;      // node row z + 2M - 1 (look-ahead of the z rings)
-    T vz;     // half row k = z + M - 1
-    T psz;    // psi_pz at half row k (CPML rows)
-    T vx;     // row z
-    T psx;    // psi_px at row z (CPML columns)
-    R br1;    // 1/rho (, rr) at row k + 1
-    R brz;    // 1/rho (, rr) at row z
-    K kd;     // dt kappa (, dt kappa dlnk) at row z
-};
-
-template <int M, bool BORN, bool WIN, bool FS>
-__device__ __forceinline__ void fwd_issue(char *st, const Step2D &a, const float *in, int xc, int z,
-                                          int zc0, int zc1, bool colok, bool vxok, bool outcol,
-                                          bool pmlxh)
+// Issues the copies of the group of rows z, z + 1 on barrier b; called by
+// whole warps, each of which issues its own field (a copy costs its issuing
+// lane 30 to 100 cycles, and the other warps would wait for one that issued
+// them all). tpn / tph: the CTA has node / half-node x CPML columns.
+template <int M, bool BORN, bool FS, bool WIN>
+__device__ __forceinline__ void fwd_issue(const Arg2D &p, int warp, char *st, char *brs, uint64_t *b, int slot, int xs,
+                                          int z, int zc0, bool tpn, bool tph)
 {
-    using T = typename FwdT<BORN>::T;
-    using R = typename FwdT<BORN>::R;
-    using K = typename FwdT<BORN>::K;
-    const GridDev &g = a.g;
-    const int pitch = g.pitch;
-    const int W = 2 * M;
-    char *sl = st + threadIdx.x * 8;
-    const T *fin = reinterpret_cast<const T *>(in);
-    const R *br = WIN ? reinterpret_cast<const R *>(in + (BORN ? W_BR2 : W_BINV) * g.plane)
-                      : (BORN ? reinterpret_cast<const R *>(a.br2) : reinterpret_cast<const R *>(a.binv));
-    const K *kk = WIN ? reinterpret_cast<const K *>(in + (BORN ? W_KD2 : W_KDT) * g.plane)
-                      : (BORN ? reinterpret_cast<const K *>(a.kd2) : reinterpret_cast<const K *>(a.kdt));
-    const int pT = (int)g.plane;   // cells per plane: the stride of one (pair) field in units of T (in-slot offsets fit 32 bits)
-    const int oP = BORN ? B_P / 2 : G_P, oVX = BORN ? B_VX / 2 : G_VX, oVZ = BORN ? B_VZ / 2 : G_VZ;
-    const int oPPX = BORN ? B_PPX / 2 : G_PPX, oPPZ = BORN ? B_PPZ / 2 : G_PPZ;
+    using L = FwdLay<M, BORN, false>;
+    const GridDev &g = p.a.g;
+    const Maps2D &m = p.m;
+    constexpr int W = 2 * M;
+    const int q = slot * (BORN ? m.pps : m.fps);
+    const CUtensorMap(&ms)[2] = BORN ? m.pr : m.fl;
+    const CUtensorMap(&mm)[2] = WIN ? ms : (BORN ? m.mb : m.md);
     const int zr = z + W - 1, k = z + M - 1;
-    const int zrs = node_src_row<FS>(g, zr), ks = half_src_row<FS>(g, k);
-    const bool okr = colok && zrs >= 0 && zrs < g.Nz;
-    const int cr = okr ? zrs * pitch + xc : 0;
-    const bool okk1 = colok && k + 1 >= 0;
-    const int ck1 = okk1 ? min(k + 1, g.Nz - 1) * pitch + xc : 0;
-    const bool okk = colok && k >= 0 && k < g.Nz;
-    const int ck = okk ? k * pitch + xc : 0;
-    const bool okks = okk && ks < g.Nz;
-    const int cks = okks ? ks * pitch + xc : 0;
-    const bool pz = okk && ((k <= g.z0 - 2) || (k >= g.z0 + g.nz));
-    const bool main = z >= zc0 && z < zc1;
-    const bool okz = colok && main;
-    const int cz = okz ? z * pitch + xc : 0;
-    const bool okv = vxok && main;
-    const bool oko = outcol && main;
-    constexpr size_t F = (size_t)NTH * 8;   // bytes between field rows of a stage
-    cpa(reinterpret_cast<T *>(sl + 0 * F), fin + oP * pT + cr, okr);
-    cpa(reinterpret_cast<T *>(sl + 1 * F), fin + oVZ * pT + cks, okks);
-    cpa_if(reinterpret_cast<T *>(sl + 2 * F), fin + oPPZ * pT + ck, pz);
-    cpa(reinterpret_cast<T *>(sl + 3 * F), fin + oVX * pT + cz, okv);
-    cpa_if(reinterpret_cast<T *>(sl + 4 * F), fin + oPPX * pT + cz, okv && pmlxh);
-    cpa(reinterpret_cast<R *>(sl + 5 * F), br + ck1, okk1);
-    cpa(reinterpret_cast<R *>(sl + 6 * F), br + cz, okz);
-    cpa(reinterpret_cast<K *>(sl + 7 * F), kk + cz, oko);
-}
-
-template <bool BORN>
-__device__ __forceinline__ FwdRow<BORN> fwd_read(const char *st)
-{
-    using T = typename FwdT<BORN>::T;
-    using R = typename FwdT<BORN>::R;
-    using K = typename FwdT<BORN>::K;
-    const char *sl = st + threadIdx.x * 8;
-    constexpr size_t F = (size_t)NTH * 8;
-    FwdRow<BORN> r;
-    r.p = *reinterpret_cast<const T *>(sl + 0 * F);
-    r.vz = *reinterpret_cast<const T *>(sl + 1 * F);
-    r.psz = *reinterpret_cast<const T *>(sl + 2 * F);
-    r.vx = *reinterpret_cast<const T *>(sl + 3 * F);
-    r.psx = *reinterpret_cast<const T *>(sl + 4 * F);
-    r.br1 = *reinterpret_cast<const R *>(sl + 5 * F);
-    r.brz = *reinterpret_cast<const R *>(sl + 6 * F);
-    r.kd = *reinterpret_cast<const K *>(sl + 7 * F);
-    return r;
+    const bool main = z >= zc0;
+    const bool pz = zpml_half(g, k) || zpml_half(g, k + 1);
+    if (warp == 0) {
+        if (tma::elect_one()) {
+            const int f = q + (BORN ? B_P / 2 : G_P);
+            if (FS && zr < g.z0)
+                copy_rows<false>(st + L::P, L::FR, ms, xs, node_src_row<FS>(g, zr), node_src_row<FS>(g, zr + 1), f, b);
+            else
+                copy_rows<true>(st + L::P, L::FR, ms, xs, zr, zr + 1, f, b);
+        }
+    } else if (warp == 1) {
+        if (tma::elect_one()) {
+            const int f = q + (BORN ? B_VZ / 2 : G_VZ);
+            if (FS && k < g.z0)
+                copy_rows<false>(st + L::VZ, L::FR, ms, xs, k < 0 ? -1 : half_src_row<FS>(g, k),
+                                 k + 1 < 0 ? -1 : half_src_row<FS>(g, k + 1), f, b);
+            else
+                copy_rows<true>(st + L::VZ, L::FR, ms, xs, k, k + 1, f, b);
+        }
+    } else if (warp == 2) {
+        if (tma::elect_one()) tma::load3(brs, mm[1], xs, k + 1, WIN ? q + (BORN ? W_BR2 / 2 : W_BINV) : 1, b);
+    } else if (warp == 3) {
+        if (main && tma::elect_one()) tma::load3(st + L::VX, ms[1], xs, z, q + (BORN ? B_VX / 2 : G_VX), b);
+    } else if (warp == 4) {
+        if (main && tma::elect_one()) tma::load3(st + L::KD, mm[1], xs, z, WIN ? q + (BORN ? W_KD2 / 2 : W_KDT) : 0, b);
+    } else if (warp == 5) {
+        if (main && tph && tma::elect_one()) tma::load3(st + L::PX, ms[1], xs, z, q + (BORN ? B_PPX / 2 : G_PPX), b);
+    } else if (warp == 6) {
+        if (pz) {
+            if (tma::elect_one()) tma::load3(st + L::PZ, ms[1], xs, k, q + (BORN ? B_PPZ / 2 : G_PPZ), b);
+        } else if (main && tpn) {   // node CPML memories along x, in the unused place of psi_pz
+            if (tma::elect_one()) tma::load3(st + L::PZ, m.pv[BORN], xs, z, slot * (BORN ? m.pvs / 2 : m.pvs) + (BORN ? B_PVX / 2 : G_PVX), b);
+        }
+    } else {
+        if (tma::elect_one())
+            tma::mbar_expect(b, (3 + (pz ? 1 : 0) + (main ? 2 + (tph ? 1 : 0) + (!pz && tpn ? 1 : 0) : 0)) * L::F);
+    }
+    __syncwarp();
 }
 
 template <int M, bool BORN, bool BANDS, bool HESS, bool WIN, bool FS>
-__global__ void __launch_bounds__(NTH, (BORN || BANDS || HESS) ? kFwdMinBlocks : kFwdPlainMinBlocks) k_fwd2d(const Step2D a)
+__device__ __forceinline__ void fwd_body(const Arg2D &p)
 {
+    const Step2D &a = p.a;
     if (guard_tripped(a.g)) return;
     using C = Cols<M>;
-    using T = typename FwdT<BORN>::T;
-    using R = typename FwdT<BORN>::R;
-    constexpr int W = C::W, HXP = C::HXP, TXO = C::TXO;
-    __shared__ T sP[NTH];
-    __shared__ R sB[NTH];
-    __shared__ T sV[NTH];
-    __shared__ float sH[HESS ? NTH : 1];
-    extern __shared__ __align__(16) char stages[];   // [PDF][kFwdSlots][NTH] x 8 bytes
+    using L = FwdLay<M, BORN, HESS>;
+    using T = typename L::T;
+    constexpr int W = C::W, HXP = C::HXP, TXO = C::TXO, NB = L::NB;
+    extern __shared__ unsigned char smraw[];
+    char *sm = reinterpret_cast<char *>(smraw + ((128u - (tma::su32(smraw) & 127u)) & 127u));
+    T *const sP = reinterpret_cast<T *>(sm + L::SP);
+    T *const sV = reinterpret_cast<T *>(sm + L::SV);
+    float *const sH = reinterpret_cast<float *>(sm + L::SH);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(sm + L::BAR);
 
     const GridDev &g = a.g;
     const int t = threadIdx.x;
@@ -288,10 +293,10 @@ __global__ void __launch_bounds__(NTH, (BORN || BANDS || HESS) ? kFwdMinBlocks :
     const int Nx = WIN ? a.win_nx[shot] + 2 * g.x0 : g.Nx;
     const int nx = WIN ? Nx - 2 * g.x0 : g.nx;
     if (WIN && (int)blockIdx.x * TXO >= Nx) return;   // no output column in this shot's window
-    const int x = (int)blockIdx.x * TXO - HXP + t;
+    const int xs = (int)blockIdx.x * TXO - HXP;
+    const int x = xs + t;
     const bool colok = x >= 0 && x < Nx;
     const bool outcol = colok && t >= HXP && t < HXP + TXO;
-    const bool vxok = colok && t >= M - 1 && t <= NTH - 1 - M;
     const int zc0 = (int)blockIdx.y * a.tzc;
     const int zc1 = min(zc0 + a.tzc, g.Nz);
     const int zstart = zc0 - W;
@@ -306,20 +311,37 @@ __global__ void __launch_bounds__(NTH, (BORN || BANDS || HESS) ? kFwdMinBlocks :
     const int x0 = g.x0, x1 = g.x0 + nx, z0 = g.z0, z1 = g.z0 + g.nz;
     const int ix = x - x0;
     const bool pmlxh = colok && ((x <= x0 - 2) || (x >= x1));
-    const bool pmlxn = colok && ((x <= x0 - 1) || (x >= x1));
-    const int px = WIN ? shot * a.pml_xstride + x : x;   // x CPML profiles of this shot's window
+    const bool pmlxn = outcol && ((x <= x0 - 1) || (x >= x1));
+    const bool tph = (xs <= x0 - 2) || (xs + NTH - 1 >= x1);   // the CTA has half-node / node x CPML columns
+    const bool tpn = (xs <= x0 - 1) || (xs + NTH - 1 >= x1);
+    const int px = WIN ? shot * a.pml_xstride + x : x;         // x CPML profiles of this shot's window
     const float ahx = pmlxh ? a.pml.ah[2][px] : 0.f, bhx = pmlxh ? a.pml.bh[2][px] : 0.f;
     const float aix = pmlxn ? a.pml.ai[2][px] : 0.f, bix = pmlxn ? a.pml.bi[2][px] : 0.f;
+    // half nodes left of the array are zero; past its end 1/rho reads zero,
+    // and the last half node replicates the last node's
+    const float hbx = x >= 0 ? 0.5f : 0.f;
+    const bool lastx = x + 1 >= Nx;
     const long long bandoff = band_base(a.bands, shot, a.n);
     const int src = a.src_cell[shot];
     const float wsrc = a.src_scale * a.wav[(a.wav_per_shot ? (long long)shot * g.nt : 0) + a.n];
     constexpr int oP = BORN ? B_P / 2 : G_P, oVX = BORN ? B_VX / 2 : G_VX, oVZ = BORN ? B_VZ / 2 : G_VZ;
     constexpr int oPPX = BORN ? B_PPX / 2 : G_PPX, oPPZ = BORN ? B_PPZ / 2 : G_PPZ;
     constexpr int oPVX = BORN ? B_PVX / 2 : G_PVX, oPVZ = BORN ? B_PVZ / 2 : G_PVZ;
+    const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);   // (known to be uniform)
 
-    // z rings, shifted by U entries after every group of U rows (entry u + m
-    // holds row z + m of P, or the half-row value written m - W + 1 rows earlier)
-    constexpr int U = W / kFwdGroupDiv > 0 ? W / kFwdGroupDiv : 1, RL = W + U - 1;
+    if (t == 0) {
+        for (int i = 0; i < NS; ++i) tma::mbar_init(bar + i);
+        tma::mbar_init_fence();
+    }
+    __syncthreads();
+    for (int j = 0; j < NS && zstart + 2 * j < zc1; ++j)
+        fwd_issue<M, BORN, FS, WIN>(p, warp, sm + j * L::STAGE, sm + L::BR + j * L::F, bar + j, slot, xs, zstart + 2 * j,
+                                    zc0, tpn, tph);
+
+    // z rings, shifted by U entries after every U rows (entry u + m holds row
+    // z + m of P, or the half-row value written m - W + 1 rows earlier)
+    constexpr int U = 2, RL = W + U - 1;
+    static_assert(U % 2 == 0, "whole groups");
     T P[RL], VZ[RL];
     float HZ[HESS ? RL : 1];
 #pragma unroll
@@ -337,568 +359,400 @@ __global__ void __launch_bounds__(NTH, (BORN || BANDS || HESS) ? kFwdMinBlocks :
             P[j] = zrs != zr ? neg_(v) : v;
         }
     }
-    R br_old = zero_<R>();
+    T br_old = zero_<T>();
     {
-        const R *br = WIN ? reinterpret_cast<const R *>(in + (BORN ? W_BR2 : W_BINV) * plane)
-                          : (BORN ? reinterpret_cast<const R *>(a.br2) : reinterpret_cast<const R *>(a.binv));
-        int k = zstart + M - 1;
+        const T *br = WIN ? reinterpret_cast<const T *>(in + (BORN ? W_BR2 : W_BINV) * plane)
+                          : (BORN ? reinterpret_cast<const T *>(a.br2) : reinterpret_cast<const T *>(a.binv));
+        const int k = zstart + M - 1;
         if (colok && k >= 0 && k < g.Nz) br_old = br[k * pitch + xc];
     }
 
-#pragma unroll
-    for (int j = 0; j < PDF - 1; ++j) {
-        if (zstart + j < zc1)
-            fwd_issue<M, BORN, WIN, FS>(stages + j * kFwdStageSlotBytes, a, in, xc, zstart + j, zc0, zc1, colok, vxok,
-                               outcol, pmlxh);
-        cp_commit();
-    }
+    // Groups whose rows (with everything their stencils reach) are interior
+    // take a form without tests of the rows (ZF), and there warps whose columns
+    // are all interior one without any boundary test (XF): straight-line code
+    // for the two rows, so their shared memory and FMA latencies overlap.
+    const bool xf = !HESS && !BANDS && __all_sync(0xffffffffu, ix >= 0 && ix < nx);
 
+    bool bad = false;      // this thread's wait gave up
+    int fail_j = -1;       // group whose stage was not consumed
+    int j = 0, bs = 0;     // group, its 1/rho slot
     for (int zb = zstart; zb < zc1; zb += U) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
+        for (int u = 0; u < U; u += 2) {
             const int z = zb + u;
             if (z >= zc1) break;
-            const int zi = z + PDF - 1;
-            if (zi < zc1)
-                fwd_issue<M, BORN, WIN, FS>(stages + ((zi - zstart) % PDF) * kFwdStageSlotBytes, a, in, xc, zi, zc0, zc1,
-                                   colok, vxok, outcol, pmlxh);
-            cp_commit();
-            cp_wait_row<PDF>();
-            const FwdRow<BORN> cur = fwd_read<BORN>(stages + ((z - zstart) % PDF) * kFwdStageSlotBytes);
-            const int k = z + M - 1;   // half row of vz computed in this iteration
-            const int sl = u + W - 1;
-            P[sl] = (FS && z + W - 1 < g.z0) ? neg_(cur.p) : cur.p;   // ghost rows hold -p(mirror)
-            // ---- vz at half row k (column-local)
-            const float buz = 0.5f * (xof(br_old) + xof(cur.br1));
-            const float rsum = yof(br_old) + yof(cur.br1);
-            br_old = cur.br1;
-            T vzn = zero_<T>();
-            float hzq = 0.f;
-            if (colok && k >= 0 && k < g.Nz) {
-                const int ck = k * pitch;
-                const bool own = outcol && k >= zc0 && k < zc1;
-                T G = stencil<M, T>(g.cz, [&](int l) { return P[u + M - 1 + l]; },
-                                    [&](int l) { return P[u + M - l]; });
-                if ((k <= z0 - 2) || (k >= z1)) {
-                    T ps = fma_(a.pml.bh[0][k], cur.psz, mul_(a.pml.ah[0][k], G));
-                    if (own) out[oPPZ * pT + ck] = ps;
-                    G = add_(G, ps);
+            char *const st = sm + (j % NS) * L::STAGE;
+            bad |= !tma::mbar_wait(bar + j % NS, (unsigned)(j / NS) & 1u);
+            const char *const stt = st + t * sizeof(T);
+            const char *const brk = sm + L::BR + bs * L::F + t * sizeof(T);
+            bs = bs + 1 == NB ? 0 : bs + 1;   // (the next group's)
+            const char *const brx = sm + L::BR + (bs + NS - 1 >= NB ? bs + NS - 1 - NB : bs + NS - 1) * L::F;
+            const bool main = z >= zc0;
+            const bool zf = !HESS && !BANDS && main && z > z0 && z + W < z1 && z + 1 < zc1;
+            if (!zf && main && outcol) {
+                // the node CPML memories of this group, read in its last stage
+                const int zn = min(z + 1, zc1 - 1);
+                if (pmlxn) {
+                    prefetch_l1(psiv + oPVX * pT + z * pitch);
+                    prefetch_l1(psiv + oPVX * pT + zn * pitch);
                 }
-                const float dtbu = dt * buz;
-                vzn = fma_(-dtbu, G, cur.vz);
-                if constexpr (BORN) vzn.y = fmaf(0.5f * dt * rsum, G.x, vzn.y);
-                if (own) {
-                    out[oVZ * pT + ck] = vzn;
-                    if (BANDS) {
-                        int iz = k - z0;
-                        if (ix >= 0 && ix < nx && in_xstrip(iz, M, g.nz))
-                            band_put(a.bands, 1, slot, bandoff, band_zstrip(iz, ix, M, g.nz, nx), xof(vzn));
-                    }
-                }
-                if (HESS) {
-                    float q = buz * xof(G);
-                    hzq = q * q;
+                if (z <= z0 - 1 || zn >= z1) {
+                    prefetch_l1(psiv + oPVZ * pT + z * pitch);
+                    prefetch_l1(psiv + oPVZ * pT + zn * pitch);
                 }
             }
-            VZ[sl] = vzn;
-            if (HESS) HZ[sl] = hzq;
-            if (z < zc0) continue;   // warm-up rows of the z rings
+            // ---- vz at half rows k = z + M - 1, z + M (column-local)
+            auto vz_stage = [&](auto zc) {
+                constexpr bool ZF = decltype(zc)::value;
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const int k = z + r + M - 1, sl = u + r + W - 1;
+                    const T pc = *reinterpret_cast<const T *>(stt + L::P + r * L::FR);
+                    P[sl] = (!ZF && FS && z + r + W - 1 < z0) ? neg_(pc) : pc;   // ghost rows hold -p(mirror)
+                    T br1 = *reinterpret_cast<const T *>(brk + r * L::FR);
+                    if (!ZF && k + 1 >= g.Nz) br1 = br_old;   // the last half row replicates the last node row
+                    const float buz = 0.5f * (xof(br_old) + xof(br1));
+                    const float rsum = yof(br_old) + yof(br1);
+                    br_old = br1;
+                    T vzn = zero_<T>();
+                    float hzq = 0.f;
+                    if (ZF || (k >= 0 && k < g.Nz)) {
+                        const int ck = k * pitch;
+                        const bool own = outcol && (ZF || k >= zc0) && k < zc1;
+                        T G = stencil<M, T>(g.cz, [&](int l) { return P[u + r + M - 1 + l]; },
+                                            [&](int l) { return P[u + r + M - l]; });
+                        if (!ZF && ((k <= z0 - 2) || (k >= z1))) {
+                            const T psz = *reinterpret_cast<const T *>(stt + L::PZ + r * L::FR);
+                            const T ps = fma_(a.pml.bh[0][k], psz, mul_(a.pml.ah[0][k], G));
+                            if (own) out[oPPZ * pT + ck] = ps;
+                            G = add_(G, ps);
+                        }
+                        const float dtbu = dt * buz;
+                        vzn = fma_(-dtbu, G, *reinterpret_cast<const T *>(stt + L::VZ + r * L::FR));
+                        if constexpr (BORN) vzn.y = fmaf(0.5f * dt * rsum, G.x, vzn.y);
+                        if (own) out[oVZ * pT + ck] = vzn;
+                        if (BANDS && own) {
+                            const int iz = k - z0;
+                            if (ix >= 0 && ix < nx && in_xstrip(iz, M, g.nz))
+                                band_put(a.bands, 1, slot, bandoff, band_zstrip(iz, ix, M, g.nz, nx), xof(vzn));
+                        }
+                        if (HESS) {
+                            const float q = buz * xof(G);
+                            hzq = q * q;
+                        }
+                    }
+                    VZ[sl] = vzn;
+                    if (HESS) HZ[sl] = hzq;
+                }
+            };
+            if (main) {
+#pragma unroll
+                for (int r = 0; r < 2; ++r) sP[r * NTH + t] = P[u + r];
+            }
+            if (zf) vz_stage(std::true_type{});
+            else vz_stage(std::false_type{});
+            // every thread is past the previous group's reads: refill its stage
+            if (__syncthreads_or(bad)) {
+                fail_j = j;
+                break;
+            }
+            if (j >= 1 && z + 2 * (NS - 1) < zc1) {
+                const int jn = j + NS - 1;
+                fwd_issue<M, BORN, FS, WIN>(p, warp, sm + (jn % NS) * L::STAGE, sm + L::BR + (jn % NB) * L::F, bar + jn % NS,
+                                            slot, xs, z + 2 * (NS - 1), zc0, tpn, tph);
+            }
+            ++j;
+            if (!main) continue;   // warm-up groups fill the z rings
 
-            // ---- row z: vx on the output columns and the halo
-            const int cz = z * pitch;
-            const T p0 = P[u];
-            sP[t] = p0;
-            sB[t] = cur.brz;
-            __syncthreads();
-            T vxn = zero_<T>();
-            float hxq = 0.f;
-            if (vxok) {
-                T G = stencil<M, T>(g.cx, [&](int l) { return sP[t + l]; }, [&](int l) { return sP[t + 1 - l]; });
-                const bool last = x + 1 >= Nx;
-                const R bn = last ? cur.brz : sB[t + 1];
-                const float bux = 0.5f * (xof(cur.brz) + xof(bn));
-                if (pmlxh) {
-                    T ps = fma_(bhx, cur.psx, mul_(ahx, G));
-                    if (outcol) out[oPPX * pT + cz] = ps;
-                    G = add_(G, ps);
-                }
-                const float dtbu = dt * bux;
-                vxn = fma_(-dtbu, G, cur.vx);
-                if constexpr (BORN) {
-                    float rs = yof(cur.brz) + (last ? 0.f : yof(bn));
-                    vxn.y = fmaf(0.5f * dt * rs, G.x, vxn.y);
-                }
-                if (outcol) {
-                    out[oVX * pT + cz] = vxn;
-                    if (BANDS) {
-                        int iz = z - z0;
+            // ---- rows z, z + 1: vx on the output columns and the halo
+            auto vx_stage = [&](auto zc, auto xc_) {
+                constexpr bool ZF = decltype(zc)::value, XF = decltype(xc_)::value;
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const T *const pr = sP + r * NTH + t;
+                    T G = stencil<M, T>(g.cx, [&](int l) { return pr[l]; }, [&](int l) { return pr[1 - l]; });
+                    const T *const b = reinterpret_cast<const T *>(brx + r * L::FR) + t;
+                    const T b0 = b[0], b1 = !XF && lastx ? b0 : b[1];
+                    const float hb = XF ? 0.5f : hbx;
+                    const float bux = hb * (xof(b0) + xof(b1));
+                    const bool own = outcol && (ZF || z + r < zc1);
+                    if (!XF && pmlxh) {
+                        const T psx = *reinterpret_cast<const T *>(stt + L::PX + r * L::FR);
+                        const T ps = fma_(bhx, psx, mul_(ahx, G));
+                        if (own) out[oPPX * pT + (z + r) * pitch] = ps;
+                        G = add_(G, ps);
+                    }
+                    const float dtbu = dt * bux;
+                    T vxn = fma_(-dtbu, G, *reinterpret_cast<const T *>(stt + L::VX + r * L::FR));
+                    if constexpr (BORN) {
+                        const float rs = yof(b0) + (!XF && lastx ? 0.f : yof(b1));
+                        vxn.y = fmaf(hb * dt * rs, G.x, vxn.y);
+                    }
+                    sV[r * NTH + t] = vxn;
+                    if (own) out[oVX * pT + (z + r) * pitch] = vxn;
+                    if (BANDS && own) {
+                        const int iz = z + r - z0;
                         if (iz >= 0 && iz < g.nz && in_xstrip(ix, M, nx))
                             band_put(a.bands, 1, slot, bandoff, band_xstrip(iz, ix, M, g.nz, nx), xof(vxn));
                     }
-                }
-                if (HESS) {
-                    float q = bux * xof(G);
-                    hxq = q * q;
-                }
-            }
-            sV[t] = vxn;
-            if (HESS) sH[t] = hxq;
-            __syncthreads();
-
-            // ---- row z: pressure on the output columns
-            if (outcol) {
-                T qx = stencil<M, T>(g.cx, [&](int l) { return sV[t + l - 1]; }, [&](int l) { return sV[t - l]; });
-                T qz = stencil<M, T>(g.cz, [&](int l) { return VZ[u + M + l - 1]; },
-                                     [&](int l) { return VZ[u + M - l]; });
-                if (pmlxn) {
-                    T ps = fma_(bix, psiv[oPVX * pT + cz], mul_(aix, qx));
-                    psiv[oPVX * pT + cz] = ps;
-                    qx = add_(qx, ps);
-                }
-                if ((z <= z0 - 1) || (z >= z1)) {
-                    T ps = fma_(a.pml.bi[0][z], psiv[oPVZ * pT + cz], mul_(a.pml.ai[0][z], qz));
-                    psiv[oPVZ * pT + cz] = ps;
-                    qz = add_(qz, ps);
-                }
-                const T Q = add_(qx, qz);
-                const float kd = xof(cur.kd);
-                T pn = fma_(-kd, Q, p0);
-                if constexpr (BORN) {
-                    pn.y = fmaf(-cur.kd.y, Q.x, pn.y);
-                    if (cz + x == src) pn.x += wsrc;
-                } else {
-                    if (cz + x == src) pn += wsrc;
-                }
-                if (FS && z <= z0) pn = zero_<T>();   // p = 0 on the free surface (ghost rows unused)
-                out[oP * pT + cz] = pn;
-                if (BANDS) {
-                    long long b = pband_index(z - z0, ix, M, g.nz, nx);
-                    if (b >= 0) band_put(a.bands, 0, slot, bandoff, b, xof(p0));
-                }
-                if (HESS) {
-                    int iz = z - z0;
-                    if (iz >= 0 && iz < g.nz && ix >= 0 && ix < nx) {
-                        float bx0 = xof(cur.brz);
-                        float hr = 0.5f * ((sH[t] + sH[t - 1]) + (HZ[u + M] + HZ[u + M - 1])) / (bx0 * bx0);
-                        float kq = kd * xof(Q) / dt;
-                        (a.hess + slot * plane)[cz + xc] += dt * (hr + kq * kq);
+                    if (HESS) {
+                        const float q = bux * xof(G);
+                        sH[r * NTH + t] = q * q;
                     }
                 }
-            }
-        }
+            };
+            if (!zf) vx_stage(std::false_type{}, std::false_type{});
+            else if (xf) vx_stage(std::true_type{}, std::true_type{});
+            else vx_stage(std::true_type{}, std::false_type{});
+            __syncthreads();
+
+            // ---- rows z, z + 1: pressure on the output columns
+            auto p_stage = [&](auto zc, auto xc_) {
+                constexpr bool ZF = decltype(zc)::value, XF = decltype(xc_)::value;
 #pragma unroll
-        for (int j = 0; j < W - 1; ++j) {
-            P[j] = P[j + U];
-            VZ[j] = VZ[j + U];
-            if (HESS) HZ[j] = HZ[j + U];
+                for (int r = 0; r < 2; ++r) {
+                    const int zr = z + r, cz = zr * pitch;
+                    const T *const vr = sV + r * NTH + t;
+                    T qx = stencil<M, T>(g.cx, [&](int l) { return vr[l - 1]; }, [&](int l) { return vr[-l]; });
+                    T qz = stencil<M, T>(g.cz, [&](int l) { return VZ[u + r + M + l - 1]; },
+                                         [&](int l) { return VZ[u + r + M - l]; });
+                    const bool own = outcol && (ZF || zr < zc1);
+                    if (!XF && own && pmlxn) {
+                        const T pv = ZF ? *reinterpret_cast<const T *>(stt + L::PZ + r * L::FR) : psiv[oPVX * pT + cz];
+                        const T ps = fma_(bix, pv, mul_(aix, qx));
+                        psiv[oPVX * pT + cz] = ps;
+                        qx = add_(qx, ps);
+                    }
+                    if (!ZF && own && ((zr <= z0 - 1) || (zr >= z1))) {
+                        const T ps = fma_(a.pml.bi[0][zr], psiv[oPVZ * pT + cz], mul_(a.pml.ai[0][zr], qz));
+                        psiv[oPVZ * pT + cz] = ps;
+                        qz = add_(qz, ps);
+                    }
+                    const T Q = add_(qx, qz);
+                    const T kd2 = *reinterpret_cast<const T *>(stt + L::KD + r * L::FR);
+                    const float kd = xof(kd2);
+                    const T p0 = P[u + r];
+                    T pn = fma_(-kd, Q, p0);
+                    const float sw = cz + x == src ? wsrc : 0.f;
+                    if constexpr (BORN) {
+                        pn.y = fmaf(-kd2.y, Q.x, pn.y);
+                        pn.x += sw;
+                    } else {
+                        pn += sw;
+                    }
+                    if (!ZF && FS && zr <= z0) pn = zero_<T>();   // p = 0 on the free surface (ghost rows unused)
+                    if (own) out[oP * pT + cz] = pn;
+                    if (BANDS && own) {
+                        const long long b = pband_index(zr - z0, ix, M, g.nz, nx);
+                        if (b >= 0) band_put(a.bands, 0, slot, bandoff, b, xof(p0));
+                    }
+                    if (HESS && own) {
+                        const int iz = zr - z0;
+                        if (iz >= 0 && iz < g.nz && ix >= 0 && ix < nx) {
+                            const float bx0 = xof(reinterpret_cast<const T *>(brx + r * L::FR)[t]);
+                            const float *const h = sH + r * NTH + t;
+                            const float hr = 0.5f * ((h[0] + h[-1]) + (HZ[u + r + M] + HZ[u + r + M - 1])) / (bx0 * bx0);
+                            const float kq = kd * xof(Q) / dt;
+                            (a.hess + slot * plane)[cz + xc] += dt * (hr + kq * kq);
+                        }
+                    }
+                }
+            };
+            if (!zf) p_stage(std::false_type{}, std::false_type{});
+            else if (xf) p_stage(std::true_type{}, std::true_type{});
+            else p_stage(std::true_type{}, std::false_type{});
         }
+        if (fail_j >= 0) break;
+#pragma unroll
+        for (int i = 0; i < W - 1; ++i) {
+            P[i] = P[i + U];
+            VZ[i] = VZ[i + U];
+            if (HESS) HZ[i] = HZ[i + U];
+        }
+    }
+
+    if (fail_j >= 0) {
+        // a wait gave up: record it, let the copies in flight land, return
+        if (t == NTH - 1) {
+            atomicOr(a.err, 1);
+            for (int jj = fail_j; jj <= max(NS - 1, fail_j + NS - 2) && zstart + 2 * jj < zc1; ++jj)
+                (void)tma::mbar_wait(bar + jj % NS, (unsigned)(jj / NS) & 1u);
+        }
+        return;
     }
 
     if (BORN || a.rec_bg) {
         // record dp^{n+1} (Born) or the background p^{n+1} (nonlinear
         // modelling) at the receivers of this CTA
         __syncthreads();
-        int tile = shot * a.trec.ntiles + blockIdx.y * gridDim.x + blockIdx.x;
-        int b = a.trec.ptr[tile], e = a.trec.ptr[tile + 1];
-        if constexpr (BORN) {
-            const float2 *po = reinterpret_cast<const float2 *>(a.out + slot * a.sstride + B_P * plane);
-            for (int i = b + t; i < e; i += NTH) {
-                int2 rc = a.trec.rec[i];
-                a.dstage[(long long)rc.y * g.nt + a.n] = a.rec_bg ? po[rc.x].x : po[rc.x].y;
-            }
-        } else {
-            const float *po = a.out + slot * a.sstride + G_P * plane;
-            for (int i = b + t; i < e; i += NTH) {
-                int2 rc = a.trec.rec[i];
-                a.dstage[(long long)rc.y * g.nt + a.n] = po[rc.x];
-            }
+        const int tile = shot * a.trec.ntiles + blockIdx.y * gridDim.x + blockIdx.x;
+        const int b = a.trec.ptr[tile], e = a.trec.ptr[tile + 1];
+        const T *po = reinterpret_cast<const T *>(a.out + slot * a.sstride) + oP * plane;
+        for (int i = b + t; i < e; i += NTH) {
+            const int2 rc = a.trec.rec[i];
+            const T v = po[rc.x];
+            a.dstage[(long long)rc.y * g.nt + a.n] = BORN && !a.rec_bg ? yof(v) : xof(v);
         }
     }
 }
 
-// ---------------------------------------------------------------------------
-// Born step with TMA row staging (shots without aperture windows): k_fwd2d's
-// Born arithmetic in the same order, with the rows ahead staged as in
-// k_adj2t (one thread issues each field row of a stage as one tile copy on
-// the stage's mbarrier; zero fill outside the grid; unused fields not copied;
-// a stage is refilled only after a barrier that follows every read of it).
-// ---------------------------------------------------------------------------
-struct Fwd2T {
-    Step2D a;
-    Maps2D m;
-};
-
-constexpr unsigned kFwdStageBytesT = (unsigned)kFwdStageSlotBytes;
-static_assert(kFwdStageBytesT % 128 == 0, "stage rows stay 128-byte aligned");
-constexpr unsigned kFwdBarOff = PDF * kFwdStageBytesT;
-constexpr unsigned kFwdSmemT = kFwdBarOff + 64 + 128;   // stages, barriers, alignment slack
-
-// Issues the copies of row z (the stage layout of fwd_issue) on barrier b;
-// tph: the CTA has half-node CPML columns.
+// The Born step of shots spanning the model, of shots with aperture windows,
+// and the background steps.
 template <int M, bool FS>
-__device__ __forceinline__ void fwd_issue_tma(const Fwd2T &p, char *st, uint64_t *b, int slot, int xs, int z,
-                                              int zc0, int zc1, bool tph)
+__global__ void __launch_bounds__(NTH, kBornMinBlocks) k_fwd2t(const __grid_constant__ Arg2D p)
 {
-    const GridDev &g = p.a.g;
-    const Maps2D &m = p.m;
-    constexpr int W = 2 * M;
-    constexpr unsigned F = NTH * 8;   // bytes of one field row
-    const int zr = z + W - 1, k = z + M - 1;
-    const int qp = slot * m.pps;
-    const bool ink = k >= 0 && k < g.Nz;
-    int rp = zr, rvz = ink ? k : -1;
-    if constexpr (FS) {
-        const int zrs = node_src_row<FS>(g, zr), ks = half_src_row<FS>(g, k);
-        rp = (zrs >= 0 && zrs < g.Nz) ? zrs : -1;
-        rvz = (ink && ks < g.Nz) ? ks : -1;
-    }
-    const int rb1 = k + 1 >= 0 ? min(k + 1, g.Nz - 1) : -1;
-    const bool pz = ink && ((k <= g.z0 - 2) || (k >= g.z0 + g.nz));
-    const bool main = z >= zc0 && z < zc1;
-    const bool px = main && tph;
-    const unsigned bytes = (3 + (pz ? 1 : 0) + (main ? 3 : 0) + (px ? 1 : 0)) * F;
-    tma::fence_proxy_async();
-    tma::mbar_expect(b, bytes);
-    tma::load3(st + 0 * F, m.pr, xs, rp, qp + B_P / 2, b);
-    tma::load3(st + 1 * F, m.pr, xs, rvz, qp + B_VZ / 2, b);
-    if (pz) tma::load3(st + 2 * F, m.pr, xs, k, qp + B_PPZ / 2, b);
-    tma::load3(st + 5 * F, m.mb, xs, rb1, 1, b);
-    if (main) {
-        tma::load3(st + 3 * F, m.pr, xs, z, qp + B_VX / 2, b);
-        tma::load3(st + 6 * F, m.mb, xs, z, 1, b);
-        tma::load3(st + 7 * F, m.mb, xs, z, 0, b);
-    }
-    if (px) tma::load3(st + 4 * F, m.pr, xs, z, qp + B_PPX / 2, b);
+    fwd_body<M, true, false, false, false, FS>(p);
 }
-
 template <int M, bool FS>
-__global__ void __launch_bounds__(NTH, kFwdTMinBlocks) k_fwd2t(const __grid_constant__ Fwd2T p)
+__global__ void __launch_bounds__(NTH, kBornMinBlocks) k_fwd2w(const __grid_constant__ Arg2D p)
 {
-    const Step2D &a = p.a;
-    if (guard_tripped(a.g)) return;
-    using C = Cols<M>;
-    using T = float2;
-    using R = float2;
-    constexpr int W = C::W, HXP = C::HXP, TXO = C::TXO;
-    static_assert(TXO % 2 == 0 && HXP % 2 == 0, "CTA column starts must be 16-byte aligned for 8-byte elements");
-    __shared__ T sP[NTH];
-    __shared__ R sB[NTH];
-    __shared__ T sV[NTH];
-    extern __shared__ unsigned char smraw[];
-    unsigned char *sm = smraw + ((128u - (tma::su32(smraw) & 127u)) & 127u);
-    char *stages = reinterpret_cast<char *>(sm);   // [PDF][kFwdSlots][NTH] x 8 bytes
-    uint64_t *bar = reinterpret_cast<uint64_t *>(sm + kFwdBarOff);
-
-    const GridDev &g = a.g;
-    const int t = threadIdx.x;
-    const int slot = blockIdx.z, shot = a.shot0 + slot;
-    const int Nx = g.Nx, nx = g.nx;
-    const int xs = (int)blockIdx.x * TXO - HXP;
-    const int x = xs + t;
-    const bool colok = x >= 0 && x < Nx;
-    const bool outcol = colok && t >= HXP && t < HXP + TXO;
-    const bool vxok = colok && t >= M - 1 && t <= NTH - 1 - M;
-    const int zc0 = (int)blockIdx.y * a.tzc;
-    const int zc1 = min(zc0 + a.tzc, g.Nz);
-    const int zstart = zc0 - W;
-    const long long plane = g.plane;
-    const int pT = (int)plane;   // in-slot offsets fit 32 bits (checked by the host)
-    const int pitch = g.pitch;
-    const int xc = colok ? x : 0;
-    const float *in = a.in + slot * a.sstride;
-    T *out = reinterpret_cast<T *>(a.out + slot * a.sstride) + xc;
-    T *psiv = reinterpret_cast<T *>(a.psiv + slot * a.vstride) + xc;
-    const float dt = g.dt;
-    const int x0 = g.x0, x1 = g.x0 + nx, z0 = g.z0, z1 = g.z0 + g.nz;
-    const bool pmlxh = colok && ((x <= x0 - 2) || (x >= x1));
-    const bool pmlxn = colok && ((x <= x0 - 1) || (x >= x1));
-    const bool tph = (xs <= x0 - 2) || (xs + NTH - 1 >= x1);   // CTA has half-node CPML columns
-    const float ahx = pmlxh ? a.pml.ah[2][x] : 0.f, bhx = pmlxh ? a.pml.bh[2][x] : 0.f;
-    const float aix = pmlxn ? a.pml.ai[2][x] : 0.f, bix = pmlxn ? a.pml.bi[2][x] : 0.f;
-    const int src = a.src_cell[shot];
-    const float wsrc = a.src_scale * a.wav[(a.wav_per_shot ? (long long)shot * g.nt : 0) + a.n];
-    constexpr int oP = B_P / 2, oVX = B_VX / 2, oVZ = B_VZ / 2, oPPX = B_PPX / 2, oPPZ = B_PPZ / 2;
-    constexpr int oPVX = B_PVX / 2, oPVZ = B_PVZ / 2;
-    constexpr int PR = NTH - 1;   // the thread that issues the copies
-
-    if (t == 0) {
-        for (int i = 0; i < PDF; ++i) tma::mbar_init(bar + i);
-        tma::mbar_init_fence();
-    }
-    __syncthreads();
-    if (t == PR) {
-        for (int j = 0; j < PDF - 1 && zstart + j < zc1; ++j)
-            fwd_issue_tma<M, FS>(p, stages + j * kFwdStageBytesT, bar + j, slot, xs, zstart + j, zc0, zc1, tph);
-    }
-
-    constexpr int U = W / kFwdGroupDiv > 0 ? W / kFwdGroupDiv : 1, RL = W + U - 1;
-    T P[RL], VZ[RL];
-#pragma unroll
-    for (int j = 0; j < RL; ++j) {
-        P[j] = zero_<T>();
-        VZ[j] = zero_<T>();
-    }
-    {
-        const T *pin = reinterpret_cast<const T *>(in) + oP * pT + xc;
-#pragma unroll
-        for (int j = 0; j < W - 1; ++j) {
-            const int zr = zstart + j, zrs = node_src_row<FS>(g, zr);
-            const T v = (colok && zrs >= 0 && zrs < g.Nz) ? pin[zrs * pitch] : zero_<T>();
-            P[j] = zrs != zr ? neg_(v) : v;
-        }
-    }
-    R br_old = zero_<R>();
-    {
-        int k = zstart + M - 1;
-        if (colok && k >= 0 && k < g.Nz) br_old = a.br2[k * pitch + xc];
-    }
-
-    bool bad = false;      // this thread's wait gave up
-    int fail_row = zc1;    // first row whose stage was not consumed
-    for (int zb = zstart; zb < zc1; zb += U) {
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int z = zb + u;
-            if (z >= zc1) break;
-            const int j = z - zstart;
-            // refill the stage of row z - 1 with row z + PDF - 1: every thread
-            // passed a barrier after reading it (the previous row's)
-            const int zi = z + PDF - 1;
-            if (t == PR && zi < zc1)
-                fwd_issue_tma<M, FS>(p, stages + ((j + PDF - 1) % PDF) * kFwdStageBytesT, bar + (j + PDF - 1) % PDF,
-                                     slot, xs, zi, zc0, zc1, tph);
-            bad |= !tma::mbar_wait(bar + j % PDF, (unsigned)(j / PDF) & 1u);
-            const FwdRow<true> cur = fwd_read<true>(stages + (j % PDF) * kFwdStageBytesT);
-            const int k = z + M - 1;   // half row of vz computed in this iteration
-            const int sl = u + W - 1;
-            P[sl] = (FS && z + W - 1 < g.z0) ? neg_(cur.p) : cur.p;   // ghost rows hold -p(mirror)
-            // ---- vz at half row k (column-local)
-            const float buz = 0.5f * (xof(br_old) + xof(cur.br1));
-            const float rsum = yof(br_old) + yof(cur.br1);
-            br_old = cur.br1;
-            T vzn = zero_<T>();
-            if (colok && k >= 0 && k < g.Nz) {
-                const int ck = k * pitch;
-                const bool own = outcol && k >= zc0 && k < zc1;
-                T G = stencil<M, T>(g.cz, [&](int l) { return P[u + M - 1 + l]; },
-                                    [&](int l) { return P[u + M - l]; });
-                if ((k <= z0 - 2) || (k >= z1)) {
-                    T ps = fma_(a.pml.bh[0][k], cur.psz, mul_(a.pml.ah[0][k], G));
-                    if (own) out[oPPZ * pT + ck] = ps;
-                    G = add_(G, ps);
-                }
-                const float dtbu = dt * buz;
-                vzn = fma_(-dtbu, G, cur.vz);
-                vzn.y = fmaf(0.5f * dt * rsum, G.x, vzn.y);
-                if (own) out[oVZ * pT + ck] = vzn;
-            }
-            VZ[sl] = vzn;
-            if (z < zc0) {
-                // warm-up row: the barrier that lets its stage be refilled
-                if (__syncthreads_or(bad)) {
-                    fail_row = z;
-                    break;
-                }
-                continue;
-            }
-
-            // ---- row z: vx on the output columns and the halo
-            const int cz = z * pitch;
-            const T p0 = P[u];
-            sP[t] = p0;
-            sB[t] = cur.brz;
-            if (__syncthreads_or(bad)) {
-                fail_row = z;
-                break;
-            }
-            T vxn = zero_<T>();
-            if (vxok) {
-                T G = stencil<M, T>(g.cx, [&](int l) { return sP[t + l]; }, [&](int l) { return sP[t + 1 - l]; });
-                const bool last = x + 1 >= Nx;
-                const R bn = last ? cur.brz : sB[t + 1];
-                const float bux = 0.5f * (xof(cur.brz) + xof(bn));
-                if (pmlxh) {
-                    T ps = fma_(bhx, cur.psx, mul_(ahx, G));
-                    if (outcol) out[oPPX * pT + cz] = ps;
-                    G = add_(G, ps);
-                }
-                const float dtbu = dt * bux;
-                vxn = fma_(-dtbu, G, cur.vx);
-                float rs = yof(cur.brz) + (last ? 0.f : yof(bn));
-                vxn.y = fmaf(0.5f * dt * rs, G.x, vxn.y);
-                if (outcol) out[oVX * pT + cz] = vxn;
-            }
-            sV[t] = vxn;
-            __syncthreads();
-
-            // ---- row z: pressure on the output columns
-            if (outcol) {
-                T qx = stencil<M, T>(g.cx, [&](int l) { return sV[t + l - 1]; }, [&](int l) { return sV[t - l]; });
-                T qz = stencil<M, T>(g.cz, [&](int l) { return VZ[u + M + l - 1]; },
-                                     [&](int l) { return VZ[u + M - l]; });
-                if (pmlxn) {
-                    T ps = fma_(bix, psiv[oPVX * pT + cz], mul_(aix, qx));
-                    psiv[oPVX * pT + cz] = ps;
-                    qx = add_(qx, ps);
-                }
-                if ((z <= z0 - 1) || (z >= z1)) {
-                    T ps = fma_(a.pml.bi[0][z], psiv[oPVZ * pT + cz], mul_(a.pml.ai[0][z], qz));
-                    psiv[oPVZ * pT + cz] = ps;
-                    qz = add_(qz, ps);
-                }
-                const T Q = add_(qx, qz);
-                const float kd = xof(cur.kd);
-                T pn = fma_(-kd, Q, p0);
-                pn.y = fmaf(-cur.kd.y, Q.x, pn.y);
-                if (cz + x == src) pn.x += wsrc;
-                if (FS && z <= z0) pn = zero_<T>();   // p = 0 on the free surface (ghost rows unused)
-                out[oP * pT + cz] = pn;
-            }
-        }
-        if (fail_row < zc1) break;
-#pragma unroll
-        for (int j = 0; j < W - 1; ++j) {
-            P[j] = P[j + U];
-            VZ[j] = VZ[j + U];
-        }
-    }
-
-    if (fail_row < zc1) {
-        // a wait gave up: record it, let the copies in flight land (rows up to
-        // fail_row + PDF - 1 were issued), return
-        if (t == PR) {
-            atomicOr(a.err, 1);
-            for (int zz = fail_row; zz <= min(fail_row + PDF - 1, zc1 - 1); ++zz) {
-                const int jj = zz - zstart;
-                (void)tma::mbar_wait(bar + jj % PDF, (unsigned)(jj / PDF) & 1u);
-            }
-        }
-        return;
-    }
-
-    // record dp^{n+1} (or the background p^{n+1} in nonlinear modelling) at
-    // the receivers of this CTA
-    __syncthreads();
-    int tile = shot * a.trec.ntiles + blockIdx.y * gridDim.x + blockIdx.x;
-    int b = a.trec.ptr[tile], e = a.trec.ptr[tile + 1];
-    const float2 *po = reinterpret_cast<const float2 *>(a.out + slot * a.sstride + B_P * plane);
-    for (int i = b + t; i < e; i += NTH) {
-        int2 rc = a.trec.rec[i];
-        a.dstage[(long long)rc.y * g.nt + a.n] = a.rec_bg ? po[rc.x].x : po[rc.x].y;
-    }
+    fwd_body<M, true, false, false, true, FS>(p);
+}
+template <int M, bool BANDS, bool HESS, bool WIN, bool FS>
+__global__ void __launch_bounds__(NTH, (BANDS || HESS) ? kBandsMinBlocks : kPlainMinBlocks) k_fwd2d(const __grid_constant__ Arg2D p)
+{
+    fwd_body<M, false, BANDS, HESS, WIN, FS>(p);
 }
 
 // ---------------------------------------------------------------------------
 // Reverse step n (n = nt-1 .. 0) of L^T. Input state: (background p^n,
-// lambda_p) with the residual of step n already added, (v^{n+1/2}, lambda_v)
-// and the lambda CPML memories. The step applies the transposed Born
-// sub-steps (S4^T, S3^T on the half nodes from lambda_p; S2^T, S1^T on the
-// nodes from lambda_v), accumulates the two zero-lag images (discrete
-// transposed forms of Eqs. gradkappa, gradrho), rebuilds p^{n-1}, v^{n-1/2}
-// in the interior from the saved boundary bands, and pre-adds the residual of
-// step n-1. The D+ stencils of (p^n, u) and the D- stencils of (v^{n+1/2}, w)
-// run as packed pairs.
+// mu = dt kappa lambda_p) with the residual of step n already added,
+// (v^{n+1/2}, lambda_v) and the lambda CPML memories. The step applies the
+// transposed Born sub-steps (S4^T, S3^T on the half nodes from mu; S2^T, S1^T
+// on the nodes from lambda_v), accumulates the two zero-lag images (discrete
+// transposed forms of Eqs. gradkappa, gradrho; the kappa image as sum Q mu),
+// rebuilds p^{n-1}, v^{n-1/2} in the interior from the saved boundary bands,
+// and pre-adds the residual of step n-1. The D+ stencils of (p^n, u) and the
+// D- stencils of (v^{n+1/2}, w) run as packed pairs.
+//
+// The adjoint pressure is carried as mu, the quantity the D+ stencils take:
+// away from the CPML strips the z ring's entry of a row then is the row's own
+// (p, mu), so a row needs neither dt kappa of its look-ahead row nor a second
+// copy of (p, lambda_p). Only the rows outside the interior (CPML rows, whose
+// ring entries hold u != mu, and ghost rows) read their own (p, mu) again, in
+// the stage rows that interior rows use for the image.
+//
+// What bounds it: 72 B a cell (70.9 from DRAM), held back like the Born step;
+// 3 tile copies a row where a row at a time took 9. The x strips' band values
+// come one group ahead by asynchronous copies (read where they are used, they
+// doubled the strip warps' time). 96 shots of 424 x 1192, order 8, FP16 bands:
+// 54.1 G cell-updates/s = 0.58 of the measured copy rate (a row at a time with
+// one issuing thread: 42.4; in groups without the straight-line form: 31.5).
 // ---------------------------------------------------------------------------
-struct AdjRow {
-    float2 pl;      // node row r = z + 2M - 1: (p^n, lambda_p)
-    float2 v2z;     // half row k: (vz^{n+1/2}, lambda_vz)
-    float2 plz;     // row z: (p^n, lambda_p)
-    float2 v2x;     // row z: (vx^{n+1/2}, lambda_vx)
-    float2 img;     // row z: image accumulators
-    float kdr, lpvzr, bz, lppz, kdz, lpsvx, lpsvz, bx, lppx;
+struct AdjLay {
+    static constexpr unsigned F2R = NTH * 8, F1R = NTH * 4, F2 = 2 * F2R, F1 = 2 * F1R;   // a row, a group's two rows
+    // stage: (p, mu) rows z + 2M - 1; v_z half rows z + M - 1; v_x rows z; image (interior rows) or (p, mu) rows z
+    static constexpr unsigned PL = 0, VZ = F2, VX = 2 * F2, IM = 3 * F2;
+    // dt kappa rows z; lambda CPML memories psi_vx and psi_px rows z (CTAs with x strips), psi_vz rows z + 2M - 1 and
+    // z, psi_pz half rows z + M - 1 (groups with z strip rows)
+    static constexpr unsigned KD = 4 * F2, LVX = KD + F1, LPX = LVX + F1, LVZR = LPX + F1, LVZ = LVZR + F1,
+                              LPZ = LVZ + F1, STAGE = LPZ + F1;
+    static constexpr unsigned B = NS * STAGE;   // 1/rho ring (FwdLay::BR)
+};
+template <int M>
+struct AdjLayM : AdjLay {
+    static constexpr int NB = M / 2 + NS;
+    static constexpr unsigned SPU = B + NB * F1;   // [2][NTH] (p^n, mu - ai_x (lpsi_vx - mu))
+    static constexpr unsigned SVW = SPU + F2;      // [2][NTH] (vx^{n+1/2}, dt*bu_x*lvx - ah_x*lpsi_px)
+    static constexpr unsigned SVN = SVW + F2;      // [2][NTH] vx^{n-1/2}
+    static constexpr unsigned SPI = SVN + F1;      // [2][8] Gx lvx of the last lane of each warp
+    static constexpr unsigned SB = SPI + 64;       // [2 groups][p, v][2 rows][2 sides][M] band values of the x strips (16-bit: in the first half)
+    static constexpr unsigned BAR = SB + 2 * 2 * 2 * 2 * M * 4 + 8;
+    static constexpr unsigned SMEM = BAR + 64 + 128;
+    static_assert(STAGE % 128 == 0, "copy destinations stay 128-byte aligned");
+    // three CTAs per SM: 228 KB, 1 KB reserved per CTA
+    static_assert(3 * (SMEM + 1024) <= 233472, "migration kernel must fit three CTAs per SM");
 };
 
-template <int M, bool WIN, bool FS>
-__device__ __forceinline__ void adj_issue(float *st, const Step2D &a, const float2 *img, const float *in,
-                                          int xc, int z, int zc0, int zc1, bool colok, bool vxok,
-                                          bool outcol, bool pmlxh, bool pmlxn, bool inner_col)
+// Issues the copies of the group of rows z, z + 1 on barrier b (as fwd_issue).
+template <int M, bool FS, bool WIN>
+__device__ __forceinline__ void adj_issue(const Arg2D &p, int warp, char *st, char *bs, uint64_t *b, int slot, int xs, int z,
+                                          int zc0, bool tpn, bool tph)
 {
-    const GridDev &g = a.g;
-    const long long plane = g.plane;
-    const long long p2 = plane;   // cells per plane: the stride of one pair field in float2 units
-    const int pitch = g.pitch;
-    const int W = 2 * M;
-    const int z0 = g.z0, z1 = g.z0 + g.nz;
-    const int t = threadIdx.x;
-    float2 *s2 = reinterpret_cast<float2 *>(st) + t;
-    float *s1 = st + 2 * kAdjF2 * NTH + t;
-    const float2 *in2 = reinterpret_cast<const float2 *>(in);
+    using L = AdjLay;
+    const GridDev &g = p.a.g;
+    const Maps2D &m = p.m;
+    constexpr int W = 2 * M;
     const int zr = z + W - 1, k = z + M - 1;
-    const bool okr = colok && zr >= 0 && zr < g.Nz;
-    const long long cr = okr ? (long long)zr * pitch + xc : 0;
-    const bool okk = colok && k >= 0 && k < g.Nz;
-    const long long ck = okk ? (long long)k * pitch + xc : 0;
-    // free surface: the pressure pair of a ghost row and v_z of a ghost half
-    // row come from their mirror rows
-    bool okrs = okr, okks = okk;
-    long long crs = cr, cks = ck;
-    if constexpr (FS) {
-        const int zrs = node_src_row<FS>(g, zr), ks = half_src_row<FS>(g, k);
-        okrs = colok && zrs >= 0 && zrs < g.Nz;
-        crs = okrs ? (long long)zrs * pitch + xc : 0;
-        okks = okk && ks < g.Nz;
-        cks = okks ? (long long)ks * pitch + xc : 0;
+    const int qp = slot * m.pps, qf = slot * m.fps;
+    const CUtensorMap(&mm)[2] = WIN ? m.fl : m.md;
+    const bool main = z >= zc0;
+    const bool lvr = zpml_node(g, zr) || zpml_node(g, zr + 1), lpz = zpml_half(g, k) || zpml_half(g, k + 1);
+    const bool lvz = main && (zpml_node(g, z) || zpml_node(g, z + 1));
+    if (warp == 0) {
+        if (tma::elect_one()) {
+            if (FS && zr < g.z0)
+                copy_rows<false>(st + L::PL, L::F2R, m.pr, xs, node_src_row<FS>(g, zr), node_src_row<FS>(g, zr + 1),
+                                 qp + A_PL / 2, b);
+            else
+                copy_rows<true>(st + L::PL, L::F2R, m.pr, xs, zr, zr + 1, qp + A_PL / 2, b);
+        }
+    } else if (warp == 1) {
+        if (tma::elect_one()) {
+            if (FS && k < g.z0)
+                copy_rows<false>(st + L::VZ, L::F2R, m.pr, xs, k < 0 ? -1 : half_src_row<FS>(g, k),
+                                 k + 1 < 0 ? -1 : half_src_row<FS>(g, k + 1), qp + A_VZ / 2, b);
+            else
+                copy_rows<true>(st + L::VZ, L::F2R, m.pr, xs, k, k + 1, qp + A_VZ / 2, b);
+        }
+    } else if (warp == 2) {
+        if (main && tma::elect_one()) tma::load3(st + L::VX, m.pr[1], xs, z, qp + A_VX / 2, b);
+    } else if (warp == 3) {
+        // the image of interior rows, (p, mu) of others
+        const bool in0 = z >= g.z0 && z < g.z0 + g.nz, in1 = z + 1 >= g.z0 && z + 1 < g.z0 + g.nz;
+        if (main && tma::elect_one()) {
+            if (in0 && in1) {
+                tma::load3(st + L::IM, m.im[1], xs, z, slot, b);
+            } else if (!in0 && !in1) {
+                tma::load3(st + L::IM, m.pr[1], xs, z, qp + A_PL / 2, b);
+            } else {
+                tma::load3(st + L::IM, in0 ? m.im[0] : m.pr[0], xs, z, in0 ? slot : qp + A_PL / 2, b);
+                tma::load3(st + L::IM + L::F2R, in1 ? m.im[0] : m.pr[0], xs, z + 1, in1 ? slot : qp + A_PL / 2, b);
+            }
+        }
+    } else if (warp == 4) {
+        if (tma::elect_one()) {
+            tma::load3(bs, mm[1], xs, k + 1, WIN ? qf + W_BINV : 1, b);
+            if (main) tma::load3(st + L::KD, mm[1], xs, z, WIN ? qf + W_KDT : 0, b);
+        }
+    } else if (warp == 5) {
+        if ((lvr || lpz) && tma::elect_one()) {
+            if (lvr) tma::load3(st + L::LVZR, m.fl[1], xs, zr, qf + A_LPVZ, b);
+            if (lpz) tma::load3(st + L::LPZ, m.fl[1], xs, k, qf + A_LPPZ, b);
+        }
+    } else if (warp == 6) {
+        if (main && (lvz || tpn) && tma::elect_one()) {
+            if (lvz) tma::load3(st + L::LVZ, m.fl[1], xs, z, qf + A_LPVZ, b);
+            if (tpn) tma::load3(st + L::LVX, m.fl[1], xs, z, qf + A_LPVX, b);
+            if (tph) tma::load3(st + L::LPX, m.fl[1], xs, z, qf + A_LPPX, b);
+        }
+    } else {
+        if (tma::elect_one()) {
+            unsigned bytes = 2 * L::F2 + (1 + (lvr ? 1 : 0) + (lpz ? 1 : 0)) * L::F1;
+            if (main) bytes += 2 * L::F2 + (1 + (lvz ? 1 : 0) + (tpn ? 1 : 0) + (tph ? 1 : 0)) * L::F1;
+            tma::mbar_expect(b, bytes);
+        }
     }
-    const bool okk1 = colok && k + 1 >= 0;
-    const long long ck1 = okk1 ? (long long)min(k + 1, g.Nz - 1) * pitch + xc : 0;
-    const bool main = z >= zc0 && z < zc1;
-    const bool okz = colok && main;
-    const long long cz = okz ? (long long)z * pitch + xc : 0;
-    const bool okv = vxok && main;
-    const int iz = z - z0;
-    cpa(s2 + 0 * NTH, in2 + (A_PL / 2) * p2 + crs, okrs);
-    cpa(s2 + 1 * NTH, in2 + (A_VZ / 2) * p2 + cks, okks);
-    cpa(s2 + 2 * NTH, in2 + (A_PL / 2) * p2 + cz, okz);
-    cpa(s2 + 3 * NTH, in2 + (A_VX / 2) * p2 + cz, okv);
-    cpa(s2 + 4 * NTH, img + cz, outcol && main && inner_col && iz >= 0 && iz < g.nz);
-    const float *kdt = WIN ? in + W_KDT * plane : a.kdt;
-    const float *binv = WIN ? in + W_BINV * plane : a.binv;
-    cpa(s1 + 0 * NTH, kdt + cr, okr);
-    cpa(s1 + 1 * NTH, in + A_LPVZ * plane + cr, okr && ((zr <= z0 - 1) || (zr >= z1)));
-    cpa(s1 + 2 * NTH, binv + ck1, okk1);
-    cpa(s1 + 3 * NTH, in + A_LPPZ * plane + ck, okk && ((k <= z0 - 2) || (k >= z1)));
-    cpa(s1 + 4 * NTH, kdt + cz, okz);
-    cpa(s1 + 5 * NTH, in + A_LPVX * plane + cz, okz && pmlxn);
-    cpa(s1 + 6 * NTH, in + A_LPVZ * plane + cz, outcol && main && ((z <= z0 - 1) || (z >= z1)));
-    cpa(s1 + 7 * NTH, binv + cz, okz);
-    cpa(s1 + 8 * NTH, in + A_LPPX * plane + cz, okv && pmlxh);
-}
-
-__device__ __forceinline__ AdjRow adj_read(const float *st)
-{
-    const int t = threadIdx.x;
-    const float2 *s2 = reinterpret_cast<const float2 *>(st) + t;
-    const float *s1 = st + 2 * kAdjF2 * NTH + t;
-    AdjRow r;
-    r.pl = s2[0 * NTH];
-    r.v2z = s2[1 * NTH];
-    r.plz = s2[2 * NTH];
-    r.v2x = s2[3 * NTH];
-    r.img = s2[4 * NTH];
-    r.kdr = s1[0 * NTH];
-    r.lpvzr = s1[1 * NTH];
-    r.bz = s1[2 * NTH];
-    r.lppz = s1[3 * NTH];
-    r.kdz = s1[4 * NTH];
-    r.lpsvx = s1[5 * NTH];
-    r.lpsvz = s1[6 * NTH];
-    r.bx = s1[7 * NTH];
-    r.lppx = s1[8 * NTH];
-    return r;
+    __syncwarp();
 }
 
 template <int M, bool WIN, bool FS>
-__global__ void __launch_bounds__(NTH, FS ? kAdjMinBlocksFS : kAdjMinBlocks) k_adj2d(const Step2D a)
+__device__ __forceinline__ void adj_body(const Arg2D &p)
 {
+    const Step2D &a = p.a;
     if (guard_tripped(a.g)) return;
     using C = Cols<M>;
-    constexpr int W = C::W, HXP = C::HXP, TXO = C::TXO;
-    __shared__ float2 sPU[NTH];   // (p^n, kdt*lp - ai_x (lpsi_vx - kdt*lp)), row z
-    __shared__ float sB[NTH];     // 1/rho, row z
-    __shared__ float2 sVW[NTH];   // (vx^{n+1/2}, dt*bu_x*lvx - ah_x*lpsi_px), row z
-    __shared__ float sVN[NTH];    // vx^{n-1/2}, row z
-    __shared__ float sPi[NTH];    // Gx * lvx, row z
-    extern __shared__ __align__(16) float stagef[];   // [PDA][kAdjStageFloats]
+    using L = AdjLayM<M>;
+    constexpr int W = C::W, HXP = C::HXP, TXO = C::TXO, NB = L::NB;
+    extern __shared__ unsigned char smraw[];
+    char *sm = reinterpret_cast<char *>(smraw + ((128u - (tma::su32(smraw) & 127u)) & 127u));
+    float2 *const sPU = reinterpret_cast<float2 *>(sm + L::SPU);
+    float2 *const sVW = reinterpret_cast<float2 *>(sm + L::SVW);
+    float *const sVN = reinterpret_cast<float *>(sm + L::SVN);
+    float *const sPi = reinterpret_cast<float *>(sm + L::SPI);
+    char *const sB = sm + L::SB;
+    float *const sScale = reinterpret_cast<float *>(sm + L::BAR - 8);   // this step's (p, v) band scales
+    uint64_t *bar = reinterpret_cast<uint64_t *>(sm + L::BAR);
 
     const GridDev &g = a.g;
     const int t = threadIdx.x;
@@ -907,357 +761,14 @@ __global__ void __launch_bounds__(NTH, FS ? kAdjMinBlocksFS : kAdjMinBlocks) k_a
     const int Nx = WIN ? a.win_nx[shot] + 2 * g.x0 : g.Nx;
     const int nx = WIN ? Nx - 2 * g.x0 : g.nx;
     if (WIN && (int)blockIdx.x * TXO >= Nx) return;   // no output column in this shot's window
-    const int x = (int)blockIdx.x * TXO - HXP + t;
-    const bool colok = x >= 0 && x < Nx;
-    const bool outcol = colok && t >= HXP && t < HXP + TXO;
-    const bool vxok = colok && t >= M - 1 && t <= NTH - 1 - M;
-    const int zc0 = (int)blockIdx.y * a.tzc;
-    const int zc1 = min(zc0 + a.tzc, g.Nz);
-    const int zstart = zc0 - W;
-    const long long plane = g.plane;
-    const long long p2 = plane;   // stride of one pair field in float2 units
-    const int pitch = g.pitch;
-    const int xc = colok ? x : 0;
-    const float *in = a.in + slot * a.sstride;
-    float *outf = a.out + slot * a.sstride + xc;
-    float2 *out2 = reinterpret_cast<float2 *>(a.out + slot * a.sstride) + xc;
-    const float dt = g.dt;
-    const int n = a.n;
-    const bool recon = n > 0;
-    const int x0 = g.x0, x1 = g.x0 + nx, z0 = g.z0, z1 = g.z0 + g.nz;
-    const int ix = x - x0;
-    const bool xint = ix >= 0 && ix < nx;
-    const bool pmlxh = colok && ((x <= x0 - 2) || (x >= x1));
-    const bool pmlxn = colok && ((x <= x0 - 1) || (x >= x1));
-    const int px = WIN ? shot * a.pml_xstride + x : x;   // x CPML profiles of this shot's window
-    const float ahx = pmlxh ? a.pml.ah[2][px] : 0.f, bhx = pmlxh ? a.pml.bh[2][px] : 0.f;
-    const float aix = pmlxn ? a.pml.ai[2][px] : 0.f, bix = pmlxn ? a.pml.bi[2][px] : 0.f;
-    const long long rowprev = band_row(a.bands, shot, n - 1);
-    const int src = a.src_cell[shot];
-    const float wsrc = recon ? a.src_scale * a.wav[(a.wav_per_shot ? (long long)shot * g.nt : 0) + n - 1] : 0.f;
-    const float2 *imgs = a.img + slot * plane;   // image accumulators of this slot
-    float2 *img = a.img + slot * plane + xc;
-
-    // z rings, shifted by U entries after every group of U rows: at row u of a
-    // group, entry u + m holds node row z + m (PU) or the half-row value
-    // written m - W + 1 rows earlier (VW, VN, PIZ), m = 0 .. W - 1
-    constexpr int U = W / kAdjGroupDiv > 0 ? W / kAdjGroupDiv : 1, RL = W + U - 1;
-    float2 PU[RL], VW[RL];
-    float VN[RL], PIZ[RL];
-#pragma unroll
-    for (int j = 0; j < RL; ++j) {
-        PU[j] = make_float2(0.f, 0.f);
-        VW[j] = make_float2(0.f, 0.f);
-        VN[j] = 0.f;
-        PIZ[j] = 0.f;
-    }
-    // (p^n, kdt*lp - ai_z (lpsi_vz - kdt*lp)) at node row r of this column
-    // (pl holds the mirror row's values for a ghost row r < z0; the surface
-    // row carries p = 0 and lambda_p = 0)
-    auto pu_node = [&](int r, float2 pl, float kd, float lpvz) -> float2 {
-        if (FS && r <= z0) {
-            if (r == z0) return make_float2(0.f, 0.f);
-            return make_float2(-pl.x, -(kd * pl.y));
-        }
-        float kl = kd * pl.y;
-        if (colok && r >= 0 && r < g.Nz && ((r <= z0 - 1) || (r >= z1))) kl -= a.pml.ai[0][r] * (lpvz - kl);
-        return make_float2(pl.x, kl);
-    };
-    {
-        const float2 *in2 = reinterpret_cast<const float2 *>(in);
-#pragma unroll
-        for (int j = 0; j < W - 1; ++j) {
-            const int r = zstart + j, rs = node_src_row<FS>(g, r);
-            const bool ok = colok && r >= 0 && r < g.Nz;
-            const long long cr = ok ? (long long)r * pitch + xc : 0;
-            const bool oks = colok && rs >= 0 && rs < g.Nz;
-            const float2 plv = oks ? in2[(A_PL / 2) * p2 + (long long)rs * pitch + xc] : make_float2(0.f, 0.f);
-            const float kd = ok ? (WIN ? in[W_KDT * plane + cr] : a.kdt[cr]) : 0.f;
-            const float lpvz = (ok && ((r <= z0 - 1) || (r >= z1))) ? in[A_LPVZ * plane + cr] : 0.f;
-            PU[j] = pu_node(r, plv, kd, lpvz);
-        }
-    }
-    float bz_old = 0.f;
-    {
-        int k = zstart + M - 1;
-        if (colok && k >= 0 && k < g.Nz)
-            bz_old = WIN ? in[W_BINV * plane + (long long)k * pitch + xc] : a.binv[(long long)k * pitch + xc];
-    }
-
-#pragma unroll
-    for (int j = 0; j < PDA - 1; ++j) {
-        if (zstart + j < zc1)
-            adj_issue<M, WIN, FS>(stagef + j * kAdjStageFloats, a, imgs, in, xc, zstart + j, zc0, zc1, colok, vxok,
-                         outcol, pmlxh, pmlxn, xint);
-        cp_commit();
-    }
-
-    for (int zb = zstart; zb < zc1; zb += U) {
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int z = zb + u;
-            if (z >= zc1) break;
-            const int zi = z + PDA - 1;
-            if (zi < zc1)
-                adj_issue<M, WIN, FS>(stagef + ((zi - zstart) % PDA) * kAdjStageFloats, a, imgs, in, xc, zi, zc0, zc1,
-                             colok, vxok, outcol, pmlxh, pmlxn, xint);
-            cp_commit();
-            cp_wait_row<PDA>();
-            const AdjRow cur = adj_read(stagef + ((z - zstart) % PDA) * kAdjStageFloats);
-            const int k = z + M - 1;
-            const int sl = u + W - 1;
-            PU[sl] = pu_node(z + W - 1, cur.pl, cur.kdr, cur.lpvzr);
-            const float buz = 0.5f * (bz_old + cur.bz);
-            bz_old = cur.bz;
-            // ---- half row k along z: lambda_vz, lambda_psi_pz, background vz^{n-1/2}
-            float wz = 0.f, vn = 0.f, piz = 0.f;
-            if (colok && k >= 0 && k < g.Nz) {
-                const long long ck = (long long)k * pitch;
-                const bool own = outcol && k >= zc0 && k < zc1;
-                // (Gz, du/dz)
-                const float2 D = stencil<M, float2>(g.cz, [&](int l) { return PU[u + M - 1 + l]; },
-                                                    [&](int l) { return PU[u + M - l]; });
-                const float lv = cur.v2z.y + D.y;
-                const float dtbu = dt * buz;
-                wz = dtbu * lv;
-                if ((k <= z0 - 2) || (k >= z1)) {
-                    float l1 = cur.lppz - dtbu * lv;
-                    wz -= a.pml.ah[0][k] * l1;
-                    if (own) outf[A_LPPZ * plane + ck] = a.pml.bh[0][k] * l1;
-                }
-                piz = D.x * lv;
-                if (recon && xint) {
-                    const int iz = k - z0;
-                    if ((iz >= 0 || FS) && iz < g.nz) vn = cur.v2z.x + dtbu * D.x;
-                    else if (in_xstrip(iz, M, g.nz))
-                        vn = band_get(a.bands, 1, rowprev, band_zstrip(iz, ix, M, g.nz, nx));
-                }
-                if (own) out2[(A_VZ / 2) * p2 + ck] = make_float2(vn, lv);
-            }
-            VW[sl] = make_float2(cur.v2z.x, wz);
-            VN[sl] = vn;
-            PIZ[sl] = piz;
-            if (z < zc0) continue;
-
-            // ---- row z: half nodes along x
-            const long long cz = (long long)z * pitch;
-            const bool surf = FS && z == z0;   // free-surface row: p = 0, lambda_p = 0
-            const float pbn = cur.plz.x;
-            const float lp1 = surf ? 0.f : cur.plz.y;
-            const float kd = cur.kdz;
-            const float kl = kd * lp1;
-            sPU[t] = make_float2(pbn, pmlxn ? kl - aix * (cur.lpsvx - kl) : kl);
-            sB[t] = cur.bx;
-            __syncthreads();
-            float2 vw = make_float2(cur.v2x.x, 0.f);
-            float vxn = 0.f, pix = 0.f;
-            if (vxok) {
-                // (Gx, du/dx)
-                const float2 D = stencil<M, float2>(g.cx, [&](int l) { return sPU[t + l]; },
-                                                    [&](int l) { return sPU[t + 1 - l]; });
-                const float bux = 0.5f * (cur.bx + (x + 1 >= Nx ? cur.bx : sB[t + 1]));
-                const float dtbu = dt * bux;
-                const float lv = cur.v2x.y + D.y;
-                float wx = dtbu * lv;
-                if (pmlxh) {
-                    float l1 = cur.lppx - dtbu * lv;
-                    wx -= ahx * l1;
-                    if (outcol) outf[A_LPPX * plane + cz] = bhx * l1;
-                }
-                vw.y = wx;
-                pix = D.x * lv;
-                if (recon) {
-                    const int iz = z - z0;
-                    if (iz >= 0 && iz < g.nz) {
-                        if (xint) vxn = cur.v2x.x + dtbu * D.x;
-                        else if (in_xstrip(ix, M, nx))
-                            vxn = band_get(a.bands, 1, rowprev, band_xstrip(iz, ix, M, g.nz, nx));
-                    }
-                }
-                if (outcol) out2[(A_VX / 2) * p2 + cz] = make_float2(vxn, lv);
-            }
-            sVW[t] = vw;
-            sVN[t] = vxn;
-            sPi[t] = pix;
-            __syncthreads();
-
-            // ---- row z: nodes on the output columns
-            if (outcol) {
-                // (Q_n, D- w) along x and z
-                const float2 Ex = stencil<M, float2>(g.cx, [&](int l) { return sVW[t + l - 1]; },
-                                                     [&](int l) { return sVW[t - l]; });
-                const float2 Ez = stencil<M, float2>(g.cz, [&](int l) { return VW[u + M + l - 1]; },
-                                                     [&](int l) { return VW[u + M - l]; });
-                const float2 E = add_(Ex, Ez);
-                float qn = 0.f;
-                if (recon)
-                    qn = stencil<M, float>(g.cx, [&](int l) { return sVN[t + l - 1]; }, [&](int l) { return sVN[t - l]; }) +
-                         stencil<M, float>(g.cz, [&](int l) { return VN[u + M + l - 1]; },
-                                           [&](int l) { return VN[u + M - l]; });
-                const int iz = z - z0;
-                const bool inner = xint && iz >= 0 && iz < g.nz;
-                if (inner) {
-                    float2 acc = cur.img;
-                    acc.x += E.x * lp1;
-                    // (on the free surface the half row above is a ghost: no product of its own)
-                    acc.y += (sPi[t] + sPi[t - 1]) + (PIZ[u + M] + (surf ? 0.f : PIZ[u + M - 1]));
-                    img[cz] = acc;
-                }
-                float pn = 0.f;
-                if (recon) {
-                    if (inner) {
-                        pn = pbn + kd * qn;
-                        if (cz + x == src) pn -= wsrc;
-                    } else {
-                        long long b = pband_index(iz, ix, M, g.nz, nx);
-                        if (b >= 0) pn = band_get(a.bands, 0, rowprev, b);
-                    }
-                }
-                out2[(A_PL / 2) * p2 + cz] = (FS && z <= z0) ? make_float2(0.f, 0.f) : make_float2(pn, lp1 + E.y);
-                if (pmlxn) outf[A_LPVX * plane + cz] = bix * (cur.lpsvx - kl);
-                if ((z <= z0 - 1) || (z >= z1)) outf[A_LPVZ * plane + cz] = a.pml.bi[0][z] * (cur.lpsvz - kl);
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < W - 1; ++j) {
-            PU[j] = PU[j + U];
-            VW[j] = VW[j + U];
-            VN[j] = VN[j + U];
-            PIZ[j] = PIZ[j + U];
-        }
-    }
-
-    if (recon) {
-        // pre-add the residual of step n-1 at the receivers of this CTA
-        __syncthreads();
-        int tile = shot * a.trec.ntiles + blockIdx.y * gridDim.x + blockIdx.x;
-        int b = a.trec.ptr[tile], e = a.trec.ptr[tile + 1];
-        float2 *plo = reinterpret_cast<float2 *>(a.out + slot * a.sstride + A_PL * plane);
-        for (int i = b + t; i < e; i += NTH) {
-            int2 rc = a.trec.rec[i];
-            if (i > b && a.trec.rec[i - 1].x == rc.x) continue;  // run handled by its first entry
-            float add = 0.f;
-            for (int q = i; q < e && a.trec.rec[q].x == rc.x; ++q)
-                add += a.dstage[(long long)a.trec.rec[q].y * g.nt + (n - 1)];
-            plo[rc.x].y += add;
-        }
-    }
-}
-
-// Start state of a reverse pass: (p, 0), (vx, 0), (vz, 0) from the saved
-// background final state [p][vx][vz] of each shot of the batch.
-// ---------------------------------------------------------------------------
-// Migration step with TMA row staging (shots without aperture windows). The
-// same arithmetic as k_adj2d, in the same order, so the results are the same
-// bits; only the loads of the rows ahead differ. One thread (the last) issues
-// every field row of a stage as one tensor-map tile copy (a kThreads2D-wide
-// row of one field) on the stage's mbarrier; the tensor maps read zeros
-// outside the padded grid, which is what the per-thread copies' zero fill
-// gives at the grid edges. Rows the per-thread copies zero-fill inside the
-// grid (a row whose source row is out of range) are read from row -1.
-// Fields a row does not use (the CPML memories outside the strips, the
-// row-z fields of the warm-up rows) are not copied; no consumer reads them.
-// A stage is refilled only after a CTA barrier that follows every read of
-// it: the previous row's barriers (a warm-up row adds one for this).
-// ---------------------------------------------------------------------------
-struct Adj2T {
-    Step2D a;
-    Maps2D m;
-};
-
-constexpr unsigned kAdjStageBytesT = (unsigned)(kAdjStageFloats * sizeof(float));
-static_assert(kAdjStageBytesT % 128 == 0, "stage rows stay 128-byte aligned");
-constexpr unsigned kAdjBarOff = PDA * kAdjStageBytesT;
-constexpr unsigned kAdjSmemT = kAdjBarOff + 64 + 128;   // stages, barriers, alignment slack
-
-// Issues the copies of row z (the stage layout of adj_issue) on barrier b.
-// xs: first column of the CTA (a multiple of 4, so every copy starts on a
-// 16-byte boundary); tpn / tph: the CTA has node / half-node CPML columns.
-template <int M, bool FS>
-__device__ __forceinline__ void adj_issue_tma(const Adj2T &p, float *st, uint64_t *b, int slot, int xs, int z,
-                                              int zc0, int zc1, bool tpn, bool tph)
-{
-    const GridDev &g = p.a.g;
-    const Maps2D &m = p.m;
-    constexpr int W = 2 * M;
-    constexpr unsigned R2 = NTH * 8, R1 = NTH * 4;   // bytes of one float2 / float field row
-    const int z0 = g.z0, z1 = g.z0 + g.nz;
-    const int zr = z + W - 1, k = z + M - 1;
-    const int qp = slot * m.pps, qf = slot * m.fps;
-    char *s2 = reinterpret_cast<char *>(st);
-    char *s1 = s2 + kAdjF2 * R2;
-    const bool inr = zr >= 0 && zr < g.Nz, ink = k >= 0 && k < g.Nz;
-    int rpl = zr, rvz = ink ? k : -1;
-    if constexpr (FS) {
-        const int zrs = node_src_row<FS>(g, zr), ks = half_src_row<FS>(g, k);
-        rpl = (zrs >= 0 && zrs < g.Nz) ? zrs : -1;
-        rvz = (ink && ks < g.Nz) ? ks : -1;
-    }
-    const int rbz = k + 1 >= 0 ? min(k + 1, g.Nz - 1) : -1;
-    const bool lpa = inr && ((zr <= z0 - 1) || (zr >= z1));
-    const bool lpz = ink && ((k <= z0 - 2) || (k >= z1));
-    const bool main = z >= zc0 && z < zc1;
-    const int iz = z - z0;
-    const bool im = main && iz >= 0 && iz < g.nz;
-    const bool lvx = main && tpn, lvz = main && ((z <= z0 - 1) || (z >= z1)), lpx = main && tph;
-    unsigned bytes = 2 * R2 + 2 * R1 + (lpa ? R1 : 0) + (lpz ? R1 : 0);
-    if (main) bytes += 2 * R2 + 2 * R1;
-    if (im) bytes += R2;
-    if (lvx) bytes += R1;
-    if (lvz) bytes += R1;
-    if (lpx) bytes += R1;
-    tma::fence_proxy_async();
-    tma::mbar_expect(b, bytes);
-    tma::load3(s2 + 0 * R2, m.pr, xs, rpl, qp + A_PL / 2, b);
-    tma::load3(s2 + 1 * R2, m.pr, xs, rvz, qp + A_VZ / 2, b);
-    tma::load3(s1 + 0 * R1, m.md, xs, zr, 0, b);
-    if (lpa) tma::load3(s1 + 1 * R1, m.fl, xs, zr, qf + A_LPVZ, b);
-    tma::load3(s1 + 2 * R1, m.md, xs, rbz, 1, b);
-    if (lpz) tma::load3(s1 + 3 * R1, m.fl, xs, k, qf + A_LPPZ, b);
-    if (main) {
-        tma::load3(s2 + 2 * R2, m.pr, xs, z, qp + A_PL / 2, b);
-        tma::load3(s2 + 3 * R2, m.pr, xs, z, qp + A_VX / 2, b);
-        tma::load3(s1 + 4 * R1, m.md, xs, z, 0, b);
-        tma::load3(s1 + 7 * R1, m.md, xs, z, 1, b);
-    }
-    if (im) tma::load3(s2 + 4 * R2, m.im, xs, z, slot, b);
-    if (lvx) tma::load3(s1 + 5 * R1, m.fl, xs, z, qf + A_LPVX, b);
-    if (lvz) tma::load3(s1 + 6 * R1, m.fl, xs, z, qf + A_LPVZ, b);
-    if (lpx) tma::load3(s1 + 8 * R1, m.fl, xs, z, qf + A_LPPX, b);
-}
-
-template <int M, bool FS>
-__global__ void __launch_bounds__(NTH, FS ? kAdjMinBlocksFS : kAdjMinBlocks) k_adj2t(const __grid_constant__ Adj2T p)
-{
-    const Step2D &a = p.a;
-    if (guard_tripped(a.g)) return;
-    using C = Cols<M>;
-    constexpr int W = C::W, HXP = C::HXP, TXO = C::TXO;
-    static_assert(TXO % 4 == 0 && HXP % 4 == 0, "CTA column starts must be 16-byte aligned for 4-byte elements");
-    __shared__ float2 sPU[NTH];   // (p^n, kdt*lp - ai_x (lpsi_vx - kdt*lp)), row z
-    __shared__ float sB[NTH];     // 1/rho, row z
-    __shared__ float2 sVW[NTH];   // (vx^{n+1/2}, dt*bu_x*lvx - ah_x*lpsi_px), row z
-    __shared__ float sVN[NTH];    // vx^{n-1/2}, row z
-    __shared__ float sPi[NTH];    // Gx * lvx, row z
-    extern __shared__ unsigned char smraw[];
-    unsigned char *sm = smraw + ((128u - (tma::su32(smraw) & 127u)) & 127u);
-    float *stagef = reinterpret_cast<float *>(sm);   // [PDA][kAdjStageFloats]
-    uint64_t *bar = reinterpret_cast<uint64_t *>(sm + kAdjBarOff);
-
-    const GridDev &g = a.g;
-    const int t = threadIdx.x;
-    const int slot = blockIdx.z, shot = a.shot0 + slot;
-    const int Nx = g.Nx, nx = g.nx;
     const int xs = (int)blockIdx.x * TXO - HXP;
     const int x = xs + t;
     const bool colok = x >= 0 && x < Nx;
     const bool outcol = colok && t >= HXP && t < HXP + TXO;
-    const bool vxok = colok && t >= M - 1 && t <= NTH - 1 - M;
     const int zc0 = (int)blockIdx.y * a.tzc;
     const int zc1 = min(zc0 + a.tzc, g.Nz);
     const int zstart = zc0 - W;
-    const long long plane = g.plane;
-    const long long p2 = plane;   // stride of one pair field in float2 units
+    const int pT = (int)g.plane;   // in-slot offsets fit 32 bits (checked by the host); the stride of a pair field in float2
     const int pitch = g.pitch;
     const int xc = colok ? x : 0;
     const float *in = a.in + slot * a.sstride;
@@ -1269,223 +780,323 @@ __global__ void __launch_bounds__(NTH, FS ? kAdjMinBlocksFS : kAdjMinBlocks) k_a
     const int x0 = g.x0, x1 = g.x0 + nx, z0 = g.z0, z1 = g.z0 + g.nz;
     const int ix = x - x0;
     const bool xint = ix >= 0 && ix < nx;
+    const bool xband = recon && in_xstrip(ix, M, nx);
+    const bool cband = recon && (xs < x0 || xs + NTH > x1);    // the CTA may have x strip columns of the bands
+    const int bc = ix < 0 ? ix + M : M + ix - nx;              // this column in a row's [2 sides][M] strip values
     const bool pmlxh = colok && ((x <= x0 - 2) || (x >= x1));
     const bool pmlxn = colok && ((x <= x0 - 1) || (x >= x1));
-    const bool tph = (xs <= x0 - 2) || (xs + NTH - 1 >= x1);   // CTA has half-node / node CPML columns
+    const bool tph = (xs <= x0 - 2) || (xs + NTH - 1 >= x1);   // the CTA has half-node / node CPML columns
     const bool tpn = (xs <= x0 - 1) || (xs + NTH - 1 >= x1);
-    const float ahx = pmlxh ? a.pml.ah[2][x] : 0.f, bhx = pmlxh ? a.pml.bh[2][x] : 0.f;
-    const float aix = pmlxn ? a.pml.ai[2][x] : 0.f, bix = pmlxn ? a.pml.bi[2][x] : 0.f;
+    const int px = WIN ? shot * a.pml_xstride + x : x;         // x CPML profiles of this shot's window
+    const float ahx = pmlxh ? a.pml.ah[2][px] : 0.f, bhx = pmlxh ? a.pml.bh[2][px] : 0.f;
+    const float aix = pmlxn ? a.pml.ai[2][px] : 0.f, bix = pmlxn ? a.pml.bi[2][px] : 0.f;
+    const float hbx = x >= 0 ? 0.5f : 0.f;   // half nodes left of the array are zero (past its end 1/rho reads zero)
+    const bool lastx = x + 1 >= Nx;
     const long long rowprev = band_row(a.bands, shot, n - 1);
     const int src = a.src_cell[shot];
     const float wsrc = recon ? a.src_scale * a.wav[(a.wav_per_shot ? (long long)shot * g.nt : 0) + n - 1] : 0.f;
-    float2 *img = a.img + slot * plane + xc;
-    constexpr int PR = NTH - 1;   // the thread that issues the copies
+    float2 *img = a.img + slot * g.plane + xc;
+    const float *kdt = WIN ? in + W_KDT * g.plane : a.kdt;
+    const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);   // (known to be uniform)
 
     if (t == 0) {
-        for (int i = 0; i < PDA; ++i) tma::mbar_init(bar + i);
+        for (int i = 0; i < NS; ++i) tma::mbar_init(bar + i);
         tma::mbar_init_fence();
+        if (cband && a.bands.fmt != BAND_F32)
+            for (int f = 0; f < 2; ++f) sScale[f] = a.bands.scale[rowprev * 2 + f];
     }
     __syncthreads();
-    if (t == PR) {
-        for (int j = 0; j < PDA - 1 && zstart + j < zc1; ++j)
-            adj_issue_tma<M, FS>(p, stagef + j * kAdjStageFloats, bar + j, slot, xs, zstart + j, zc0, zc1, tpn, tph);
-    }
+    for (int j = 0; j < NS && zstart + 2 * j < zc1; ++j)
+        adj_issue<M, FS, WIN>(p, warp, sm + j * L::STAGE, sm + L::B + j * L::F1, bar + j, slot, xs, zstart + 2 * j, zc0, tpn,
+                              tph);
 
-    constexpr int U = W / kAdjGroupDiv > 0 ? W / kAdjGroupDiv : 1, RL = W + U - 1;
+    // z rings, shifted by U entries after every U rows: at row u of a pass,
+    // entry u + m holds node row z + m (PU) or the half-row value written m -
+    // W + 1 rows earlier (VW, VN), m = 0 .. W - 1; PIZ entry u + m half row z
+    // - 1 + m, m = 0 .. M
+    constexpr int U = 2, RL = W + U - 1, RP = M + U;
     float2 PU[RL], VW[RL];
-    float VN[RL], PIZ[RL];
+    float VN[RL], PIZ[RP];
 #pragma unroll
-    for (int j = 0; j < RL; ++j) {
-        PU[j] = make_float2(0.f, 0.f);
-        VW[j] = make_float2(0.f, 0.f);
-        VN[j] = 0.f;
-        PIZ[j] = 0.f;
+    for (int i = 0; i < RL; ++i) {
+        PU[i] = make_float2(0.f, 0.f);
+        VW[i] = make_float2(0.f, 0.f);
+        VN[i] = 0.f;
     }
-    auto pu_node = [&](int r, float2 pl, float kd, float lpvz) -> float2 {
+#pragma unroll
+    for (int i = 0; i < RP; ++i) PIZ[i] = 0.f;
+    // (p^n, mu - ai_z (lpsi_vz - mu)) at node row r of this column (pl holds
+    // the mirror row's values for a ghost row r < z0; the surface row carries
+    // p = 0 and mu = 0)
+    auto pu_node = [&](int r, float2 pl, float lpvz) -> float2 {
         if (FS && r <= z0) {
             if (r == z0) return make_float2(0.f, 0.f);
-            return make_float2(-pl.x, -(kd * pl.y));
+            return make_float2(-pl.x, -pl.y);
         }
-        float kl = kd * pl.y;
-        if (colok && r >= 0 && r < g.Nz && ((r <= z0 - 1) || (r >= z1))) kl -= a.pml.ai[0][r] * (lpvz - kl);
-        return make_float2(pl.x, kl);
+        if (zpml_node(g, r)) pl.y -= a.pml.ai[0][r] * (lpvz - pl.y);
+        return pl;
     };
     {
-        const float2 *in2 = reinterpret_cast<const float2 *>(in);
+        const float2 *in2 = reinterpret_cast<const float2 *>(in) + (A_PL / 2) * pT + xc;
 #pragma unroll
-        for (int j = 0; j < W - 1; ++j) {
-            const int r = zstart + j, rs = node_src_row<FS>(g, r);
-            const bool ok = colok && r >= 0 && r < g.Nz;
-            const long long cr = ok ? (long long)r * pitch + xc : 0;
-            const bool oks = colok && rs >= 0 && rs < g.Nz;
-            const float2 plv = oks ? in2[(A_PL / 2) * p2 + (long long)rs * pitch + xc] : make_float2(0.f, 0.f);
-            const float kd = ok ? a.kdt[cr] : 0.f;
-            const float lpvz = (ok && ((r <= z0 - 1) || (r >= z1))) ? in[A_LPVZ * plane + cr] : 0.f;
-            PU[j] = pu_node(r, plv, kd, lpvz);
+        for (int i = 0; i < W - 1; ++i) {
+            const int r = zstart + i, rs = node_src_row<FS>(g, r);
+            const float2 plv = (colok && rs >= 0 && rs < g.Nz) ? in2[rs * pitch] : make_float2(0.f, 0.f);
+            const float lpvz = colok && zpml_node(g, r) ? in[A_LPVZ * pT + r * pitch + xc] : 0.f;
+            PU[i] = pu_node(r, plv, lpvz);
         }
     }
     float bz_old = 0.f;
     {
-        int k = zstart + M - 1;
-        if (colok && k >= 0 && k < g.Nz) bz_old = a.binv[(long long)k * pitch + xc];
+        const int k = zstart + M - 1;
+        if (colok && k >= 0 && k < g.Nz) bz_old = (WIN ? in + W_BINV * g.plane : a.binv)[k * pitch + xc];
     }
+
+    // forms without row (ZF) and column (XF) tests, as in fwd_body
+    const bool xf = __all_sync(0xffffffffu, xint);
+
+    // The x strips' band values of the group of rows zg, zg + 1 (buffer bf),
+    // fetched one group ahead by asynchronous copies of 4 bytes: one value, or
+    // two 16-bit ones by the even columns (rows of a strip hold M values, M
+    // even, so their pairs are 4-byte aligned).
+    auto band_fetch = [&](int zg, int bf) {
+        const bool f32 = a.bands.fmt == BAND_F32;
+        if (xband && (f32 || (bc & 1) == 0)) {
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int iz = zg + r - z0;
+                if (iz < 0 || iz >= g.nz) continue;
+                const long long o = rowprev * a.bands.nb + band_xstrip(iz, ix, M, g.nz, nx);
+                const int e = (bf * 4 + r) * 2 * M + bc;   // field 0; field 1 at + 2 * 2M
+                const int sz = f32 ? 4 : 2;
+                cp_async4(sB + e * sz, static_cast<const char *>(a.bands.p) + o * sz);
+                cp_async4(sB + (e + 4 * M) * sz, static_cast<const char *>(a.bands.v) + o * sz);
+            }
+        }
+    };
+    auto band_val = [&](int field, int bf, int r) -> float {
+        const int e = (bf * 4 + field * 2 + r) * 2 * M + bc;
+        if (a.bands.fmt == BAND_F32) return reinterpret_cast<const float *>(sB)[e];
+        if (a.bands.fmt == BAND_BF16S) return sScale[field] * __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(sB)[e]);
+        return sScale[field] * __half2float(reinterpret_cast<const __half *>(sB)[e]);
+    };
 
     bool bad = false;      // this thread's wait gave up
-    int fail_row = zc1;    // first row whose stage was not consumed
-    for (int zb = zstart; zb < zc1; zb += U) {
+    int fail_j = -1;       // group whose stage was not consumed
+    int j = 0, bs = 0;     // group, its 1/rho slot
+    for (int z = zstart; z < zc1; z += U) {
+        char *const st = sm + (j % NS) * L::STAGE;
+        bad |= !tma::mbar_wait(bar + j % NS, (unsigned)(j / NS) & 1u);
+        const char *const st2 = st + t * 8;
+        const char *const st1 = st + t * 4;
+        const char *const bk = sm + L::B + bs * L::F1 + t * 4;
+        bs = bs + 1 == NB ? 0 : bs + 1;   // (the next group's)
+        const char *const brx = sm + L::B + (bs + NS - 1 >= NB ? bs + NS - 1 - NB : bs + NS - 1) * L::F1;
+        const bool main = z >= zc0;
+        const bool zf = recon && main && z > z0 && z + W < z1 && z + 1 < zc1;
+        // ---- rows z, z + 1: (p, mu) of the row itself
+        float2 pm[2];
+        auto own_row = [&](auto zc, auto xc_) {
+            constexpr bool ZF = decltype(zc)::value, XF = decltype(xc_)::value;
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int z = zb + u;
-            if (z >= zc1) break;
-            const int j = z - zstart;
-            // refill the stage of row z - 1 with row z + PDA - 1: every thread
-            // passed a barrier after reading it (the previous row's)
-            const int zi = z + PDA - 1;
-            if (t == PR && zi < zc1)
-                adj_issue_tma<M, FS>(p, stagef + ((j + PDA - 1) % PDA) * kAdjStageFloats, bar + (j + PDA - 1) % PDA,
-                                     slot, xs, zi, zc0, zc1, tpn, tph);
-            bad |= !tma::mbar_wait(bar + j % PDA, (unsigned)(j / PDA) & 1u);
-            const AdjRow cur = adj_read(stagef + (j % PDA) * kAdjStageFloats);
-            const int k = z + M - 1;
-            const int sl = u + W - 1;
-            PU[sl] = pu_node(z + W - 1, cur.pl, cur.kdr, cur.lpvzr);
-            const float buz = 0.5f * (bz_old + cur.bz);
-            bz_old = cur.bz;
-            // ---- half row k along z: lambda_vz, lambda_psi_pz, background vz^{n-1/2}
-            float wz = 0.f, vn = 0.f, piz = 0.f;
-            if (colok && k >= 0 && k < g.Nz) {
-                const long long ck = (long long)k * pitch;
-                const bool own = outcol && k >= zc0 && k < zc1;
-                const float2 D = stencil<M, float2>(g.cz, [&](int l) { return PU[u + M - 1 + l]; },
-                                                    [&](int l) { return PU[u + M - l]; });
-                const float lv = cur.v2z.y + D.y;
-                const float dtbu = dt * buz;
-                wz = dtbu * lv;
-                if ((k <= z0 - 2) || (k >= z1)) {
-                    float l1 = cur.lppz - dtbu * lv;
-                    wz -= a.pml.ah[0][k] * l1;
-                    if (own) outf[A_LPPZ * plane + ck] = a.pml.bh[0][k] * l1;
-                }
-                piz = D.x * lv;
-                if (recon && xint) {
-                    const int iz = k - z0;
-                    if ((iz >= 0 || FS) && iz < g.nz) vn = cur.v2z.x + dtbu * D.x;
-                    else if (in_xstrip(iz, M, g.nz))
-                        vn = band_get(a.bands, 1, rowprev, band_zstrip(iz, ix, M, g.nz, nx));
-                }
-                if (own) out2[(A_VZ / 2) * p2 + ck] = make_float2(vn, lv);
+            for (int r = 0; r < 2; ++r) {
+                const int iz = z + r - z0;
+                pm[r] = (ZF || (iz >= 0 && iz < g.nz)) ? PU[r] : *reinterpret_cast<const float2 *>(st2 + L::IM + r * L::F2R);
+                float u = pm[r].y;
+                if (!XF && pmlxn) u -= aix * (*reinterpret_cast<const float *>(st1 + L::LVX + r * L::F1R) - u);
+                sPU[r * NTH + t] = make_float2(pm[r].x, u);
             }
-            VW[sl] = make_float2(cur.v2z.x, wz);
-            VN[sl] = vn;
-            PIZ[sl] = piz;
-            if (z < zc0) {
-                // warm-up row: the barrier that lets its stage be refilled
-                if (__syncthreads_or(bad)) {
-                    fail_row = z;
-                    break;
-                }
-                continue;
-            }
-
-            // ---- row z: half nodes along x
-            const long long cz = (long long)z * pitch;
-            const bool surf = FS && z == z0;   // free-surface row: p = 0, lambda_p = 0
-            const float pbn = cur.plz.x;
-            const float lp1 = surf ? 0.f : cur.plz.y;
-            const float kd = cur.kdz;
-            const float kl = kd * lp1;
-            sPU[t] = make_float2(pbn, pmlxn ? kl - aix * (cur.lpsvx - kl) : kl);
-            sB[t] = cur.bx;
-            if (__syncthreads_or(bad)) {
-                fail_row = z;
-                break;
-            }
-            float2 vw = make_float2(cur.v2x.x, 0.f);
-            float vxn = 0.f, pix = 0.f;
-            if (vxok) {
-                const float2 D = stencil<M, float2>(g.cx, [&](int l) { return sPU[t + l]; },
-                                                    [&](int l) { return sPU[t + 1 - l]; });
-                const float bux = 0.5f * (cur.bx + (x + 1 >= Nx ? cur.bx : sB[t + 1]));
-                const float dtbu = dt * bux;
-                const float lv = cur.v2x.y + D.y;
-                float wx = dtbu * lv;
-                if (pmlxh) {
-                    float l1 = cur.lppx - dtbu * lv;
-                    wx -= ahx * l1;
-                    if (outcol) outf[A_LPPX * plane + cz] = bhx * l1;
-                }
-                vw.y = wx;
-                pix = D.x * lv;
-                if (recon) {
-                    const int iz = z - z0;
-                    if (iz >= 0 && iz < g.nz) {
-                        if (xint) vxn = cur.v2x.x + dtbu * D.x;
-                        else if (in_xstrip(ix, M, nx))
-                            vxn = band_get(a.bands, 1, rowprev, band_xstrip(iz, ix, M, g.nz, nx));
+        };
+        // ---- half rows k along z: lambda_vz, lambda_psi_pz, background vz^{n-1/2}
+        auto vz_stage = [&](auto zc) {
+            constexpr bool ZF = decltype(zc)::value;
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int zr = z + r + W - 1, k = z + r + M - 1, sl = r + W - 1;
+                const float2 pl = *reinterpret_cast<const float2 *>(st2 + L::PL + r * L::F2R);
+                if (ZF) PU[sl] = pl;
+                else PU[sl] = pu_node(zr, pl, *reinterpret_cast<const float *>(st1 + L::LVZR + r * L::F1R));
+                float b1 = *reinterpret_cast<const float *>(bk + r * L::F1R);
+                if (!ZF && k + 1 >= g.Nz) b1 = bz_old;   // the last half row replicates the last node row
+                const float buz = 0.5f * (bz_old + b1);
+                bz_old = b1;
+                const float2 v2z = *reinterpret_cast<const float2 *>(st2 + L::VZ + r * L::F2R);
+                float wz = 0.f, vn = 0.f, piz = 0.f;
+                if (ZF || (k >= 0 && k < g.Nz)) {
+                    const int ck = k * pitch;
+                    const bool own = outcol && (ZF || k >= zc0) && k < zc1;
+                    // (Gz, du/dz)
+                    const float2 D = stencil<M, float2>(g.cz, [&](int l) { return PU[r + M - 1 + l]; },
+                                                        [&](int l) { return PU[r + M - l]; });
+                    const float lv = v2z.y + D.y;
+                    const float dtbu = dt * buz;
+                    wz = dtbu * lv;
+                    if (!ZF && ((k <= z0 - 2) || (k >= z1))) {
+                        const float l1 = *reinterpret_cast<const float *>(st1 + L::LPZ + r * L::F1R) - dtbu * lv;
+                        wz -= a.pml.ah[0][k] * l1;
+                        if (own) outf[A_LPPZ * pT + ck] = a.pml.bh[0][k] * l1;
                     }
+                    piz = D.x * lv;
+                    if (ZF) {
+                        vn = xint ? v2z.x + dtbu * D.x : 0.f;
+                    } else if (recon && xint) {
+                        const int iz = k - z0;
+                        if ((iz >= 0 || FS) && iz < g.nz) vn = v2z.x + dtbu * D.x;
+                        else if (in_xstrip(iz, M, g.nz))
+                            vn = band_get(a.bands, 1, rowprev, band_zstrip(iz, ix, M, g.nz, nx));
+                    }
+                    if (own) out2[(A_VZ / 2) * pT + ck] = make_float2(vn, lv);
                 }
-                if (outcol) out2[(A_VX / 2) * p2 + cz] = make_float2(vxn, lv);
+                VW[sl] = make_float2(v2z.x, wz);
+                VN[sl] = vn;
+                PIZ[r + M] = piz;
             }
-            sVW[t] = vw;
-            sVN[t] = vxn;
-            sPi[t] = pix;
+        };
+        if (!zf) {
+            if (main) own_row(std::false_type{}, std::false_type{});
+            vz_stage(std::false_type{});
+        } else {
+            if (xf) own_row(std::true_type{}, std::true_type{});
+            else own_row(std::true_type{}, std::false_type{});
+            vz_stage(std::true_type{});
+        }
+        if (cband) cp_async_wait();   // (the barrier makes this group's band values visible to the other lanes)
+        // every thread is past the previous group's reads: refill its stage
+        if (__syncthreads_or(bad)) {
+            fail_j = j;
+            break;
+        }
+        if (j >= 1 && z + 2 * (NS - 1) < zc1) {
+            const int jn = j + NS - 1;
+            adj_issue<M, FS, WIN>(p, warp, sm + (jn % NS) * L::STAGE, sm + L::B + (jn % NB) * L::F1, bar + jn % NS, slot, xs,
+                                  z + 2 * (NS - 1), zc0, tpn, tph);
+        }
+        ++j;
+        if (cband && z + 2 >= zc0) band_fetch(z + 2, j & 1);   // the next group's
+        if (main) {
+            // ---- rows z, z + 1: half nodes along x
+            float pix[2];
+            const int bf = (j - 1) & 1;   // band values of this group (j counts the next one by now)
+            auto vx_stage = [&](auto zc, auto xc_) {
+                constexpr bool ZF = decltype(zc)::value, XF = decltype(xc_)::value;
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const int zr = z + r, cz = zr * pitch, iz = zr - z0;
+                    const float2 *const pu = sPU + r * NTH + t;
+                    // (Gx, du/dx)
+                    const float2 D = stencil<M, float2>(g.cx, [&](int l) { return pu[l]; }, [&](int l) { return pu[1 - l]; });
+                    const float2 v2x = *reinterpret_cast<const float2 *>(st2 + L::VX + r * L::F2R);
+                    const float *const b = reinterpret_cast<const float *>(brx + r * L::F1R) + t;
+                    const float bux = (XF ? 0.5f : hbx) * (b[0] + (!XF && lastx ? b[0] : b[1]));
+                    const float dtbu = dt * bux;
+                    const float lv = v2x.y + D.y;
+                    const bool own = outcol && (ZF || zr < zc1);
+                    float wx = dtbu * lv;
+                    if (!XF && pmlxh) {
+                        const float l1 = *reinterpret_cast<const float *>(st1 + L::LPX + r * L::F1R) - dtbu * lv;
+                        wx -= ahx * l1;
+                        if (own) outf[A_LPPX * pT + cz] = bhx * l1;
+                    }
+                    pix[r] = D.x * lv;
+                    float vxn = 0.f;
+                    if (XF) {
+                        vxn = v2x.x + dtbu * D.x;
+                    } else if (ZF || (recon && iz >= 0 && iz < g.nz)) {
+                        if (xint) vxn = v2x.x + dtbu * D.x;
+                        else if (xband) vxn = band_val(1, bf, r);
+                    }
+                    if (own) out2[(A_VX / 2) * pT + cz] = make_float2(vxn, lv);
+                    sVW[r * NTH + t] = make_float2(v2x.x, wx);
+                    sVN[r * NTH + t] = vxn;
+                    if ((t & 31) == 31) sPi[r * (NTH / 32) + (t >> 5)] = pix[r];
+                }
+            };
+            if (!zf) vx_stage(std::false_type{}, std::false_type{});
+            else if (xf) vx_stage(std::true_type{}, std::true_type{});
+            else vx_stage(std::true_type{}, std::false_type{});
             __syncthreads();
-
-            // ---- row z: nodes on the output columns
-            if (outcol) {
-                const float2 Ex = stencil<M, float2>(g.cx, [&](int l) { return sVW[t + l - 1]; },
-                                                     [&](int l) { return sVW[t - l]; });
-                const float2 Ez = stencil<M, float2>(g.cz, [&](int l) { return VW[u + M + l - 1]; },
-                                                     [&](int l) { return VW[u + M - l]; });
-                const float2 E = add_(Ex, Ez);
-                float qn = 0.f;
-                if (recon)
-                    qn = stencil<M, float>(g.cx, [&](int l) { return sVN[t + l - 1]; }, [&](int l) { return sVN[t - l]; }) +
-                         stencil<M, float>(g.cz, [&](int l) { return VN[u + M + l - 1]; },
-                                           [&](int l) { return VN[u + M - l]; });
-                const int iz = z - z0;
-                const bool inner = xint && iz >= 0 && iz < g.nz;
-                if (inner) {
-                    float2 acc = cur.img;
-                    acc.x += E.x * lp1;
-                    // (on the free surface the half row above is a ghost: no product of its own)
-                    acc.y += (sPi[t] + sPi[t - 1]) + (PIZ[u + M] + (surf ? 0.f : PIZ[u + M - 1]));
-                    img[cz] = acc;
-                }
-                float pn = 0.f;
-                if (recon) {
-                    if (inner) {
-                        pn = pbn + kd * qn;
-                        if (cz + x == src) pn -= wsrc;
-                    } else {
-                        long long b = pband_index(iz, ix, M, g.nz, nx);
-                        if (b >= 0) pn = band_get(a.bands, 0, rowprev, b);
-                    }
-                }
-                out2[(A_PL / 2) * p2 + cz] = (FS && z <= z0) ? make_float2(0.f, 0.f) : make_float2(pn, lp1 + E.y);
-                if (pmlxn) outf[A_LPVX * plane + cz] = bix * (cur.lpsvx - kl);
-                if ((z <= z0 - 1) || (z >= z1)) outf[A_LPVZ * plane + cz] = a.pml.bi[0][z] * (cur.lpsvz - kl);
-            }
-        }
-        if (fail_row < zc1) break;
+            // Gx lvx of the half node to the left: the lane below's, or the
+            // last lane's of the warp below (the first warp's first lane
+            // owns no output column)
+            float pil[2];
 #pragma unroll
-        for (int j = 0; j < W - 1; ++j) {
-            PU[j] = PU[j + U];
-            VW[j] = VW[j + U];
-            VN[j] = VN[j + U];
-            PIZ[j] = PIZ[j + U];
+            for (int r = 0; r < 2; ++r) {
+                pil[r] = __shfl_up_sync(0xffffffffu, pix[r], 1);
+                const float left = sPi[r * (NTH / 32) + max((t >> 5) - 1, 0)];
+                if ((t & 31) == 0) pil[r] = left;
+            }
+            // ---- rows z, z + 1: nodes on the output columns
+            auto node_stage = [&](auto zc, auto xc_) {
+                constexpr bool ZF = decltype(zc)::value, XF = decltype(xc_)::value;
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const int zr = z + r, cz = zr * pitch, iz = zr - z0;
+                    const bool own = outcol && (ZF || zr < zc1);
+                    const bool surf = !ZF && FS && zr == z0;   // free-surface row: p = 0, mu = 0
+                    const float2 *const vw = sVW + r * NTH + t;
+                    const float *const vn = sVN + r * NTH + t;
+                    // (Q_n, D- w) along x and z
+                    const float2 Ex = stencil<M, float2>(g.cx, [&](int l) { return vw[l - 1]; }, [&](int l) { return vw[-l]; });
+                    const float2 Ez = stencil<M, float2>(g.cz, [&](int l) { return VW[r + M + l - 1]; },
+                                                         [&](int l) { return VW[r + M - l]; });
+                    const float2 E = add_(Ex, Ez);
+                    float qn = 0.f;
+                    if (ZF || recon)
+                        qn = stencil<M, float>(g.cx, [&](int l) { return vn[l - 1]; }, [&](int l) { return vn[-l]; }) +
+                             stencil<M, float>(g.cz, [&](int l) { return VN[r + M + l - 1]; },
+                                               [&](int l) { return VN[r + M - l]; });
+                    const float kd = *reinterpret_cast<const float *>(st1 + L::KD + r * L::F1R);
+                    const float mu = pm[r].y;
+                    const bool inner = XF || (xint && (ZF || (iz >= 0 && iz < g.nz)));
+                    if (inner) {
+                        float2 acc = *reinterpret_cast<const float2 *>(st2 + L::IM + r * L::F2R);
+                        acc.x += E.x * mu;
+                        // (on the free surface the half row above is a ghost: no product of its own)
+                        acc.y += (pix[r] + pil[r]) + (PIZ[r + 1] + (surf ? 0.f : PIZ[r]));
+                        if (own) img[cz] = acc;
+                    }
+                    float pn = 0.f;
+                    if (ZF || recon) {
+                        if (inner) {
+                            pn = pm[r].x + kd * qn;
+                            pn -= cz + x == src ? wsrc : 0.f;
+                        } else if (ZF || (iz >= 0 && iz < g.nz)) {
+                            if (xband) pn = band_val(0, bf, r);
+                        } else if (xint && in_xstrip(iz, M, g.nz)) {
+                            pn = band_get(a.bands, 0, rowprev, band_zstrip(iz, ix, M, g.nz, nx));
+                        }
+                    }
+                    float2 pmn = make_float2(pn, fmaf(kd, E.y, mu));
+                    if (!ZF && FS && zr <= z0) pmn = make_float2(0.f, 0.f);
+                    if (own) out2[(A_PL / 2) * pT + cz] = pmn;
+                    if (!XF && own && pmlxn)
+                        outf[A_LPVX * pT + cz] = bix * (*reinterpret_cast<const float *>(st1 + L::LVX + r * L::F1R) - mu);
+                    if (!ZF && own && ((zr <= z0 - 1) || (zr >= z1)))
+                        outf[A_LPVZ * pT + cz] =
+                            a.pml.bi[0][zr] * (*reinterpret_cast<const float *>(st1 + L::LVZ + r * L::F1R) - mu);
+                }
+            };
+            if (!zf) node_stage(std::false_type{}, std::false_type{});
+            else if (xf) node_stage(std::true_type{}, std::true_type{});
+            else node_stage(std::true_type{}, std::false_type{});
         }
+#pragma unroll
+        for (int i = 0; i < W - 1; ++i) {
+            PU[i] = PU[i + U];
+            VW[i] = VW[i + U];
+            VN[i] = VN[i + U];
+        }
+#pragma unroll
+        for (int i = 0; i < M; ++i) PIZ[i] = PIZ[i + U];
     }
 
-    if (fail_row < zc1) {
-        // a wait gave up: record it, let the copies in flight land (rows up to
-        // fail_row + PDA - 1 were issued), return
-        if (t == PR) {
+    if (cband) cp_async_wait();
+    if (fail_j >= 0) {
+        // a wait gave up: record it, let the copies in flight land, return
+        if (t == NTH - 1) {
             atomicOr(a.err, 1);
-            for (int zz = fail_row; zz <= min(fail_row + PDA - 1, zc1 - 1); ++zz) {
-                const int jj = zz - zstart;
-                (void)tma::mbar_wait(bar + jj % PDA, (unsigned)(jj / PDA) & 1u);
-            }
+            for (int jj = fail_j; jj <= max(NS - 1, fail_j + NS - 2) && zstart + 2 * jj < zc1; ++jj)
+                (void)tma::mbar_wait(bar + jj % NS, (unsigned)(jj / NS) & 1u);
         }
         return;
     }
@@ -1493,20 +1104,34 @@ __global__ void __launch_bounds__(NTH, FS ? kAdjMinBlocksFS : kAdjMinBlocks) k_a
     if (recon) {
         // pre-add the residual of step n-1 at the receivers of this CTA
         __syncthreads();
-        int tile = shot * a.trec.ntiles + blockIdx.y * gridDim.x + blockIdx.x;
-        int b = a.trec.ptr[tile], e = a.trec.ptr[tile + 1];
-        float2 *plo = reinterpret_cast<float2 *>(a.out + slot * a.sstride + A_PL * plane);
+        const int tile = shot * a.trec.ntiles + blockIdx.y * gridDim.x + blockIdx.x;
+        const int b = a.trec.ptr[tile], e = a.trec.ptr[tile + 1];
+        float2 *plo = reinterpret_cast<float2 *>(a.out + slot * a.sstride) + (A_PL / 2) * pT;
         for (int i = b + t; i < e; i += NTH) {
-            int2 rc = a.trec.rec[i];
+            const int2 rc = a.trec.rec[i];
             if (i > b && a.trec.rec[i - 1].x == rc.x) continue;  // run handled by its first entry
             float add = 0.f;
             for (int q = i; q < e && a.trec.rec[q].x == rc.x; ++q)
                 add += a.dstage[(long long)a.trec.rec[q].y * g.nt + (n - 1)];
-            plo[rc.x].y += add;
+            plo[rc.x].y += kdt[rc.x] * add;
         }
     }
 }
 
+// Migration step of shots spanning the model and of shots with aperture windows.
+template <int M, bool FS>
+__global__ void __launch_bounds__(NTH, kAdjMinBlocks) k_adj2t(const __grid_constant__ Arg2D p)
+{
+    adj_body<M, false, FS>(p);
+}
+template <int M, bool FS>
+__global__ void __launch_bounds__(NTH, kAdjMinBlocks) k_adj2d(const __grid_constant__ Arg2D p)
+{
+    adj_body<M, true, FS>(p);
+}
+
+// Start state of a reverse pass: (p, 0), (vx, 0), (vz, 0) from the saved
+// background final state [p][vx][vz] of each shot of the batch.
 __global__ void k_pack_adj(const GridDev g, const float *final_state, int shot0, int batch, float *st,
                            long long sstride)
 {
@@ -1521,96 +1146,6 @@ __global__ void k_pack_adj(const GridDev g, const float *final_state, int shot0,
         o[(A_VX / 2) * plane + c] = make_float2(fs[plane + c], 0.f);
         o[(A_VZ / 2) * plane + c] = make_float2(fs[2 * plane + c], 0.f);
     }
-}
-
-template <int M, bool BORN, bool BANDS, bool HESS, bool WIN>
-cudaError_t launch_fwd_t(const Step2D &a, dim3 grid, cudaStream_t s)
-{
-    if (a.g.fs) k_fwd2d<M, BORN, BANDS, HESS, WIN, true><<<grid, NTH, kFwdStageBytes, s>>>(a);
-    else k_fwd2d<M, BORN, BANDS, HESS, WIN, false><<<grid, NTH, kFwdStageBytes, s>>>(a);
-    return cudaGetLastError();
-}
-
-template <int M, bool BORN, bool BANDS, bool HESS>
-cudaError_t attr_fwd()
-{
-    cudaError_t e;
-    const int b = (int)kFwdStageBytes;
-    const auto at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    if ((e = cudaFuncSetAttribute(k_fwd2d<M, BORN, BANDS, HESS, false, false>, at, b)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_fwd2d<M, BORN, BANDS, HESS, true, false>, at, b)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_fwd2d<M, BORN, BANDS, HESS, false, true>, at, b)) != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_fwd2d<M, BORN, BANDS, HESS, true, true>, at, b);
-}
-
-template <int M>
-cudaError_t attr_M()
-{
-    cudaError_t e;
-    if ((e = attr_fwd<M, true, false, false>()) != cudaSuccess) return e;
-    if ((e = attr_fwd<M, false, true, true>()) != cudaSuccess) return e;
-    if ((e = attr_fwd<M, false, true, false>()) != cudaSuccess) return e;
-    if ((e = attr_fwd<M, false, false, true>()) != cudaSuccess) return e;
-    if ((e = attr_fwd<M, false, false, false>()) != cudaSuccess) return e;
-    const int b = (int)kAdjStageBytes;
-    const auto at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    if ((e = cudaFuncSetAttribute(k_adj2d<M, false, false>, at, b)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_adj2d<M, true, false>, at, b)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_adj2d<M, false, true>, at, b)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_adj2d<M, true, true>, at, b)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_fwd2t<M, false>, at, (int)kFwdSmemT)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_fwd2t<M, true>, at, (int)kFwdSmemT)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_adj2t<M, false>, at, (int)kAdjSmemT)) != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_adj2t<M, true>, at, (int)kAdjSmemT);
-}
-
-template <int M, bool WIN>
-cudaError_t launch_fwd_MW(const Step2D &a, dim3 grid, bool born, bool bands, bool hess, cudaStream_t s)
-{
-    if (born) return launch_fwd_t<M, true, false, false, WIN>(a, grid, s);
-    if (bands && hess) return launch_fwd_t<M, false, true, true, WIN>(a, grid, s);
-    if (bands) return launch_fwd_t<M, false, true, false, WIN>(a, grid, s);
-    if (hess) return launch_fwd_t<M, false, false, true, WIN>(a, grid, s);
-    return launch_fwd_t<M, false, false, false, WIN>(a, grid, s);
-}
-
-template <int M>
-cudaError_t launch_fwd_M(const Step2D &a, int batch, bool born, bool bands, bool hess, cudaStream_t s,
-                         const Maps2D *maps)
-{
-    dim3 grid((a.g.Nx + Cols<M>::TXO - 1) / Cols<M>::TXO, (a.g.Nz + a.tzc - 1) / a.tzc, batch);
-    if (born && maps && !a.win_nx) {
-        if (!a.err) return cudaErrorInvalidValue;
-        Fwd2T p;
-        p.a = a;
-        p.m = *maps;
-        if (a.g.fs) k_fwd2t<M, true><<<grid, NTH, kFwdSmemT, s>>>(p);
-        else k_fwd2t<M, false><<<grid, NTH, kFwdSmemT, s>>>(p);
-        return cudaGetLastError();
-    }
-    if (a.win_nx) return launch_fwd_MW<M, true>(a, grid, born, bands, hess, s);
-    return launch_fwd_MW<M, false>(a, grid, born, bands, hess, s);
-}
-
-template <int M>
-cudaError_t launch_adj_M(const Step2D &a, const Maps2D *maps, int batch, cudaStream_t s)
-{
-    dim3 grid((a.g.Nx + Cols<M>::TXO - 1) / Cols<M>::TXO, (a.g.Nz + a.tzc - 1) / a.tzc, batch);
-    const bool w = a.win_nx != nullptr, f = a.g.fs != 0;
-    if (maps && !w) {
-        if (!a.err) return cudaErrorInvalidValue;
-        Adj2T p;
-        p.a = a;
-        p.m = *maps;
-        if (f) k_adj2t<M, true><<<grid, NTH, kAdjSmemT, s>>>(p);
-        else k_adj2t<M, false><<<grid, NTH, kAdjSmemT, s>>>(p);
-        return cudaGetLastError();
-    }
-    if (w && f) k_adj2d<M, true, true><<<grid, NTH, kAdjStageBytes, s>>>(a);
-    else if (w) k_adj2d<M, true, false><<<grid, NTH, kAdjStageBytes, s>>>(a);
-    else if (f) k_adj2d<M, false, true><<<grid, NTH, kAdjStageBytes, s>>>(a);
-    else k_adj2d<M, false, false><<<grid, NTH, kAdjStageBytes, s>>>(a);
-    return cudaGetLastError();
 }
 
 __global__ void k_window_model(const GridDev gm, const GridDev g, const int *win_x0, const int *win_nx, int shot0,
@@ -1655,6 +1190,87 @@ __global__ void k_window_model(const GridDev gm, const GridDev g, const int *win
     }
 }
 
+
+template <class K>
+cudaError_t set_smem(K k, unsigned bytes)
+{
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+// Calls f(WIN, FS) as compile-time constants.
+template <class F>
+cudaError_t with_flags(bool win, bool fs, F &&f)
+{
+    using T = std::true_type;
+    using N = std::false_type;
+    if (win) return fs ? f(T{}, T{}) : f(T{}, N{});
+    return fs ? f(N{}, T{}) : f(N{}, N{});
+}
+
+template <int M, bool BANDS, bool HESS>
+cudaError_t launch_bg(const Arg2D &p, dim3 grid, cudaStream_t s)
+{
+    return with_flags(p.a.win_nx != nullptr, p.a.g.fs != 0, [&](auto w, auto f) {
+        k_fwd2d<M, BANDS, HESS, decltype(w)::value, decltype(f)::value><<<grid, NTH, FwdLay<M, false, HESS>::SMEM, s>>>(p);
+        return cudaGetLastError();
+    });
+}
+
+template <int M>
+cudaError_t launch_fwd_M(const Arg2D &p, int batch, bool born, bool bands, bool hess, cudaStream_t s)
+{
+    const Step2D &a = p.a;
+    const dim3 grid((a.g.Nx + Cols<M>::TXO - 1) / Cols<M>::TXO, (a.g.Nz + a.tzc - 1) / a.tzc, batch);
+    if (born)
+        return with_flags(a.win_nx != nullptr, a.g.fs != 0, [&](auto w, auto f) {
+            if constexpr (decltype(w)::value) k_fwd2w<M, decltype(f)::value><<<grid, NTH, FwdLay<M, true, false>::SMEM, s>>>(p);
+            else k_fwd2t<M, decltype(f)::value><<<grid, NTH, FwdLay<M, true, false>::SMEM, s>>>(p);
+            return cudaGetLastError();
+        });
+    if (bands && hess) return launch_bg<M, true, true>(p, grid, s);
+    if (bands) return launch_bg<M, true, false>(p, grid, s);
+    if (hess) return launch_bg<M, false, true>(p, grid, s);
+    return launch_bg<M, false, false>(p, grid, s);
+}
+
+template <int M>
+cudaError_t launch_adj_M(const Arg2D &p, int batch, cudaStream_t s)
+{
+    const Step2D &a = p.a;
+    const dim3 grid((a.g.Nx + Cols<M>::TXO - 1) / Cols<M>::TXO, (a.g.Nz + a.tzc - 1) / a.tzc, batch);
+    return with_flags(a.win_nx != nullptr, a.g.fs != 0, [&](auto w, auto f) {
+        if constexpr (decltype(w)::value) k_adj2d<M, decltype(f)::value><<<grid, NTH, AdjLayM<M>::SMEM, s>>>(p);
+        else k_adj2t<M, decltype(f)::value><<<grid, NTH, AdjLayM<M>::SMEM, s>>>(p);
+        return cudaGetLastError();
+    });
+}
+
+template <int M>
+cudaError_t attr_M()
+{
+    cudaError_t e = cudaSuccess;
+    auto set = [&](auto k, unsigned bytes) {
+        if (e == cudaSuccess) e = set_smem(k, bytes);
+    };
+    for (int i = 0; i < 4; ++i)
+        with_flags(i & 1, i & 2, [&](auto w, auto f) {
+            constexpr bool WIN = decltype(w)::value, FS = decltype(f)::value;
+            set(k_fwd2d<M, true, true, WIN, FS>, FwdLay<M, false, true>::SMEM);
+            set(k_fwd2d<M, true, false, WIN, FS>, FwdLay<M, false, false>::SMEM);
+            set(k_fwd2d<M, false, true, WIN, FS>, FwdLay<M, false, true>::SMEM);
+            set(k_fwd2d<M, false, false, WIN, FS>, FwdLay<M, false, false>::SMEM);
+            if constexpr (WIN) {
+                set(k_fwd2w<M, FS>, FwdLay<M, true, false>::SMEM);
+                set(k_adj2d<M, FS>, AdjLayM<M>::SMEM);
+            } else {
+                set(k_fwd2t<M, FS>, FwdLay<M, true, false>::SMEM);
+                set(k_adj2t<M, FS>, AdjLayM<M>::SMEM);
+            }
+            return cudaSuccess;
+        });
+    return e;
+}
+
 }  // namespace
 
 int march2d_txo(int M) { return M == 2 ? Cols<2>::TXO : Cols<4>::TXO; }
@@ -1685,39 +1301,57 @@ cudaError_t ensure_kernels_configured()
     return cudaSuccess;
 }
 
-cudaError_t launch_fwd2d(const Step2D &a, int batch, bool born, bool save_bands, bool hess, cudaStream_t s,
-                         const Maps2D *maps)
+cudaError_t launch_fwd2d(const Step2D &a, const Maps2D &maps, int batch, bool born, bool save_bands, bool hess, cudaStream_t s)
 {
-    if (a.g.M == 2) return launch_fwd_M<2>(a, batch, born, save_bands, hess, s, maps);
-    return launch_fwd_M<4>(a, batch, born, save_bands, hess, s, maps);
+    if (!a.err) return cudaErrorInvalidValue;
+    const Arg2D p{a, maps};
+    if (a.g.M == 2) return launch_fwd_M<2>(p, batch, born, save_bands, hess, s);
+    return launch_fwd_M<4>(p, batch, born, save_bands, hess, s);
 }
 
-cudaError_t launch_adj2d(const Step2D &a, const Maps2D *maps, int batch, cudaStream_t s)
+cudaError_t launch_adj2d(const Step2D &a, const Maps2D &maps, int batch, cudaStream_t s)
 {
-    if (a.g.M == 2) return launch_adj_M<2>(a, maps, batch, s);
-    return launch_adj_M<4>(a, maps, batch, s);
+    if (!a.err) return cudaErrorInvalidValue;
+    const Arg2D p{a, maps};
+    if (a.g.M == 2) return launch_adj_M<2>(p, batch, s);
+    return launch_adj_M<4>(p, batch, s);
 }
 
-cudaError_t maps2d(Maps2D *m, const GridDev &g, const float *st, long long sstride, const float *kdt,
-                   const float *binv, const float2 *kd2, const float2 *br2, const float2 *img, int batch)
+cudaError_t maps2d(Maps2D *m, const GridDev &gm, const GridDev &g, const float *st, long long sstride, const float *kdt,
+                   const float *binv, const float2 *kd2, const float2 *br2, const float2 *img, const float *psiv,
+                   long long vstride, int batch)
 {
     // the two model arrays of each kind are one map: their planes must be adjacent
-    if (binv != kdt + g.plane || br2 != kd2 + g.plane || sstride % (2 * g.plane)) return cudaErrorInvalidValue;
+    if (binv != kdt + gm.plane || br2 != kd2 + gm.plane) return cudaErrorInvalidValue;
+    // (the pair map of a slot with an odd number of planes, a background-only
+    // state, is never read)
     m->pps = (int)(sstride / (2 * g.plane));
     m->fps = (int)(sstride / g.plane);
-    const cuuint32_t box[3] = {(cuuint32_t)NTH, 1, 1};
+    m->pvs = (int)(vstride / g.plane);
+    const auto u64 = CU_TENSOR_MAP_DATA_TYPE_UINT64, f32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     const cuuint64_t s8[2] = {(cuuint64_t)g.pitch * 8, (cuuint64_t)g.plane * 8};
     const cuuint64_t s4[2] = {(cuuint64_t)g.pitch * 4, (cuuint64_t)g.plane * 4};
-    const cuuint64_t dpr[3] = {(cuuint64_t)g.Nx, (cuuint64_t)g.Nz, (cuuint64_t)batch * m->pps};
-    const cuuint64_t dfl[3] = {(cuuint64_t)g.Nx, (cuuint64_t)g.Nz, (cuuint64_t)batch * m->fps};
-    const cuuint64_t dmd[3] = {(cuuint64_t)g.Nx, (cuuint64_t)g.Nz, 2};
-    const cuuint64_t dim[3] = {(cuuint64_t)g.Nx, (cuuint64_t)g.Nz, (cuuint64_t)batch};
-    cudaError_t e;
-    if ((e = encode_tmap(&m->pr, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, st, dpr, s8, box)) != cudaSuccess) return e;
-    if ((e = encode_tmap(&m->fl, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, st, dfl, s4, box)) != cudaSuccess) return e;
-    if ((e = encode_tmap(&m->md, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, kdt, dmd, s4, box)) != cudaSuccess) return e;
-    if ((e = encode_tmap(&m->mb, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, kd2, dmd, s8, box)) != cudaSuccess) return e;
-    return encode_tmap(&m->im, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, img, dim, s8, box);
+    const cuuint64_t nx = (cuuint64_t)g.Nx, nz = (cuuint64_t)g.Nz;
+    const cuuint64_t dpr[3] = {nx, nz, (cuuint64_t)batch * m->pps}, dfl[3] = {nx, nz, (cuuint64_t)batch * m->fps};
+    const cuuint64_t dim[3] = {nx, nz, (cuuint64_t)batch};
+    // the model grid (without aperture windows the slots' own grid)
+    const cuuint64_t dmd[3] = {(cuuint64_t)gm.Nx, (cuuint64_t)gm.Nz, 2};
+    const cuuint64_t m8[2] = {(cuuint64_t)gm.pitch * 8, (cuuint64_t)gm.plane * 8};
+    const cuuint64_t m4[2] = {(cuuint64_t)gm.pitch * 4, (cuuint64_t)gm.plane * 4};
+    for (int r = 0; r < 2; ++r) {
+        const cuuint32_t box[3] = {(cuuint32_t)NTH, (cuuint32_t)(r + 1), 1};
+        cudaError_t e;
+        if ((e = encode_tmap(&m->pr[r], u64, 3, st, dpr, s8, box)) != cudaSuccess) return e;
+        if ((e = encode_tmap(&m->fl[r], f32, 3, st, dfl, s4, box)) != cudaSuccess) return e;
+        if ((e = encode_tmap(&m->md[r], f32, 3, kdt, dmd, m4, box)) != cudaSuccess) return e;
+        if ((e = encode_tmap(&m->mb[r], u64, 3, kd2, dmd, m8, box)) != cudaSuccess) return e;
+        // two-row boxes over its floats and its pairs
+        const cuuint64_t dpv[3] = {nx, nz, (cuuint64_t)batch * (r ? m->pvs / 2 : m->pvs)};
+        const cuuint32_t box2[3] = {(cuuint32_t)NTH, 2, 1};
+        if ((e = encode_tmap(&m->pv[r], r ? u64 : f32, 3, psiv, dpv, r ? s8 : s4, box2)) != cudaSuccess) return e;
+        if (img && (e = encode_tmap(&m->im[r], u64, 3, img, dim, s8, box)) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_window_model(const GridDev &gm, const GridDev &g, const int *win_x0, const int *win_nx,

@@ -75,8 +75,8 @@ __global__ void k_pert_prep(GridDev g, const float *dm, const float *kdt, const 
     }
 }
 
-__global__ void k_inject(GridDev g, TileRecs tr, int shot0, const float *dstage, int n, float2 *pl,
-                         long long sstride2)
+__global__ void k_inject(GridDev gm, GridDev g, TileRecs tr, int shot0, const float *dstage, int n, const float *kdt,
+                         const int *win_x0, float2 *pl, long long sstride2)
 {
     int slot = blockIdx.y;
     int t = (shot0 + slot) * tr.ntiles + blockIdx.x;
@@ -88,6 +88,11 @@ __global__ void k_inject(GridDev g, TileRecs tr, int shot0, const float *dstage,
         float add = 0.f;
         for (int k = i; k < e && tr.rec[k].x == rc.x; ++k)
             add += dstage[(long long)tr.rec[k].y * g.nt + n];
+        if (kdt) {
+            // node of the model grid (windowed shots, 2D: z and the column in the window)
+            const long long c = win_x0 ? (long long)(rc.x / g.pitch) * gm.pitch + rc.x % g.pitch + win_x0[shot0 + slot] : rc.x;
+            add *= kdt[c];
+        }
         dst[rc.x].y += add;
     }
 }
@@ -166,7 +171,7 @@ __global__ void k_image_fin(GridDev g, const double2 *acc, const float *kdt, con
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < nint;
          k += (long long)gridDim.x * blockDim.x) {
         long long c = pad_of(g, k);
-        double gk = -(double)kdt[c] * acc[k].x;
+        double gk = g.ndim == 2 ? -acc[k].x : -(double)kdt[c] * acc[k].x;   // (2D: acc.x holds sum Q dt kappa lp)
         double gr = 0.5 * (double)g.dt * (double)binv[c] * acc[k].y;
         gout[k] = (float)(gk - gr);
         gout[nint + k] = (float)(gk + gr);
@@ -530,12 +535,12 @@ cudaError_t launch_pert_prep(const GridDev &g, const float *dm, const float *kdt
     return cudaGetLastError();
 }
 
-cudaError_t launch_inject_residual(const GridDev &g, const TileRecs &tr, int batch, int shot0,
-                                   const float *dstage, int n, float2 *pl, long long sstride2,
-                                   cudaStream_t s)
+cudaError_t launch_inject_residual(const GridDev &gm, const GridDev &g, const TileRecs &tr, int batch, int shot0,
+                                   const float *dstage, int n, const float *kdt, const int *win_x0, float2 *pl,
+                                   long long sstride2, cudaStream_t s)
 {
     dim3 grid(tr.ntiles, batch);
-    k_inject<<<grid, 64, 0, s>>>(g, tr, shot0, dstage, n, pl, sstride2);
+    k_inject<<<grid, 64, 0, s>>>(gm, g, tr, shot0, dstage, n, kdt, win_x0, pl, sstride2);
     return cudaGetLastError();
 }
 

@@ -127,7 +127,7 @@ struct TileRecs {
     int ntiles;           // tiles per shot
 };
 
-// Arguments of the fused 2D time-step kernels.
+// Arguments of the 2D time-step kernels.
 struct Step2D {
     GridDev g;
     Pml pml;
@@ -269,26 +269,27 @@ constexpr int kThreads2D = 256;
 int march2d_txo(int M);
 
 // Launchers (kernels2d.cu). Return the cudaError of the launch.
-struct Maps2D;
-// maps (Born modelling only): TMA row staging, as for launch_adj2d.
-cudaError_t launch_fwd2d(const Step2D &a, int batch, bool born, bool save_bands, bool hess,
-                         cudaStream_t s, const Maps2D *maps = nullptr);
-// TMA row maps of the 2D Born and migration kernels reading one state buffer
-// (boxes one kThreads2D-wide row of one field): pr over the float2 pair planes
-// of every slot (8-byte elements; coordinates x, z, slot * pps + pair), fl
-// over its float planes (x, z, slot * fps + plane), md over dt kappa and
-// 1/rho (x, z, 0 | 1), mb over the Born model pairs (dt kappa, dt kappa
+// TMA row maps of the 2D kernels reading one state buffer, [0] with boxes of
+// one and [1] of two kThreads2D-wide rows of one field: pr over the float2
+// pair planes of every slot (8-byte elements; coordinates x, z, slot * pps +
+// pair), fl over its float planes (x, z, slot * fps + plane), md over dt kappa
+// and 1/rho (x, z, 0 | 1), mb over the Born model pairs (dt kappa, dt kappa
 // dlnk), (1/rho, rr) (x, z, 0 | 1), im over the image accumulators (x, z,
-// slot). Outside the padded grid the copies read zeros.
+// slot). pv: two-row boxes over the in-place node CPML memories (pvs planes a
+// slot) as floats [0] (x, z, slot * pvs + plane) and float2 pairs [1].
+// Outside the padded grid the copies read zeros. gm is the model's grid,
+// g the slots' (the same without aperture windows); img may be null where no
+// migration step uses the maps.
 struct Maps2D {
-    CUtensorMap pr, fl, md, mb, im;
-    int pps, fps;
+    CUtensorMap pr[2], fl[2], md[2], mb[2], im[2], pv[2];
+    int pps, fps, pvs;
 };
-cudaError_t maps2d(Maps2D *m, const GridDev &g, const float *st, long long sstride, const float *kdt,
-                   const float *binv, const float2 *kd2, const float2 *br2, const float2 *img, int batch);
-// maps: TMA row staging (shots without aperture windows), or null for the
-// per-thread asynchronous copies.
-cudaError_t launch_adj2d(const Step2D &a, const Maps2D *maps, int batch, cudaStream_t s);
+cudaError_t maps2d(Maps2D *m, const GridDev &gm, const GridDev &g, const float *st, long long sstride, const float *kdt,
+                   const float *binv, const float2 *kd2, const float2 *br2, const float2 *img, const float *psiv,
+                   long long vstride, int batch);
+cudaError_t launch_fwd2d(const Step2D &a, const Maps2D &maps, int batch, bool born, bool save_bands, bool hess,
+                         cudaStream_t s);
+cudaError_t launch_adj2d(const Step2D &a, const Maps2D &maps, int batch, cudaStream_t s);
 // cuTensorMapEncodeTiled (element strides 1, no swizzle, zero fill).
 cudaError_t encode_tmap(CUtensorMap *m, CUtensorMapDataType type, int rank, const void *base, const cuuint64_t *dims,
                         const cuuint64_t *strides, const cuuint32_t *box);
@@ -343,15 +344,19 @@ cudaError_t launch_model_prep(const GridDev &g, const float *vp, const float *rh
                               float *binv, cudaStream_t s);
 cudaError_t launch_pert_prep(const GridDev &g, const float *dm, const float *kdt,
                              const float *binv, float2 *kd2, float2 *br2, cudaStream_t s);
-// Adds the residual of step n to lambda_p (the .y of the (p, lambda_p) pairs).
-cudaError_t launch_inject_residual(const GridDev &g, const TileRecs &tr, int batch, int shot0,
-                                   const float *dstage, int n, float2 *pl, long long sstride2,
-                                   cudaStream_t s);
+// Adds the residual of step n to lambda_p (the .y of the (p, lambda_p)
+// pairs), times dt kappa of the node where the state carries dt kappa lambda_p
+// (kdt non-null: planes of the model grid gm, of which shot s's slot grid g
+// takes the columns from win_x0[s], or all with win_x0 null).
+cudaError_t launch_inject_residual(const GridDev &gm, const GridDev &g, const TileRecs &tr, int batch, int shot0,
+                                   const float *dstage, int n, const float *kdt, const int *win_x0, float2 *pl,
+                                   long long sstride2, cudaStream_t s);
 // Stacks the batch's per-slot images (grid g) into the FP64 interior image of
 // the model grid gm; with aperture windows (win_x0 non-null) slot b covers the
 // columns [win_x0, win_x0 + win_nx) of shot shot0 + b.
 cudaError_t launch_image_accumulate(const GridDev &gm, const GridDev &g, const float2 *img, int batch, int shot0,
                                     const int *win_x0, const int *win_nx, double2 *acc, cudaStream_t s);
+// The kappa image of 2D grids holds sum Q dt kappa lambda_p, of 3D grids sum Q lambda_p.
 cudaError_t launch_image_finalize(const GridDev &g, const double2 *acc, const float *kdt,
                                   const float *binv, float *gout, cudaStream_t s);
 cudaError_t launch_hess_accumulate(const GridDev &gm, const GridDev &g, const float *hess, int batch, int shot0,

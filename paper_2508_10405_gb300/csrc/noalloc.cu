@@ -240,10 +240,10 @@ extern "C" lsrtm_status lsrtm_born_static(const lsrtm_config *cfg, const float *
     // carve the static workspace
     const size_t P = (size_t)g.plane;
     size_t off[16], sz[16];
-    sz[0] = P * 4;                          // kdt
-    sz[1] = P * 4;                          // binv
-    sz[2] = P * 8;                          // kd2
-    sz[3] = P * 8;                          // br2
+    sz[0] = 2 * align256(P * 4);            // kdt, binv (adjacent: one tensor map covers both)
+    sz[1] = 0;
+    sz[2] = 2 * align256(P * 8);            // kd2, br2 (adjacent)
+    sz[3] = 0;
     sz[4] = 4 * ((size_t)g.Nz + 1 + g.Nx) * 4;   // CPML profiles
     sz[5] = (size_t)nshot * 4;              // src_idx copy
     sz[6] = (size_t)(nshot + 1) * 4;        // rec_ptr copy
@@ -281,9 +281,9 @@ extern "C" lsrtm_status lsrtm_born_static(const lsrtm_config *cfg, const float *
     } while (0)
 
     float *kdt = reinterpret_cast<float *>(at(0));
-    float *binv = reinterpret_cast<float *>(at(1));
+    float *binv = kdt + P;
     float2 *kd2 = reinterpret_cast<float2 *>(at(2));
-    float2 *br2 = reinterpret_cast<float2 *>(at(3));
+    float2 *br2 = kd2 + P;
     float *prof = reinterpret_cast<float *>(at(4));
     int *src_copy = reinterpret_cast<int *>(at(5));
     int *rp_copy = reinterpret_cast<int *>(at(6));
@@ -298,7 +298,6 @@ extern "C" lsrtm_status lsrtm_born_static(const lsrtm_config *cfg, const float *
 
     // model, perturbation and profiles
     SCU(cudaMemsetAsync(kdt, 0, sz[0], s));
-    SCU(cudaMemsetAsync(binv, 0, sz[1], s));
     SCU(launch_model_prep(g, vp, rho, kdt, binv, s));
     SCU(launch_pert_prep(g, dm, kdt, binv, kd2, br2, s));
     Pml pml{};
@@ -351,6 +350,12 @@ extern "C" lsrtm_status lsrtm_born_static(const lsrtm_config *cfg, const float *
     a.trec.rec = trec;
     a.trec.ntiles = ntiles;
     a.dstage = d;   // records go straight to the caller's output
+    // the kernels' error word takes the first tile cursor's place once the tables are built
+    a.err = tcur;
+    SCU(cudaMemsetAsync(a.err, 0, sizeof(int), s));
+    Maps2D maps[2];
+    SCU(maps2d(&maps[0], g, g, st0, a.sstride, kdt, binv, kd2, br2, nullptr, psiv, a.vstride, 1));
+    SCU(maps2d(&maps[1], g, g, st1, a.sstride, kdt, binv, kd2, br2, nullptr, psiv, a.vstride, 1));
     for (int shot = 0; shot < nshot; ++shot) {
         SCU(cudaMemsetAsync(st0, 0, sz[12], s));
         SCU(cudaMemsetAsync(st1, 0, sz[13], s));
@@ -360,7 +365,7 @@ extern "C" lsrtm_status lsrtm_born_static(const lsrtm_config *cfg, const float *
             a.n = n;
             a.in = (n & 1) ? st1 : st0;
             a.out = (n & 1) ? st0 : st1;
-            SCU(launch_fwd2d(a, 1, true, false, false, s));
+            SCU(launch_fwd2d(a, maps[n & 1], 1, true, false, false, s));
         }
     }
 #undef SCU
