@@ -1340,7 +1340,7 @@ lsrtm_status create_impl(const lsrtm_config *cfg, const float *vp, const float *
         g.cx[l] = (float)(cl / cfg->dx);
     }
     h->nint = (long long)g.nz * g.ny * g.nx;
-    // CTA blocking: output columns fixed by the kernel, z-chunks of about 112 rows
+    // CTA blocking: output columns fixed by the kernel, z-chunks by the work
     h->txo = march2d_txo(g.M);
     if (d3) {
         // enough CTAs for two waves of one CTA per SM, chunks of at least 8M rows
@@ -1349,8 +1349,17 @@ lsrtm_status create_impl(const lsrtm_config *cfg, const float *vp, const float *
         const int nchunk = std::max(1, std::min(want, g.Nz / (8 * g.M)));
         h->tzc = (g.Nz + nchunk - 1) / nchunk;
     } else {
-        int nchunk = std::max(1, (g.Nz + 56) / 112);
-        h->tzc = (g.Nz + nchunk - 1) / nchunk;
+        // CTAs over the columns of a batch's shots (all shots, unless the plan
+        // or the caller says fewer; a batch that memory limits fills the GPU)
+        const int ns = geo_nshot(geo), per = cfg->plan == LSRTM_PLAN_PLAIN ? 1 : cfg->shots_per_batch;
+        const int bs = per > 0 ? std::min(per, ns) : ns;
+        long long ctas = 0;
+        for (int s = 0; s < bs; ++s) {
+            const bool w = geo && geo->win_x0 && geo->win_nx && geo->nshot > 0;
+            const long long nx = (w ? std::max(1, std::min(geo->win_nx[s], g.nx)) : g.nx) + 2LL * cfg->npml;
+            ctas += (nx + h->txo - 1) / h->txo;
+        }
+        h->tzc = march2d_rows(g.M, g.Nz, ctas);
     }
     h->src_scale = (float)(d3 ? cfg->dt / (cfg->dz * cfg->dy * cfg->dx) : cfg->dt / (cfg->dz * cfg->dx));
 

@@ -28,6 +28,7 @@
 // their slot) and x CPML profiles; CTAs past a shot's width exit at once.
 // Every state and model plane of a slot is zero past the shot's width.
 #include <algorithm>
+#include <cmath>
 #include <mutex>
 #include <type_traits>
 
@@ -1274,6 +1275,36 @@ cudaError_t attr_M()
 }  // namespace
 
 int march2d_txo(int M) { return M == 2 ? Cols<2>::TXO : Cols<4>::TXO; }
+
+// A chunk of t rows costs its CTA t + 2M rows (the warm-up ones included) and a
+// start of about 7 rows' time (barriers, first copies, the ring's prologue).
+// Up to three CTAs share an SM almost for free (a CTA alone waits for its own
+// latencies most of the time: 1.1x its time with two on the SM, 1.25x with
+// three), so a small batch is split until every SM has one to three CTAs: 1
+// shot of 141 x 141 (order 4) 258 us a Born and migration step in one chunk, 23
+// in chunks of 4; 16 shots of 240 x 240 209 -> 46 (10 rows); 12 shots of 227 x
+// 451 (order 8) 284 -> 77 (12 rows). Past three, the starts hide behind other
+// CTAs and what counts is the work repeated and the last wave (0.7 of one on
+// average): 96 shots of 424 x 1192 take 1483 us in chunks of 106 rows, 1453 in
+// 72, 1484 in 40, 1763 in 14.
+int march2d_rows(int M, int Nz, long long ctas)
+{
+    constexpr double sms = 152.0, three = 1.25;
+    double best = 1e300;
+    int rows = Nz;
+    for (int nc = 1; nc <= std::max(1, Nz / 2); ++nc) {
+        int t = (Nz + nc - 1) / nc;
+        t += t & 1;   // whole groups of two rows
+        const double n = (double)ctas * ((Nz + t - 1) / t), q = std::ceil(n / sms);
+        const double c = q <= 3.0 ? (t + 2 * M + 7) * (q <= 1.0 ? 1.0 : (q <= 2.0 ? 1.1 : three))
+                                  : (t + M + 3) * three * (n / (3.0 * sms) + 0.7);
+        if (c < best) {
+            best = c;
+            rows = t;
+        }
+    }
+    return rows;
+}
 
 cudaError_t configure_2d_kernels()
 {

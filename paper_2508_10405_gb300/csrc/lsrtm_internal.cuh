@@ -267,6 +267,9 @@ cudaError_t launch_fwd3d(const Step3D &a, int batch, bool bands, bool hess, int 
 // march2d_txo(M) output columns and a z-chunk of Step2D::tzc rows.
 constexpr int kThreads2D = 256;
 int march2d_txo(int M);
+// Rows per z-chunk for a padded depth Nz when a chunk has `ctas` CTAs over the
+// columns and the shots of a batch (kernels2d.cu).
+int march2d_rows(int M, int Nz, long long ctas);
 
 // Launchers (kernels2d.cu). Return the cudaError of the launch.
 // TMA row maps of the 2D kernels reading one state buffer, [0] with boxes of

@@ -232,10 +232,11 @@ extern "C" lsrtm_status lsrtm_born_static(const lsrtm_config *cfg, const float *
         if (geom->rec_idx[r] < 0 || geom->rec_idx[r] >= nint)
             return fail(LSRTM_ERR_GEOMETRY, "receiver outside the interior grid");
     const int txo = march2d_txo(M);
-    const int nchunk = (g.Nz + 56) / 112 > 1 ? (g.Nz + 56) / 112 : 1;
-    const int tzc = (g.Nz + nchunk - 1) / nchunk;
-    const int ntx = (g.Nx + txo - 1) / txo, ntz = (g.Nz + tzc - 1) / tzc;
-    const int ntiles = ntx * ntz;
+    const int ntx = (g.Nx + txo - 1) / txo;
+    // z-chunks for one shot's CTAs; where their receiver tables would not fit
+    // the workspace, chunks of about 112 rows
+    const int nfew = (g.Nz + 56) / 112 > 1 ? (g.Nz + 56) / 112 : 1;
+    int tzc = march2d_rows(M, g.Nz, ntx), ntiles = 0;
 
     // carve the static workspace
     const size_t P = (size_t)g.plane;
@@ -249,16 +250,22 @@ extern "C" lsrtm_status lsrtm_born_static(const lsrtm_config *cfg, const float *
     sz[6] = (size_t)(nshot + 1) * 4;        // rec_ptr copy
     sz[7] = (size_t)(nrec > 0 ? nrec : 1) * 4;   // rec_idx copy
     sz[8] = (size_t)nshot * 4;              // src_cell
-    sz[9] = ((size_t)nshot * ntiles + 1) * 4;    // tile receiver offsets
-    sz[10] = (size_t)nshot * ntiles * 4;    // tile cursors
     sz[11] = (size_t)(nrec > 0 ? nrec : 1) * 8;  // tile receivers
     sz[12] = 10 * P * 4;                    // wavefield ping
     sz[13] = 10 * P * 4;                    // wavefield pong
     sz[14] = 4 * P * 4;                     // node CPML memories
     size_t total = 0;
-    for (int i = 0; i < 15; ++i) {
-        off[i] = total;
-        total += align256(sz[i]);
+    for (int fewer = 0; fewer < 2; ++fewer) {
+        if (fewer) tzc = (g.Nz + nfew - 1) / nfew;
+        ntiles = ntx * ((g.Nz + tzc - 1) / tzc);
+        sz[9] = ((size_t)nshot * ntiles + 1) * 4;    // tile receiver offsets
+        sz[10] = (size_t)nshot * ntiles * 4;    // tile cursors
+        total = 0;
+        for (int i = 0; i < 15; ++i) {
+            off[i] = total;
+            total += align256(sz[i]);
+        }
+        if (total <= kStaticBytes) break;
     }
     if (total > kStaticBytes) {
         char buf[200];
