@@ -912,7 +912,7 @@ lsrtm_status adjoint_core_ckpt(lsrtm_handle *h, float *gout, bool want_hess)
         h->launches++;
         h->hess_ready = true;
     }
-    CU(launch_image_finalize(h->gm, h->img_acc, h->kdt, h->binv, gout, h->work));
+    CU(launch_image_finalize(h->gm, h->img_acc, h->binv, gout, h->work));
     h->launches++;
     return LSRTM_OK;
 }
@@ -966,7 +966,7 @@ lsrtm_status adjoint_core(lsrtm_handle *h, float *gout, bool want_hess)
             h->launches++;
         }
     }
-    CU(launch_image_finalize(h->gm, h->img_acc, h->kdt, h->binv, gout, h->work));
+    CU(launch_image_finalize(h->gm, h->img_acc, h->binv, gout, h->work));
     h->launches++;
     return LSRTM_OK;
 }
@@ -1265,7 +1265,7 @@ lsrtm_status adj3f_step(lsrtm_handle *h, int i, int n, int s0, const Bands &band
 lsrtm_status adj3f_start(lsrtm_handle *h, int fs0, int s0, int bs)
 {
     CU(launch_pack3f(h->g, h->final_state, fs0, bs, h->st[0], h->sstride, h->work));
-    CU(launch_inject_residual(h->gm, h->g, h->trv, bs, s0, h->dstage, h->g.nt - 1, nullptr, nullptr,
+    CU(launch_inject_residual(h->gm, h->g, h->trv, bs, s0, h->dstage, h->g.nt - 1, h->kdt, nullptr,
                               reinterpret_cast<float2 *>(h->st[0]), h->sstride / 2, h->work));
     h->launches += 2;
     return LSRTM_OK;
@@ -1342,24 +1342,26 @@ lsrtm_status create_impl(const lsrtm_config *cfg, const float *vp, const float *
     h->nint = (long long)g.nz * g.ny * g.nx;
     // CTA blocking: output columns fixed by the kernel, z-chunks by the work
     h->txo = march2d_txo(g.M);
-    if (d3) {
-        // enough CTAs for two waves of one CTA per SM, chunks of at least 8M rows
-        const int ntxy = ((g.Nx + kTile3X - 1) / kTile3X) * ((g.Ny + kTile3Y - 1) / kTile3Y);
-        const int want = (2 * 152 + ntxy * geo_nshot(geo) - 1) / std::max(1, ntxy * geo_nshot(geo));
-        const int nchunk = std::max(1, std::min(want, g.Nz / (8 * g.M)));
-        h->tzc = (g.Nz + nchunk - 1) / nchunk;
-    } else {
+    {
         // CTAs over the columns of a batch's shots (all shots, unless the plan
         // or the caller says fewer; a batch that memory limits fills the GPU)
         const int ns = geo_nshot(geo), per = cfg->plan == LSRTM_PLAN_PLAIN ? 1 : cfg->shots_per_batch;
         const int bs = per > 0 ? std::min(per, ns) : ns;
-        long long ctas = 0;
-        for (int s = 0; s < bs; ++s) {
+        if (d3) {
+            const long long ntxy = (long long)((g.Nx + kTile3X - 1) / kTile3X) * ((g.Ny + kTile3Y - 1) / kTile3Y);
+            // enough CTAs for two waves of one CTA per SM, chunks of at least 8M rows
+            const long long want = (2 * 152 + ntxy * ns - 1) / std::max(1LL, ntxy * ns);
+            const int nchunk = (int)std::max(1LL, std::min(want, (long long)(g.Nz / (8 * g.M))));
+            h->tzc = (g.Nz + nchunk - 1) / nchunk;
+        } else {
             const bool w = geo && geo->win_x0 && geo->win_nx && geo->nshot > 0;
-            const long long nx = (w ? std::max(1, std::min(geo->win_nx[s], g.nx)) : g.nx) + 2LL * cfg->npml;
-            ctas += (nx + h->txo - 1) / h->txo;
+            long long ctas = 0;
+            for (int s = 0; s < bs; ++s) {
+                const long long nx = (w ? std::max(1, std::min(geo->win_nx[s], g.nx)) : g.nx) + 2LL * cfg->npml;
+                ctas += (nx + h->txo - 1) / h->txo;
+            }
+            h->tzc = march2d_rows(g.M, g.Nz, ctas);
         }
-        h->tzc = march2d_rows(g.M, g.Nz, ctas);
     }
     h->src_scale = (float)(d3 ? cfg->dt / (cfg->dz * cfg->dy * cfg->dx) : cfg->dt / (cfg->dz * cfg->dx));
 

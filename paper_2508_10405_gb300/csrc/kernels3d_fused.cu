@@ -5,13 +5,13 @@
 //
 // A CTA of 384 threads owns a 32 x 12 tile of (x, y) columns, one column per
 // thread, and marches down a z-chunk (two CTAs per SM):
-//   * z stencils: per-thread register rings of length 2M (+1 look-ahead),
-//     shifted after every row;
+//   * z stencils: per-thread register rings of length 2M, shifted after every
+//     row;
 //   * x and y stencils: shared-memory tiles of the current row. Every tile a
 //     row needs (the centre column block, the x-extended and y-extended
-//     halo blocks, the model) arrives by TMA (cp.async.bulk.tensor, one
-//     elected thread) into a 2-deep stage ring guarded by mbarriers, one
-//     row ahead of the compute; the tensor maps zero-fill outside the padded
+//     halo blocks, the model) arrives by TMA (cp.async.bulk.tensor, one or
+//     two copies an elected lane of every warp) into a 2-deep stage ring
+//     guarded by mbarriers, one row ahead of the compute; the tensor maps zero-fill outside the padded
 //     array, which is the operators' boundary convention;
 //   * the velocity (half-node) stage is recomputed on the x and y halos, so
 //     the pressure stage of the same row needs nothing from other CTAs and a
@@ -26,7 +26,9 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <cmath>
 #include <mutex>
+#include <type_traits>
 
 #include "lsrtm_internal.cuh"
 #include "tma.cuh"
@@ -76,6 +78,15 @@ __device__ __forceinline__ float st1(const float *c, FA fa, FB fb)
 __device__ __forceinline__ int node_src_row(const GridDev &g, int r) { return (g.fs && r < g.z0) ? fs_node_row(g, r) : r; }
 __device__ __forceinline__ int half_src_row(const GridDev &g, int k) { return (g.fs && k < g.z0) ? fs_half_row(g, k) : k; }
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+// Half-node and node z CPML rows.
+__device__ __forceinline__ bool zpml_half(const GridDev &g, int k)
+{
+    return k >= 0 && k < g.Nz && (k <= g.z0 - 2 || k >= g.z0 + g.nz);
+}
+__device__ __forceinline__ bool zpml_node(const GridDev &g, int r)
+{
+    return r >= 0 && r < g.Nz && (r <= g.z0 - 1 || r >= g.z0 + g.nz);
+}
 
 // ---- shared memory, mbarriers and TMA (tma.cuh)
 using tma::al128;
@@ -102,14 +113,26 @@ struct Geo {
     static constexpr int W = 2 * M;
     static constexpr int XO1 = 4, XW1 = TX + 8;
     static constexpr int XO2 = (2 * M + 3) / 4 * 4, XW2 = TX + 2 * XO2;
+    static constexpr int XH1 = TX + 2 * M - 1;   // half nodes [x0-M, x0+TX+M-2]
     static constexpr int YO1 = M, YH1 = TY + 2 * M - 1, YHB = TY + 2 * M;
     static constexpr int YO2 = 2 * M - 1, YH2 = TY + 4 * M - 2;
-    static constexpr int NXI = TX + 2 * M - 1;   // half nodes per row of the x halo stage
     static_assert(XO1 >= M && XO2 >= 2 * M - 1, "halo offsets");
 };
 
 // ---------------------------------------------------------------------------
 // Born modelling step n -> n+1.
+//
+// What bounds it: 80 B a cell in one pass (112 measured: the tiles' halos come
+// from DRAM again where neighbours run apart in z) and the issue slots of the
+// halo work. So every warp issues one of a row's tile copies (one thread that
+// issued all eleven was waited for by the CTA), the half nodes of a row are
+// dealt to the threads once per launch (its own x and y half node and at most
+// one of the halo's), tiles and rows away from the strips run a form without
+// boundary tests, and strip tiles apply the CPML terms to all columns with
+// profiles that are zero outside the strips. 2 shots of 168 x 296 x 296 cells,
+// order 8: 107.2 -> 84.6 ms in 96 steps, 26.4 -> 33.4 G cell-updates/s in the
+// same chunk of 168 rows; 73.7 ms = 38.4 G = 0.46 of the measured copy rate
+// with march3d_rows' chunks.
 // ---------------------------------------------------------------------------
 template <int M>
 struct BornSmem {
@@ -130,7 +153,11 @@ struct BornSmem {
     // after the stages: the new vx / vy of the row (half-node halos)
     static constexpr unsigned OVX = PD * STAGE;
     static constexpr unsigned OVY = OVX + al128(G::XW1 * TY * 8);
-    static constexpr unsigned BAR = OVY + al128(TX * G::YH1 * 8);
+    // CPML profiles over the tile, zero outside the strips: a, b at the half
+    // nodes along x and y (halo included), a, b at the nodes
+    static constexpr unsigned TAB = OVY + al128(TX * G::YH1 * 8);
+    static constexpr int HX = 0, HY = HX + 2 * G::XH1, NX = HY + 2 * G::YH1, NY = NX + 2 * TX, NTAB = NY + 2 * TY;
+    static constexpr unsigned BAR = TAB + al128(NTAB * 4);
     static constexpr unsigned TOTAL = BAR + 64 + 128;   // + alignment slack
 };
 
@@ -140,8 +167,9 @@ size_t fused3d_born_smem(int M) { return M == 2 ? BornSmem<2>::TOTAL : BornSmem<
 
 namespace {
 
+// One of the row's copies per warp (called by whole warps).
 template <int M>
-__device__ __forceinline__ void born_issue(const Step3F &a, unsigned char *st, uint64_t *bar, int slot, int x0,
+__device__ __forceinline__ void born_issue(const Step3F &a, int warp, unsigned char *st, uint64_t *bar, int slot, int x0,
                                            int y0, int z, int zc0, bool px, bool py)
 {
     using G = Geo<M>;
@@ -149,34 +177,42 @@ __device__ __forceinline__ void born_issue(const Step3F &a, unsigned char *st, u
     const GridDev &g = a.g;
     const int k = z + M - 1, r = z + G::W - 1;
     const bool main = z >= zc0;
-    const bool pzs = k >= 0 && k < g.Nz && (k <= g.z0 - 2 || k >= g.z0 + g.nz);
+    const bool pzs = zpml_half(g, k);
     const int q = slot * a.in_pairs;   // pair-plane index of the slot's first field
-    unsigned bytes = 3 * TX * TY * 8 + (pzs ? TX * TY * 8 : 0);
-    if (main) {
-        bytes += TX * TY * 8 + G::XW2 * G::YH2 * 8 + G::XW1 * TY * 8 + TX * G::YH1 * 8 + G::XW1 * G::YHB * 8;
-        if (px) bytes += G::XW1 * TY * 8;
-        if (py) bytes += TX * G::YH1 * 8;
-    }
     // x coordinates in floats (pairs x 2); each a multiple of 4 (16 bytes)
     const int xc = 2 * x0, x1 = 2 * (x0 - G::XO1), x2 = 2 * (x0 - G::XO2);
-    if ((xc | x1 | x2) & 3) {   // never issue a misaligned copy
-        atomicOr(a.err, 2);
-        return;
+    if (warp == 0) {
+        if (tma::elect_one()) tma4(st + S::PA, a.in_core, xc, y0, node_src_row(g, r), q + F3_P, bar);
+    } else if (warp == 1) {
+        if (tma::elect_one()) tma4(st + S::VZ, a.in_core, xc, y0, half_src_row(g, k), q + F3_VZ, bar);
+    } else if (warp == 2) {
+        if (tma::elect_one()) tma4(st + S::BK, a.m_core, xc, y0, k + 1, 1, bar);
+    } else if (warp == 3) {
+        if (pzs && tma::elect_one()) tma4(st + S::PZ, a.in_core, xc, y0, k, q + F3_PPZ, bar);
+    } else if (warp == 4) {
+        if (main && tma::elect_one()) tma4(st + S::KD, a.m_core, xc, y0, z, 0, bar);
+    } else if (warp == 5) {
+        if (main && tma::elect_one()) tma4(st + S::PW, a.in_wide, x2, y0 - G::YO2, z, q + F3_P, bar);
+    } else if (warp == 6) {
+        if (main && tma::elect_one()) tma4(st + S::VX, a.in_xbox, x1, y0, z, q + F3_VX, bar);
+    } else if (warp == 7) {
+        if (main && tma::elect_one()) tma4(st + S::VY, a.in_ybox, xc, y0 - G::YO1, z, q + F3_VY, bar);
+    } else if (warp == 8) {
+        if (main && tma::elect_one()) tma4(st + S::BR, a.m_ybr, x1, y0 - G::YO1, z, 1, bar);
+    } else if (warp == 9) {
+        if (main && px && tma::elect_one()) tma4(st + S::PX, a.in_xbox, x1, y0, z, q + F3_PPX, bar);
+    } else if (warp == 10) {
+        if (main && py && tma::elect_one()) tma4(st + S::PY, a.in_ybox, xc, y0 - G::YO1, z, q + F3_PPY, bar);
+    } else if (tma::elect_one()) {
+        unsigned bytes = 3 * TX * TY * 8 + (pzs ? TX * TY * 8 : 0);
+        if (main) {
+            bytes += TX * TY * 8 + G::XW2 * G::YH2 * 8 + G::XW1 * TY * 8 + TX * G::YH1 * 8 + G::XW1 * G::YHB * 8;
+            if (px) bytes += G::XW1 * TY * 8;
+            if (py) bytes += TX * G::YH1 * 8;
+        }
+        mbar_expect(bar, bytes);
     }
-    mbar_expect(bar, bytes);
-    tma4(st + S::PA, a.in_core, xc, y0, node_src_row(g, r), q + F3_P, bar);
-    tma4(st + S::VZ, a.in_core, xc, y0, half_src_row(g, k), q + F3_VZ, bar);
-    tma4(st + S::BK, a.m_core, xc, y0, k + 1, 1, bar);
-    if (pzs) tma4(st + S::PZ, a.in_core, xc, y0, k, q + F3_PPZ, bar);
-    if (main) {
-        tma4(st + S::KD, a.m_core, xc, y0, z, 0, bar);
-        tma4(st + S::PW, a.in_wide, x2, y0 - G::YO2, z, q + F3_P, bar);
-        tma4(st + S::VX, a.in_xbox, x1, y0, z, q + F3_VX, bar);
-        tma4(st + S::VY, a.in_ybox, xc, y0 - G::YO1, z, q + F3_VY, bar);
-        tma4(st + S::BR, a.m_ybr, x1, y0 - G::YO1, z, 1, bar);
-        if (px) tma4(st + S::PX, a.in_xbox, x1, y0, z, q + F3_PPX, bar);
-        if (py) tma4(st + S::PY, a.in_ybox, xc, y0 - G::YO1, z, q + F3_PPY, bar);
-    }
+    __syncwarp();
 }
 
 template <int M>
@@ -194,6 +230,7 @@ __global__ void __launch_bounds__(NTH, kMinBlocks) k3f_born(const __grid_constan
 
     const GridDev &g = a.g;
     const int t = threadIdx.x, tx = t % TX, ty = t / TX;
+    const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);   // (known to be uniform)
     const int nzc = (g.Nz + a.tzc - 1) / a.tzc;
     const int slot = blockIdx.z / nzc, zcn = blockIdx.z - slot * nzc;
     const int shot = a.shot0 + slot;
@@ -208,34 +245,85 @@ __global__ void __launch_bounds__(NTH, kMinBlocks) k3f_born(const __grid_constan
     // CTA-uniform: does the tile's x (y) halo reach a CPML strip?
     const bool px = (x0 - M <= g.x0 - 2) || (x0 + TX + M - 2 >= g.x0 + g.nx);
     const bool py = (y0 - M <= g.y0 - 2) || (y0 + TY + M - 2 >= g.y0 + g.ny);
+    const bool xyf = !px && !py;   // (then every node and half node of the tile and its halo is interior)
     float2 *out = reinterpret_cast<float2 *>(a.out) + slot * a.out_pairs * plane;
     float2 *psv = reinterpret_cast<float2 *>(a.psiv) + slot * a.psiv_pairs * plane;   // in place: x y z
     const int src = a.src_cell[shot];
     const float wsrc = a.src_scale * a.wav[(a.wav_per_shot ? (long long)shot * g.nt : 0) + a.n];
 
+    float *tab = reinterpret_cast<float *>(sm + S::TAB);
     if (t == 0) {
         for (int i = 0; i < PD; ++i) mbar_init(bar + i);
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        tma::mbar_init_fence();
+    }
+    for (int i = t; i < S::NTAB; i += NTH) {
+        int d, e;   // axis, and entry in its (a, b) table
+        const float *pa, *pb;
+        if (i < S::NX) {
+            d = i < S::HY ? 2 : 1;
+            e = i < S::HY ? i : i - S::HY;
+            pa = a.pml.ah[d], pb = a.pml.bh[d];
+        } else {
+            d = i < S::NY ? 2 : 1;
+            e = i < S::NY ? i - S::NX : i - S::NY;
+            pa = a.pml.ai[d], pb = a.pml.bi[d];
+        }
+        const int len = i < S::NX ? (d == 2 ? G::XH1 : G::YH1) : (d == 2 ? TX : TY);
+        const int q = e % len, c0 = (d == 2 ? x0 : y0) - (i < S::NX ? M : 0) + q, N = d == 2 ? g.Nx : g.Ny;
+        tab[i] = c0 >= 0 && c0 < N ? (e < len ? pa : pb)[c0] : 0.f;
     }
     __syncthreads();
-    if (t == 0) {
-        for (int j = 0; j < PD - 1; ++j)
-            if (zstart + j < zc1) born_issue<M>(a, sm + j * S::STAGE, bar + j, slot, x0, y0, zstart + j, zc0, px, py);
-    }
+    for (int j = 0; j < PD - 1; ++j)
+        if (zstart + j < zc1) born_issue<M>(a, warp, sm + j * S::STAGE, bar + j, slot, x0, y0, zstart + j, zc0, px, py);
 
-    // z rings: P[m] = p^n at row z + m (m = 0..W-1, P[W-1] filled each row),
-    // VZ[m] = vz^{n+1/2} at half row z + m - M.
-    float2 P[W], VZ[W];
+    // This thread's half nodes: its column's x and y ones (all offsets around
+    // the centre of the wide and ybr tiles), and one of the halo's: vy rows
+    // outside the tile for the first 2M - 1 warps, vx columns outside it for
+    // the next threads. Half nodes before the array's start are zero (past its
+    // end 1/rho reads zero), the last one replicates the last node's 1/rho.
+    constexpr int NH = 2 * M - 1;
+    static_assert(NH + (TY * NH + 31) / 32 <= TY, "one halo item per thread");
+    const int wc = (ty + G::YO2) * G::XW2 + tx + G::XO2, bc = (ty + M) * G::XW1 + tx + G::XO1;
+    const int vxi = ty * G::XW1 + tx + G::XO1, vyi = (ty + M) * TX + tx;
+    const bool halo_y = warp < NH;
+    const int he = (warp - NH) * 32 + tx;
+    const bool halo_x = !halo_y && he < TY * NH;
+    int hw = 0, hb = 0, hv = 0, ho = 0, hi = 0, hq = 0;   // entries in the wide, ybr, v and output tiles; index along the axis, in its table
+    if (halo_y) {
+        const int jy = warp < M ? warp : warp + TY;
+        hw = (jy + M - 1) * G::XW2 + tx + G::XO2;
+        hb = jy * G::XW1 + tx + G::XO1;
+        hv = ho = jy * TX + tx;
+        hi = y0 - M + jy;
+        hq = S::HY + jy;
+    } else if (halo_x) {
+        const int iy = he / NH, q = he - iy * NH, jx = q < M ? q : q + TX;
+        hw = (iy + G::YO2) * G::XW2 + (jx - M + G::XO2);
+        hb = (iy + M) * G::XW1 + (jx - M + G::XO1);
+        hv = iy * G::XW1 + (jx - M + G::XO1);
+        ho = iy * G::XW1 + jx;
+        hi = x0 - M + jx;
+        hq = S::HX + jx;
+    }
+    const float hscale = hi >= 0 ? 0.5f : 0.f;
+
+    // z rings, shifted by U entries after every U rows: entry u + m holds p^n
+    // at row z + m (P) or vz^{n+1/2} at half row z + m - M (VZ) of the pass's
+    // row u
+    constexpr int U = 1, RL = W + U - 1;
+    float2 P[RL], VZ[RL];
     {
         const float2 *pin = reinterpret_cast<const float2 *>(a.in) + slot * a.in_pairs * plane + F3_P * plane;
 #pragma unroll
-        for (int m = 0; m < W - 1; ++m) {
-            const int zr = zstart + m, zs = node_src_row(g, zr);
-            const float2 v = (colok && zs >= 0 && zs < g.Nz) ? pin[zs * g.rowz + cxy] : make_float2(0.f, 0.f);
-            P[m] = zs != zr ? neg2(v) : v;
+        for (int m = 0; m < RL; ++m) {
+            P[m] = make_float2(0.f, 0.f);
+            if (m < W - 1) {
+                const int zr = zstart + m, zs = node_src_row(g, zr);
+                const float2 v = (colok && zs >= 0 && zs < g.Nz) ? pin[zs * g.rowz + cxy] : make_float2(0.f, 0.f);
+                P[m] = zs != zr ? neg2(v) : v;
+            }
+            VZ[m] = make_float2(0.f, 0.f);
         }
-#pragma unroll
-        for (int m = 0; m < W; ++m) VZ[m] = make_float2(0.f, 0.f);
     }
     float2 br_old = make_float2(0.f, 0.f);
     {
@@ -243,169 +331,173 @@ __global__ void __launch_bounds__(NTH, kMinBlocks) k3f_born(const __grid_constan
         if (colok && kk >= 0 && kk < g.Nz) br_old = a.br2[kk * g.rowz + cxy];
     }
 
+    // this column's strips of the node CPML memories
+    const bool xp = colok && (x <= g.x0 - 1 || x >= g.x0 + g.nx), yp = colok && (y <= g.y0 - 1 || y >= g.y0 + g.ny);
     bool failed = false;
     int fail_row = 0;
     const int pl = (int)plane;   // in-slot offsets fit in 32 bits (checked by the host)
     const int rowz = (int)g.rowz, pitch = g.pitch;
     const int cxy32 = y * pitch + x;
-    for (int z = zstart; z < zc1; ++z) {
-        const int j = z - zstart;
-        const bool to = !mbar_wait(bar + j % PD, (unsigned)(j / PD) & 1u);
-        // (this barrier also certifies that every thread is done with row z-1,
-        // its stage and the vx / vy tiles)
-        if (__syncthreads_or(to)) {
-            failed = true;
-            fail_row = z;
-            break;
-        }
-        // the last warp has no item in the last round of the halo loop: it
-        // refills the stage of row z-1 with row z+PD-1
-        if (t == NTH - 1 && z + PD - 1 < zc1) {
-            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-            born_issue<M>(a, sm + ((j + PD - 1) % PD) * S::STAGE, bar + (j + PD - 1) % PD, slot, x0, y0, z + PD - 1,
-                          zc0, px, py);
-        }
-        const unsigned char *st = sm + (j % PD) * S::STAGE;
-        const float2 *cPA = reinterpret_cast<const float2 *>(st + S::PA);
-        const float2 *cVZ = reinterpret_cast<const float2 *>(st + S::VZ);
-        const float2 *cBK = reinterpret_cast<const float2 *>(st + S::BK);
-        const float2 *cPZ = reinterpret_cast<const float2 *>(st + S::PZ);
-        const int k = z + M - 1;
-
-        // ---- vz at half row k (column-local)
-        P[W - 1] = (g.fs && z + W - 1 < g.z0) ? neg2(cPA[t]) : cPA[t];   // ghost rows: -p(mirror)
-        // (the last half row replicates the last node row's buoyancy)
-        const float2 brk1 = k + 1 < g.Nz ? cBK[t] : make_float2(br_old.x, 0.f);
-        float2 vzn = make_float2(0.f, 0.f);
-        if (colok && k >= 0 && k < g.Nz) {
-            float2 Gz = st2<M>(g.cz, [&](int l) { return P[M - 1 + l]; }, [&](int l) { return P[M - l]; });
-            const bool own = k >= zc0 && k < zc1;
-            if (k <= g.z0 - 2 || k >= g.z0 + g.nz) {
-                const float2 ps = fma2(a.pml.bh[0][k], cPZ[t], mul2(a.pml.ah[0][k], Gz));
-                if (own) out[F3_PPZ * pl + k * rowz + cxy32] = ps;
-                Gz = add2(Gz, ps);
+    for (int zb = zstart; zb < zc1 && !failed; zb += U) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int z = zb + u;
+            if (z >= zc1) break;
+            const int j = z - zstart;
+            const bool to = !mbar_wait(bar + j % PD, (unsigned)(j / PD) & 1u);
+            // (this barrier also certifies that every thread is done with row
+            // z-1, its stage and the vx / vy tiles)
+            if (__syncthreads_or(to)) {
+                failed = true;
+                fail_row = z;
+                break;
             }
-            const float bu = 0.5f * (br_old.x + brk1.x);
-            vzn = fma2(-dt * bu, Gz, cVZ[t]);
-            vzn.y = fmaf(0.5f * dt * (br_old.y + brk1.y), Gz.x, vzn.y);
-            if (own) out[F3_VZ * pl + k * rowz + cxy32] = vzn;
-        }
-        br_old = brk1;
-        VZ[W - 1] = vzn;
-
-        if (z >= zc0) {
-            const float2 *cKD = reinterpret_cast<const float2 *>(st + S::KD);
-            const float2 *wP = reinterpret_cast<const float2 *>(st + S::PW);
-            const float2 *bVX = reinterpret_cast<const float2 *>(st + S::VX);
-            const float2 *bVY = reinterpret_cast<const float2 *>(st + S::VY);
-            const float2 *bBR = reinterpret_cast<const float2 *>(st + S::BR);
-            const float2 *bPX = reinterpret_cast<const float2 *>(st + S::PX);
-            const float2 *bPY = reinterpret_cast<const float2 *>(st + S::PY);
-            const int rz = z * rowz;
-            // ---- velocities on the halos of the row, one loop over both:
-            // items [0, NVX) are vx at half nodes xh = x0 - M + jx of row iy,
-            // the rest vy at half nodes yh = y0 - M + jy of column ix
-            constexpr int NVX = TY * G::NXI, NIT = NVX + G::YH1 * TX;
-            for (int i = t; i < NIT; i += NTH) {
-                if (i < NVX) {
-                    const int iy = i / G::NXI, jx = i - iy * G::NXI;
-                    const int xh = x0 - M + jx, yy = y0 + iy;
-                    float2 v = make_float2(0.f, 0.f);
-                    if (xh >= 0 && xh < g.Nx && yy < g.Ny) {
-                        const float2 *pr = wP + (iy + G::YO2) * G::XW2 + (jx - M + G::XO2);
-                        float2 Gx = st2<M>(g.cx, [&](int l) { return pr[l]; }, [&](int l) { return pr[1 - l]; });
-                        const int cb = iy * G::XW1 + jx - M + G::XO1;   // xbox entry of half node xh
-                        const bool own = jx >= M && jx < M + TX;
-                        const int o = rz + yy * pitch + xh;
-                        if (px && (xh <= g.x0 - 2 || xh >= g.x0 + g.nx)) {
-                            const float2 ps = fma2(a.pml.bh[2][xh], bPX[cb], mul2(a.pml.ah[2][xh], Gx));
-                            if (own) out[F3_PPX * pl + o] = ps;
-                            Gx = add2(Gx, ps);
-                        }
-                        const float2 *brr = bBR + M * G::XW1 + cb;
-                        const float2 b0 = brr[0];
-                        const float2 b1 = xh + 1 >= g.Nx ? make_float2(b0.x, 0.f) : brr[1];
-                        v = fma2(-dt * 0.5f * (b0.x + b1.x), Gx, bVX[cb]);
-                        v.y = fmaf(0.5f * dt * (b0.y + b1.y), Gx.x, v.y);
-                        if (own) out[F3_VX * pl + o] = v;
+            if (z + PD - 1 < zc1)   // refill the stage of row z-1 with row z+PD-1
+                born_issue<M>(a, warp, sm + ((j + PD - 1) % PD) * S::STAGE, bar + (j + PD - 1) % PD, slot, x0, y0,
+                              z + PD - 1, zc0, px, py);
+            const unsigned char *st = sm + (j % PD) * S::STAGE;
+            auto tile = [&](unsigned off) { return reinterpret_cast<const float2 *>(st + off); };
+            const int k = z + M - 1, c = z * rowz + cxy32;
+            const bool main = z >= zc0;
+            const bool zf = main && z > g.z0 && z + W < g.z0 + g.nz;
+            // node CPML memories, for the last stage
+            float2 mx = make_float2(0.f, 0.f), my = mx, mz = mx;
+            if (!xyf && main) {
+                if (xp) mx = psv[c];
+                if (yp) my = psv[pl + c];
+            }
+            const bool zs = main && !zf && zpml_node(g, z);
+            if (zs && colok) mz = psv[2 * pl + c];
+            // ---- vz at half row k (column-local), then the half nodes of row
+            // z. ZF: rows without tests (the rows and all they reach are
+            // interior); XY: tiles without strips. In strip tiles the CPML
+            // terms run on every column, with zero profiles outside the strips.
+            auto v_stage = [&](auto zc, auto xyc) {
+                constexpr bool ZF = decltype(zc)::value, XY = decltype(xyc)::value;
+                const float2 pa = tile(S::PA)[t];
+                P[u + W - 1] = (!ZF && g.fs && z + W - 1 < g.z0) ? neg2(pa) : pa;   // ghost rows: -p(mirror)
+                // (the last half row replicates the last node row's buoyancy)
+                float2 brk1 = tile(S::BK)[t];
+                if (!ZF && k + 1 >= g.Nz) brk1 = make_float2(br_old.x, 0.f);
+                float2 vzn = make_float2(0.f, 0.f);
+                if (ZF || (k >= 0 && k < g.Nz)) {
+                    float2 Gz = st2<M>(g.cz, [&](int l) { return P[u + M - 1 + l]; }, [&](int l) { return P[u + M - l]; });
+                    const bool own = (XY || colok) && (ZF || k >= zc0) && k < zc1;
+                    if (!ZF && (k <= g.z0 - 2 || k >= g.z0 + g.nz)) {
+                        const float2 ps = fma2(a.pml.bh[0][k], tile(S::PZ)[t], mul2(a.pml.ah[0][k], Gz));
+                        if (own) out[F3_PPZ * pl + k * rowz + cxy32] = ps;
+                        Gz = add2(Gz, ps);
                     }
-                    oVX[iy * G::XW1 + jx] = v;
-                } else {
-                    const int i2 = i - NVX;
-                    const int jy = i2 / TX, ix = i2 - jy * TX;
-                    const int yh = y0 - M + jy, xx = x0 + ix;
-                    float2 v = make_float2(0.f, 0.f);
-                    if (yh >= 0 && yh < g.Ny && xx < g.Nx) {
-                        const float2 *pc = wP + (jy + M - 1) * G::XW2 + (ix + G::XO2);
-                        float2 Gy = st2<M>(g.cy, [&](int l) { return pc[l * G::XW2]; },
-                                           [&](int l) { return pc[(1 - l) * G::XW2]; });
-                        const bool own = jy >= M && jy < M + TY;
-                        const int o = rz + yh * pitch + xx;
-                        if (py && (yh <= g.y0 - 2 || yh >= g.y0 + g.ny)) {
-                            const float2 ps = fma2(a.pml.bh[1][yh], bPY[i2], mul2(a.pml.ah[1][yh], Gy));
-                            if (own) out[F3_PPY * pl + o] = ps;
-                            Gy = add2(Gy, ps);
-                        }
-                        const float2 *brc = bBR + jy * G::XW1 + ix + G::XO1;
-                        const float2 b0 = brc[0];
-                        const float2 b1 = yh + 1 >= g.Ny ? make_float2(b0.x, 0.f) : brc[G::XW1];
-                        v = fma2(-dt * 0.5f * (b0.x + b1.x), Gy, bVY[i2]);
-                        v.y = fmaf(0.5f * dt * (b0.y + b1.y), Gy.x, v.y);
-                        if (own) out[F3_VY * pl + o] = v;
-                    }
-                    oVY[i2] = v;
+                    const float bu = 0.5f * (br_old.x + brk1.x);
+                    vzn = fma2(-dt * bu, Gz, tile(S::VZ)[t]);
+                    vzn.y = fmaf(0.5f * dt * (br_old.y + brk1.y), Gz.x, vzn.y);
+                    if (own) out[F3_VZ * pl + k * rowz + cxy32] = vzn;
                 }
-            }
-            __syncthreads();
+                br_old = brk1;
+                VZ[u + W - 1] = vzn;
+                if (!ZF && !main) return;
+                // one half node: entries in the wide and ybr tiles, tap strides
+                // there, the stored velocity; strip: its table entries a (at q)
+                // and b (len further), its memory
+                auto half = [&](const float *cf, int w, int ws, int b, int bst, float2 v0, float hs, bool last, bool strip,
+                                int q, int len, const float2 *psi, float2 *ps_out) -> float2 {
+                    const float2 *p = tile(S::PW) + w;
+                    float2 Gd = st2<M>(cf, [&](int l) { return p[l * ws]; }, [&](int l) { return p[(1 - l) * ws]; });
+                    if (!XY && strip) {
+                        const float pb = tab[q + len];
+                        const float2 ps = fma2(pb, *psi, mul2(tab[q], Gd));
+                        if (ps_out && pb != 0.f) *ps_out = ps;
+                        Gd = add2(Gd, ps);
+                    }
+                    const float2 b0 = tile(S::BR)[b];
+                    float2 b1 = tile(S::BR)[b + bst];
+                    if (!XY && last) b1 = make_float2(b0.x, 0.f);
+                    float2 v = fma2(-dt * (hs * (b0.x + b1.x)), Gd, v0);
+                    v.y = fmaf(hs * dt * (b0.y + b1.y), Gd.x, v.y);
+                    return v;
+                };
+                {
+                    const float2 v = half(g.cx, wc, 1, bc, 1, tile(S::VX)[vxi], 0.5f, x + 1 >= g.Nx, px, S::HX + tx + M, G::XH1,
+                                          tile(S::PX) + vxi, colok ? out + F3_PPX * pl + c : nullptr);
+                    oVX[ty * G::XW1 + tx + M] = v;
+                    if (XY || colok) out[F3_VX * pl + c] = v;
+                }
+                {
+                    const float2 v = half(g.cy, wc, G::XW2, bc, G::XW1, tile(S::VY)[vyi], 0.5f, y + 1 >= g.Ny, py,
+                                          S::HY + ty + M, G::YH1, tile(S::PY) + vyi, colok ? out + F3_PPY * pl + c : nullptr);
+                    oVY[vyi] = v;
+                    if (XY || colok) out[F3_VY * pl + c] = v;
+                }
+                if (halo_y)
+                    oVY[ho] = half(g.cy, hw, G::XW2, hb, G::XW1, tile(S::VY)[hv], XY ? 0.5f : hscale, hi + 1 >= g.Ny, py, hq,
+                                   G::YH1, tile(S::PY) + hv, nullptr);
+                else if (halo_x)
+                    oVX[ho] = half(g.cx, hw, 1, hb, 1, tile(S::VX)[hv], XY ? 0.5f : hscale, hi + 1 >= g.Nx, px, hq, G::XH1,
+                                   tile(S::PX) + hv, nullptr);
+            };
             // ---- pressure at row z on the thread's own column
-            if (colok) {
+            auto p_stage = [&](auto zc, auto xyc) {
+                constexpr bool ZF = decltype(zc)::value, XY = decltype(xyc)::value;
                 const float2 *vxr = oVX + ty * G::XW1 + tx + M;
-                const float2 *vyc = oVY + (ty + M) * TX + tx;
+                const float2 *vyc = oVY + vyi;
                 float2 Qx = st2<M>(g.cx, [&](int l) { return vxr[l - 1]; }, [&](int l) { return vxr[-l]; });
                 float2 Qy = st2<M>(g.cy, [&](int l) { return vyc[(l - 1) * TX]; }, [&](int l) { return vyc[-l * TX]; });
-                float2 Qz = st2<M>(g.cz, [&](int l) { return VZ[M + l - 1]; }, [&](int l) { return VZ[M - l]; });
-                const int c = rz + cxy32;
-                if (x <= g.x0 - 1 || x >= g.x0 + g.nx) {
-                    float2 *m = psv + c;
-                    const float2 ps = fma2(a.pml.bi[2][x], *m, mul2(a.pml.ai[2][x], Qx));
-                    *m = ps;
+                float2 Qz = st2<M>(g.cz, [&](int l) { return VZ[u + M + l - 1]; }, [&](int l) { return VZ[u + M - l]; });
+                if (!XY && px) {
+                    const float2 ps = fma2(tab[S::NX + TX + tx], mx, mul2(tab[S::NX + tx], Qx));
+                    if (xp) psv[c] = ps;
                     Qx = add2(Qx, ps);
                 }
-                if (y <= g.y0 - 1 || y >= g.y0 + g.ny) {
-                    float2 *m = psv + pl + c;
-                    const float2 ps = fma2(a.pml.bi[1][y], *m, mul2(a.pml.ai[1][y], Qy));
-                    *m = ps;
+                if (!XY && py) {
+                    const float2 ps = fma2(tab[S::NY + TY + ty], my, mul2(tab[S::NY + ty], Qy));
+                    if (yp) psv[pl + c] = ps;
                     Qy = add2(Qy, ps);
                 }
-                if (z <= g.z0 - 1 || z >= g.z0 + g.nz) {
-                    float2 *m = psv + 2 * pl + c;
-                    const float2 ps = fma2(a.pml.bi[0][z], *m, mul2(a.pml.ai[0][z], Qz));
-                    *m = ps;
+                if (!ZF && zs) {
+                    const float2 ps = fma2(a.pml.bi[0][z], mz, mul2(a.pml.ai[0][z], Qz));
+                    if (colok) psv[2 * pl + c] = ps;
                     Qz = add2(Qz, ps);
                 }
                 const float2 Q = add2(add2(Qx, Qy), Qz);
-                const float2 kd = cKD[t];
-                const float2 p0 = wP[(ty + G::YO2) * G::XW2 + tx + G::XO2];
-                float2 pn = fma2(-kd.x, Q, p0);
+                const float2 kd = tile(S::KD)[t];
+                float2 pn = fma2(-kd.x, Q, P[u]);
                 pn.y = fmaf(-kd.y, Q.x, pn.y);
-                if (c == src) pn.x += wsrc;
-                if (g.fs && z <= g.z0) pn = make_float2(0.f, 0.f);   // p = 0 on the free surface
-                out[F3_P * pl + c] = pn;
+                pn.x += c == src ? wsrc : 0.f;
+                if (!ZF && g.fs && z <= g.z0) pn = make_float2(0.f, 0.f);   // p = 0 on the free surface
+                if (XY || colok) out[F3_P * pl + c] = pn;
+            };
+            const std::true_type Y{};
+            const std::false_type N{};
+            if (xyf) {
+                if (zf) v_stage(Y, Y);
+                else v_stage(N, Y);
+            } else {
+                if (zf) v_stage(Y, N);
+                else v_stage(N, N);
+            }
+            if (!main) continue;
+            __syncthreads();
+            if (xyf) {
+                if (zf) p_stage(Y, Y);
+                else p_stage(N, Y);
+            } else {
+                if (zf) p_stage(Y, N);
+                else p_stage(N, N);
             }
         }
 #pragma unroll
         for (int m = 0; m < W - 1; ++m) {
-            P[m] = P[m + 1];
-            VZ[m] = VZ[m + 1];
+            P[m] = P[m + U];
+            VZ[m] = VZ[m + U];
         }
     }
 
     if (failed) {
         if (t == 0) {
             atomicOr(a.err, 1);
-            // rows issued and not yet consumed: jf .. jf + PD - 1 (bounded waits)
+            // rows issued and not yet consumed: jf .. jf + PD - 2 (bounded waits)
             const int jf = fail_row - zstart;
-            for (int jj = jf; jj < jf + PD && zstart + jj < zc1; ++jj)
+            for (int jj = jf; jj < jf + PD - 1 && zstart + jj < zc1; ++jj)
                 (void)mbar_wait(bar + jj % PD, (unsigned)(jj / PD) & 1u);
         }
         return;
@@ -413,8 +505,8 @@ __global__ void __launch_bounds__(NTH, kMinBlocks) k3f_born(const __grid_constan
     // records dp^{n+1} at the receivers of this tile
     __syncthreads();
     const int ntile = (int)(gridDim.x * gridDim.y) * nzc;
-    const int tile = shot * ntile + (zcn * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-    const int b = a.trec.ptr[tile], e = a.trec.ptr[tile + 1];
+    const int rt = shot * ntile + (zcn * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    const int b = a.trec.ptr[rt], e = a.trec.ptr[rt + 1];
     for (int i = b + t; i < e; i += NTH) {
         const int2 rc = a.trec.rec[i];
         a.dstage[(long long)rc.y * g.nt + a.n] = out[F3_P * plane + rc.x].y;   // (all rows written: barrier above)
@@ -426,10 +518,22 @@ __global__ void __launch_bounds__(NTH, kMinBlocks) k3f_born(const __grid_constan
 // sub-steps, the zero-lag imaging condition and the reconstruction of the
 // background p^{n-1}, v^{n-1/2} from p^n, v^{n+1/2} and the boundary bands
 // (App. A), arranged as in the 2D kernel. State pairs (background, adjoint):
-// (p, lambda_p) at nodes, (v_d, lambda_v_d) at half nodes; the lambda CPML
-// memories as float planes. For the half-node stencils each node carries
-// (p, u_d) with u_d = dt kappa lambda_p - a_d (lambda_psi_v_d - dt kappa
-// lambda_p) (a_d nonzero only in the d strips).
+// (p, mu = dt kappa lambda_p) at nodes, (v_d, lambda_v_d) at half nodes; the
+// lambda CPML memories as float planes. For the half-node stencils each node
+// carries (p, u_d) with u_d = mu - a_d (lambda_psi_v_d - mu) (a_d nonzero only
+// in the d strips, where u_d is formed once per node).
+//
+// What bounds it: 88 B a cell in one pass, but the kernel is held back by
+// latencies and instructions (51% of the issue slots used): four outputs a half
+// node instead of one. Against the form it replaces: mu in place of lambda_p
+// needs no pass over the wide tile and no dt kappa there; the four values of a
+// half node lie in one float4, read by one load a tap; the image comes by TMA
+// (read where it was used, every row waited for it); band values of the strips
+// are loaded a stage ahead at offsets formed once; registers that did not fit
+// went to L2 (16 KB of L1 are left beside the tiles), so offsets are formed
+// anew instead. 2 shots of 168 x 296 x 296, order 8, BF16 bands: 229.0 ->
+// 154.2 ms in 96 steps in one chunk of 168 rows, 120.5 ms = 23.5 G
+// cell-updates/s = 0.31 of the measured copy rate with march3d_rows' chunks.
 // ---------------------------------------------------------------------------
 
 // Face bands (as written by the 3D background kernels):
@@ -457,28 +561,32 @@ __device__ __forceinline__ long long fband(const GridDev &g, int d, int iz, int 
 template <int M>
 struct AdjSmem {
     using G = Geo<M>;
-    static constexpr unsigned PA = 0;                                  // (p, lp) row z+W-1, core
+    static constexpr unsigned PA = 0;                                  // (p, mu) row z+W-1, core
     static constexpr unsigned LA = PA + al128(TX * TY * 8);            // lpsi_vz, row z+W-1 (strip)
     static constexpr unsigned VZ = LA + al128(TX * TY * 4);            // (vz, lvz) half row z+M-1
     static constexpr unsigned BK = VZ + al128(TX * TY * 8);            // 1/rho, row z+M
     static constexpr unsigned PZ = BK + al128(TX * TY * 4);            // lpsi_pz half row z+M-1 (strip)
-    static constexpr unsigned PW = PZ + al128(TX * TY * 4);            // (p, lp) row z, wide
-    static constexpr unsigned KW = PW + al128(G::XW2 * G::YH2 * 8);    // kdt row z, wide
-    static constexpr unsigned LX = KW + al128(G::XW2 * G::YH2 * 4);    // lpsi_vx, x-wide (strip tiles)
-    static constexpr unsigned LY = LX + al128(G::XW2 * TY * 4);        // lpsi_vy, y-wide (strip tiles)
+    static constexpr unsigned KD = PZ + al128(TX * TY * 4);            // dt kappa, row z
+    static constexpr unsigned PW = KD + al128(TX * TY * 4);            // (p, mu) row z, wide
+    static constexpr unsigned LX = PW + al128(G::XW2 * G::YH2 * 8);    // lpsi_vx, x-wide (strip tiles), then u_x
+    static constexpr unsigned LY = LX + al128(G::XW2 * TY * 4);        // lpsi_vy, y-wide (strip tiles), then u_y
     static constexpr unsigned VX = LY + al128(TX * G::YH2 * 4);        // (vx, lvx) xbox
     static constexpr unsigned VY = VX + al128(G::XW1 * TY * 8);        // (vy, lvy) ybox
     static constexpr unsigned BB = VY + al128(TX * G::YH1 * 8);        // 1/rho ybr
     static constexpr unsigned QX = BB + al128(G::XW1 * G::YHB * 4);    // lpsi_px xbox (strip tiles)
     static constexpr unsigned QY = QX + al128(G::XW1 * TY * 4);        // lpsi_py ybox (strip tiles)
-    static constexpr unsigned STAGE = QY + al128(TX * G::YH1 * 4);
-    static constexpr unsigned OWX = PD * STAGE;                        // (v^{n+1/2}, w) x half nodes
-    static constexpr unsigned ONX = OWX + al128(G::XW1 * TY * 8);      // v^{n-1/2} x
-    static constexpr unsigned OIX = ONX + al128(G::XW1 * TY * 4);      // G lambda_v products x
-    static constexpr unsigned OWY = OIX + al128(G::XW1 * TY * 4);
-    static constexpr unsigned ONY = OWY + al128(TX * G::YH1 * 8);
-    static constexpr unsigned OIY = ONY + al128(TX * G::YH1 * 4);
-    static constexpr unsigned BAR = OIY + al128(TX * G::YH1 * 4);
+    static constexpr unsigned IM = QY + al128(TX * G::YH1 * 4);        // image, row z, core (interior rows)
+    static constexpr unsigned STAGE = IM + al128(TX * TY * 8);
+    // the half nodes of the row: (v^{n+1/2}, w, v^{n-1/2}, G lambda_v)
+    static constexpr unsigned OX = PD * STAGE;
+    static constexpr unsigned OY = OX + al128(G::XW1 * TY * 16);
+    // CPML profiles over the tile, zero outside the strips: a, b at the half
+    // nodes along x and y, a at the nodes of the wide tile, b at the own nodes;
+    // then the step's (p, v) band scales
+    static constexpr unsigned TAB = OY + al128(TX * G::YH1 * 16);
+    static constexpr int HX = 0, HY = HX + 2 * G::XH1, WX = HY + 2 * G::YH1, WY = WX + G::XW2, NX = WY + G::YH2,
+                         NY = NX + TX, SC = NY + TY, NTAB = SC + 2;
+    static constexpr unsigned BAR = TAB + al128(NTAB * 4);
     static constexpr unsigned TOTAL = BAR + 64 + 128;
 };
 
@@ -492,49 +600,64 @@ size_t fused3d_adj_smem(int M) { return M == 2 ? AdjSmem<2>::TOTAL : AdjSmem<4>:
 
 namespace {
 
+// A row's copies, dealt to the warps (called by whole warps).
 template <int M>
-__device__ __forceinline__ void adj_issue(const Adj3F &a, unsigned char *st, uint64_t *bar, int slot, int x0, int y0,
-                                          int z, int zc0, bool px, bool py, bool px2, bool py2)
+__device__ __forceinline__ void adj_issue(const Adj3F &a, int warp, unsigned char *st, uint64_t *bar, int slot, int x0,
+                                          int y0, int z, int zc0, bool px, bool py, bool px2, bool py2)
 {
     using G = Geo<M>;
     using S = AdjSmem<M>;
     const GridDev &g = a.g;
     const int k = z + M - 1, r = z + G::W - 1;
-    const bool main = z >= zc0;
-    const bool rs = r >= 0 && r < g.Nz && (r <= g.z0 - 1 || r >= g.z0 + g.nz);   // node z strip
-    const bool ks = k >= 0 && k < g.Nz && (k <= g.z0 - 2 || k >= g.z0 + g.nz);   // half-node z strip
+    const bool main = z >= zc0, im = main && z >= g.z0 && z < g.z0 + g.nz;
+    const bool rs = zpml_node(g, r), ks = zpml_half(g, k);
     const int qp = slot * (a.in_planes / 2), qf = slot * a.in_planes;
     constexpr unsigned C8 = TX * TY * 8, C4 = TX * TY * 4;
-    unsigned bytes = C8 + C8 + C4 + (rs ? C4 : 0) + (ks ? C4 : 0);
-    if (main) {
-        bytes += G::XW2 * G::YH2 * 12 + G::XW1 * TY * 8 + TX * G::YH1 * 8 + G::XW1 * G::YHB * 4;
-        if (px2) bytes += G::XW2 * TY * 4;
-        if (py2) bytes += TX * G::YH2 * 4;
-        if (px) bytes += G::XW1 * TY * 4;
-        if (py) bytes += TX * G::YH1 * 4;
+    const int xc = x0, x1 = x0 - G::XO1, x2 = x0 - G::XO2;   // floats, each a multiple of 4 (16 bytes); pairs use 2x
+    if (warp == 0) {
+        if (tma::elect_one()) tma4(st + S::PA, a.p_core, 2 * xc, y0, node_src_row(g, r), qp + A3F_PL / 2, bar);
+    } else if (warp == 1) {
+        if (tma::elect_one()) tma4(st + S::VZ, a.p_core, 2 * xc, y0, half_src_row(g, k), qp + A3F_VZ / 2, bar);
+    } else if (warp == 2) {
+        if (tma::elect_one()) {
+            tma4(st + S::BK, a.m_core, xc, y0, k + 1, 1, bar);
+            if (main) tma4(st + S::KD, a.m_core, xc, y0, z, 0, bar);
+        }
+    } else if (warp == 3) {
+        if ((rs || ks || im) && tma::elect_one()) {
+            if (im) tma4(st + S::IM, a.im, 2 * xc, y0, z, slot, bar);
+            if (rs) tma4(st + S::LA, a.f_core, xc, y0, r, qf + A3F_LPVZ, bar);
+            if (ks) tma4(st + S::PZ, a.f_core, xc, y0, k, qf + A3F_LPPZ, bar);
+        }
+    } else if (warp == 4) {
+        if (main && tma::elect_one()) tma4(st + S::PW, a.p_wide, 2 * x2, y0 - G::YO2, z, qp + A3F_PL / 2, bar);
+    } else if (warp == 5) {
+        if (main && tma::elect_one()) tma4(st + S::VX, a.p_xbox, 2 * x1, y0, z, qp + A3F_VX / 2, bar);
+    } else if (warp == 6) {
+        if (main && tma::elect_one()) tma4(st + S::VY, a.p_ybox, 2 * xc, y0 - G::YO1, z, qp + A3F_VY / 2, bar);
+    } else if (warp == 7) {
+        if (main && tma::elect_one()) tma4(st + S::BB, a.m_ybr, x1, y0 - G::YO1, z, 1, bar);
+    } else if (warp == 8) {
+        if (main && px2 && tma::elect_one()) tma4(st + S::LX, a.f_xwide, x2, y0, z, qf + A3F_LPVX, bar);
+    } else if (warp == 9) {
+        if (main && py2 && tma::elect_one()) tma4(st + S::LY, a.f_ywide, xc, y0 - G::YO2, z, qf + A3F_LPVY, bar);
+    } else if (warp == 10) {
+        if (main && (px || py) && tma::elect_one()) {
+            if (px) tma4(st + S::QX, a.f_xbox, x1, y0, z, qf + A3F_LPPX, bar);
+            if (py) tma4(st + S::QY, a.f_ybox, xc, y0 - G::YO1, z, qf + A3F_LPPY, bar);
+        }
+    } else if (tma::elect_one()) {
+        unsigned bytes = C8 + C8 + C4 + (rs ? C4 : 0) + (ks ? C4 : 0) + (im ? C8 : 0);
+        if (main) {
+            bytes += C4 + G::XW2 * G::YH2 * 8 + G::XW1 * TY * 8 + TX * G::YH1 * 8 + G::XW1 * G::YHB * 4;
+            if (px2) bytes += G::XW2 * TY * 4;
+            if (py2) bytes += TX * G::YH2 * 4;
+            if (px) bytes += G::XW1 * TY * 4;
+            if (py) bytes += TX * G::YH1 * 4;
+        }
+        mbar_expect(bar, bytes);
     }
-    const int xc = x0, x1 = x0 - G::XO1, x2 = x0 - G::XO2;   // floats; pairs use 2x
-    if ((xc | x1 | x2) & 3) {
-        atomicOr(a.err, 2);
-        return;
-    }
-    mbar_expect(bar, bytes);
-    tma4(st + S::PA, a.p_core, 2 * xc, y0, node_src_row(g, r), qp + A3F_PL / 2, bar);
-    if (rs) tma4(st + S::LA, a.f_core, xc, y0, r, qf + A3F_LPVZ, bar);
-    tma4(st + S::VZ, a.p_core, 2 * xc, y0, half_src_row(g, k), qp + A3F_VZ / 2, bar);
-    tma4(st + S::BK, a.m_core, xc, y0, k + 1, 1, bar);
-    if (ks) tma4(st + S::PZ, a.f_core, xc, y0, k, qf + A3F_LPPZ, bar);
-    if (main) {
-        tma4(st + S::PW, a.p_wide, 2 * x2, y0 - G::YO2, z, qp + A3F_PL / 2, bar);
-        tma4(st + S::KW, a.m_wide, x2, y0 - G::YO2, z, 0, bar);
-        if (px2) tma4(st + S::LX, a.f_xwide, x2, y0, z, qf + A3F_LPVX, bar);
-        if (py2) tma4(st + S::LY, a.f_ywide, xc, y0 - G::YO2, z, qf + A3F_LPVY, bar);
-        tma4(st + S::VX, a.p_xbox, 2 * x1, y0, z, qp + A3F_VX / 2, bar);
-        tma4(st + S::VY, a.p_ybox, 2 * xc, y0 - G::YO1, z, qp + A3F_VY / 2, bar);
-        tma4(st + S::BB, a.m_ybr, x1, y0 - G::YO1, z, 1, bar);
-        if (px) tma4(st + S::QX, a.f_xbox, x1, y0, z, qf + A3F_LPPX, bar);
-        if (py) tma4(st + S::QY, a.f_ybox, xc, y0 - G::YO1, z, qf + A3F_LPPY, bar);
-    }
+    __syncwarp();
 }
 
 template <int M>
@@ -547,15 +670,12 @@ __global__ void __launch_bounds__(NTH, kMinBlocks) k3f_adj(const __grid_constant
     extern __shared__ unsigned char smem_raw[];
     unsigned char *sm = smem_raw + ((128u - (su32(smem_raw) & 127u)) & 127u);
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + S::BAR);
-    float2 *oWX = reinterpret_cast<float2 *>(sm + S::OWX);
-    float *oNX = reinterpret_cast<float *>(sm + S::ONX);
-    float *oIX = reinterpret_cast<float *>(sm + S::OIX);
-    float2 *oWY = reinterpret_cast<float2 *>(sm + S::OWY);
-    float *oNY = reinterpret_cast<float *>(sm + S::ONY);
-    float *oIY = reinterpret_cast<float *>(sm + S::OIY);
+    float4 *oX = reinterpret_cast<float4 *>(sm + S::OX);
+    float4 *oY = reinterpret_cast<float4 *>(sm + S::OY);
 
     const GridDev &g = a.g;
     const int t = threadIdx.x, tx = t % TX, ty = t / TX;
+    const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);   // (known to be uniform)
     const int nzc = (g.Nz + a.tzc - 1) / a.tzc;
     const int slot = blockIdx.z / nzc, zcn = blockIdx.z - slot * nzc;
     const int shot = a.shot0 + slot;
@@ -576,6 +696,7 @@ __global__ void __launch_bounds__(NTH, kMinBlocks) k3f_adj(const __grid_constant
     const bool py = (y0 - M <= g.y0 - 2) || (y0 + TY + M - 2 >= g.y0 + g.ny);
     const bool px2 = (x0 - 2 * M + 1 <= g.x0 - 1) || (x0 + TX + 2 * M - 2 >= g.x0 + g.nx);
     const bool py2 = (y0 - 2 * M + 1 <= g.y0 - 1) || (y0 + TY + 2 * M - 2 >= g.y0 + g.ny);
+    const bool xyf = !px2 && !py2;   // every node and half node the tile reads is interior
     const float *in = a.in + (long long)slot * a.in_planes * g.plane;
     float *outf = a.out + (long long)slot * a.out_planes * g.plane;
     float2 *out2 = reinterpret_cast<float2 *>(outf);
@@ -584,46 +705,87 @@ __global__ void __launch_bounds__(NTH, kMinBlocks) k3f_adj(const __grid_constant
     const int src = a.src_cell[shot];
     const float wsrc = recon ? a.src_scale * a.wav[(a.wav_per_shot ? (long long)shot * g.nt : 0) + n - 1] : 0.f;
 
+    float *tab = reinterpret_cast<float *>(sm + S::TAB);
     if (t == 0) {
         for (int i = 0; i < PD; ++i) mbar_init(bar + i);
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        tma::mbar_init_fence();
+        for (int f = 0; f < 2; ++f) tab[S::SC + f] = recon && a.bands.fmt != BAND_F32 ? a.bands.scale[rowprev * 2 + f] : 1.f;
+    }
+    for (int i = t; i < S::SC; i += NTH) {
+        const float *pr;
+        int c0, N;
+        if (i < S::HY) pr = i < G::XH1 ? a.pml.ah[2] : a.pml.bh[2], c0 = x0 - M + i % G::XH1, N = g.Nx;
+        else if (i < S::WX) pr = i - S::HY < G::YH1 ? a.pml.ah[1] : a.pml.bh[1], c0 = y0 - M + (i - S::HY) % G::YH1, N = g.Ny;
+        else if (i < S::WY) pr = a.pml.ai[2], c0 = x0 - G::XO2 + i - S::WX, N = g.Nx;
+        else if (i < S::NX) pr = a.pml.ai[1], c0 = y0 - G::YO2 + i - S::WY, N = g.Ny;
+        else if (i < S::NY) pr = a.pml.bi[2], c0 = x0 + i - S::NX, N = g.Nx;
+        else pr = a.pml.bi[1], c0 = y0 + i - S::NY, N = g.Ny;
+        tab[i] = c0 >= 0 && c0 < N ? pr[c0] : 0.f;
     }
     __syncthreads();
-    if (t == 0) {
-        for (int j = 0; j < PD - 1; ++j)
-            if (zstart + j < zc1)
-                adj_issue<M>(a, sm + j * S::STAGE, bar + j, slot, x0, y0, zstart + j, zc0, px, py, px2, py2);
-    }
+    for (int j = 0; j < PD - 1; ++j)
+        if (zstart + j < zc1)
+            adj_issue<M>(a, warp, sm + j * S::STAGE, bar + j, slot, x0, y0, zstart + j, zc0, px, py, px2, py2);
+
+    // this thread's half nodes (k3f_born): its own column's and at most one of
+    // the halo's, whose offsets are formed anew in every row (the z rings leave
+    // no registers to keep them; a spilled one comes from L2)
+    constexpr int NH = 2 * M - 1;
+    const int wc = (ty + G::YO2) * G::XW2 + tx + G::XO2, bc = (ty + M) * G::XW1 + tx + G::XO1;
+    const bool halo_y = warp < NH;
+    const int jy = warp < M ? warp : warp + TY;   // halo_y: its row of half nodes
+    const int he = (warp - NH) * 32 + tx;
+    const bool halo_x = !halo_y && he < TY * NH;
+    const int hy0 = he / NH, hx0 = he - hy0 * NH < M ? he - hy0 * NH : he - hy0 * NH + TX;
+    const int hpack = hy0 | hx0 << 8;   // halo_x: its row and half node, in one register
+    // Strip band values of an interior row iz: those of this column (its v is
+    // the strip's normal one, along x or y) at b_off + iz times the strip's
+    // values a row, those of the halo item at h_off (-1: none)
+    const int xstr = 2 * M * g.ny, ystr = 2 * M * g.nx;
+    auto strip_off = [&](int jx, int jy) -> int {   // interior offsets of a half node or node
+        const bool ix_in = jx >= 0 && jx < g.nx, iy_in = jy >= 0 && jy < g.ny;
+        const int sx = jx < 0 ? jx + M : M + jx - g.nx, sy = jy < 0 ? jy + M : M + jy - g.ny;
+        if (iy_in && !ix_in && sx >= 0 && sx < 2 * M) return jy * 2 * M + sx;
+        if (ix_in && !iy_in && sy >= 0 && sy < 2 * M) return 2 * M * g.nz * g.ny + sy * g.nx + jx;
+        return -1;
+    };
+    const int b_off = recon && colok && !xyf ? strip_off(ixg, iyg) : -1;
+    const int h_off = !recon ? -1 : (halo_y ? strip_off(ixg, y0 - M + jy - g.y0)
+                                            : (halo_x ? strip_off(x0 - M + hx0 - g.x0, y0 + hy0 - g.y0) : -1));
+    auto band_raw = [&](int field, int o) -> float {
+        const long long e = rowprev * a.bands.nb + o;
+        const void *b = field ? a.bands.v : a.bands.p;
+        if (a.bands.fmt == BAND_F32) return reinterpret_cast<const float *>(b)[e];
+        if (a.bands.fmt == BAND_BF16S) return tab[S::SC + field] * __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(b)[e]);
+        return tab[S::SC + field] * __half2float(reinterpret_cast<const __half *>(b)[e]);
+    };
 
     // (p^n, u_z) at node row rr of this column
     // (pq holds the mirror row's values for a ghost row rr < z0; the surface
-    // row carries p = 0 and lambda_p = 0)
-    auto pu_node = [&](int rr, float2 pq, float kd, float lpvz) -> float2 {
-        if (g.fs && rr <= g.z0) return rr == g.z0 ? make_float2(0.f, 0.f) : make_float2(-pq.x, -(kd * pq.y));
-        float u = kd * pq.y;
-        if (colok && rr >= 0 && rr < g.Nz && (rr <= g.z0 - 1 || rr >= g.z0 + g.nz)) u -= a.pml.ai[0][rr] * (lpvz - u);
-        return make_float2(pq.x, u);
+    // row carries p = 0 and mu = 0)
+    auto pu_node = [&](int rr, float2 pq, float lpvz) -> float2 {
+        if (g.fs && rr <= g.z0) return rr == g.z0 ? make_float2(0.f, 0.f) : neg2(pq);
+        if (zpml_node(g, rr)) pq.y -= a.pml.ai[0][rr] * (lpvz - pq.y);
+        return pq;
     };
-    // z rings: PU[m] node row z + m; VW, VN, PIZ half row z + m - M
+    // z rings: PU[m] node row z + m; VW, VN half row z + m - M; PIZ half row z + m - 1
     float2 PU[W], VW[W];
-    float VN[W], PIZ[W];
+    float VN[W], PIZ[M + 1];
 #pragma unroll
     for (int m = 0; m < W; ++m) {
         VW[m] = make_float2(0.f, 0.f);
         VN[m] = 0.f;
-        PIZ[m] = 0.f;
     }
+#pragma unroll
+    for (int m = 0; m <= M; ++m) PIZ[m] = 0.f;
     {
         const float2 *pin = reinterpret_cast<const float2 *>(in) + (A3F_PL / 2) * (long long)pl;
 #pragma unroll
         for (int m = 0; m < W - 1; ++m) {
             const int rr = zstart + m, rs = node_src_row(g, rr);
-            const bool ok = colok && rr >= 0 && rr < g.Nz;
-            const int c = ok ? rr * rowz + cxy : 0;
             const float2 pq = (colok && rs >= 0 && rs < g.Nz) ? pin[rs * rowz + cxy] : make_float2(0.f, 0.f);
-            const float kd = ok ? a.kdt[c] : 0.f;
-            const float lv = (ok && (rr <= g.z0 - 1 || rr >= g.z0 + g.nz)) ? in[A3F_LPVZ * (long long)pl + c] : 0.f;
-            PU[m] = pu_node(rr, pq, kd, lv);
+            const float lv = colok && zpml_node(g, rr) ? in[A3F_LPVZ * (long long)pl + rr * rowz + cxy] : 0.f;
+            PU[m] = pu_node(rr, pq, lv);
         }
     }
     float bz_old = 0.f;
@@ -631,9 +793,6 @@ __global__ void __launch_bounds__(NTH, kMinBlocks) k3f_adj(const __grid_constant
         const int kk = zstart + M - 1;
         if (colok && kk >= 0 && kk < g.Nz) bz_old = a.binv[kk * rowz + cxy];
     }
-    // dt kappa of the look-ahead node row, loaded one row ahead
-    auto kd_at = [&](int rr) { return (colok && rr >= 0 && rr < g.Nz) ? a.kdt[rr * rowz + cxy] : 0.f; };
-    float kd_r = kd_at(zstart + W - 1);
 
     bool failed = false;
     int fail_row = 0;
@@ -645,40 +804,96 @@ __global__ void __launch_bounds__(NTH, kMinBlocks) k3f_adj(const __grid_constant
             fail_row = z;
             break;
         }
-        if (t == NTH - 1 && z + PD - 1 < zc1) {
-            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-            adj_issue<M>(a, sm + ((j + PD - 1) % PD) * S::STAGE, bar + (j + PD - 1) % PD, slot, x0, y0, z + PD - 1,
+        if (z + PD - 1 < zc1)
+            adj_issue<M>(a, warp, sm + ((j + PD - 1) % PD) * S::STAGE, bar + (j + PD - 1) % PD, slot, x0, y0, z + PD - 1,
                          zc0, px, py, px2, py2);
-        }
         unsigned char *st = sm + (j % PD) * S::STAGE;
-        const int k = z + M - 1, r = z + W - 1;
-        {
-            const float2 pq = reinterpret_cast<const float2 *>(st + S::PA)[t];
-            const bool rs = r >= 0 && r < g.Nz && (r <= g.z0 - 1 || r >= g.z0 + g.nz);
-            PU[W - 1] = pu_node(r, pq, kd_r, rs ? reinterpret_cast<const float *>(st + S::LA)[t] : 0.f);
-            kd_r = kd_at(r + 1);
+        auto tile2 = [&](unsigned off) { return reinterpret_cast<const float2 *>(st + off); };
+        auto tile1 = [&](unsigned off) { return reinterpret_cast<const float *>(st + off); };
+        const int k = z + M - 1, c = z * rowz + cxy, izg = z - g.z0;
+        const bool main = z >= zc0;
+        const bool zin = izg >= 0 && izg < g.nz;
+        const bool inner = xin && yin && zin;
+        const bool zf = recon && main && z > g.z0 && z + W < g.z0 + g.nz;
+        const bool surf = g.fs && z == g.z0;   // free-surface row: p = 0, mu = 0
+        // band values of this thread's half nodes in the strips, loaded ahead
+        float bv = 0.f, bvh = 0.f;
+        if (main && !xyf && zin) {
+            if (b_off >= 0) bv = band_raw(1, izg * (yin ? xstr : ystr) + b_off);
+            if (h_off >= 0) {
+                const int hy = (halo_y ? y0 - M + jy : y0 + (hpack & 255)) - g.y0;
+                bvh = band_raw(1, izg * (hy >= 0 && hy < g.ny ? xstr : ystr) + h_off);
+            }
         }
-        // ---- half row k along z: lambda_vz, lambda_psi_pz, background vz^{n-1/2}
-        {
-            const float2 v2 = reinterpret_cast<const float2 *>(st + S::VZ)[t];
-            const float bk1 = k + 1 < g.Nz ? reinterpret_cast<const float *>(st + S::BK)[t] : bz_old;
+        // ---- strip tiles: u_x and u_y of every node the half nodes' stencils
+        // reach, in place of the lambda CPML memories (after the own node's
+        // are advanced)
+        if (main && (px2 || py2)) {
+            const float2 *wP = tile2(S::PW);
+            const float mu = surf ? 0.f : wP[wc].y;
+            if (px2) {
+                float *LX = reinterpret_cast<float *>(st + S::LX);
+                auto put = [&](int l, int w, int cc) {
+                    const float u = wP[w].y;
+                    LX[l] = u - tab[S::WX + cc] * (LX[l] - u);
+                };
+                const int lxc = ty * G::XW2 + tx + G::XO2;
+                if (colok && !(ixg >= 0 && ixg < g.nx)) outf[A3F_LPVX * pl + c] = tab[S::NX + tx] * (LX[lxc] - mu);
+                put(lxc, wc, tx + G::XO2);
+                constexpr int NX2 = 2 * G::XO2;
+                if (t < TY * NX2) {
+                    const int iy = t / NX2, q = t - iy * NX2, cc = q < G::XO2 ? q : q + TX;
+                    put(iy * G::XW2 + cc, (iy + G::YO2) * G::XW2 + cc, cc);
+                }
+            }
+            if (py2) {
+                float *LY = reinterpret_cast<float *>(st + S::LY);
+                auto put = [&](int l, int w, int rr) {
+                    const float u = wP[w].y;
+                    LY[l] = u - tab[S::WY + rr] * (LY[l] - u);
+                };
+                const int lyc = (ty + G::YO2) * TX + tx;
+                if (colok && !(iyg >= 0 && iyg < g.ny)) outf[A3F_LPVY * pl + c] = tab[S::NY + ty] * (LY[lyc] - mu);
+                put(lyc, wc, ty + G::YO2);
+                for (int q = warp; q < 2 * G::YO2; q += TY) {
+                    const int rr = q < G::YO2 ? q : q + TY;
+                    put(rr * TX + tx, rr * G::XW2 + tx + G::XO2, rr);
+                }
+            }
+            // the generic-proxy writes to the stage must be ordered before the
+            // TMA copy that refills it (issued after the next row's barrier)
+            tma::fence_proxy_async();
+            __syncthreads();
+        }
+        // ---- half row k along z: lambda_vz, lambda_psi_pz, background vz^{n-1/2}; half nodes of row z
+        // (ZF: rows without tests, XY: tiles without strips, as in k3f_born)
+        auto v_stage = [&](auto zc, auto xyc) {
+            constexpr bool ZF = decltype(zc)::value, XY = decltype(xyc)::value;
+            const float2 pq = tile2(S::PA)[t];
+            if (ZF) PU[W - 1] = pq;
+            else PU[W - 1] = pu_node(z + W - 1, pq, tile1(S::LA)[t]);
+            const float2 v2z = tile2(S::VZ)[t];
+            float bk1 = tile1(S::BK)[t];
+            if (!ZF && k + 1 >= g.Nz) bk1 = bz_old;   // the last half row replicates the last node row
             float wz = 0.f, vn = 0.f, piz = 0.f;
-            if (colok && k >= 0 && k < g.Nz) {
-                const bool own = k >= zc0 && k < zc1;
+            if (ZF || (k >= 0 && k < g.Nz)) {
+                const bool own = (XY || colok) && (ZF || k >= zc0) && k < zc1;
                 const int ck = k * rowz + cxy;
                 const float2 D = st2<M>(g.cz, [&](int l) { return PU[M - 1 + l]; }, [&](int l) { return PU[M - l]; });
-                const float lv = v2.y + D.y;
+                const float lv = v2z.y + D.y;
                 const float dtbu = dt * 0.5f * (bz_old + bk1);
                 wz = dtbu * lv;
-                if (k <= g.z0 - 2 || k >= g.z0 + g.nz) {
-                    const float l1 = reinterpret_cast<const float *>(st + S::PZ)[t] - dtbu * lv;
+                if (!ZF && (k <= g.z0 - 2 || k >= g.z0 + g.nz)) {
+                    const float l1 = tile1(S::PZ)[t] - dtbu * lv;
                     wz -= a.pml.ah[0][k] * l1;
                     if (own) outf[A3F_LPPZ * pl + ck] = a.pml.bh[0][k] * l1;
                 }
                 piz = D.x * lv;
-                if (recon && xin && yin) {
+                if (ZF) {
+                    vn = XY || (xin && yin) ? v2z.x + dtbu * D.x : 0.f;
+                } else if (recon && xin && yin) {
                     const int iz = k - g.z0;
-                    if ((iz >= 0 || g.fs) && iz < g.nz) vn = v2.x + dtbu * D.x;   // ghost half rows: mirrors
+                    if ((iz >= 0 || g.fs) && iz < g.nz) vn = v2z.x + dtbu * D.x;   // ghost half rows: mirrors
                     else {
                         const long long b = fband(g, 0, iz, iyg, ixg);
                         if (b >= 0) vn = band_get(a.bands, 1, rowprev, b);
@@ -687,194 +902,150 @@ __global__ void __launch_bounds__(NTH, kMinBlocks) k3f_adj(const __grid_constant
                 if (own) out2[(A3F_VZ / 2) * pl + ck] = make_float2(vn, lv);
             }
             bz_old = bk1;
-            VW[W - 1] = make_float2(v2.x, wz);
+            VW[W - 1] = make_float2(v2z.x, wz);
             VN[W - 1] = vn;
-            PIZ[W - 1] = piz;
-        }
-
-        if (z >= zc0) {
-            float2 *wP = reinterpret_cast<float2 *>(st + S::PW);
-            const float *wK = reinterpret_cast<const float *>(st + S::KW);
-            const float *bLX = reinterpret_cast<const float *>(st + S::LX);
-            const float *bLY = reinterpret_cast<const float *>(st + S::LY);
-            const float2 *bVX = reinterpret_cast<const float2 *>(st + S::VX);
-            const float2 *bVY = reinterpret_cast<const float2 *>(st + S::VY);
-            const float *bBB = reinterpret_cast<const float *>(st + S::BB);
-            const float *bQX = reinterpret_cast<const float *>(st + S::QX);
-            const float *bQY = reinterpret_cast<const float *>(st + S::QY);
-            const int rz = z * rowz;
-            // ---- (p, lambda_p) -> (p, dt kappa lambda_p) over the wide tile;
-            // the thread's own node first (it keeps p^n and lambda_p)
-            const int own_w = (ty + G::YO2) * G::XW2 + tx + G::XO2;
-            const bool surf = g.fs && z == g.z0;   // free-surface row: p = 0, lambda_p = 0
-            const float lsc = surf ? 0.f : 1.f;
-            float2 pl1 = wP[own_w];
-            pl1.y *= lsc;
-            const float kd = wK[own_w];
-            const float kl = kd * pl1.y;
-            wP[own_w] = make_float2(pl1.x, kl);
-            for (int i = t; i < G::XW2 * G::YH2; i += NTH) {
-                const int rr = i / G::XW2, cc = i - rr * G::XW2;
-                if (rr >= G::YO2 && rr < G::YO2 + TY && cc >= G::XO2 && cc < G::XO2 + TX) continue;
-                const float2 v = wP[i];
-                wP[i] = make_float2(v.x, wK[i] * (v.y * lsc));
-            }
-            // these generic-proxy writes to the stage must be ordered before the
-            // TMA copy that refills it (issued after the next row's barrier):
-            // every writing thread fences its own writes
-            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-            __syncthreads();
-            // ---- half nodes on the x and y halos of the row
-            constexpr int NVX = TY * G::NXI, NIT = NVX + G::YH1 * TX;
-            for (int i = t; i < NIT; i += NTH) {
-                if (i < NVX) {
-                    const int iy = i / G::NXI, jx = i - iy * G::NXI;
-                    const int xh = x0 - M + jx, yy = y0 + iy;
-                    float2 vw = make_float2(0.f, 0.f);
-                    float vn = 0.f, pi = 0.f;
-                    const int cb = iy * G::XW1 + jx - M + G::XO1;   // xbox entry of half node xh
-                    if (xh >= 0 && xh < g.Nx && yy < g.Ny) {
-                        const int c0 = (iy + G::YO2) * G::XW2 + (jx - M + G::XO2);   // wide entry of node xh
-                        const int l0 = iy * G::XW2 + (jx - M + G::XO2);              // x-wide entry of node xh
-                        auto tap = [&](int l) -> float2 {
-                            float2 v = wP[c0 + l];
-                            if (px2) {
-                                const int xn = xh + l;
-                                if (xn >= 0 && xn < g.Nx && (xn <= g.x0 - 1 || xn >= g.x0 + g.nx))
-                                    v.y -= a.pml.ai[2][xn] * (bLX[l0 + l] - v.y);
-                            }
-                            return v;
-                        };
-                        const float2 D = st2<M>(g.cx, [&](int l) { return tap(l); }, [&](int l) { return tap(1 - l); });
-                        const float2 v2 = bVX[cb];
-                        const float lv = v2.y + D.y;
-                        const float b0 = bBB[M * G::XW1 + cb];
-                        const float b1 = xh + 1 >= g.Nx ? b0 : bBB[M * G::XW1 + cb + 1];
-                        const float dtbu = dt * 0.5f * (b0 + b1);
-                        float w = dtbu * lv;
-                        const bool own = jx >= M && jx < M + TX;
-                        const int o = rz + yy * pitch + xh;
-                        if (px && (xh <= g.x0 - 2 || xh >= g.x0 + g.nx)) {
-                            const float l1 = bQX[cb] - dtbu * lv;
-                            w -= a.pml.ah[2][xh] * l1;
-                            if (own) outf[A3F_LPPX * pl + o] = a.pml.bh[2][xh] * l1;
-                        }
-                        pi = D.x * lv;
-                        if (recon) {
-                            const int iz = z - g.z0, iy2 = yy - g.y0, ix2 = xh - g.x0;
-                            if (iz >= 0 && iz < g.nz && iy2 >= 0 && iy2 < g.ny) {
-                                if (ix2 >= 0 && ix2 < g.nx) vn = v2.x + dtbu * D.x;
-                                else {
-                                    const long long b = fband(g, 2, iz, iy2, ix2);
-                                    if (b >= 0) vn = band_get(a.bands, 1, rowprev, b);
-                                }
-                            }
-                        }
-                        if (own) out2[(A3F_VX / 2) * pl + o] = make_float2(vn, lv);
-                        vw = make_float2(v2.x, w);
-                    }
-                    oWX[iy * G::XW1 + jx] = vw;
-                    oNX[iy * G::XW1 + jx] = vn;
-                    oIX[iy * G::XW1 + jx] = pi;
+            PIZ[M] = piz;
+            if (!ZF && !main) return;
+            // one half node: (v^{n+1/2}, w, v^{n-1/2}, G lambda_v). strip: its u
+            // tile lt (entry l0) in node strip tiles, its table entries a (at q)
+            // and b (len further) and memory psi in half-node strip tiles
+            auto half = [&](const float *cf, int w, int ws, int b, int bst, float2 v2, float hs, bool last, bool p2,
+                            const float *lt, int l0, bool strip, int q, int len, const float *psi, float *psi_out, bool vin,
+                            float band, float2 *v_out) -> float4 {
+                const float2 *p = tile2(S::PW) + w;
+                float2 D;
+                if (XY || !p2) {
+                    D = st2<M>(cf, [&](int l) { return p[l * ws]; }, [&](int l) { return p[(1 - l) * ws]; });
                 } else {
-                    const int i2 = i - NVX;
-                    const int jy = i2 / TX, ix = i2 - jy * TX;
-                    const int yh = y0 - M + jy, xx = x0 + ix;
-                    float2 vw = make_float2(0.f, 0.f);
-                    float vn = 0.f, pi = 0.f;
-                    if (yh >= 0 && yh < g.Ny && xx < g.Nx) {
-                        const int c0 = (jy + M - 1) * G::XW2 + ix + G::XO2;   // wide entry of node yh
-                        const int l0 = (jy + M - 1) * TX + ix;                // y-wide entry of node yh
-                        auto tap = [&](int l) -> float2 {
-                            float2 v = wP[c0 + l * G::XW2];
-                            if (py2) {
-                                const int yn = yh + l;
-                                if (yn >= 0 && yn < g.Ny && (yn <= g.y0 - 1 || yn >= g.y0 + g.ny))
-                                    v.y -= a.pml.ai[1][yn] * (bLY[l0 + l * TX] - v.y);
-                            }
-                            return v;
-                        };
-                        const float2 D = st2<M>(g.cy, [&](int l) { return tap(l); }, [&](int l) { return tap(1 - l); });
-                        const float2 v2 = bVY[i2];
-                        const float lv = v2.y + D.y;
-                        const float *bc = bBB + jy * G::XW1 + ix + G::XO1;
-                        const float b0 = bc[0];
-                        const float b1 = yh + 1 >= g.Ny ? b0 : bc[G::XW1];
-                        const float dtbu = dt * 0.5f * (b0 + b1);
-                        float w = dtbu * lv;
-                        const bool own = jy >= M && jy < M + TY;
-                        const int o = rz + yh * pitch + xx;
-                        if (py && (yh <= g.y0 - 2 || yh >= g.y0 + g.ny)) {
-                            const float l1 = bQY[i2] - dtbu * lv;
-                            w -= a.pml.ah[1][yh] * l1;
-                            if (own) outf[A3F_LPPY * pl + o] = a.pml.bh[1][yh] * l1;
-                        }
-                        pi = D.x * lv;
-                        if (recon) {
-                            const int iz = z - g.z0, iy2 = yh - g.y0, ix2 = xx - g.x0;
-                            if (iz >= 0 && iz < g.nz && ix2 >= 0 && ix2 < g.nx) {
-                                if (iy2 >= 0 && iy2 < g.ny) vn = v2.x + dtbu * D.x;
-                                else {
-                                    const long long b = fband(g, 1, iz, iy2, ix2);
-                                    if (b >= 0) vn = band_get(a.bands, 1, rowprev, b);
-                                }
-                            }
-                        }
-                        if (own) out2[(A3F_VY / 2) * pl + o] = make_float2(vn, lv);
-                        vw = make_float2(v2.x, w);
-                    }
-                    oWY[i2] = vw;
-                    oNY[i2] = vn;
-                    oIY[i2] = pi;
+                    const int ls = ws == 1 ? 1 : TX;
+                    D.x = st1<M>(cf, [&](int l) { return p[l * ws].x; }, [&](int l) { return p[(1 - l) * ws].x; });
+                    D.y = st1<M>(cf, [&](int l) { return lt[l0 + l * ls]; }, [&](int l) { return lt[l0 + (1 - l) * ls]; });
                 }
+                if (!ZF && surf) D.y = 0.f;
+                const float lv = v2.y + D.y;
+                const float b0 = tile1(S::BB)[b];
+                const float b1 = !XY && last ? b0 : tile1(S::BB)[b + bst];
+                const float dtbu = dt * (hs * (b0 + b1));
+                float wv = dtbu * lv;
+                if (!XY && strip) {
+                    const float ah = tab[q], bh = tab[q + len];
+                    const float l1 = *psi - dtbu * lv;
+                    wv -= ah * l1;
+                    if (psi_out && bh != 0.f) *psi_out = bh * l1;
+                }
+                const float vn1 = (ZF && XY) || vin ? v2.x + dtbu * D.x : band;
+                if (v_out) *v_out = make_float2(vn1, lv);
+                return make_float4(v2.x, wv, vn1, D.x * lv);
+            };
+            const bool rz = ZF || (recon && zin);
+            {
+                const int vi = ty * G::XW1 + tx + G::XO1;
+                oX[ty * G::XW1 + tx + M] =
+                    half(g.cx, wc, 1, bc, 1, tile2(S::VX)[vi], 0.5f, x + 1 >= g.Nx, px2, tile1(S::LX),
+                         ty * G::XW2 + tx + G::XO2, px, S::HX + tx + M, G::XH1, tile1(S::QX) + vi,
+                         colok ? outf + A3F_LPPX * pl + c : nullptr, rz && xin && yin, yin ? bv : 0.f,
+                         XY || colok ? out2 + (A3F_VX / 2) * pl + c : nullptr);
             }
+            {
+                const int vi = (ty + M) * TX + tx;
+                oY[vi] = half(g.cy, wc, G::XW2, bc, G::XW1, tile2(S::VY)[vi], 0.5f, y + 1 >= g.Ny, py2, tile1(S::LY),
+                              (ty + G::YO2) * TX + tx, py, S::HY + ty + M, G::YH1, tile1(S::QY) + vi,
+                              colok ? outf + A3F_LPPY * pl + c : nullptr, rz && xin && yin, xin ? bv : 0.f,
+                              XY || colok ? out2 + (A3F_VY / 2) * pl + c : nullptr);
+            }
+            if (halo_y) {
+                const int hi = y0 - M + jy, vi = jy * TX + tx;
+                const bool vin = rz && xin && hi >= g.y0 && hi < g.y0 + g.ny;
+                oY[vi] = half(g.cy, (jy + M - 1) * G::XW2 + tx + G::XO2, G::XW2, jy * G::XW1 + tx + G::XO1, G::XW1,
+                              tile2(S::VY)[vi], XY || hi >= 0 ? 0.5f : 0.f, hi + 1 >= g.Ny, py2, tile1(S::LY),
+                              (jy + M - 1) * TX + tx, py, S::HY + jy, G::YH1, tile1(S::QY) + vi, nullptr, vin, bvh, nullptr);
+            } else if (halo_x) {
+                int h = hpack;
+                const int hiy = h & 255, hjx = h >> 8, hi = x0 - M + hjx, hj = y0 + hiy, vi = hiy * G::XW1 + hjx - M + G::XO1;
+                const bool vin = rz && hj >= g.y0 && hj < g.y0 + g.ny && hi >= g.x0 && hi < g.x0 + g.nx;
+                oX[hiy * G::XW1 + hjx] =
+                    half(g.cx, (hiy + G::YO2) * G::XW2 + hjx - M + G::XO2, 1, (hiy + M) * G::XW1 + hjx - M + G::XO1, 1,
+                         tile2(S::VX)[vi], XY || hi >= 0 ? 0.5f : 0.f, hi + 1 >= g.Nx, px2, tile1(S::LX),
+                         hiy * G::XW2 + hjx - M + G::XO2, px, S::HX + hjx, G::XH1, tile1(S::QX) + vi, nullptr, vin, bvh, nullptr);
+            }
+        };
+        const std::true_type Y{};
+        const std::false_type N{};
+        if (xyf) {
+            if (zf) v_stage(Y, Y);
+            else v_stage(N, Y);
+        } else {
+            if (zf) v_stage(Y, N);
+            else v_stage(N, N);
+        }
+        // the node's band value, or z strip memory
+        float bp = 0.f;
+        if (main && !(xyf && zf)) {
+            if (zin) {
+                if (b_off >= 0) bp = band_raw(0, izg * (yin ? xstr : ystr) + b_off);
+            } else if (recon && colok) {
+                const long long b = fband(g, 0, izg, iyg, ixg);
+                if (b >= 0) bp = band_raw(0, (int)b);
+            }
+            if (!zf && colok && zpml_node(g, z))
+                outf[A3F_LPVZ * pl + c] = a.pml.bi[0][z] * (in[A3F_LPVZ * pl + c] - (surf ? 0.f : tile2(S::PW)[wc].y));
+        }
+        if (main) {
             __syncthreads();
             // ---- node of the thread's own column at row z
-            if (colok) {
-                const int hx = ty * G::XW1 + tx + M;     // x half node x (x + 1/2)
-                const int hy = (ty + M) * TX + tx;       // y half node y
-                const float2 Ex = st2<M>(g.cx, [&](int l) { return oWX[hx + l - 1]; }, [&](int l) { return oWX[hx - l]; });
-                const float2 Ey = st2<M>(g.cy, [&](int l) { return oWY[hy + (l - 1) * TX]; },
-                                         [&](int l) { return oWY[hy - l * TX]; });
+            auto node_stage = [&](auto zc, auto xyc) {
+                constexpr bool ZF = decltype(zc)::value, XY = decltype(xyc)::value;
+                // (Q_n, D- w) and D- v^{n-1/2} along an axis, and the two adjacent G lambda_v products
+                auto axis = [&](const float *cf, const float4 *o, int st_, float2 &E, float &q, float &pi) {
+                    float2 d2[M];
+                    float dn[M];
+#pragma unroll
+                    for (int l = 0; l < M; ++l) {
+                        const float4 u = o[l * st_], v = o[-(l + 1) * st_];
+                        d2[l] = sub2(make_float2(u.x, u.y), make_float2(v.x, v.y));
+                        dn[l] = u.z - v.z;
+                        if (l == 0) pi = u.w + v.w;
+                    }
+                    E = mul2(cf[0], d2[0]);
+                    q = cf[0] * dn[0];
+#pragma unroll
+                    for (int l = 1; l < M; ++l) {
+                        E = fma2(cf[l], d2[l], E);
+                        q = fmaf(cf[l], dn[l], q);
+                    }
+                };
+                float2 Ex, Ey;
+                float qx, qy, pix, piy;
+                axis(g.cx, oX + ty * G::XW1 + tx + M, 1, Ex, qx, pix);
+                axis(g.cy, oY + (ty + M) * TX + tx, TX, Ey, qy, piy);
                 const float2 Ez = st2<M>(g.cz, [&](int l) { return VW[M + l - 1]; }, [&](int l) { return VW[M - l]; });
                 const float2 E = add2(add2(Ex, Ey), Ez);   // (Q_n = D- . v^{n+1/2}, D- . w)
-                const int c = rz + cxy;
-                const int izg = z - g.z0;
-                const bool inner = xin && yin && izg >= 0 && izg < g.nz;
                 // D- . v^{n-1/2}, summed z, y, x as the background pass sums
                 // it, so the rebuilt p^{n-1} undoes that pass's rounding
-                float qn = 0.f;
-                if (recon)
-                    qn = (st1<M>(g.cz, [&](int l) { return VN[M + l - 1]; }, [&](int l) { return VN[M - l]; }) +
-                          st1<M>(g.cy, [&](int l) { return oNY[hy + (l - 1) * TX]; },
-                                 [&](int l) { return oNY[hy - l * TX]; })) +
-                         st1<M>(g.cx, [&](int l) { return oNX[hx + l - 1]; }, [&](int l) { return oNX[hx - l]; });
-                if (inner) {
-                    float2 acc = img[c];
-                    acc.x += E.x * pl1.y;
+                const float qn = (st1<M>(g.cz, [&](int l) { return VN[M + l - 1]; }, [&](int l) { return VN[M - l]; }) + qy) + qx;
+                float2 pm = tile2(S::PW)[wc];
+                if (!ZF && surf) pm.y = 0.f;
+                const float kd = tile1(S::KD)[t];
+                const bool in_ = (ZF && XY) || inner;
+                if (in_) {
+                    float2 acc = tile2(S::IM)[t];
+                    acc.x += E.x * pm.y;
                     // (on the free surface the half row above is a ghost: no product of its own)
-                    acc.y += (oIX[hx] + oIX[hx - 1]) + (oIY[hy] + oIY[hy - TX]) + (PIZ[M] + (surf ? 0.f : PIZ[M - 1]));
+                    acc.y += pix + piy + (PIZ[1] + (!ZF && surf ? 0.f : PIZ[0]));
                     img[c] = acc;
                 }
-                float pn = 0.f;
-                if (recon) {
-                    if (inner) {
-                        pn = pl1.x + kd * qn;
-                        if (c == src) pn -= wsrc;
-                    } else {
-                        long long b = -1;
-                        for (int d = 0; d < 3 && b < 0; ++d) b = fband(g, d, izg, iyg, ixg);
-                        if (b >= 0) pn = band_get(a.bands, 0, rowprev, b);
-                    }
-                }
-                out2[(A3F_PL / 2) * pl + c] =
-                    (g.fs && z <= g.z0) ? make_float2(0.f, 0.f) : make_float2(pn, pl1.y + E.y);
-                if (x <= g.x0 - 1 || x >= g.x0 + g.nx)
-                    outf[A3F_LPVX * pl + c] = a.pml.bi[2][x] * (bLX[ty * G::XW2 + tx + G::XO2] - kl);
-                if (y <= g.y0 - 1 || y >= g.y0 + g.ny)
-                    outf[A3F_LPVY * pl + c] = a.pml.bi[1][y] * (bLY[(ty + G::YO2) * TX + tx] - kl);
-                if (z <= g.z0 - 1 || z >= g.z0 + g.nz)
-                    outf[A3F_LPVZ * pl + c] = a.pml.bi[0][z] * (in[A3F_LPVZ * pl + c] - kl);
+                float pn = in_ && (ZF || recon) ? pm.x + kd * qn : bp;
+                pn -= c == src ? wsrc : 0.f;   // (a source node is an interior one; wsrc = 0 at the last reverse step)
+                float2 pmn = make_float2(pn, fmaf(kd, E.y, pm.y));
+                if (!ZF && g.fs && z <= g.z0) pmn = make_float2(0.f, 0.f);
+                if (XY || colok) out2[(A3F_PL / 2) * pl + c] = pmn;
+            };
+            if (xyf) {
+                if (zf) node_stage(Y, Y);
+                else node_stage(N, Y);
+            } else {
+                if (zf) node_stage(Y, N);
+                else node_stage(N, N);
             }
         }
 #pragma unroll
@@ -882,15 +1053,16 @@ __global__ void __launch_bounds__(NTH, kMinBlocks) k3f_adj(const __grid_constant
             PU[m] = PU[m + 1];
             VW[m] = VW[m + 1];
             VN[m] = VN[m + 1];
-            PIZ[m] = PIZ[m + 1];
         }
+#pragma unroll
+        for (int m = 0; m < M; ++m) PIZ[m] = PIZ[m + 1];
     }
 
     if (failed) {
         if (t == 0) {
             atomicOr(a.err, 1);
             const int jf = fail_row - zstart;
-            for (int jj = jf; jj < jf + PD && zstart + jj < zc1; ++jj)
+            for (int jj = jf; jj < jf + PD - 1 && zstart + jj < zc1; ++jj)
                 (void)mbar_wait(bar + jj % PD, (unsigned)(jj / PD) & 1u);
         }
         return;
@@ -899,15 +1071,15 @@ __global__ void __launch_bounds__(NTH, kMinBlocks) k3f_adj(const __grid_constant
         // pre-add the residual of step n-1 at the receivers of this tile
         __syncthreads();
         const int ntile = (int)(gridDim.x * gridDim.y) * nzc;
-        const int tile = shot * ntile + (zcn * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-        const int b = a.trec.ptr[tile], e = a.trec.ptr[tile + 1];
+        const int rt = shot * ntile + (zcn * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+        const int b = a.trec.ptr[rt], e = a.trec.ptr[rt + 1];
         for (int i = b + t; i < e; i += NTH) {
             const int2 rc = a.trec.rec[i];
             if (i > b && a.trec.rec[i - 1].x == rc.x) continue;   // run handled by its first entry
             float add = 0.f;
             for (int q = i; q < e && a.trec.rec[q].x == rc.x; ++q)
                 add += a.dstage[(long long)a.trec.rec[q].y * g.nt + (n - 1)];
-            out2[(A3F_PL / 2) * pl + rc.x].y += add;
+            out2[(A3F_PL / 2) * pl + rc.x].y += a.kdt[rc.x] * add;
         }
     }
 }
@@ -1046,8 +1218,33 @@ cudaError_t fused3d_adj_maps(Adj3F &a, const float *kdt, const float *binv, int 
     // model: plane 0 dt kappa, plane 1 1/rho (adjacent)
     if (binv - kdt != (ptrdiff_t)g.plane) return cudaErrorInvalidValue;
     if ((e = make_tmap3(&a.m_core, kdt, g, 4, 2, TX, TY)) != cudaSuccess) return e;
-    if ((e = make_tmap3(&a.m_wide, kdt, g, 4, 2, XW2, YH2)) != cudaSuccess) return e;
+    if ((e = make_tmap3(&a.im, a.img, g, 8, batch, TX, TY)) != cudaSuccess) return e;
     return make_tmap3(&a.m_ybr, kdt, g, 4, 2, XW1, YHB);
+}
+
+// A chunk of t rows marches t + 2M. A CTA that shares its SM with another one
+// takes 1.25x its time alone; past two a SM the warm-up rows hide behind other
+// CTAs and what counts is the work repeated and the last wave (0.6 of one on
+// average): the model's relative costs a row, 1, 1.25 and 1.06 a wave, follow
+// from a Born and migration step of 168 x 296 x 296 cells: 1 shot 1300 us in
+// one chunk, 1253 in 84 rows, 1053 in 24, 1066 in 16; 2 shots 2449, 2090,
+// 2002, 2076, and 1969 in 34; 16 shots 14415, 14250 (84), 15271, 16235; 100 x
+// 120 x 130 cells, 1 shot: 658 in one chunk, 252 in 25 rows, 182 in 17.
+int march3d_rows(int M, int Nz, long long ctas)
+{
+    constexpr double sms = 152.0;
+    double best = 1e300;
+    int rows = Nz;
+    for (int nc = 1; nc <= Nz; ++nc) {
+        const int t = (Nz + nc - 1) / nc;
+        const double n = (double)ctas * ((Nz + t - 1) / t), q = std::ceil(n / sms);
+        const double c = q <= 2.0 ? (t + 2 * M) * (q <= 1.0 ? 1.0 : 1.25) : (t + 0.5 * M) * 1.06 * (n / (2.0 * sms) + 0.6);
+        if (c < best) {
+            best = c;
+            rows = t;
+        }
+    }
+    return rows;
 }
 
 cudaError_t configure_3d_kernels()

@@ -88,12 +88,9 @@ __global__ void k_inject(GridDev gm, GridDev g, TileRecs tr, int shot0, const fl
         float add = 0.f;
         for (int k = i; k < e && tr.rec[k].x == rc.x; ++k)
             add += dstage[(long long)tr.rec[k].y * g.nt + n];
-        if (kdt) {
-            // node of the model grid (windowed shots, 2D: z and the column in the window)
-            const long long c = win_x0 ? (long long)(rc.x / g.pitch) * gm.pitch + rc.x % g.pitch + win_x0[shot0 + slot] : rc.x;
-            add *= kdt[c];
-        }
-        dst[rc.x].y += add;
+        // node of the model grid (windowed shots, 2D: z and the column in the window)
+        const long long c = win_x0 ? (long long)(rc.x / g.pitch) * gm.pitch + rc.x % g.pitch + win_x0[shot0 + slot] : rc.x;
+        dst[rc.x].y += kdt[c] * add;
     }
 }
 
@@ -162,16 +159,15 @@ __global__ void k_band_pack(Bands b, int shot0, int n)
     }
 }
 
-// g_kappa = -dt kappa sum_n Q lp, g_rho = (dt / 2) / rho * sum_n (products at
+// g_kappa = -sum_n Q (dt kappa lp), g_rho = (dt / 2) / rho * sum_n (products at
 // the adjacent half nodes); g_Vp = g_kappa - g_rho, g_Ip = g_kappa + g_rho.
-__global__ void k_image_fin(GridDev g, const double2 *acc, const float *kdt, const float *binv,
-                            float *gout)
+__global__ void k_image_fin(GridDev g, const double2 *acc, const float *binv, float *gout)
 {
     long long nint = (long long)g.nz * g.ny * g.nx;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < nint;
          k += (long long)gridDim.x * blockDim.x) {
         long long c = pad_of(g, k);
-        double gk = g.ndim == 2 ? -acc[k].x : -(double)kdt[c] * acc[k].x;   // (2D: acc.x holds sum Q dt kappa lp)
+        double gk = -acc[k].x;
         double gr = 0.5 * (double)g.dt * (double)binv[c] * acc[k].y;
         gout[k] = (float)(gk - gr);
         gout[nint + k] = (float)(gk + gr);
@@ -558,11 +554,11 @@ cudaError_t launch_band_pack(const Bands &b, int batch, int shot0, int n, cudaSt
     return cudaGetLastError();
 }
 
-cudaError_t launch_image_finalize(const GridDev &g, const double2 *acc, const float *kdt,
-                                  const float *binv, float *gout, cudaStream_t s)
+cudaError_t launch_image_finalize(const GridDev &g, const double2 *acc, const float *binv, float *gout,
+                                  cudaStream_t s)
 {
     long long n = (long long)g.nz * g.ny * g.nx;
-    k_image_fin<<<grid_for(n), NT, 0, s>>>(g, acc, kdt, binv, gout);
+    k_image_fin<<<grid_for(n), NT, 0, s>>>(g, acc, binv, gout);
     return cudaGetLastError();
 }
 

@@ -191,6 +191,9 @@ struct Step3D {
 // Fused 3D time-step kernels (kernels3d_fused.cu): CTAs of kTile3X x kTile3Y
 // (x, y) columns marching a z-chunk of tzc rows, ping-pong state buffers.
 constexpr int kTile3X = 32, kTile3Y = 12;
+// Rows per z-chunk for a padded depth Nz when a chunk has `ctas` CTAs over the
+// columns and the shots of a batch (kernels3d_fused.cu).
+int march3d_rows(int M, int Nz, long long ctas);
 // Pair-plane offsets within a slot. Born ping-pong: (p, dp), (vx, dvx),
 // (vy, dvy), (vz, dvz), (psi_p, dpsi_p) x y z; the node CPML memories
 // (psi_v, dpsi_v) x y z live in a separate in-place block.
@@ -217,7 +220,7 @@ struct Step3F {
     float *dstage;            // records [nrec_total][nt]
     int *err;                 // error word: 1 = a wait gave up, 2 = a misaligned copy was refused
 };
-// Fused 3D adjoint layout (float planes of a slot): pairs (p, lambda_p) 0-1,
+// Fused 3D adjoint layout (float planes of a slot): pairs (p, dt kappa lambda_p) 0-1,
 // (vx, lambda_vx) 2-3, (vy, lambda_vy) 4-5, (vz, lambda_vz) 6-7, then the
 // lambda CPML memories psi_p x y z (8-10) and psi_v x y z (11-13).
 enum { A3F_PL = 0, A3F_VX = 2, A3F_VY = 4, A3F_VZ = 6, A3F_LPPX = 8, A3F_LPPY = 9, A3F_LPPZ = 10,
@@ -227,16 +230,17 @@ constexpr int kAdjPlanes3F = 14;
 struct Adj3F {
     // input-state pair planes (core, wide, xbox, ybox), input-state float
     // planes (core, xwide, ywide, xbox, ybox), model float planes (plane 0
-    // dt kappa, plane 1 1/rho: core, wide, ybr)
+    // dt kappa, plane 1 1/rho: core, ybr)
     CUtensorMap p_core, p_wide, p_xbox, p_ybox;
     CUtensorMap f_core, f_xwide, f_ywide, f_xbox, f_ybox;
-    CUtensorMap m_core, m_wide, m_ybr;
+    CUtensorMap m_core, m_ybr;
+    CUtensorMap im;           // image accumulators: float2 planes of the slots, core
     GridDev g;
     Pml pml;
     const float *in;          // input state, slot stride in_planes float planes
     float *out;               // output state, slot stride out_planes
     int in_planes, out_planes;
-    const float *kdt, *binv;  // for the first rows of a march
+    const float *kdt, *binv;  // for the first rows of a march and the residual
     float2 *img;              // [batch][plane] image accumulators (in place)
     int n, tzc, shot0;
     const float *wav;
@@ -347,10 +351,9 @@ cudaError_t launch_model_prep(const GridDev &g, const float *vp, const float *rh
                               float *binv, cudaStream_t s);
 cudaError_t launch_pert_prep(const GridDev &g, const float *dm, const float *kdt,
                              const float *binv, float2 *kd2, float2 *br2, cudaStream_t s);
-// Adds the residual of step n to lambda_p (the .y of the (p, lambda_p)
-// pairs), times dt kappa of the node where the state carries dt kappa lambda_p
-// (kdt non-null: planes of the model grid gm, of which shot s's slot grid g
-// takes the columns from win_x0[s], or all with win_x0 null).
+// Adds dt kappa times the residual of step n to dt kappa lambda_p (the .y of
+// the (p, dt kappa lambda_p) pairs). kdt: of the model grid gm, of which shot
+// s's slot grid g takes the columns from win_x0[s], or all with win_x0 null.
 cudaError_t launch_inject_residual(const GridDev &gm, const GridDev &g, const TileRecs &tr, int batch, int shot0,
                                    const float *dstage, int n, const float *kdt, const int *win_x0, float2 *pl,
                                    long long sstride2, cudaStream_t s);
@@ -359,9 +362,9 @@ cudaError_t launch_inject_residual(const GridDev &gm, const GridDev &g, const Ti
 // columns [win_x0, win_x0 + win_nx) of shot shot0 + b.
 cudaError_t launch_image_accumulate(const GridDev &gm, const GridDev &g, const float2 *img, int batch, int shot0,
                                     const int *win_x0, const int *win_nx, double2 *acc, cudaStream_t s);
-// The kappa image of 2D grids holds sum Q dt kappa lambda_p, of 3D grids sum Q lambda_p.
-cudaError_t launch_image_finalize(const GridDev &g, const double2 *acc, const float *kdt,
-                                  const float *binv, float *gout, cudaStream_t s);
+// acc: (sum Q dt kappa lambda_p, sum of the adjacent half nodes' products).
+cudaError_t launch_image_finalize(const GridDev &g, const double2 *acc, const float *binv, float *gout,
+                                  cudaStream_t s);
 cudaError_t launch_hess_accumulate(const GridDev &gm, const GridDev &g, const float *hess, int batch, int shot0,
                                    const int *win_x0, const int *win_nx, double *acc, cudaStream_t s);
 cudaError_t launch_hess_finalize(const GridDev &g, const double *acc, float *out,
