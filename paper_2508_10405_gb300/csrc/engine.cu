@@ -1349,10 +1349,7 @@ lsrtm_status create_impl(const lsrtm_config *cfg, const float *vp, const float *
         const int bs = per > 0 ? std::min(per, ns) : ns;
         if (d3) {
             const long long ntxy = (long long)((g.Nx + kTile3X - 1) / kTile3X) * ((g.Ny + kTile3Y - 1) / kTile3Y);
-            // enough CTAs for two waves of one CTA per SM, chunks of at least 8M rows
-            const long long want = (2 * 152 + ntxy * ns - 1) / std::max(1LL, ntxy * ns);
-            const int nchunk = (int)std::max(1LL, std::min(want, (long long)(g.Nz / (8 * g.M))));
-            h->tzc = (g.Nz + nchunk - 1) / nchunk;
+            h->tzc = march3d_rows(g.M, g.Nz, ntxy * bs);
         } else {
             const bool w = geo && geo->win_x0 && geo->win_nx && geo->nshot > 0;
             long long ctas = 0;
