@@ -13,7 +13,8 @@
 // parameter j. The parameter mask restricts the operator to P H P.
 //
 // k_psfh_patches: the node windows, packed per (node, offset) as one float4
-//   of the four blocks (00, 01, 10, 11), so one 16-byte load serves all four.
+//   of the four blocks (00, 01, 10, 11; for H^T 00, 10, 01, 11), so one 16-byte
+//   load serves all four and its halves are the pairs of packed products.
 // k_psfh_apply<MASK, TR, R>: one thread per output column and R consecutive
 //   rows (R = the largest of 8, 4, 2, 1 not above s), CTAs of 32 columns x
 //   2 R rows (small CTAs spread the one wave evenly over the SMs). The input
@@ -23,7 +24,13 @@
 //   (three node rows, two node columns; R <= s rows cross at most one node
 //   row) through L1, interpolates along x once and along z per row: one
 //   loaded value serves R pixels, which keeps the L1 return path (the limit
-//   of a one-pixel-per-thread form) below the FMA pipe.
+//   of a one-pixel-per-thread form) below the FMA pipe. A warp's rows are the
+//   same for all its lanes, and most warps' (12 of 20 positions at s = 20, R = 8)
+//   lie between two node rows: those load four node values an offset, not six,
+//   and interpolate with one multiply-add. 300 x 2000, s = 20, 19 x 19 windows,
+//   two parameters: 239 -> 180 us an application (packed products and this;
+//   packed products alone 219, with two offsets loaded ahead 300: 160
+//   registers). What bounds it now: the L1 return path (68%) and its latency.
 //   TR = false: y(r) = sum_a H(r, r - a) x(r - a), the columns gathered at r;
 //   TR = true:  y(c) = sum_a H(c + a, c) x(c + a), the transpose.
 // k_psfh3_patches, k_psfh3_rows: the same for 3D images, with the eight
@@ -31,6 +38,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "lsrtm_internal.cuh"
 #include "psfhess3d.cuh"
@@ -69,7 +77,7 @@ __device__ __forceinline__ Corner corner_of(int c, int n, int s, int nk)
 }
 
 __global__ void k_psfh_patches(const float *psf_vp, const float *psf_ip, int nz, int nx, int s, int half,
-                               int nkz, int nkx, int mask, float4 *pt)
+                               int nkz, int nkx, int mask, bool transpose, float4 *pt)
 {
     const int L = 2 * half + 1, LL = L * L;
     const long long plane = (long long)nz * nx;
@@ -89,20 +97,27 @@ __global__ void k_psfh_patches(const float *psf_vp, const float *psf_ip, int nz,
             const bool use = inside && src && ((mask >> po) & 1) && ((mask >> pi) & 1);
             v[b] = use ? src[po * plane + (long long)z * nx + x] : 0.f;
         }
-        pt[i] = make_float4(v[0], v[1], v[2], v[3]);
+        pt[i] = make_float4(v[0], transpose ? v[2] : v[1], transpose ? v[1] : v[2], v[3]);
     }
 }
 
-// Parameter-block values: a float4 of the four blocks (two parameters) or
-// the one block of a single-parameter mask.
+// Parameter-block values: the four blocks (two parameters) as two pairs, each
+// pair the two blocks whose products with an input pixel's two planes make up
+// one output plane, or the one block of a single-parameter mask. Pairs take
+// packed FP32x2 arithmetic: with scalars the interpolation and the products
+// were bound by issue slots.
+struct Pairs {
+    float2 a, b;
+};
 template <int MASK>
 struct Blk {
     using T = float;
 };
 template <>
 struct Blk<3> {
-    using T = float4;
+    using T = Pairs;
 };
+__device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
 
 template <int BM>
 __device__ __forceinline__ float load_blk(const float4 *pt, int i, float)
@@ -110,44 +125,90 @@ __device__ __forceinline__ float load_blk(const float4 *pt, int i, float)
     return __ldg(reinterpret_cast<const float *>(pt) + 4 * i + BM);
 }
 template <int BM>
-__device__ __forceinline__ float4 load_blk(const float4 *pt, int i, float4)
+__device__ __forceinline__ Pairs load_blk(const float4 *pt, int i, Pairs)
 {
-    return __ldg(pt + i);
+    const float4 v = __ldg(pt + i);
+    return Pairs{make_float2(v.x, v.y), make_float2(v.z, v.w)};
 }
 // p0 + w (p1 - p0)
-__device__ __forceinline__ float lerp_(float p0, float p1, float w) { return fmaf(w, p1 - p0, p0); }
-__device__ __forceinline__ float4 lerp_(float4 p0, float4 p1, float w)
-{
-    return make_float4(lerp_(p0.x, p1.x, w), lerp_(p0.y, p1.y, w), lerp_(p0.z, p1.z, w), lerp_(p0.w, p1.w, w));
-}
 __device__ __forceinline__ float sub_(float a, float b) { return a - b; }
-__device__ __forceinline__ float4 sub_(float4 a, float4 b) { return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w); }
+__device__ __forceinline__ float2 sub_(float2 a, float2 b) { return __ffma2_rn(dup(-1.f), b, a); }
+__device__ __forceinline__ Pairs sub_(Pairs a, Pairs b) { return Pairs{sub_(a.a, b.a), sub_(a.b, b.b)}; }
+__device__ __forceinline__ float lerp_(float p0, float p1, float w) { return fmaf(w, p1 - p0, p0); }
+__device__ __forceinline__ float2 lerp_(float2 p0, float2 p1, float w) { return __ffma2_rn(dup(w), sub_(p1, p0), p0); }
+__device__ __forceinline__ Pairs lerp_(Pairs p0, Pairs p1, float w) { return Pairs{lerp_(p0.a, p1.a, w), lerp_(p0.b, p1.b, w)}; }
 // q0 + b d1 + c d2 (= (1 - b - c) q0 + b q1 + c q2 with d1 = q1 - q0, d2 = q2 - q0)
 __device__ __forceinline__ float mix3(float q0, float d1, float d2, float b, float c)
 {
     return fmaf(c, d2, fmaf(b, d1, q0));
 }
-__device__ __forceinline__ float4 mix3(float4 q0, float4 d1, float4 d2, float b, float c)
+__device__ __forceinline__ float2 mix3(float2 q0, float2 d1, float2 d2, float2 b, float2 c)
 {
-    return make_float4(mix3(q0.x, d1.x, d2.x, b, c), mix3(q0.y, d1.y, d2.y, b, c), mix3(q0.z, d1.z, d2.z, b, c),
-                       mix3(q0.w, d1.w, d2.w, b, c));
+    return __ffma2_rn(c, d2, __ffma2_rn(b, d1, q0));
 }
+__device__ __forceinline__ Pairs mix3(Pairs q0, Pairs d1, Pairs d2, float2 b, float2 c)
+{
+    return Pairs{mix3(q0.a, d1.a, d2.a, b, c), mix3(q0.b, d1.b, d2.b, b, c)};
+}
+// q0 + b d1: rows that no node row separates
+__device__ __forceinline__ float mix2(float q0, float d1, float b) { return fmaf(b, d1, q0); }
+__device__ __forceinline__ Pairs mix2(Pairs q0, Pairs d1, float2 b)
+{
+    return Pairs{__ffma2_rn(b, d1.a, q0.a), __ffma2_rn(b, d1.b, q0.b)};
+}
+// Row weights: a scalar, or the pair both of a Pairs' products take.
+template <int MASK>
+struct Wgt {
+    using T = float;
+    static __device__ __forceinline__ T of(float w) { return w; }
+};
+template <>
+struct Wgt<3> {
+    using T = float2;
+    static __device__ __forceinline__ T of(float w) { return dup(w); }
+};
+// Accumulators of one output pixel: a scalar, or per output plane the two
+// input planes' sums.
+__device__ __forceinline__ void accum(float &acc, float C, float x) { acc = fmaf(C, x, acc); }
+__device__ __forceinline__ void accum(Pairs &acc, Pairs C, float2 x)
+{
+    acc.a = __ffma2_rn(C.a, x, acc.a);
+    acc.b = __ffma2_rn(C.b, x, acc.b);
+}
+__device__ __forceinline__ float plane0(float a) { return a; }
+__device__ __forceinline__ float plane0(Pairs a) { return a.a.x + a.a.y; }
+__device__ __forceinline__ float plane1(float) { return 0.f; }
+__device__ __forceinline__ float plane1(Pairs a) { return a.b.x + a.b.y; }
 
 // Weights of R consecutive rows (first corner row kf) on the node rows
 // kf + 1 and kf + 2 (the rest, on kf, is implied): row r puts 1 - w on its k0
 // and w on its k1. R <= s keeps every k0 in {kf, kf + 1} and every k1 in
 // {kf, .., kf + 2}.
-template <int R>
-__device__ __forceinline__ void row_weights(const Corner *zc, int kf, float (&wb)[R], float (&wc)[R])
+template <int MASK, int R>
+__device__ __forceinline__ void row_weights(const Corner *zc, int kf, typename Wgt<MASK>::T (&wb)[R],
+                                            typename Wgt<MASK>::T (&wc)[R])
 {
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const Corner Z = zc[r];
         const int s0 = Z.k0 - kf, s1 = Z.k1 - kf;
         const float u = 1.f - Z.w, w = Z.w;
-        wb[r] = (s0 == 1 ? u : 0.f) + (s1 == 1 ? w : 0.f);
-        wc[r] = s1 == 2 ? w : 0.f;
+        wb[r] = Wgt<MASK>::of((s0 == 1 ? u : 0.f) + (s1 == 1 ? w : 0.f));
+        wc[r] = Wgt<MASK>::of(s1 == 2 ? w : 0.f);
     }
+}
+
+// Whether a node row separates the R rows (a weight on kf + 2). The rows of a
+// warp are the same for all its lanes.
+__device__ __forceinline__ bool nonzero(float w) { return w != 0.f; }
+__device__ __forceinline__ bool nonzero(float2 w) { return w.x != 0.f; }
+template <int MASK, int R>
+__device__ __forceinline__ bool any_weight(const typename Wgt<MASK>::T (&wc)[R])
+{
+    bool any = false;
+#pragma unroll
+    for (int r = 0; r < R; ++r) any |= nonzero(wc[r]);
+    return any;
 }
 
 // One thread per column and R consecutive rows; CTAs of 32 columns x kRowThreads
@@ -196,12 +257,13 @@ __global__ void __launch_bounds__(kApplyThreads) k_psfh_apply(const PsfHessDev a
 
     const float4 *pt = a.pt;
     const int nkx = a.nkx, nkz1 = a.nkz - 1;
-    const float2 *t2 = reinterpret_cast<const float2 *>(tile);
     const V zero = V{};
-    float acc0[R], acc1[R];
+    using X = typename std::conditional<MASK == 3, float2, float>::type;
+    const X *in_t = reinterpret_cast<const X *>(tile);
+    V acc[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) acc0[r] = acc1[r] = 0.f;
-    float wb[R], wc[R];
+    for (int r = 0; r < R; ++r) acc[r] = V{};
+    typename Wgt<MASK>::T wb[R], wc[R];
 
     if (!TR) {
         // y(r) = sum_a [sum_corners(c) w P(a)] x(c), c = r - a: for offset
@@ -209,87 +271,78 @@ __global__ void __launch_bounds__(kApplyThreads) k_psfh_apply(const PsfHessDev a
         for (int dz = -h; dz <= h; ++dz) {
             const int row0 = ty * R + h - dz;   // tile row of c = rz0 - dz
             const int kf = zc[row0].k0;
-            row_weights<R>(zc + row0, kf, wb, wc);
+            row_weights<MASK, R>(zc + row0, kf, wb, wc);
             const int n0 = kf * nkx, n1 = min(kf + 1, nkz1) * nkx, n2 = min(kf + 2, nkz1) * nkx;
             const int arow = (dz + h) * L + h;
             // node values of offset dx = -h, then of dx + 1 while dx is used
-            int col = tx + 2 * h;
-            int xk0 = xc[col].k0, xk1 = xc[col].k1;
-            float wx = xc[col].w;
-            V p00 = load_blk<BM>(pt, (n0 + xk0) * LL + arow - h, zero);
-            V p01 = load_blk<BM>(pt, (n0 + xk1) * LL + arow - h, zero);
-            V p10 = load_blk<BM>(pt, (n1 + xk0) * LL + arow - h, zero);
-            V p11 = load_blk<BM>(pt, (n1 + xk1) * LL + arow - h, zero);
-            V p20 = load_blk<BM>(pt, (n2 + xk0) * LL + arow - h, zero);
-            V p21 = load_blk<BM>(pt, (n2 + xk1) * LL + arow - h, zero);
-            for (int dx = -h; dx <= h; ++dx) {
-                const int dn = min(dx + 1, h), cn = tx + h - dn, an = arow + dn;
-                const int yk0 = xc[cn].k0, yk1 = xc[cn].k1;
-                const float wn = xc[cn].w;
-                const V n00 = load_blk<BM>(pt, (n0 + yk0) * LL + an, zero);
-                const V n01 = load_blk<BM>(pt, (n0 + yk1) * LL + an, zero);
-                const V n10 = load_blk<BM>(pt, (n1 + yk0) * LL + an, zero);
-                const V n11 = load_blk<BM>(pt, (n1 + yk1) * LL + an, zero);
-                const V n20 = load_blk<BM>(pt, (n2 + yk0) * LL + an, zero);
-                const V n21 = load_blk<BM>(pt, (n2 + yk1) * LL + an, zero);
-                const V q0 = lerp_(p00, p01, wx), q1 = lerp_(p10, p11, wx), q2 = lerp_(p20, p21, wx);
-                const V d1 = sub_(q1, q0), d2 = sub_(q2, q0);
+            const float4 *q0 = pt + n0 * LL + arow, *q1 = pt + n1 * LL + arow, *q2 = pt + n2 * LL + arow;
+            auto sweep = [&](auto cross) {
+                constexpr bool CROSS = decltype(cross)::value;
+                V p00, p01, p10, p11, p20 = V{}, p21 = V{};
+                float wx;
+                auto load = [&](int dx) {
+                    const Corner Xc = xc[tx + h - dx];
+                    const int k0 = Xc.k0 * LL + dx, k1 = Xc.k1 * LL + dx;
+                    wx = Xc.w;
+                    p00 = load_blk<BM>(q0, k0, zero), p01 = load_blk<BM>(q0, k1, zero);
+                    p10 = load_blk<BM>(q1, k0, zero), p11 = load_blk<BM>(q1, k1, zero);
+                    if (CROSS) p20 = load_blk<BM>(q2, k0, zero), p21 = load_blk<BM>(q2, k1, zero);
+                };
+                load(-h);
+                const X *xin = in_t + row0 * TCW + tx + 2 * h;   // input of offset dx = -h
+                for (int dx = -h; dx <= h; ++dx) {
+                    const V m0 = lerp_(p00, p01, wx), d1 = sub_(lerp_(p10, p11, wx), m0);
+                    V d2 = V{};
+                    if (CROSS) d2 = sub_(lerp_(p20, p21, wx), m0);
+                    load(min(dx + 1, h));
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const V C = mix3(q0, d1, d2, wb[r], wc[r]);
-                    const int o = (row0 + r) * TCW + col;
-                    if constexpr (MASK == 3) {
-                        const float2 xv = t2[o];
-                        acc0[r] = fmaf(C.x, xv.x, fmaf(C.y, xv.y, acc0[r]));
-                        acc1[r] = fmaf(C.z, xv.x, fmaf(C.w, xv.y, acc1[r]));
-                    } else {
-                        acc0[r] = fmaf(C, tile[o], acc0[r]);
-                    }
+                    for (int r = 0; r < R; ++r)
+                        accum(acc[r], CROSS ? mix3(m0, d1, d2, wb[r], wc[r]) : mix2(m0, d1, wb[r]), xin[r * TCW]);
+                    --xin;
                 }
-                p00 = n00, p01 = n01, p10 = n10, p11 = n11, p20 = n20, p21 = n21;
-                col = cn, wx = wn;
-            }
+            };
+            if (any_weight<MASK, R>(wc)) sweep(std::true_type{});
+            else sweep(std::false_type{});
         }
     } else {
         // y(c) = sum_a [sum_corners(c) w P(a)] x(c + a): the thread's rows c
         // and column are fixed, so are their corners
         const int row0 = ty * R + h;   // tile row of c = rz0
         const int kf = zc[row0].k0;
-        row_weights<R>(zc + row0, kf, wb, wc);
+        row_weights<MASK, R>(zc + row0, kf, wb, wc);
         const int xk0 = xc[tx + h].k0, xk1 = xc[tx + h].k1;
         const float wx = xc[tx + h].w;
         const int n0 = kf * nkx, n1 = min(kf + 1, nkz1) * nkx, n2 = min(kf + 2, nkz1) * nkx;
         const int b00 = (n0 + xk0) * LL, b01 = (n0 + xk1) * LL, b10 = (n1 + xk0) * LL;
         const int b11 = (n1 + xk1) * LL, b20 = (n2 + xk0) * LL, b21 = (n2 + xk1) * LL;
-        // the window offsets in storage order, the next offset's six node
-        // values loaded while the current one is used
-        V p00 = load_blk<BM>(pt, b00, zero), p01 = load_blk<BM>(pt, b01, zero);
-        V p10 = load_blk<BM>(pt, b10, zero), p11 = load_blk<BM>(pt, b11, zero);
-        V p20 = load_blk<BM>(pt, b20, zero), p21 = load_blk<BM>(pt, b21, zero);
-        int dz = -h, dx = -h;
-        for (int ai = 0; ai < LL; ++ai) {
-            const int an = min(ai + 1, LL - 1);
-            const V n00 = load_blk<BM>(pt, b00 + an, zero), n01 = load_blk<BM>(pt, b01 + an, zero);
-            const V n10 = load_blk<BM>(pt, b10 + an, zero), n11 = load_blk<BM>(pt, b11 + an, zero);
-            const V n20 = load_blk<BM>(pt, b20 + an, zero), n21 = load_blk<BM>(pt, b21 + an, zero);
-            const V q0 = lerp_(p00, p01, wx), q1 = lerp_(p10, p11, wx), q2 = lerp_(p20, p21, wx);
-            const V d1 = sub_(q1, q0), d2 = sub_(q2, q0);
-            const int ob = (row0 + dz) * TCW + tx + h + dx;
+        // the window offsets in storage order, the next offset's node values
+        // loaded while the current one's are used
+        const float4 *q00 = pt + b00, *q01 = pt + b01, *q10 = pt + b10, *q11 = pt + b11, *q20 = pt + b20, *q21 = pt + b21;
+        auto sweep = [&](auto cross) {
+            constexpr bool CROSS = decltype(cross)::value;
+            V p00 = load_blk<BM>(q00, 0, zero), p01 = load_blk<BM>(q01, 0, zero);
+            V p10 = load_blk<BM>(q10, 0, zero), p11 = load_blk<BM>(q11, 0, zero);
+            V p20 = V{}, p21 = V{};
+            if (CROSS) p20 = load_blk<BM>(q20, 0, zero), p21 = load_blk<BM>(q21, 0, zero);
+            const X *xin = in_t + (row0 - h) * TCW + tx;   // input of offset (-h, -h)
+            int dx = -h;
+            for (int ai = 0; ai < LL; ++ai) {
+                const V m0 = lerp_(p00, p01, wx), d1 = sub_(lerp_(p10, p11, wx), m0);
+                V d2 = V{};
+                if (CROSS) d2 = sub_(lerp_(p20, p21, wx), m0);
+                const int an = min(ai + 1, LL - 1);
+                p00 = load_blk<BM>(q00, an, zero), p01 = load_blk<BM>(q01, an, zero);
+                p10 = load_blk<BM>(q10, an, zero), p11 = load_blk<BM>(q11, an, zero);
+                if (CROSS) p20 = load_blk<BM>(q20, an, zero), p21 = load_blk<BM>(q21, an, zero);
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const V C = mix3(q0, d1, d2, wb[r], wc[r]);
-                const int o = ob + r * TCW;
-                if constexpr (MASK == 3) {
-                    const float2 yv = t2[o];
-                    acc0[r] = fmaf(C.x, yv.x, fmaf(C.z, yv.y, acc0[r]));
-                    acc1[r] = fmaf(C.y, yv.x, fmaf(C.w, yv.y, acc1[r]));
-                } else {
-                    acc0[r] = fmaf(C, tile[o], acc0[r]);
-                }
+                for (int r = 0; r < R; ++r)
+                    accum(acc[r], CROSS ? mix3(m0, d1, d2, wb[r], wc[r]) : mix2(m0, d1, wb[r]), xin[r * TCW]);
+                ++xin;
+                if (++dx > h) dx = -h, xin += TCW - L;
             }
-            p00 = n00, p01 = n01, p10 = n10, p11 = n11, p20 = n20, p21 = n21;
-            if (++dx > h) dx = -h, ++dz;
-        }
+        };
+        if (any_weight<MASK, R>(wc)) sweep(std::true_type{});
+        else sweep(std::false_type{});
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -297,10 +350,10 @@ __global__ void __launch_bounds__(kApplyThreads) k_psfh_apply(const PsfHessDev a
         if (z >= a.nz) break;
         const long long o = (long long)z * a.nx + rx;
         if (MASK == 3) {
-            out[o] = acc0[r];
-            out[plane + o] = acc1[r];
+            out[o] = plane0(acc[r]);
+            out[plane + o] = plane1(acc[r]);
         } else {
-            out[P0 * plane + o] = acc0[r];
+            out[P0 * plane + o] = plane0(acc[r]);
             out[(1 - P0) * plane + o] = 0.f;
         }
     }
@@ -340,7 +393,7 @@ cudaError_t launch_r(const PsfHessDev &a, const float *in, float *out, cudaStrea
 // ---------------------------------------------------------------------------
 constexpr int k3X = 32, k3Y = 4, k3Threads = k3X * k3Y;
 
-__global__ void k_psfh3_patches(const float *psf_vp, const float *psf_ip, const PsfHess3Dev a, float4 *pt)
+__global__ void k_psfh3_patches(const float *psf_vp, const float *psf_ip, const PsfHess3Dev a, bool transpose, float4 *pt)
 {
     const int L = 2 * a.half + 1, LL = L * L, LLL = LL * L;
     const long long vol = (long long)a.nz * a.ny * a.nx;
@@ -362,7 +415,7 @@ __global__ void k_psfh3_patches(const float *psf_vp, const float *psf_ip, const 
             const bool use = inside && src && ((a.mask >> po) & 1) && ((a.mask >> pi) & 1);
             e[b] = use ? src[po * vol + v] : 0.f;
         }
-        pt[i] = make_float4(e[0], e[1], e[2], e[3]);
+        pt[i] = make_float4(e[0], transpose ? e[2] : e[1], transpose ? e[1] : e[2], e[3]);
     }
 }
 
@@ -396,14 +449,15 @@ __global__ void __launch_bounds__(k3Threads) k_psfh3_rows(const PsfHess3Dev a, c
     const float4 *pt = a.pt;
     const int nky = a.nky, nkx = a.nkx, nkz1 = a.nkz - 1;
     const V zero = V{};
-    float acc0[R], acc1[R], wb[R], wc[R];
+    V acc[R];
+    typename Wgt<MASK>::T wb[R], wc[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) acc0[r] = acc1[r] = 0.f;
+    for (int r = 0; r < R; ++r) acc[r] = V{};
     if (!TR) {
         for (int dz = -h; dz <= h; ++dz) {
             const int row0 = h - dz;   // zc index of c_z = Z0 - dz
             const int kf = zc[row0].k0;
-            row_weights<R>(zc + row0, kf, wb, wc);
+            row_weights<MASK, R>(zc + row0, kf, wb, wc);
             const int nq[3] = {kf, min(kf + 1, nkz1), min(kf + 2, nkz1)};
             for (int dy = -h; dy <= h; ++dy) {
                 const int cy = y - dy;
@@ -432,20 +486,15 @@ __global__ void __launch_bounds__(k3Threads) k_psfh3_rows(const PsfHess3Dev a, c
                         if (cz < 0 || cz >= a.nz) continue;
                         const V C = mix3(Q[0], d1, d2, wb[r], wc[r]);
                         const long long c = cz * rowz + cb;
-                        if constexpr (MASK == 3) {
-                            const float v0 = __ldg(in0 + c), v1 = __ldg(in1 + c);
-                            acc0[r] = fmaf(C.x, v0, fmaf(C.y, v1, acc0[r]));
-                            acc1[r] = fmaf(C.z, v0, fmaf(C.w, v1, acc1[r]));
-                        } else {
-                            acc0[r] = fmaf(C, __ldg(in0 + c), acc0[r]);
-                        }
+                        if constexpr (MASK == 3) accum(acc[r], C, make_float2(__ldg(in0 + c), __ldg(in1 + c)));
+                        else accum(acc[r], C, __ldg(in0 + c));
                     }
                 }
             }
         }
     } else {
         const int kf = zc[h].k0;
-        row_weights<R>(zc + h, kf, wb, wc);
+        row_weights<MASK, R>(zc + h, kf, wb, wc);
         const Corner Y = yc[ty + h], X = xc[tx + h];
         int base[3][2][2];
 #pragma unroll
@@ -481,13 +530,8 @@ __global__ void __launch_bounds__(k3Threads) k_psfh3_rows(const PsfHess3Dev a, c
                         if (cz < 0 || cz >= a.nz) continue;
                         const V C = mix3(Q[0], d1, d2, wb[r], wc[r]);
                         const long long c = cz * rowz + cb;
-                        if constexpr (MASK == 3) {
-                            const float v0 = __ldg(in0 + c), v1 = __ldg(in1 + c);
-                            acc0[r] = fmaf(C.x, v0, fmaf(C.z, v1, acc0[r]));
-                            acc1[r] = fmaf(C.y, v0, fmaf(C.w, v1, acc1[r]));
-                        } else {
-                            acc0[r] = fmaf(C, __ldg(in0 + c), acc0[r]);
-                        }
+                        if constexpr (MASK == 3) accum(acc[r], C, make_float2(__ldg(in0 + c), __ldg(in1 + c)));
+                        else accum(acc[r], C, __ldg(in0 + c));
                     }
                 }
             }
@@ -499,10 +543,10 @@ __global__ void __launch_bounds__(k3Threads) k_psfh3_rows(const PsfHess3Dev a, c
         if (z >= a.nz) break;
         const long long o = z * rowz + (long long)y * a.nx + x;
         if (MASK == 3) {
-            out[o] = acc0[r];
-            out[vol + o] = acc1[r];
+            out[o] = plane0(acc[r]);
+            out[vol + o] = plane1(acc[r]);
         } else {
-            out[P0 * vol + o] = acc0[r];
+            out[P0 * vol + o] = plane0(acc[r]);
             out[(1 - P0) * vol + o] = 0.f;
         }
     }
@@ -529,13 +573,13 @@ cudaError_t launch3_t(const PsfHess3Dev &a, const float *in, float *out, cudaStr
 
 int psfh_max_half() { return kPsfHessMaxHalf; }
 
-cudaError_t launch_psfh3_patches(const float *psf_vp, const float *psf_ip, const PsfHess3Dev &a, float4 *pt,
-                                 cudaStream_t st)
+cudaError_t launch_psfh3_patches(const float *psf_vp, const float *psf_ip, const PsfHess3Dev &a, bool transpose,
+                                 float4 *pt, cudaStream_t st)
 {
     const long long L = 2 * a.half + 1;
     const long long n = (long long)a.nkz * a.nky * a.nkx * L * L * L;
     const int blocks = (int)std::min<long long>((n + 255) / 256, 152 * 16);
-    k_psfh3_patches<<<blocks, 256, 0, st>>>(psf_vp, psf_ip, a, pt);
+    k_psfh3_patches<<<blocks, 256, 0, st>>>(psf_vp, psf_ip, a, transpose, pt);
     return cudaGetLastError();
 }
 
@@ -553,11 +597,11 @@ cudaError_t launch_psfh3_apply(const PsfHess3Dev &a, bool transpose, const float
 }
 
 cudaError_t launch_psfh_patches(const float *psf_vp, const float *psf_ip, int nz, int nx, int s, int half,
-                                int nkz, int nkx, int mask, float4 *pt, cudaStream_t st)
+                                int nkz, int nkx, int mask, bool transpose, float4 *pt, cudaStream_t st)
 {
     const long long n = (long long)nkz * nkx * (2 * half + 1) * (2 * half + 1);
     const int blocks = (int)std::min<long long>((n + 255) / 256, 4096);
-    k_psfh_patches<<<blocks, 256, 0, st>>>(psf_vp, psf_ip, nz, nx, s, half, nkz, nkx, mask, pt);
+    k_psfh_patches<<<blocks, 256, 0, st>>>(psf_vp, psf_ip, nz, nx, s, half, nkz, nkx, mask, transpose, pt);
     return cudaGetLastError();
 }
 
