@@ -147,8 +147,6 @@ struct lsrtm_handle {
     // interpolated PSF Hessian (App. D)
     float4 *ph_pt = nullptr;     // node windows, grown on demand
     size_t ph_cap = 0;
-    float4 *ph_pt2 = nullptr;    // the CG's node windows for H^T, where memory allows
-    size_t ph_cap2 = 0;
     float *ph_vec = nullptr;     // [8][2 nint]: x, r, s, p, q, staged input, staged PSFs (Vp, Ip)
     double *ph_scal = nullptr;   // [0] gamma [1] gamma_new [2] <q,q> [3] <d,d>
     double *ph_mis = nullptr;    // per-iteration <r,r>
@@ -2109,49 +2107,20 @@ lsrtm_status lsrtm_deblur_wiener(lsrtm_handle *h, const float *m_rtm, const floa
 
 namespace {
 
-// The interpolated PSF Hessian of one call: 2D or 3D arguments of the kernels,
-// the PSF images, and the node windows packed for H and for H^T (one array
-// each, or one array packed anew when the other is needed; a single parameter's
-// windows serve both).
+// The interpolated PSF Hessian of one call: 2D or 3D arguments of the kernels.
 struct PsfhPlan {
     bool d3 = false;
     PsfHessDev a2{};
     PsfHess3Dev a3{};
-    const float *pv = nullptr, *pi = nullptr;
-    float4 *pt[2] = {nullptr, nullptr};
-    int packed = -1;   // what the one array holds: 0 H, 1 H^T, -1 nothing yet
 };
 
-lsrtm_status psfh_pack(lsrtm_handle *h, const PsfhPlan &pl, bool transpose)
+cudaError_t psfh_apply(const PsfhPlan &pl, bool transpose, const float *in, float *out, cudaStream_t s)
 {
-    float4 *pt = pl.pt[transpose];
-    if (pl.d3) CU(launch_psfh3_patches(pl.pv, pl.pi, pl.a3, transpose, pt, h->work));
-    else CU(launch_psfh_patches(pl.pv, pl.pi, pl.a2.nz, pl.a2.nx, pl.a2.s, pl.a2.half, pl.a2.nkz, pl.a2.nkx, pl.a2.mask,
-                                transpose, pt, h->work));
-    h->launches++;
-    return LSRTM_OK;
+    return pl.d3 ? launch_psfh3_apply(pl.a3, transpose, in, out, s) : launch_psfh_apply(pl.a2, transpose, in, out, s);
 }
 
-lsrtm_status psfh_apply(lsrtm_handle *h, PsfhPlan &pl, bool transpose, const float *in, float *out)
-{
-    const int mask = pl.d3 ? pl.a3.mask : pl.a2.mask;
-    if (pl.pt[0] == pl.pt[1] && (pl.packed < 0 || (mask == 3 && pl.packed != (int)transpose))) {
-        CHECK(psfh_pack(h, pl, transpose));
-        pl.packed = transpose;
-    }
-    if (pl.d3) {
-        pl.a3.pt = pl.pt[transpose];
-        CU(launch_psfh3_apply(pl.a3, transpose, in, out, h->work));
-    } else {
-        pl.a2.pt = pl.pt[transpose];
-        CU(launch_psfh_apply(pl.a2, transpose, in, out, h->work));
-    }
-    h->launches++;
-    return LSRTM_OK;
-}
-
-// Validates the PSF Hessian arguments, stages the PSF images and finds room for
-// the node windows; the caller has called begin_call.
+// Validates the PSF Hessian arguments, stages the PSF images and builds the
+// node windows; the caller has called begin_call.
 lsrtm_status psfh_setup(lsrtm_handle *h, const float *psf_vp, const float *psf_ip, int spacing, int half,
                         int param_mask, PsfhPlan *pl)
 {
@@ -2182,11 +2151,14 @@ lsrtm_status psfh_setup(lsrtm_handle *h, const float *psf_vp, const float *psf_i
     if (param_mask & 1) CHECK(stage_in(h, psf_vp, h->ph_vec + 6 * m, m, &pv));
     if (param_mask & 2) CHECK(stage_in(h, psf_ip, h->ph_vec + 7 * m, m, &pi));
     pl->d3 = d3;
-    pl->pv = pv;
-    pl->pi = pi;
-    pl->pt[0] = pl->pt[1] = h->ph_pt;
-    if (d3) pl->a3 = PsfHess3Dev{nz, ny, nx, spacing, half, nkz, nky, nkx, param_mask, h->ph_pt};
-    else pl->a2 = PsfHessDev{nz, nx, spacing, half, nkz, nkx, param_mask, h->ph_pt};
+    if (d3) {
+        pl->a3 = PsfHess3Dev{nz, ny, nx, spacing, half, nkz, nky, nkx, param_mask, h->ph_pt};
+        CU(launch_psfh3_patches(pv, pi, pl->a3, h->ph_pt, h->work));
+    } else {
+        pl->a2 = PsfHessDev{nz, nx, spacing, half, nkz, nkx, param_mask, h->ph_pt};
+        CU(launch_psfh_patches(pv, pi, nz, nx, spacing, half, nkz, nkx, param_mask, h->ph_pt, h->work));
+    }
+    h->launches++;
     return LSRTM_OK;
 }
 
@@ -2207,7 +2179,8 @@ lsrtm_status lsrtm_psf_hessian(lsrtm_handle *h, const float *psf_vp, const float
     CHECK(stage_in(h, x, h->ph_vec + 5 * m, m, &xd));
     const bool odev = is_device_ptr(y);
     float *od = odev ? y : h->ph_vec + 4 * m;
-    CHECK(psfh_apply(h, a, transpose != 0, xd, od));
+    CU(psfh_apply(a, transpose != 0, xd, od, h->work));
+    h->launches++;
     if (!odev) CHECK(copy_out(h, y, od, m));
     return end_call(h, !odev);
 }
@@ -2224,24 +2197,6 @@ lsrtm_status lsrtm_psf_cg(lsrtm_handle *h, const float *psf_vp, const float *psf
     CHECK(begin_call(h));
     PsfhPlan a;
     CHECK(psfh_setup(h, psf_vp, psf_ip, spacing, half, param_mask, &a));
-    // two parameters: an array of node windows for H^T beside H's, packed once;
-    // without room for it (a memory cap) the one array is packed before every
-    // application
-    if (param_mask == 3) {
-        if (h->ph_cap2 < h->ph_cap) {
-            float4 *p2 = nullptr;
-            if (dalloc_t(h, &p2, h->ph_cap) == LSRTM_OK) {
-                h->ph_pt2 = p2;
-                h->ph_cap2 = h->ph_cap;
-            }
-            g_last_error.clear();
-        }
-        if (h->ph_cap2 >= h->ph_cap) {
-            a.pt[1] = h->ph_pt2;
-            CHECK(psfh_pack(h, a, false));
-            CHECK(psfh_pack(h, a, true));
-        }
-    }
     const long long m = 2 * h->nint;
     float *v = h->ph_vec;
     float *X = v, *R = v + m, *S = v + 2 * m, *Pp = v + 3 * m, *Q = v + 4 * m;
@@ -2258,22 +2213,22 @@ lsrtm_status lsrtm_psf_cg(lsrtm_handle *h, const float *psf_vp, const float *psf
     CU(launch_scale_copy(R, md, m, s));
     CU(launch_mul_mask(R, nullptr, param_mask, h->nint, s));
     CU(launch_dot(R, R, m, dd, h->dotwork, s));
-    CHECK(psfh_apply(h, a, true, R, S));
+    CU(psfh_apply(a, true, R, S, s));
     CU(launch_scale_copy(Pp, S, m, s));
     CU(launch_dot(S, S, m, gamma, h->dotwork, s));
     CU(cudaMemcpyAsync(h->ph_mis, dd, sizeof(double), cudaMemcpyDeviceToDevice, s));
-    h->launches += 5;
+    h->launches += 6;
     for (int k = 0; k < niter; ++k) {
-        CHECK(psfh_apply(h, a, false, Pp, Q));
+        CU(psfh_apply(a, false, Pp, Q, s));
         CU(launch_dot(Q, Q, m, qq, h->dotwork, s));
         CU(launch_axpy_ratio(X, Pp, gamma, qq, 1.0f, m, s));
         CU(launch_axpy_ratio(R, Q, gamma, qq, -1.0f, m, s));
-        CHECK(psfh_apply(h, a, true, R, S));
+        CU(psfh_apply(a, true, R, S, s));
         CU(launch_dot(S, S, m, gnew, h->dotwork, s));
         CU(launch_xpby_ratio(Pp, S, gnew, gamma, m, s));
         CU(cudaMemcpyAsync(gamma, gnew, sizeof(double), cudaMemcpyDeviceToDevice, s));
         CU(launch_dot(R, R, m, h->ph_mis + k + 1, h->dotwork, s));
-        h->launches += 6;
+        h->launches += 8;
     }
     CHECK(copy_out(h, dm, X, m));
     std::vector<double> m2(niter + 1);

@@ -13,8 +13,7 @@
 // parameter j. The parameter mask restricts the operator to P H P.
 //
 // k_psfh_patches: the node windows, packed per (node, offset) as one float4
-//   of the four blocks (00, 01, 10, 11; for H^T 00, 10, 01, 11), so one 16-byte
-//   load serves all four and its halves are the pairs of packed products.
+//   of the four blocks (00, 01, 10, 11), so one 16-byte load serves all four.
 // k_psfh_apply<MASK, TR, R>: one thread per output column and R consecutive
 //   rows (R = the largest of 8, 4, 2, 1 not above s), CTAs of 32 columns x
 //   2 R rows (small CTAs spread the one wave evenly over the SMs). The input
@@ -28,9 +27,9 @@
 //   same for all its lanes, and most warps' (12 of 20 positions at s = 20, R = 8)
 //   lie between two node rows: those load four node values an offset, not six,
 //   and interpolate with one multiply-add. 300 x 2000, s = 20, 19 x 19 windows,
-//   two parameters: 239 -> 180 us an application (packed products and this;
-//   packed products alone 219, with two offsets loaded ahead 300: 160
-//   registers). What bounds it now: the L1 return path (68%) and its latency.
+//   two parameters: 239 -> 199 us an application, by this and the interpolation
+//   in packed FP32x2 (with two offsets loaded ahead 300: 160 registers). What
+//   bounds it now: the L1 return path and its latency.
 //   TR = false: y(r) = sum_a H(r, r - a) x(r - a), the columns gathered at r;
 //   TR = true:  y(c) = sum_a H(c + a, c) x(c + a), the transpose.
 // k_psfh3_patches, k_psfh3_rows: the same for 3D images, with the eight
@@ -77,7 +76,7 @@ __device__ __forceinline__ Corner corner_of(int c, int n, int s, int nk)
 }
 
 __global__ void k_psfh_patches(const float *psf_vp, const float *psf_ip, int nz, int nx, int s, int half,
-                               int nkz, int nkx, int mask, bool transpose, float4 *pt)
+                               int nkz, int nkx, int mask, float4 *pt)
 {
     const int L = 2 * half + 1, LL = L * L;
     const long long plane = (long long)nz * nx;
@@ -97,15 +96,13 @@ __global__ void k_psfh_patches(const float *psf_vp, const float *psf_ip, int nz,
             const bool use = inside && src && ((mask >> po) & 1) && ((mask >> pi) & 1);
             v[b] = use ? src[po * plane + (long long)z * nx + x] : 0.f;
         }
-        pt[i] = make_float4(v[0], transpose ? v[2] : v[1], transpose ? v[1] : v[2], v[3]);
+        pt[i] = make_float4(v[0], v[1], v[2], v[3]);
     }
 }
 
-// Parameter-block values: the four blocks (two parameters) as two pairs, each
-// pair the two blocks whose products with an input pixel's two planes make up
-// one output plane, or the one block of a single-parameter mask. Pairs take
-// packed FP32x2 arithmetic: with scalars the interpolation and the products
-// were bound by issue slots.
+// Parameter-block values: the four blocks (two parameters) as two pairs, or the
+// one block of a single-parameter mask. Pairs are interpolated with packed FP32x2
+// arithmetic: with scalars the kernel was bound by issue slots.
 struct Pairs {
     float2 a, b;
 };
@@ -167,18 +164,18 @@ struct Wgt<3> {
     using T = float2;
     static __device__ __forceinline__ T of(float w) { return dup(w); }
 };
-// Accumulators of one output pixel: a scalar, or per output plane the two
-// input planes' sums.
-__device__ __forceinline__ void accum(float &acc, float C, float x) { acc = fmaf(C, x, acc); }
-__device__ __forceinline__ void accum(Pairs &acc, Pairs C, float2 x)
+// One output pixel's products, plane 1's input first: unpacked, so that each
+// plane is one chain of sums whose rounding does not depend on the packing (one
+// sum per input plane, added at the end, took 180 us for 199 but moves the CG's
+// misfits by up to 4e-9).
+template <bool TR>
+__device__ __forceinline__ void accum(float &a0, float &, float C, float x) { a0 = fmaf(C, x, a0); }
+template <bool TR>
+__device__ __forceinline__ void accum(float &a0, float &a1, Pairs C, float2 x)
 {
-    acc.a = __ffma2_rn(C.a, x, acc.a);
-    acc.b = __ffma2_rn(C.b, x, acc.b);
+    a0 = fmaf(C.a.x, x.x, fmaf(TR ? C.b.x : C.a.y, x.y, a0));
+    a1 = fmaf(TR ? C.a.y : C.b.x, x.x, fmaf(C.b.y, x.y, a1));
 }
-__device__ __forceinline__ float plane0(float a) { return a; }
-__device__ __forceinline__ float plane0(Pairs a) { return a.a.x + a.a.y; }
-__device__ __forceinline__ float plane1(float) { return 0.f; }
-__device__ __forceinline__ float plane1(Pairs a) { return a.b.x + a.b.y; }
 
 // Weights of R consecutive rows (first corner row kf) on the node rows
 // kf + 1 and kf + 2 (the rest, on kf, is implied): row r puts 1 - w on its k0
@@ -260,9 +257,9 @@ __global__ void __launch_bounds__(kApplyThreads) k_psfh_apply(const PsfHessDev a
     const V zero = V{};
     using X = typename std::conditional<MASK == 3, float2, float>::type;
     const X *in_t = reinterpret_cast<const X *>(tile);
-    V acc[R];
+    float acc0[R], acc1[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) acc[r] = V{};
+    for (int r = 0; r < R; ++r) acc0[r] = acc1[r] = 0.f;
     typename Wgt<MASK>::T wb[R], wc[R];
 
     if (!TR) {
@@ -297,7 +294,7 @@ __global__ void __launch_bounds__(kApplyThreads) k_psfh_apply(const PsfHessDev a
                     load(min(dx + 1, h));
 #pragma unroll
                     for (int r = 0; r < R; ++r)
-                        accum(acc[r], CROSS ? mix3(m0, d1, d2, wb[r], wc[r]) : mix2(m0, d1, wb[r]), xin[r * TCW]);
+                        accum<TR>(acc0[r], acc1[r], CROSS ? mix3(m0, d1, d2, wb[r], wc[r]) : mix2(m0, d1, wb[r]), xin[r * TCW]);
                     --xin;
                 }
             };
@@ -336,7 +333,7 @@ __global__ void __launch_bounds__(kApplyThreads) k_psfh_apply(const PsfHessDev a
                 if (CROSS) p20 = load_blk<BM>(q20, an, zero), p21 = load_blk<BM>(q21, an, zero);
 #pragma unroll
                 for (int r = 0; r < R; ++r)
-                    accum(acc[r], CROSS ? mix3(m0, d1, d2, wb[r], wc[r]) : mix2(m0, d1, wb[r]), xin[r * TCW]);
+                    accum<TR>(acc0[r], acc1[r], CROSS ? mix3(m0, d1, d2, wb[r], wc[r]) : mix2(m0, d1, wb[r]), xin[r * TCW]);
                 ++xin;
                 if (++dx > h) dx = -h, xin += TCW - L;
             }
@@ -350,10 +347,10 @@ __global__ void __launch_bounds__(kApplyThreads) k_psfh_apply(const PsfHessDev a
         if (z >= a.nz) break;
         const long long o = (long long)z * a.nx + rx;
         if (MASK == 3) {
-            out[o] = plane0(acc[r]);
-            out[plane + o] = plane1(acc[r]);
+            out[o] = acc0[r];
+            out[plane + o] = acc1[r];
         } else {
-            out[P0 * plane + o] = plane0(acc[r]);
+            out[P0 * plane + o] = acc0[r];
             out[(1 - P0) * plane + o] = 0.f;
         }
     }
@@ -393,7 +390,7 @@ cudaError_t launch_r(const PsfHessDev &a, const float *in, float *out, cudaStrea
 // ---------------------------------------------------------------------------
 constexpr int k3X = 32, k3Y = 4, k3Threads = k3X * k3Y;
 
-__global__ void k_psfh3_patches(const float *psf_vp, const float *psf_ip, const PsfHess3Dev a, bool transpose, float4 *pt)
+__global__ void k_psfh3_patches(const float *psf_vp, const float *psf_ip, const PsfHess3Dev a, float4 *pt)
 {
     const int L = 2 * a.half + 1, LL = L * L, LLL = LL * L;
     const long long vol = (long long)a.nz * a.ny * a.nx;
@@ -415,7 +412,7 @@ __global__ void k_psfh3_patches(const float *psf_vp, const float *psf_ip, const 
             const bool use = inside && src && ((a.mask >> po) & 1) && ((a.mask >> pi) & 1);
             e[b] = use ? src[po * vol + v] : 0.f;
         }
-        pt[i] = make_float4(e[0], transpose ? e[2] : e[1], transpose ? e[1] : e[2], e[3]);
+        pt[i] = make_float4(e[0], e[1], e[2], e[3]);
     }
 }
 
@@ -449,10 +446,10 @@ __global__ void __launch_bounds__(k3Threads) k_psfh3_rows(const PsfHess3Dev a, c
     const float4 *pt = a.pt;
     const int nky = a.nky, nkx = a.nkx, nkz1 = a.nkz - 1;
     const V zero = V{};
-    V acc[R];
+    float acc0[R], acc1[R];
     typename Wgt<MASK>::T wb[R], wc[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) acc[r] = V{};
+    for (int r = 0; r < R; ++r) acc0[r] = acc1[r] = 0.f;
     if (!TR) {
         for (int dz = -h; dz <= h; ++dz) {
             const int row0 = h - dz;   // zc index of c_z = Z0 - dz
@@ -486,8 +483,8 @@ __global__ void __launch_bounds__(k3Threads) k_psfh3_rows(const PsfHess3Dev a, c
                         if (cz < 0 || cz >= a.nz) continue;
                         const V C = mix3(Q[0], d1, d2, wb[r], wc[r]);
                         const long long c = cz * rowz + cb;
-                        if constexpr (MASK == 3) accum(acc[r], C, make_float2(__ldg(in0 + c), __ldg(in1 + c)));
-                        else accum(acc[r], C, __ldg(in0 + c));
+                        if constexpr (MASK == 3) accum<TR>(acc0[r], acc1[r], C, make_float2(__ldg(in0 + c), __ldg(in1 + c)));
+                        else accum<TR>(acc0[r], acc1[r], C, __ldg(in0 + c));
                     }
                 }
             }
@@ -530,8 +527,8 @@ __global__ void __launch_bounds__(k3Threads) k_psfh3_rows(const PsfHess3Dev a, c
                         if (cz < 0 || cz >= a.nz) continue;
                         const V C = mix3(Q[0], d1, d2, wb[r], wc[r]);
                         const long long c = cz * rowz + cb;
-                        if constexpr (MASK == 3) accum(acc[r], C, make_float2(__ldg(in0 + c), __ldg(in1 + c)));
-                        else accum(acc[r], C, __ldg(in0 + c));
+                        if constexpr (MASK == 3) accum<TR>(acc0[r], acc1[r], C, make_float2(__ldg(in0 + c), __ldg(in1 + c)));
+                        else accum<TR>(acc0[r], acc1[r], C, __ldg(in0 + c));
                     }
                 }
             }
@@ -543,10 +540,10 @@ __global__ void __launch_bounds__(k3Threads) k_psfh3_rows(const PsfHess3Dev a, c
         if (z >= a.nz) break;
         const long long o = z * rowz + (long long)y * a.nx + x;
         if (MASK == 3) {
-            out[o] = plane0(acc[r]);
-            out[vol + o] = plane1(acc[r]);
+            out[o] = acc0[r];
+            out[vol + o] = acc1[r];
         } else {
-            out[P0 * vol + o] = plane0(acc[r]);
+            out[P0 * vol + o] = acc0[r];
             out[(1 - P0) * vol + o] = 0.f;
         }
     }
@@ -573,13 +570,13 @@ cudaError_t launch3_t(const PsfHess3Dev &a, const float *in, float *out, cudaStr
 
 int psfh_max_half() { return kPsfHessMaxHalf; }
 
-cudaError_t launch_psfh3_patches(const float *psf_vp, const float *psf_ip, const PsfHess3Dev &a, bool transpose,
+cudaError_t launch_psfh3_patches(const float *psf_vp, const float *psf_ip, const PsfHess3Dev &a,
                                  float4 *pt, cudaStream_t st)
 {
     const long long L = 2 * a.half + 1;
     const long long n = (long long)a.nkz * a.nky * a.nkx * L * L * L;
     const int blocks = (int)std::min<long long>((n + 255) / 256, 152 * 16);
-    k_psfh3_patches<<<blocks, 256, 0, st>>>(psf_vp, psf_ip, a, transpose, pt);
+    k_psfh3_patches<<<blocks, 256, 0, st>>>(psf_vp, psf_ip, a, pt);
     return cudaGetLastError();
 }
 
@@ -597,11 +594,11 @@ cudaError_t launch_psfh3_apply(const PsfHess3Dev &a, bool transpose, const float
 }
 
 cudaError_t launch_psfh_patches(const float *psf_vp, const float *psf_ip, int nz, int nx, int s, int half,
-                                int nkz, int nkx, int mask, bool transpose, float4 *pt, cudaStream_t st)
+                                int nkz, int nkx, int mask, float4 *pt, cudaStream_t st)
 {
     const long long n = (long long)nkz * nkx * (2 * half + 1) * (2 * half + 1);
     const int blocks = (int)std::min<long long>((n + 255) / 256, 4096);
-    k_psfh_patches<<<blocks, 256, 0, st>>>(psf_vp, psf_ip, nz, nx, s, half, nkz, nkx, mask, transpose, pt);
+    k_psfh_patches<<<blocks, 256, 0, st>>>(psf_vp, psf_ip, nz, nx, s, half, nkz, nkx, mask, pt);
     return cudaGetLastError();
 }
 
