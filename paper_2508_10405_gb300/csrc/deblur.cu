@@ -31,6 +31,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "lsrtm_internal.cuh"
 #include "wiener.cuh"
@@ -237,14 +238,34 @@ __global__ void k_deblur_apply(const float *mref, const float *filt, int nz, int
 // (zero when m'' is zero), and the blocks are blended with the bilinear
 // valence of the space-domain filters.
 //
-// k_wiener_block: one CTA per (node, plane); the block, its spectra and a
-// transform buffer sit in shared memory as complex FP32; each 2D DFT runs
-// along the rows, then the columns, each as one Cooley-Tukey split N = N1 N2
-// (dft2) with a twiddle table; the block result goes to
-// blk[plane][node][N*N].
-// k_wiener_blend: one thread per pixel, the (up to) four covering blocks.
+// k_wiener_node (N = N1 N2 with both factors at most 8, every even N up to 64
+// but those with a larger prime factor, 50, 54 and 60): one CTA per node, both
+// planes. The blocks of m'' and m_rtm are real, so one complex transform of
+// a + i b gives both spectra, A = (Z(k) + conj Z(-k)) / 2 and B = (Z(k) - conj
+// Z(-k)) / 2i, and the two planes' results, real again, come from one inverse
+// transform: three transforms a node where six were made. What is packed
+// together is first scaled to about the same norm by powers of two, so neither
+// part loses precision to the other; mean|A|^2 is sum a^2 (Parseval). A 2D transform is one Cooley-Tukey split per
+// axis; a thread forms a whole length-N1 or N2 transform in registers, so a
+// value is read once instead of N1 or N2 times. The inverse is the forward
+// transform with real and imaginary parts exchanged before and after.
+// Bound by issue slots and the shared memory around the twelve passes with a
+// barrier after each (57% of issue, 56% of L1): 300 x 2000, s = 20 (1500 nodes,
+// N = 40) 100 us with the blend, at 64 registers a thread, three CTAs an SM
+// (9% more at 81 registers, two); k_wiener_block took 533 us there.
+// k_wiener_block: the other N; one CTA per (node, plane); the block, its
+// spectra and a transform buffer sit in shared memory as complex FP32; each 2D
+// DFT runs along the rows, then the columns, each as one Cooley-Tukey split
+// (dft2) with a twiddle table and one output a thread.
+// Both write blk[node][N*N][plane].
+// k_wiener_blend: one thread per pixel, both planes, the (up to) four covering
+// blocks.
 // ---------------------------------------------------------------------------
 constexpr int kWienerThreads = 256, kWienerMaxS = 32;
+// m'' is packed 2^3 above m_rtm: the filter amplifies an error of A by up to
+// 1 / sqrt(eps), one of B not at all (error 5.4e-6 with both alike, 4.0e-6 so,
+// 6.8e-6 at 2^6, of the result at 300 x 2000).
+constexpr int kWienerBias = 3;
 
 // One Cooley-Tukey split of a length-N DFT, N = N1 N2 (N1 the divisor of N
 // nearest sqrt N; 5 x 8 for N = 40): with n = N2 n1 + n2 and k = k1 + N1 k2,
@@ -380,21 +401,315 @@ __global__ void __launch_bounds__(kWienerThreads) k_wiener_block(const float *mr
     }
     __syncthreads();
     dft2(P, Q, A, tw, N, true);
-    float *out = blk + ((long long)plane * gridDim.x + node) * NN;
+    float *out = blk + (long long)node * NN * 2 + plane;
     const float scale = 1.f / (float)NN;
-    for (int idx = threadIdx.x; idx < NN; idx += blockDim.x) out[idx] = A[idx].x * scale;
+    for (int idx = threadIdx.x; idx < NN; idx += blockDim.x) out[2 * idx] = A[idx].x * scale;
 }
 
-__global__ void k_wiener_blend(const float *blk, int nz, int nx, int s, int nkz, int nkx, float *out)
+// ---- forward DFTs of length R in registers, v[k] = sum_n v[n] exp(-2 pi i n k / R)
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ float2 cmul(float2 a, float2 b)
+{
+    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+}
+// a w, the twiddle w as a rounded value (x, y) and what rounding took off (z, w)
+__device__ __forceinline__ float2 ctwiddle(float2 a, float4 w)
+{
+    return make_float2(fmaf(a.x, w.x, fmaf(-a.y, w.y, fmaf(a.x, w.z, -a.y * w.w))),
+                       fmaf(a.x, w.y, fmaf(a.y, w.x, fmaf(a.x, w.w, a.y * w.z))));
+}
+// cos and sin of 2 pi j / R, j = 0 .. R - 1, for R = 3, 5, 7
+template <int R>
+__device__ constexpr float cos_of(int j)
+{
+    if (2 * j > R) j = R - j;
+    if (j == 0) return 1.f;
+    if (R == 3) return -0.5f;
+    if (R == 5) return j == 1 ? 0.309016994374947424f : -0.809016994374947424f;
+    return j == 1 ? 0.623489801858733531f : (j == 2 ? -0.222520933956314404f : -0.900968867902419126f);
+}
+template <int R>
+__device__ constexpr float sin_of(int j)
+{
+    if (2 * j > R) return -sin_of<R>(R - j);
+    if (j == 0) return 0.f;
+    if (R == 3) return 0.866025403784438647f;
+    if (R == 5) return j == 1 ? 0.951056516295153572f : 0.587785252292473129f;
+    return j == 1 ? 0.781831482468029809f : (j == 2 ? 0.974927912181823607f : 0.433883739117558120f);
+}
+template <int R>
+__device__ __forceinline__ void dft_reg(float2 (&v)[R])
+{
+    if constexpr (R == 2) {
+        const float2 a = v[0];
+        v[0] = cadd(a, v[1]);
+        v[1] = csub(a, v[1]);
+    } else if constexpr (R % 2 == 1) {
+        // with p = v_j + v_{R-j}, m = v_j - v_{R-j}: V_k, V_{R-k} = (v_0 + sum c_jk p_j) -+ i sum s_jk m_j
+        constexpr int H = (R - 1) / 2;
+        float2 p[H], m[H], sum = v[0];
+#pragma unroll
+        for (int j = 0; j < H; ++j) {
+            p[j] = cadd(v[j + 1], v[R - 1 - j]);
+            m[j] = csub(v[j + 1], v[R - 1 - j]);
+            sum = cadd(sum, p[j]);
+        }
+        const float2 v0 = v[0];
+        v[0] = sum;
+#pragma unroll
+        for (int k = 1; k <= H; ++k) {
+            float2 a = v0, b = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int j = 1; j <= H; ++j) {
+                const float c = cos_of<R>(j * k % R), s = sin_of<R>(j * k % R);
+                a = make_float2(fmaf(c, p[j - 1].x, a.x), fmaf(c, p[j - 1].y, a.y));
+                b = make_float2(fmaf(s, m[j - 1].x, b.x), fmaf(s, m[j - 1].y, b.y));
+            }
+            v[k] = make_float2(a.x + b.y, a.y - b.x);
+            v[R - k] = make_float2(a.x - b.y, a.y + b.x);
+        }
+    } else {
+        // even and odd halves, V_k = E_k + w^k O_k, V_{k+R/2} = E_k - w^k O_k
+        constexpr int H = R / 2;
+        float2 e[H], o[H];
+#pragma unroll
+        for (int j = 0; j < H; ++j) {
+            e[j] = v[2 * j];
+            o[j] = v[2 * j + 1];
+        }
+        dft_reg<H>(e);
+        dft_reg<H>(o);
+        constexpr float r2 = 0.707106781186547524f, r3 = 0.866025403784438647f;
+#pragma unroll
+        for (int k = 0; k < H; ++k) {
+            float2 t = o[k];
+            if (R == 4 && k == 1) t = make_float2(t.y, -t.x);
+            if (R == 8 && k == 1) t = make_float2(r2 * (t.x + t.y), r2 * (t.y - t.x));
+            if (R == 8 && k == 2) t = make_float2(t.y, -t.x);
+            if (R == 8 && k == 3) t = make_float2(r2 * (t.y - t.x), -r2 * (t.x + t.y));
+            if (R == 6 && k == 1) t = cmul(t, make_float2(0.5f, -r3));
+            if (R == 6 && k == 2) t = cmul(t, make_float2(-0.5f, -r3));
+            v[k] = cadd(e[k], t);
+            v[k + H] = csub(e[k], t);
+        }
+    }
+}
+
+// One pass over every line of an N x N block (line stride ls, element stride
+// es): with e = N2 n1 + n2, A forms the length-N1 transforms over n1 and the
+// twiddle w^(n2 k1) into n2 N1 + k1; B the length-N2 transforms over n2 into
+// k1 + N1 k2. Lanes run along the contiguous direction.
+template <int N1, int N2, int P, bool COLS, bool PASS_B>
+__device__ __forceinline__ void dft_lines(const float2 *src, float2 *dst, const float4 *tw)
+{
+    constexpr int N = N1 * N2, R = PASS_B ? N2 : N1, C = N / R;   // C transforms of length R a line
+    constexpr int ls = COLS ? 1 : P, es = COLS ? P : 1;
+    for (int i = threadIdx.x; i < N * C; i += blockDim.x) {
+        const int line = COLS ? i % N : i / C, m = COLS ? i / N : i % C;   // m: n2 (A) or k1 (B)
+        const float2 *a = src + line * ls;
+        float2 *b = dst + line * ls;
+        float2 v[R];
+#pragma unroll
+        for (int q = 0; q < R; ++q) v[q] = a[(PASS_B ? q * N1 + m : N2 * q + m) * es];
+        dft_reg<R>(v);
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+            if (PASS_B) b[(m + N1 * q) * es] = v[q];
+            else b[(m * N1 + q) * es] = q == 0 ? v[q] : ctwiddle(v[q], tw[m * q]);
+        }
+    }
+    __syncthreads();
+}
+
+// Block sum (or maximum) of two values; every thread gets both.
+template <bool MAX>
+__device__ __forceinline__ float2 block_reduce2(float a, float b, float2 *red)
+{
+    auto op = [](float u, float v) { return MAX ? fmaxf(u, v) : u + v; };
+    for (int o = 16; o > 0; o >>= 1) {
+        a = op(a, __shfl_xor_sync(0xffffffffu, a, o));
+        b = op(b, __shfl_xor_sync(0xffffffffu, b, o));
+    }
+    __syncthreads();   // (red may still be read from an earlier reduction)
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_float2(a, b);
+    __syncthreads();
+    float2 t = red[0];
+    for (unsigned w = 1; w < (blockDim.x + 31) / 32; ++w) t = make_float2(op(t.x, red[w].x), op(t.y, red[w].y));
+    return t;
+}
+// The exponent e for which 2^e m is about one (0 for zero and non-finite m).
+__device__ __forceinline__ int unit_exp(float m)
+{
+    return m > 0.f && isfinite(m) ? -ilogbf(m) : 0;
+}
+// v 2^e for |e| up to 252, as two factors in the normal range.
+struct Scale {
+    float a, b;
+    __device__ __forceinline__ explicit Scale(int e) : a(ldexpf(1.f, e / 2)), b(ldexpf(1.f, e - e / 2)) {}
+    __device__ __forceinline__ float operator*(float v) const { return v * a * b; }
+};
+
+// exp(-2 pi i k / N), each part as a float and the rest of it: the rounding of the
+// twiddles was the largest part of the error (4.0e-6 -> 3.1e-6 of the result with
+// the rests; with this form's packing, before it, 3.7e-6 for one DFT a plane).
+template <int N>
+struct WienerTwiddles {
+    float4 w[N];
+};
+
+template <int N1, int N2>
+struct WienerCfg {
+    static constexpr int N = N1 * N2, P = N + 1;   // row pitch
+    static constexpr int items = N * (N1 > N2 ? N1 : N2);
+    static constexpr int threads = items >= 512 ? 512 : (items + 31) / 32 * 32;
+    static constexpr size_t smem = N * sizeof(float4) + 3 * (size_t)N * P * sizeof(float2);
+    static constexpr int blocks = 1024 / threads;   // 64 registers a thread
+};
+
+template <int N1, int N2>
+__global__ void __launch_bounds__(WienerCfg<N1, N2>::threads, WienerCfg<N1, N2>::blocks) k_wiener_node(const float *mref, const float *mrem, int nz,
+                                                                            int nx, int nkx, float eps, float *blk,
+        const WienerTwiddles<N1 * N2> table)
+{
+    using C = WienerCfg<N1, N2>;
+    constexpr int N = C::N, P = C::P, NN = N * N, s = N / 2, NT = C::threads, PER = (NN + NT - 1) / NT;
+    extern __shared__ __align__(16) float4 wsm4[];
+    float4 *tw = wsm4;                                  // [N] exp(-2 pi i k / N)
+    float2 *X = reinterpret_cast<float2 *>(tw + N);     // [N][P]
+    float2 *Y = X + N * P;         // [N][P]
+    float2 *W = Y + N * P;         // [N][P] the first plane's product
+    __shared__ float2 red[16];
+    const int node = blockIdx.x, t = threadIdx.x;
+    const int kz = node / nkx, kx = node - kz * nkx;
+    const int zb = s / 2 + kz * s - s, xb = s / 2 + kx * s - s;   // first pixel of the block
+    const long long pl = (long long)nz * nx;
+    for (int k = t; k < N; k += NT) tw[k] = table.w[k];
+    int out_exp[2];                               // the result's scale of each plane
+    float pmax0 = 0.f;                            // the first product's largest part
+    bool bad[2] = {false, false};                 // a plane's product is not finite
+    float norm[2] = {1.f / (float)NN, 1.f / (float)NN};   // 1 / N^2, or what a plane without a result gets
+    for (int q = 0; q < 3; ++q) {
+        if (q < 2) {
+            // the plane's two blocks, scaled, as a + i b
+            float2 v[PER];
+            float ma = 0.f, mb = 0.f;
+#pragma unroll
+            for (int i = 0; i < PER; ++i) {
+                const int idx = t + i * NT, a = idx / N, b = idx - a * N, z = zb + a, x = xb + b;
+                const bool ok = idx < NN && z >= 0 && z < nz && x >= 0 && x < nx;
+                const long long g = q * pl + (long long)z * nx + x;
+                v[i] = ok ? make_float2(mrem[g], mref[g]) : make_float2(0.f, 0.f);
+                ma = fmaxf(ma, fabsf(v[i].x));
+                mb = fmaxf(mb, fabsf(v[i].y));
+            }
+            // scaled to norms of about one (by the largest value first: sums
+            // of squares could overflow)
+            const float2 mx = block_reduce2<true>(ma, mb, red);
+            const int ea = unit_exp(mx.x), eb = unit_exp(mx.y);
+            const Scale fa(ea), fb(eb);
+            float sa = 0.f, sb = 0.f;
+#pragma unroll
+            for (int i = 0; i < PER; ++i) {
+                v[i] = make_float2(fa * v[i].x, fb * v[i].y);
+                sa = fmaf(v[i].x, v[i].x, sa);
+                sb = fmaf(v[i].y, v[i].y, sb);
+            }
+            const float2 sq = block_reduce2<false>(sa, sb, red);
+            const int na = unit_exp(sqrtf(sq.x)) + kWienerBias, nb = unit_exp(sqrtf(sq.y));
+            const float ga = ldexpf(1.f, na), gb = ldexpf(1.f, nb);
+#pragma unroll
+            for (int i = 0; i < PER; ++i) {
+                const int idx = t + i * NT, a = idx / N, b = idx - a * N;
+                if (idx < NN) X[a * P + b] = make_float2(v[i].x * ga, v[i].y * gb);
+            }
+            __syncthreads();
+            const float eps_k = eps * (sq.x * ga * ga);   // sum a^2 = mean |A|^2 of the scaled block
+            // (a zero or non-finite m'' gives zero, and so does a zero m_rtm)
+            const bool live = sq.x > 0.f && isfinite(sq.x) && !(sq.y == 0.f);
+            dft_lines<N1, N2, P, false, false>(X, Y, tw);
+            dft_lines<N1, N2, P, false, true>(Y, X, tw);
+            dft_lines<N1, N2, P, true, false>(X, Y, tw);
+            dft_lines<N1, N2, P, true, true>(Y, X, tw);
+            // conj(A) B B / (|A|^2 + eps_k)
+            float2 *dst = q == 0 ? W : Y;
+            float pm = 0.f;
+            bool nf = false;
+            for (int idx = t; idx < NN; idx += NT) {
+                const int a = idx / N, b = idx - a * N;
+                const float2 z1 = X[a * P + b], z2 = X[(a ? N - a : 0) * P + (b ? N - b : 0)];
+                const float2 A = make_float2(0.5f * (z1.x + z2.x), 0.5f * (z1.y - z2.y));
+                const float2 B = make_float2(0.5f * (z1.y + z2.y), 0.5f * (z2.x - z1.x));
+                float2 r = make_float2(0.f, 0.f);
+                if (live) {
+                    const float den = fmaf(A.x, A.x, fmaf(A.y, A.y, eps_k));
+                    const float2 l = make_float2((A.x * B.x + A.y * B.y) / den, (A.x * B.y - A.y * B.x) / den);
+                    r = make_float2(l.x * B.x - l.y * B.y, l.x * B.y + l.y * B.x);
+                }
+                dst[a * P + b] = r;
+                pm = fmaxf(pm, fmaxf(fabsf(r.x), fabsf(r.y)));
+                nf |= !(isfinite(r.x) && isfinite(r.y));
+            }
+            bad[q] = __syncthreads_or(nf);
+            // conj(A) B B / (|A|^2 + eps_k) goes as b^2 / a
+            out_exp[q] = ea + na - 2 * (eb + nb);
+            if (!live) norm[q] = 0.f;
+            if (bad[q]) norm[q] = __int_as_float(0x7fffffff);
+            if (q == 0) {
+                pmax0 = pm;
+            } else {
+                // both planes' products as P0 + i P1, scaled to norms of about
+                // one, parts exchanged; one that is not finite stays out of the
+                // other's result (its own is then not a number)
+                const float2 mp = block_reduce2<true>(pmax0, pm, red);
+                const int e0 = unit_exp(mp.x), e1 = unit_exp(mp.y);
+                const Scale f0(e0), f1(e1);
+                float s0 = 0.f, s1 = 0.f;
+                for (int idx = t; idx < NN; idx += NT) {
+                    const int e = idx / N * P + idx % N;
+                    const float2 p0 = W[e], p1 = Y[e];
+                    const float2 u0 = make_float2(f0 * p0.x, f0 * p0.y), u1 = make_float2(f1 * p1.x, f1 * p1.y);
+                    W[e] = u0, Y[e] = u1;
+                    s0 = fmaf(u0.x, u0.x, fmaf(u0.y, u0.y, s0));
+                    s1 = fmaf(u1.x, u1.x, fmaf(u1.y, u1.y, s1));
+                }
+                const float2 sp = block_reduce2<false>(s0, s1, red);
+                const int n0 = unit_exp(sqrtf(sp.x)), n1 = unit_exp(sqrtf(sp.y));
+                const float g0 = ldexpf(1.f, n0), g1 = ldexpf(1.f, n1);
+                out_exp[0] -= e0 + n0;
+                out_exp[1] -= e1 + n1;
+                for (int idx = t; idx < NN; idx += NT) {
+                    const int a = idx / N, b = idx - a * N;
+                    const float2 zero = make_float2(0.f, 0.f);
+                    const float2 p0 = bad[0] ? zero : W[a * P + b], p1 = bad[1] ? zero : Y[a * P + b];
+                    X[a * P + b] = make_float2(g0 * p0.y + g1 * p1.x, g0 * p0.x - g1 * p1.y);
+                }
+                __syncthreads();
+            }
+        } else {
+            dft_lines<N1, N2, P, false, false>(X, Y, tw);
+            dft_lines<N1, N2, P, false, true>(Y, X, tw);
+            dft_lines<N1, N2, P, true, false>(X, Y, tw);
+            dft_lines<N1, N2, P, true, true>(Y, X, tw);
+        }
+    }
+    float2 *out = reinterpret_cast<float2 *>(blk) + (long long)node * NN;
+    for (int idx = t; idx < NN; idx += NT) {
+        const int a = idx / N, b = idx - a * N;
+        const float2 r = X[a * P + b];   // (imaginary, real) of the inverse: (plane 1, plane 0)
+        out[idx] = make_float2(ldexpf(r.y * norm[0], out_exp[0]), ldexpf(r.x * norm[1], out_exp[1]));
+    }
+}
+
+__global__ void k_wiener_blend(const float2 *blk, int nz, int nx, int s, int nkz, int nkx, float *out)
 {
     const long long plane = (long long)nz * nx;
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= plane) return;
-    const int param = blockIdx.y;
     const int z = (int)(i / nx), x = (int)(i - (long long)(i / nx) * nx);
     const int N = 2 * s, NN = N * N;
     const int iz = z >= s / 2 ? (z - s / 2) / s : -1, ix = x >= s / 2 ? (x - s / 2) / s : -1;
-    float num = 0.f, den = 0.f;
+    float num0 = 0.f, num1 = 0.f, den = 0.f;
     for (int a = 0; a < 2; ++a) {
         const int kz = iz + a;
         if (kz < 0 || kz >= nkz) continue;
@@ -406,11 +721,30 @@ __global__ void k_wiener_blend(const float *blk, int nz, int nx, int s, int nkz,
             const int dx = x - (s / 2 + kx * s);
             const float w = wz * fmaxf(0.f, 1.f - fabsf((float)dx) / s);
             if (w <= 0.f) continue;
-            num = fmaf(w, blk[(((long long)param * nkz + kz) * nkx + kx) * NN + (dz + s) * N + (dx + s)], num);
+            const float2 v = blk[((long long)kz * nkx + kx) * NN + (dz + s) * N + (dx + s)];
+            num0 = fmaf(w, v.x, num0);
+            num1 = fmaf(w, v.y, num1);
             den += w;
         }
     }
-    out[param * plane + i] = den > 0.f ? num / den : 0.f;
+    out[i] = den > 0.f ? num0 / den : 0.f;
+    out[plane + i] = den > 0.f ? num1 / den : 0.f;
+}
+
+template <int N1, int N2>
+cudaError_t wiener_node(const float *mref, const float *mrem, int nz, int nx, int nkz, int nkx, double eps, float *blk,
+                        cudaStream_t st)
+{
+    using C = WienerCfg<N1, N2>;
+    const cudaError_t e = cudaFuncSetAttribute(k_wiener_node<N1, N2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem);
+    if (e != cudaSuccess) return e;
+    WienerTwiddles<C::N> tw;
+    for (int k = 0; k < C::N; ++k) {
+        const double a = 2.0 * M_PI * k / C::N, c = std::cos(a), s = -std::sin(a);
+        tw.w[k] = make_float4((float)c, (float)s, (float)(c - (float)c), (float)(s - (float)s));
+    }
+    k_wiener_node<N1, N2><<<nkz * nkx, C::threads, C::smem, st>>>(mref, mrem, nz, nx, nkx, (float)eps, blk, tw);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -427,13 +761,40 @@ cudaError_t launch_wiener(const float *mref, const float *mrem, int nz, int nx, 
                           float *out, cudaStream_t st)
 {
     const int nkz = deblur_nodes(nz, s), nkx = deblur_nodes(nx, s);
-    const size_t sm = wiener_smem(s);
-    cudaError_t e = cudaFuncSetAttribute(k_wiener_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = cudaSuccess;
+    auto node = [&](auto f) { e = f(mref, mrem, nz, nx, nkz, nkx, eps, blk, st); };
+    switch (2 * s) {   // the factors nearest the square root
+    case 4: node(wiener_node<2, 2>); break;
+    case 6: node(wiener_node<2, 3>); break;
+    case 8: node(wiener_node<2, 4>); break;
+    case 10: node(wiener_node<2, 5>); break;
+    case 12: node(wiener_node<3, 4>); break;
+    case 14: node(wiener_node<2, 7>); break;
+    case 16: node(wiener_node<4, 4>); break;
+    case 18: node(wiener_node<3, 6>); break;
+    case 20: node(wiener_node<4, 5>); break;
+    case 24: node(wiener_node<4, 6>); break;
+    case 28: node(wiener_node<4, 7>); break;
+    case 30: node(wiener_node<5, 6>); break;
+    case 32: node(wiener_node<4, 8>); break;
+    case 36: node(wiener_node<6, 6>); break;
+    case 40: node(wiener_node<5, 8>); break;
+    case 42: node(wiener_node<6, 7>); break;
+    case 48: node(wiener_node<6, 8>); break;
+    case 56: node(wiener_node<7, 8>); break;
+    case 64: node(wiener_node<8, 8>); break;
+    default: {
+        const size_t sm = wiener_smem(s);
+        e = cudaFuncSetAttribute(k_wiener_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e != cudaSuccess) return e;
+        k_wiener_block<<<dim3(nkz * nkx, 2), kWienerThreads, sm, st>>>(mref, mrem, nz, nx, s, nkx, (float)eps, blk);
+        e = cudaGetLastError();
+    }
+    }
     if (e != cudaSuccess) return e;
-    k_wiener_block<<<dim3(nkz * nkx, 2), kWienerThreads, sm, st>>>(mref, mrem, nz, nx, s, nkx, (float)eps, blk);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const long long plane = (long long)nz * nx;
-    k_wiener_blend<<<dim3((unsigned)((plane + 255) / 256), 2), 256, 0, st>>>(blk, nz, nx, s, nkz, nkx, out);
+    k_wiener_blend<<<(unsigned)((plane + 255) / 256), 256, 0, st>>>(reinterpret_cast<const float2 *>(blk), nz, nx, s, nkz, nkx,
+                                                                    out);
     return cudaGetLastError();
 }
 
