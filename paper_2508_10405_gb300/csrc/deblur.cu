@@ -14,16 +14,24 @@
 //
 // k_deblur_solve: one CTA per (node, parameter plane). The window's patch of
 // m'' (window + h on each side, zero outside the image) sits in shared memory
-// as float. Entry (u, v) of A^T A is the sum of P(q) P(q + d) over the window
+// as double: a conversion costs the FP64 pipe as much as the multiply-add it
+// feeds. Entry (u, v) of A^T A is the sum of P(q) P(q + d) over the window
 // shifted to tap u's origin, d = origin(v) - origin(u): the products depend on
-// the lag d only, so per lag one warp forms, for every patch row, the
-// running sums of the row's lagged products over the window width at every
-// origin column (one pass along the row), then slides those along z over the
-// window height at every origin row. That is 15x fewer FP64 operations than
-// summing each entry over the window (products of two floats are exact in
-// FP64; sums in FP64). The matrix, factorised in place by a right-looking
-// Cholesky, and the right-hand side stay in shared memory (121 x 121 doubles
-// = 117 KB for flen = 11).
+// the lag d only, so per lag and patch row a thread forms the running sums of
+// the row's lagged products over the window width at every origin column (one
+// pass along the row), and per lag and origin column a thread slides those
+// along z over the window height at every origin row: 15x fewer FP64
+// operations than summing each entry over the window (products of two floats
+// are exact in FP64; sums in FP64). The (dz, row) pairs of one dx are dealt
+// over all threads together: one lag's 41 to 51 rows fill two warps to 72%,
+// and an FP64 instruction takes its 64 cycles of a scheduler whatever lanes it
+// has. The matrix is kept as its packed lower triangle with the right-hand side
+// as one more row (60 KB for flen = 11, two CTAs per SM: the serial parts of
+// one run under the other's sums), factorised in panels of eight columns: the
+// diagonal block in the registers of one warp, a panel row per thread, and one
+// pass over the rest for all eight columns.
+// Bound by the FP64 pipe (2 multiply-adds a clock and SM: about 1.1M of them a
+// window). @@MEASURED@@
 // k_deblur_apply: one thread per pixel and plane; FP32 taps, at most four
 // covering nodes.
 // The paper's own Fourier form of the filter (per-block Wiener ratio) follows
@@ -40,147 +48,225 @@ namespace lsrtm {
 
 namespace {
 
-constexpr int kSolveThreads = 256;
+constexpr int kSolveThreads = 256, kSolvePanel = 8;
 
-__global__ void __launch_bounds__(kSolveThreads) k_deblur_solve(const float *mref, const float *mrem, int nz,
-                                                                 int nx, int s, int flen, double eps,
-                                                                 float *filt, int *flag, int nrs)
+__device__ __forceinline__ int tri(int i) { return i * (i + 1) / 2; }
+
+// Row of entry e of a packed lower triangle.
+__device__ __forceinline__ int tri_row(int e)
+{
+    int i = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+    if (tri(i) > e) --i;
+    if (tri(i + 1) <= e) ++i;
+    return i;
+}
+
+// ulen: doubles of the region U, at least one lag's row sums, PZ * flen.
+__global__ void __launch_bounds__(kSolveThreads, 3) k_deblur_solve(const float *mref, const float *mrem, int nz,
+                                                                    int nx, int s, int flen, double eps,
+                                                                    float *filt, int *flag, int ulen)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int n = flen * flen, h = flen / 2;
+    const int n = flen * flen, h = flen / 2, w2 = 2 * h;
     const int nkz = gridDim.y, nkx = gridDim.x;
     const int param = blockIdx.z;
     const int zk = s / 2 + (int)blockIdx.y * s, xk = s / 2 + (int)blockIdx.x * s;
     const int z0 = max(0, zk - s), z1 = min(nz, zk + s + 1);
     const int x0 = max(0, xk - s), x1 = min(nx, xk + s + 1);
     const int WZ = z1 - z0, WX = x1 - x0;
-    const int PZ = WZ + 2 * h, PX = WX + 2 * h;
-    double *G = reinterpret_cast<double *>(smem);   // [n][n]
-    double *rhs = G + n * n;                        // [n]
-    double *red = rhs + n;                          // [2]: trace, pivot status
-    double *RS = red + 2;                           // [nrs warps][PZ][2h + 1] row sums of one lag
-    float *P = reinterpret_cast<float *>(RS + (size_t)nrs * PZ * (2 * h + 1));   // [PZ][PX]
+    const int PZ = WZ + w2, PX = WX + w2, PS = PX | 1;   // odd row stride: lanes on consecutive rows hit all banks
+    double *G = reinterpret_cast<double *>(smem);   // rows 0..n packed; row n: the right-hand side
+    double *red = G + tri(n + 1);                   // [2]: trace, pivot status
+    double *U = red + 2;                            // row sums; then rows of m'; then the panel [8][n + 1]
+    double *P = U + ulen;                           // [PZ][PS]
     const long long plane = (long long)nz * nx;
     const float *m2 = mrem + param * plane;
     const float *m1 = mref + param * plane;
-    const int t = threadIdx.x;
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
 
-    for (int i = t; i < PZ * PX; i += blockDim.x) {
-        int pz = i / PX, px = i - pz * PX;
-        int z = z0 - h + pz, x = x0 - h + px;
-        P[i] = (z >= 0 && z < nz && x >= 0 && x < nx) ? m2[(long long)z * nx + x] : 0.f;
+    for (int i = t; i < PZ * PX; i += kSolveThreads) {
+        const int pz = i / PX, px = i - pz * PX;
+        const int z = z0 - h + pz, x = x0 - h + px;
+        P[pz * PS + px] = (z >= 0 && z < nz && x >= 0 && x < nx) ? (double)m2[(long long)z * nx + x] : 0.0;
     }
-    if (t == 0) {
-        red[0] = 0.0;
-        red[1] = 0.0;
-    }
+    if (t == 0) red[1] = 0.0;
     __syncthreads();
 
     // A[p, u] = m''(p - (a, b)) = P[pz + oz_u][px + ox_u], u = (a + h) flen + (b + h),
-    // origin (oz_u, ox_u) = (2h - u / flen, 2h - u % flen) in [0, 2h]^2
-    {
-        const int warp = t >> 5, lane = t & 31, W2 = 2 * h + 1;
-        double *rs = RS + (size_t)warp * PZ * W2;
-        const int nlag = 2 * h * (4 * h + 1) + (2 * h + 1);   // dz > 0, or dz = 0 and dx >= 0
-        for (int li = warp; li < nlag && warp < nrs; li += nrs) {
-            const int dz = li < 2 * h + 1 ? 0 : 1 + (li - (2 * h + 1)) / (4 * h + 1);
-            const int dx = li < 2 * h + 1 ? li : (li - (2 * h + 1)) % (4 * h + 1) - 2 * h;
-            const int oz0 = max(0, -dz), oz1 = min(2 * h, 2 * h - dz);   // origins of u with u + d a tap
-            const int ox0 = max(0, -dx), ox1 = min(2 * h, 2 * h - dx);
-            // rs[r][ox] = sum_{c = ox}^{ox + WX - 1} P[r][c] P[r + dz][c + dx]
-            for (int r = oz0 + lane; r < oz1 + WZ; r += 32) {
-                const float *a = P + r * PX, *b = P + (r + dz) * PX + dx;
+    // origin (oz_u, ox_u) = (2h - u / flen, 2h - u % flen) in [0, 2h]^2. Lags dz > 0, or dz = 0 and dx >= 0.
+    for (int dx = -w2; dx <= w2; ++dx) {
+        const int ox0 = max(0, -dx), ox1 = min(w2, w2 - dx), nox = ox1 - ox0 + 1, nos = nox | 1;
+        const int chunk = ulen / (PZ * nos);
+        for (int d0 = dx < 0 ? 1 : 0; d0 <= w2; d0 += chunk) {
+            const int cnt = min(chunk, w2 + 1 - d0);
+            // rs[(dz, r)][ox] = sum_{c = ox}^{ox + WX - 1} P[r][c] P[r + dz][c + dx], the PZ - dz rows of each dz in turn
+            const int items = cnt * (PZ - d0) - cnt * (cnt - 1) / 2;
+            for (int e = t; e < items; e += kSolveThreads) {
+                int r = e, dz = d0;
+                while (r >= PZ - dz) {
+                    r -= PZ - dz;
+                    ++dz;
+                }
+                const double *a = P + r * PS, *b = P + (r + dz) * PS + dx;
+                double *rs = U + e * nos - ox0;
                 double acc = 0.0;
-                for (int c = ox0; c < ox0 + WX; ++c) acc = fma((double)a[c], (double)b[c], acc);
-                rs[r * W2 + ox0] = acc;
+#pragma unroll 4
+                for (int c = ox0; c < ox0 + WX; ++c) acc = fma(a[c], b[c], acc);
+                rs[ox0] = acc;
                 for (int ox = ox0 + 1; ox <= ox1; ++ox) {
-                    acc = fma((double)a[ox + WX - 1], (double)b[ox + WX - 1], acc);
-                    acc = fma(-(double)a[ox - 1], (double)b[ox - 1], acc);
-                    rs[r * W2 + ox] = acc;
+                    acc = fma(a[ox + WX - 1], b[ox + WX - 1], acc);
+                    acc = fma(-a[ox - 1], b[ox - 1], acc);
+                    rs[ox] = acc;
                 }
             }
-            __syncwarp();
-            // S(oz, ox) = sum_{r = oz}^{oz + WZ - 1} rs[r][ox] -> G[u][v] and G[v][u]
-            for (int ox = ox0 + lane; ox <= ox1; ox += 32) {
+            __syncthreads();
+            // S(oz, ox) = sum_{r = oz}^{oz + WZ - 1} rs[r][ox] -> G[u][v]; d >= 0 in the order of taps: v <= u
+            for (int e = t; e < cnt * nox; e += kSolveThreads) {
+                const int j = e / nox, ox = ox0 + e - j * nox, dz = d0 + j;
+                const double *rs = U + (j * (PZ - d0) - j * (j - 1) / 2) * nos + (ox - ox0);
                 double acc = 0.0;
-                for (int r = oz0; r < oz0 + WZ; ++r) acc += rs[r * W2 + ox];
-                for (int oz = oz0; oz <= oz1; ++oz) {
-                    if (oz > oz0) acc += rs[(oz + WZ - 1) * W2 + ox] - rs[(oz - 1) * W2 + ox];
-                    const int u = (2 * h - oz) * flen + (2 * h - ox);
-                    const int v = (2 * h - oz - dz) * flen + (2 * h - ox - dx);
-                    G[u * n + v] = acc;
-                    G[v * n + u] = acc;
+#pragma unroll 4
+                for (int r = 0; r < WZ; ++r) acc += rs[r * nos];
+                for (int oz = 0; oz <= w2 - dz; ++oz) {
+                    if (oz > 0) acc += rs[(oz + WZ - 1) * nos] - rs[(oz - 1) * nos];
+                    const int u = (w2 - oz) * flen + (w2 - ox);
+                    G[tri(u) + u - dz * flen - dx] = acc;
                 }
             }
-            __syncwarp();
+            __syncthreads();
         }
     }
-    for (int u = t; u < n; u += blockDim.x) {
-        const int ozu = 2 * h - u / flen, oxu = 2 * h - u % flen;
+    // right-hand side: a thread per tap, m' in pieces
+    {
+        const int u = min(t, n - 1), ou = (w2 - u / flen) * PS + w2 - u % flen;
         double acc = 0.0;
-        for (int pz = 0; pz < WZ; ++pz) {
-            const float *ru = P + (pz + ozu) * PX + oxu;
-            const float *r1 = m1 + (long long)(z0 + pz) * nx + x0;
-            for (int px = 0; px < WX; ++px) acc = fma((double)ru[px], (double)r1[px], acc);
+        for (int q0 = 0; q0 < WZ * WX; q0 += ulen) {
+            const int q1 = min(WZ * WX, q0 + ulen);
+            for (int q = q0 + t; q < q1; q += kSolveThreads) {
+                const int pz = q / WX;
+                U[q - q0] = (double)m1[(long long)(z0 + pz) * nx + x0 + q - pz * WX];
+            }
+            __syncthreads();
+            if (warp * 32 < n) {
+                int pz = q0 / WX, px = q0 - pz * WX;
+                for (int q = q0; q < q1;) {
+                    const int len = min(WX - px, q1 - q);
+                    const double *ru = P + pz * PS + ou + px, *r1 = U + (q - q0);
+#pragma unroll 4
+                    for (int i = 0; i < len; ++i) acc = fma(ru[i], r1[i], acc);
+                    q += len;
+                    px = 0;
+                    ++pz;
+                }
+            }
+            __syncthreads();
         }
-        rhs[u] = acc;
+        if (t < n) G[tri(n) + t] = acc;
     }
-    __syncthreads();
-    if (t == 0) {
+    if (warp == 0) {
         double tr = 0.0;
-        for (int u = 0; u < n; ++u) tr += G[u * n + u];
-        red[0] = tr;
+        for (int u = lane; u < n; u += 32) tr += G[tri(u) + u];
+        for (int o = 16; o; o >>= 1) tr += __shfl_xor_sync(~0u, tr, o);
+        if (lane == 0) red[0] = tr;
     }
     __syncthreads();
     const double tr = red[0];
     float *out = filt + (((long long)param * nkz + blockIdx.y) * nkx + blockIdx.x) * n;
     if (tr == 0.0) {   // all-zero remigrated window: zero filter
-        for (int u = t; u < n; u += blockDim.x) out[u] = 0.f;
+        for (int u = t; u < n; u += kSolveThreads) out[u] = 0.f;
         return;
     }
     const double reg = eps * tr / n;
-    for (int u = t; u < n; u += blockDim.x) G[u * n + u] += reg;
+    for (int u = t; u < n; u += kSolveThreads) G[tri(u) + u] += reg;
     __syncthreads();
 
-    // Cholesky G = L L^T, L in the lower triangle
-    for (int k = 0; k < n; ++k) {
-        if (t == 0) {
-            double d = G[k * n + k];
-            if (!(d > 0.0)) {
-                red[1] = 1.0;
-                d = 1.0;
+    // Cholesky G = L L^T with 1 / L_kk on the diagonal; row n becomes y of L y = rhs
+    double *panel = U;   // [8][m + 1]: the panel's rows below its diagonal block
+    for (int k0 = 0; k0 < n; k0 += kSolvePanel) {
+        const int nb = min(kSolvePanel, n - k0), k1 = k0 + nb, m = n - k1;
+        if (warp == 0) {
+            double g[kSolvePanel];
+            double *row = G + tri(k0 + lane) + k0;
+#pragma unroll
+            for (int c = 0; c < kSolvePanel; ++c) g[c] = (lane < nb && c <= lane) ? row[c] : 0.0;
+            bool bad = false;
+#pragma unroll
+            for (int c = 0; c < kSolvePanel; ++c) {
+                if (c >= nb) break;
+                double d = __shfl_sync(~0u, g[c], c);
+                if (!(d > 0.0)) {
+                    bad = true;
+                    d = 1.0;
+                }
+                const double r = rsqrt(d);
+                g[c] = lane == c ? r : g[c] * r;
+#pragma unroll
+                for (int j = c + 1; j < kSolvePanel; ++j)
+                    g[j] = fma(-g[c], __shfl_sync(~0u, g[c], j), g[j]);
             }
-            G[k * n + k] = sqrt(d);
+#pragma unroll
+            for (int c = 0; c < kSolvePanel; ++c)
+                if (lane < nb && c <= lane) row[c] = g[c];
+            if (bad && lane == 0) red[1] = 1.0;
         }
         __syncthreads();
-        const double dk = G[k * n + k];
-        for (int i = k + 1 + t; i < n; i += blockDim.x) G[i * n + k] /= dk;
+        for (int i = t; i <= m; i += kSolveThreads) {
+            double *row = G + tri(k1 + i) + k0;
+            double x[kSolvePanel];
+#pragma unroll
+            for (int c = 0; c < kSolvePanel; ++c) x[c] = c < nb ? row[c] : 0.0;
+#pragma unroll
+            for (int c = 0; c < kSolvePanel; ++c) {
+                if (c >= nb) break;
+                x[c] *= G[tri(k0 + c) + k0 + c];
+                row[c] = x[c];
+                panel[c * (m + 1) + i] = x[c];
+#pragma unroll
+                for (int j = c + 1; j < kSolvePanel; ++j)
+                    if (j < nb) x[j] = fma(-x[c], G[tri(k0 + j) + k0 + c], x[j]);
+            }
+        }
         __syncthreads();
-        const int m = n - k - 1;
-        for (int e = t; e < m * m; e += blockDim.x) {
-            const int i = k + 1 + e / m, j = k + 1 + e % m;
-            if (j <= i) G[i * n + j] -= G[i * n + k] * G[j * n + k];
+        // the rest, rows k1..n of columns k1..n-1; m > 0 only below a full panel
+        const int rest = tri(m + 1) - 1;
+        for (int e = t; e < rest; e += 2 * kSolveThreads) {
+            const bool two = e + kSolveThreads < rest;   // two entries a thread, for two chains
+            const int e1 = two ? e + kSolveThreads : e;
+            const int ia = tri_row(e), ja = e - tri(ia), ib = tri_row(e1), jb = e1 - tri(ib);
+            double *ga = G + tri(k1 + ia) + k1 + ja, *gb = G + tri(k1 + ib) + k1 + jb;
+            double va = *ga, vb = *gb;
+#pragma unroll
+            for (int c = 0; c < kSolvePanel; ++c) {
+                const double *l = panel + c * (m + 1);
+                va = fma(-l[ia], l[ja], va);
+                vb = fma(-l[ib], l[jb], vb);
+            }
+            *ga = va;
+            if (two) *gb = vb;
         }
         __syncthreads();
     }
-    // L y = rhs, then L^T f = y (in place in rhs)
-    for (int k = 0; k < n; ++k) {
-        if (t == 0) rhs[k] /= G[k * n + k];
-        __syncthreads();
-        const double yk = rhs[k];
-        for (int i = k + 1 + t; i < n; i += blockDim.x) rhs[i] -= G[i * n + k] * yk;
-        __syncthreads();
-    }
-    for (int k = n - 1; k >= 0; --k) {
-        if (t == 0) rhs[k] /= G[k * n + k];
-        __syncthreads();
-        const double fk = rhs[k];
-        for (int i = t; i < k; i += blockDim.x) rhs[i] -= G[k * n + i] * fk;
-        __syncthreads();
+    if (warp > 0) return;
+    // L^T f = y: a warp, f[lane + 32 q] in its registers
+    double f[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) f[q] = 32 * q + lane < n ? G[tri(n) + 32 * q + lane] : 0.0;
+#pragma unroll
+    for (int q = 3; q >= 0; --q) {
+        for (int k = min(n, 32 * q + 32) - 1; k >= 32 * q; --k) {
+            const double *row = G + tri(k);
+            const double fk = __shfl_sync(~0u, f[q], k & 31) * row[k];
+            if (lane == (k & 31)) f[q] = fk;
+#pragma unroll
+            for (int p = 0; p <= q; ++p)
+                if (32 * p + lane < k) f[p] = fma(-row[32 * p + lane], fk, f[p]);
+        }
     }
     const bool bad = red[1] != 0.0;
-    if (bad && t == 0) atomicOr(flag, 1);
-    for (int u = t; u < n; u += blockDim.x) out[u] = bad ? 0.f : (float)rhs[u];
+    if (bad && lane == 0) atomicOr(flag, 1);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if (32 * q + lane < n) out[32 * q + lane] = bad ? 0.f : (float)f[q];
 }
 
 __global__ void k_deblur_apply(const float *mref, const float *filt, int nz, int nx, int s, int flen, int nkz,
@@ -798,22 +884,25 @@ cudaError_t launch_wiener(const float *mref, const float *mrem, int nz, int nx, 
     return cudaGetLastError();
 }
 
-// Shared memory of k_deblur_solve with nrs warps forming lag sums.
-size_t deblur_solve_smem(int nz, int nx, int s, int flen, int nrs)
+// Doubles of k_deblur_solve's region U, and its shared memory in bytes. The
+// patch and the matrix leave two CTAs an SM (three for flen <= 9) at the usual
+// spacings; U, at least one lag's row sums and the panel, takes the rest of
+// the share, up to what all lags of a dx need.
+int deblur_solve_region(int nz, int nx, int s, int flen, size_t *bytes)
 {
-    const int n = flen * flen, h = flen / 2;
-    const int wz = std::min(nz, 2 * s + 1), wx = std::min(nx, 2 * s + 1);
-    return ((size_t)n * n + n + 2 + (size_t)nrs * (wz + 2 * h) * (2 * h + 1)) * sizeof(double) +
-           (size_t)(wz + 2 * h) * (wx + 2 * h) * sizeof(float);
-}
-
-// Warps of k_deblur_solve that form lag sums: as many as fit (at most all),
-// 0 if not even one does.
-int deblur_solve_warps(int nz, int nx, int s, int flen)
-{
-    int nrs = kSolveThreads / 32;
-    while (nrs > 0 && deblur_solve_smem(nz, nx, s, flen, nrs) > kDeblurSmemLimit) --nrs;
-    return nrs;
+    const int n = flen * flen, pz = std::min(nz, 2 * s + 1) + flen - 1, px = std::min(nx, 2 * s + 1) + flen - 1;
+    const size_t fixed = ((size_t)(n + 1) * (n + 2) / 2 + 2 + (size_t)pz * (px | 1)) * sizeof(double);
+    const int least = std::max(pz * flen, kSolvePanel * (n + 1)), most = std::max(least, pz * flen * flen);
+    const int wish = std::max(least, 4 * pz * flen);
+    int ulen = least;
+    for (int ctas = 3; ctas >= 1; --ctas) {
+        const size_t share = std::min<size_t>(228 * 1024 / ctas - 1024, kDeblurSmemLimit);
+        if (fixed + (size_t)(ctas > 1 ? wish : least) * sizeof(double) > share) continue;
+        ulen = (int)std::min<size_t>(most, (share - fixed) / sizeof(double));
+        break;
+    }
+    *bytes = fixed + (size_t)ulen * sizeof(double);
+    return ulen;
 }
 
 int deblur_nodes(int n, int s) { return n > s / 2 ? (n - 1 - s / 2) / s + 1 : 0; }
@@ -822,12 +911,12 @@ cudaError_t launch_deblur(const float *mref, const float *mrem, int nz, int nx, 
                           float *filt, float *out, int *flag, cudaStream_t st)
 {
     const int nkz = deblur_nodes(nz, s), nkx = deblur_nodes(nx, s);
-    const int nrs = deblur_solve_warps(nz, nx, s, flen);
-    if (nrs < 1) return cudaErrorInvalidValue;
-    const size_t sm = deblur_solve_smem(nz, nx, s, flen, nrs);
+    size_t sm = 0;
+    const int ulen = deblur_solve_region(nz, nx, s, flen, &sm);
+    if (sm > kDeblurSmemLimit) return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(k_deblur_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k_deblur_solve<<<dim3(nkx, nkz, 2), kSolveThreads, sm, st>>>(mref, mrem, nz, nx, s, flen, eps, filt, flag, nrs);
+    k_deblur_solve<<<dim3(nkx, nkz, 2), kSolveThreads, sm, st>>>(mref, mrem, nz, nx, s, flen, eps, filt, flag, ulen);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const long long plane = (long long)nz * nx;
     k_deblur_apply<<<dim3((unsigned)((plane + 255) / 256), 2), 256, 0, st>>>(mref, filt, nz, nx, s, flen, nkz, nkx,
