@@ -47,12 +47,13 @@ lsrtm_status fail(lsrtm_status st, const std::string &msg)
         if (s_ != LSRTM_OK) return s_;         \
     } while (0)
 
-// Planes per wavefield slot: 10 ping-pong planes (Born: (p, dp) (vx, dvx)
-// (vz, dvz) (psi_px, dpsi_px) (psi_pz, dpsi_pz) as float2 pairs; background
-// only: p vx vz psi_px psi_pz; adjoint: (p, dt kappa lambda_p) (vx,
-// lambda_vx) (vz, lambda_vz) pairs and four lambda CPML memories), 4 in-place
-// node CPML planes (forward).
-constexpr int kStatePlanes2D = 10;
+// Planes per wavefield slot: 12 ping-pong planes (Born, 10 of them: (p, dp)
+// (vx, dvx) (vz, dvz) (psi_px, dpsi_px) (psi_pz, dpsi_pz) as float2 pairs;
+// background only: p vx vz psi_px psi_pz; adjoint: (p, dt kappa lambda_p)
+// (vx, lambda_vx) (vz, lambda_vz) pairs, four lambda CPML memories and
+// lambda_p; one unused, pairs go by twos), 4 in-place node CPML planes
+// (forward).
+constexpr int kStatePlanes2D = 12;
 constexpr int kPsivPlanes2D = 4;
 constexpr int kStatePlanes3D = 20;
 
@@ -894,7 +895,7 @@ lsrtm_status adjoint_core_ckpt(lsrtm_handle *h, float *gout, bool want_hess)
             CU(launch_pack_adjoint(h->g, h->final_state, 0, bs, h->st[0], h->sstride, h->work));
             CU(launch_inject_residual(h->gm, h->g, h->trv, bs, s0, h->dstage, nt - 1, h->kdt,
                                       h->win ? h->win_x0_d : nullptr, reinterpret_cast<float2 *>(h->st[0]),
-                                      h->sstride / 2, h->work));
+                                      h->sstride / 2, h->st[0] + kAdjLambda2D * plane, h->work));
             h->launches += 2;
         }
         for (int j = h->ck_nseg - 1; j >= 0; --j) {
@@ -912,7 +913,7 @@ lsrtm_status adjoint_core_ckpt(lsrtm_handle *h, float *gout, bool want_hess)
         h->launches++;
         h->hess_ready = true;
     }
-    CU(launch_image_finalize(h->gm, h->img_acc, h->binv, gout, h->work));
+    CU(launch_image_finalize(h->gm, h->img_acc, is3d(h) ? nullptr : h->kdt, h->binv, gout, h->work));
     h->launches++;
     return LSRTM_OK;
 }
@@ -947,7 +948,7 @@ lsrtm_status adjoint_core(lsrtm_handle *h, float *gout, bool want_hess)
             CU(launch_pack_adjoint(h->g, h->final_state, s0, bs, h->st[0], h->sstride, h->work));
             CU(launch_inject_residual(h->gm, h->g, h->trv, bs, s0, h->dstage, nt - 1, h->kdt,
                                       h->win ? h->win_x0_d : nullptr, reinterpret_cast<float2 *>(h->st[0]),
-                                      h->sstride / 2, h->work));
+                                      h->sstride / 2, h->st[0] + kAdjLambda2D * plane, h->work));
             h->launches += 2;
             CHECK(run_loop(h, G_ADJ, s0, bs, [&]() -> lsrtm_status {
                 CHECK(gather_model(h, s0, bs, false));
@@ -966,7 +967,7 @@ lsrtm_status adjoint_core(lsrtm_handle *h, float *gout, bool want_hess)
             h->launches++;
         }
     }
-    CU(launch_image_finalize(h->gm, h->img_acc, h->binv, gout, h->work));
+    CU(launch_image_finalize(h->gm, h->img_acc, is3d(h) ? nullptr : h->kdt, h->binv, gout, h->work));
     h->launches++;
     return LSRTM_OK;
 }
@@ -1266,7 +1267,7 @@ lsrtm_status adj3f_start(lsrtm_handle *h, int fs0, int s0, int bs)
 {
     CU(launch_pack3f(h->g, h->final_state, fs0, bs, h->st[0], h->sstride, h->work));
     CU(launch_inject_residual(h->gm, h->g, h->trv, bs, s0, h->dstage, h->g.nt - 1, h->kdt, nullptr,
-                              reinterpret_cast<float2 *>(h->st[0]), h->sstride / 2, h->work));
+                              reinterpret_cast<float2 *>(h->st[0]), h->sstride / 2, nullptr, h->work));
     h->launches += 2;
     return LSRTM_OK;
 }
@@ -1488,7 +1489,8 @@ lsrtm_status create_impl(const lsrtm_config *cfg, const float *vp, const float *
     // last 6 as the in-place node CPML memories), st[1] (14 planes, pong), the
     // float2 image plane and the pseudo-Hessian plane
     h->sstride1 = d3 ? 2LL * kBornPairs3F * g.plane : h->sstride;
-    if (h->sstride >= (1LL << 31))   // the time-step kernels index within a slot with 32-bit offsets
+    // the time-step kernels index within a slot with 32-bit offsets (2D: but for the planes of lambda_p)
+    if (h->sstride - (d3 ? 0 : 2 * (long long)g.plane) >= (1LL << 31))
         return fail(LSRTM_ERR_ARG, "grid too large: a wavefield slot exceeds 2^31 floats");
     size_t per_slot = d3 ? ((size_t)h->sstride + h->sstride1 + 3 * g.plane) * sizeof(float)
                          : (2 * (size_t)h->sstride + h->vstride + 2 * g.plane + g.plane) * sizeof(float);

@@ -52,13 +52,13 @@ enum { B_PVX = 0, B_PVZ = 2 };                 // in-place node CPML memories
 // Background only (band saving, pseudo-Hessian): float.
 enum { G_P = 0, G_VX = 1, G_VZ = 2, G_PPX = 3, G_PPZ = 4 };
 enum { G_PVX = 0, G_PVZ = 1 };
-// Adjoint: float2 pairs (p, dt kappa lambda_p), (v, lambda_v) and float
-// lambda CPML memories.
-enum { A_PL = 0, A_VX = 2, A_VZ = 4, A_LPPX = 6, A_LPPZ = 7, A_LPVX = 8, A_LPVZ = 9 };
+// Adjoint: float2 pairs (p, dt kappa lambda_p), (v, lambda_v), float lambda
+// CPML memories and lambda_p.
+enum { A_PL = 0, A_VX = 2, A_VZ = 4, A_LPPX = 6, A_LPPZ = 7, A_LPVX = 8, A_LPVZ = 9, A_L = 10 };
 // Slots of aperture-windowed shots carry the window's own model after the
 // state: dt kappa and 1/rho (float planes), and the Born pairs (float2).
-enum { W_KDT = 10, W_BINV = 11, W_KD2 = 12, W_BR2 = 14 };
-static_assert(W_BR2 + 2 == kWinStatePlanes2D, "window slot layout");
+enum { W_KDT = 12, W_BINV = 13, W_KD2 = 14, W_BR2 = 16 };
+static_assert(W_BR2 + 2 == kWinStatePlanes2D && A_L == kAdjLambda2D, "slot layout");
 
 // ---- packed arithmetic for T = float or float2
 __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
@@ -324,7 +324,7 @@ __device__ __forceinline__ void fwd_body(const Arg2D &p)
     const bool lastx = x + 1 >= Nx;
     const long long bandoff = band_base(a.bands, shot, a.n);
     const int src = a.src_cell[shot];
-    const float wsrc = a.src_scale * a.wav[(a.wav_per_shot ? (long long)shot * g.nt : 0) + a.n];
+    const float wsrc = a.wav[(a.wav_per_shot ? (long long)shot * g.nt : 0) + a.n];
     constexpr int oP = BORN ? B_P / 2 : G_P, oVX = BORN ? B_VX / 2 : G_VX, oVZ = BORN ? B_VZ / 2 : G_VZ;
     constexpr int oPPX = BORN ? B_PPX / 2 : G_PPX, oPPZ = BORN ? B_PPZ / 2 : G_PPZ;
     constexpr int oPVX = BORN ? B_PVX / 2 : G_PVX, oPVZ = BORN ? B_PVZ / 2 : G_PVZ;
@@ -537,9 +537,9 @@ __device__ __forceinline__ void fwd_body(const Arg2D &p)
                     const float sw = cz + x == src ? wsrc : 0.f;
                     if constexpr (BORN) {
                         pn.y = fmaf(-kd2.y, Q.x, pn.y);
-                        pn.x += sw;
+                        pn.x = fmaf(a.src_scale, sw, pn.x);
                     } else {
-                        pn += sw;
+                        pn = fmaf(a.src_scale, sw, pn);
                     }
                     if (!ZF && FS && zr <= z0) pn = zero_<T>();   // p = 0 on the free surface (ghost rows unused)
                     if (own) out[oP * pT + cz] = pn;
@@ -626,28 +626,30 @@ __global__ void __launch_bounds__(NTH, (BANDS || HESS) ? kBandsMinBlocks : kPlai
 // and pre-adds the residual of step n-1. The D+ stencils of (p^n, u) and the
 // D- stencils of (v^{n+1/2}, w) run as packed pairs.
 //
-// The adjoint pressure is carried as mu, the quantity the D+ stencils take:
-// away from the CPML strips the z ring's entry of a row then is the row's own
-// (p, mu), so a row needs neither dt kappa of its look-ahead row nor a second
-// copy of (p, lambda_p). Only the rows outside the interior (CPML rows, whose
-// ring entries hold u != mu, and ghost rows) read their own (p, mu) again, in
-// the stage rows that interior rows use for the image.
+// The adjoint pressure is carried twice: as mu in the pairs, the quantity the
+// D+ stencils take, and as lambda_p in a plane of its own, what the images and
+// the update take. Away from the z strips the ring's entry of a row then is
+// the row's own (p, mu): a row needs neither dt kappa of its look-ahead row nor
+// a second copy of the pairs. (With mu alone, 72 B a cell: 55.2 G; but
+// lambda_p then is rounded as mu, and the 64-bit misfits of a CG move by 1e-8.) Which products of the CPML terms are fused into the
+// subtractions, and in the forward step the source's, is written out for the
+// same reason: left to the compiler, it changes with the code around them.
 //
-// What bounds it: 72 B a cell (70.9 from DRAM), held back like the Born step;
+// What bounds it: 80 B a cell, held back like the Born step;
 // 3 tile copies a row where a row at a time took 9. The x strips' band values
 // come one group ahead by asynchronous copies (read where they are used, they
 // doubled the strip warps' time). 96 shots of 424 x 1192, order 8, FP16 bands:
-// 54.1 G cell-updates/s = 0.58 of the measured copy rate (a row at a time with
+// 53.7 G cell-updates/s = 0.64 of the measured copy rate (a row at a time with
 // one issuing thread: 42.4; in groups without the straight-line form: 31.5).
 // ---------------------------------------------------------------------------
 struct AdjLay {
     static constexpr unsigned F2R = NTH * 8, F1R = NTH * 4, F2 = 2 * F2R, F1 = 2 * F1R;   // a row, a group's two rows
-    // stage: (p, mu) rows z + 2M - 1; v_z half rows z + M - 1; v_x rows z; image (interior rows) or (p, mu) rows z
+    // stage: (p, mu) rows z + 2M - 1; v_z half rows z + M - 1; v_x rows z; image (interior rows) or lambda psi_vz rows z
     static constexpr unsigned PL = 0, VZ = F2, VX = 2 * F2, IM = 3 * F2;
-    // dt kappa rows z; lambda CPML memories psi_vx and psi_px rows z (CTAs with x strips), psi_vz rows z + 2M - 1 and
-    // z, psi_pz half rows z + M - 1 (groups with z strip rows)
-    static constexpr unsigned KD = 4 * F2, LVX = KD + F1, LPX = LVX + F1, LVZR = LPX + F1, LVZ = LVZR + F1,
-                              LPZ = LVZ + F1, STAGE = LPZ + F1;
+    // dt kappa and lambda_p rows z; lambda CPML memories psi_vx and psi_px rows z (CTAs with x strips), psi_vz rows
+    // z + 2M - 1, psi_pz half rows z + M - 1 (groups with z strip rows)
+    static constexpr unsigned KD = 4 * F2, LAM = KD + F1, LVX = LAM + F1, LPX = LVX + F1, LVZR = LPX + F1,
+                              LPZ = LVZR + F1, STAGE = LPZ + F1;
     static constexpr unsigned B = NS * STAGE;   // 1/rho ring (FwdLay::BR)
 };
 template <int M>
@@ -679,7 +681,7 @@ __device__ __forceinline__ void adj_issue(const Arg2D &p, int warp, char *st, ch
     const CUtensorMap(&mm)[2] = WIN ? m.fl : m.md;
     const bool main = z >= zc0;
     const bool lvr = zpml_node(g, zr) || zpml_node(g, zr + 1), lpz = zpml_half(g, k) || zpml_half(g, k + 1);
-    const bool lvz = main && (zpml_node(g, z) || zpml_node(g, z + 1));
+    const bool in0 = z >= g.z0 && z < g.z0 + g.nz, in1 = z + 1 >= g.z0 && z + 1 < g.z0 + g.nz;
     if (warp == 0) {
         if (tma::elect_one()) {
             if (FS && zr < g.z0)
@@ -699,16 +701,13 @@ __device__ __forceinline__ void adj_issue(const Arg2D &p, int warp, char *st, ch
     } else if (warp == 2) {
         if (main && tma::elect_one()) tma::load3(st + L::VX, m.pr[1], xs, z, qp + A_VX / 2, b);
     } else if (warp == 3) {
-        // the image of interior rows, (p, mu) of others
-        const bool in0 = z >= g.z0 && z < g.z0 + g.nz, in1 = z + 1 >= g.z0 && z + 1 < g.z0 + g.nz;
+        // the image of interior rows, lambda psi_vz of others
         if (main && tma::elect_one()) {
             if (in0 && in1) {
                 tma::load3(st + L::IM, m.im[1], xs, z, slot, b);
-            } else if (!in0 && !in1) {
-                tma::load3(st + L::IM, m.pr[1], xs, z, qp + A_PL / 2, b);
             } else {
-                tma::load3(st + L::IM, in0 ? m.im[0] : m.pr[0], xs, z, in0 ? slot : qp + A_PL / 2, b);
-                tma::load3(st + L::IM + L::F2R, in1 ? m.im[0] : m.pr[0], xs, z + 1, in1 ? slot : qp + A_PL / 2, b);
+                tma::load3(st + L::IM, in0 ? m.im[0] : m.fl[0], xs, z, in0 ? slot : qf + A_LPVZ, b);
+                tma::load3(st + L::IM + L::F2R, in1 ? m.im[0] : m.fl[0], xs, z + 1, in1 ? slot : qf + A_LPVZ, b);
             }
         }
     } else if (warp == 4) {
@@ -722,15 +721,15 @@ __device__ __forceinline__ void adj_issue(const Arg2D &p, int warp, char *st, ch
             if (lpz) tma::load3(st + L::LPZ, m.fl[1], xs, k, qf + A_LPPZ, b);
         }
     } else if (warp == 6) {
-        if (main && (lvz || tpn) && tma::elect_one()) {
-            if (lvz) tma::load3(st + L::LVZ, m.fl[1], xs, z, qf + A_LPVZ, b);
+        if (main && tma::elect_one()) {
+            tma::load3(st + L::LAM, m.fl[1], xs, z, qf + A_L, b);
             if (tpn) tma::load3(st + L::LVX, m.fl[1], xs, z, qf + A_LPVX, b);
             if (tph) tma::load3(st + L::LPX, m.fl[1], xs, z, qf + A_LPPX, b);
         }
     } else {
         if (tma::elect_one()) {
             unsigned bytes = 2 * L::F2 + (1 + (lvr ? 1 : 0) + (lpz ? 1 : 0)) * L::F1;
-            if (main) bytes += 2 * L::F2 + (1 + (lvz ? 1 : 0) + (tpn ? 1 : 0) + (tph ? 1 : 0)) * L::F1;
+            if (main) bytes += L::F2 + (in0 ? L::F2R : L::F1R) + (in1 ? L::F2R : L::F1R) + (2 + (tpn ? 1 : 0) + (tph ? 1 : 0)) * L::F1;
             tma::mbar_expect(b, bytes);
         }
     }
@@ -774,6 +773,7 @@ __device__ __forceinline__ void adj_body(const Arg2D &p)
     const int xc = colok ? x : 0;
     const float *in = a.in + slot * a.sstride;
     float *outf = a.out + slot * a.sstride + xc;
+    float *outl = a.out + slot * a.sstride + A_L * g.plane + xc;
     float2 *out2 = reinterpret_cast<float2 *>(a.out + slot * a.sstride) + xc;
     const float dt = g.dt;
     const int n = a.n;
@@ -895,17 +895,20 @@ __device__ __forceinline__ void adj_body(const Arg2D &p)
         const char *const brx = sm + L::B + (bs + NS - 1 >= NB ? bs + NS - 1 - NB : bs + NS - 1) * L::F1;
         const bool main = z >= zc0;
         const bool zf = recon && main && z > z0 && z + W < z1 && z + 1 < zc1;
-        // ---- rows z, z + 1: (p, mu) of the row itself
-        float2 pm[2];
+        // ---- rows z, z + 1: (p, mu) of the row itself (the ring's entries of rows in the z strips hold u != mu)
+        float pr[2];
+        auto own_lam = [&](int r, bool ZF) {   // zero on the free surface
+            return (!ZF && FS && z + r == z0) ? 0.f : *reinterpret_cast<const float *>(st1 + L::LAM + r * L::F1R);
+        };
         auto own_row = [&](auto zc, auto xc_) {
             constexpr bool ZF = decltype(zc)::value, XF = decltype(xc_)::value;
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
-                const int iz = z + r - z0;
-                pm[r] = (ZF || (iz >= 0 && iz < g.nz)) ? PU[r] : *reinterpret_cast<const float2 *>(st2 + L::IM + r * L::F2R);
-                float u = pm[r].y;
-                if (!XF && pmlxn) u -= aix * (*reinterpret_cast<const float *>(st1 + L::LVX + r * L::F1R) - u);
-                sPU[r * NTH + t] = make_float2(pm[r].x, u);
+                pr[r] = (!ZF && FS && z + r < z0) ? 0.f : PU[r].x;
+                float u = PU[r].y;
+                if (!ZF) u = __fmul_rn(*reinterpret_cast<const float *>(st1 + L::KD + r * L::F1R), own_lam(r, ZF));
+                if (!XF && pmlxn) u = fmaf(-aix, *reinterpret_cast<const float *>(st1 + L::LVX + r * L::F1R) - u, u);
+                sPU[r * NTH + t] = make_float2(pr[r], u);
             }
         };
         // ---- half rows k along z: lambda_vz, lambda_psi_pz, background vz^{n-1/2}
@@ -931,10 +934,10 @@ __device__ __forceinline__ void adj_body(const Arg2D &p)
                                                         [&](int l) { return PU[r + M - l]; });
                     const float lv = v2z.y + D.y;
                     const float dtbu = dt * buz;
-                    wz = dtbu * lv;
+                    wz = __fmul_rn(dtbu, lv);
                     if (!ZF && ((k <= z0 - 2) || (k >= z1))) {
-                        const float l1 = *reinterpret_cast<const float *>(st1 + L::LPZ + r * L::F1R) - dtbu * lv;
-                        wz -= a.pml.ah[0][k] * l1;
+                        const float l1 = *reinterpret_cast<const float *>(st1 + L::LPZ + r * L::F1R) - wz;
+                        wz = fmaf(-a.pml.ah[0][k], l1, wz);
                         if (own) outf[A_LPPZ * pT + ck] = a.pml.bh[0][k] * l1;
                     }
                     piz = D.x * lv;
@@ -992,10 +995,10 @@ __device__ __forceinline__ void adj_body(const Arg2D &p)
                     const float dtbu = dt * bux;
                     const float lv = v2x.y + D.y;
                     const bool own = outcol && (ZF || zr < zc1);
-                    float wx = dtbu * lv;
+                    float wx = __fmul_rn(dtbu, lv);
                     if (!XF && pmlxh) {
-                        const float l1 = *reinterpret_cast<const float *>(st1 + L::LPX + r * L::F1R) - dtbu * lv;
-                        wx -= ahx * l1;
+                        const float l1 = *reinterpret_cast<const float *>(st1 + L::LPX + r * L::F1R) - wx;
+                        wx = M == 4 && !FS ? fmaf(dtbu, lv, -__fmul_rn(ahx, l1)) : fmaf(-ahx, l1, wx);
                         if (own) outf[A_LPPX * pT + cz] = bhx * l1;
                     }
                     pix[r] = D.x * lv;
@@ -1047,11 +1050,11 @@ __device__ __forceinline__ void adj_body(const Arg2D &p)
                              stencil<M, float>(g.cz, [&](int l) { return VN[r + M + l - 1]; },
                                                [&](int l) { return VN[r + M - l]; });
                     const float kd = *reinterpret_cast<const float *>(st1 + L::KD + r * L::F1R);
-                    const float mu = pm[r].y;
+                    const float lam = own_lam(r, ZF);
                     const bool inner = XF || (xint && (ZF || (iz >= 0 && iz < g.nz)));
                     if (inner) {
                         float2 acc = *reinterpret_cast<const float2 *>(st2 + L::IM + r * L::F2R);
-                        acc.x += E.x * mu;
+                        acc.x += E.x * lam;
                         // (on the free surface the half row above is a ghost: no product of its own)
                         acc.y += (pix[r] + pil[r]) + (PIZ[r + 1] + (surf ? 0.f : PIZ[r]));
                         if (own) img[cz] = acc;
@@ -1059,7 +1062,7 @@ __device__ __forceinline__ void adj_body(const Arg2D &p)
                     float pn = 0.f;
                     if (ZF || recon) {
                         if (inner) {
-                            pn = pm[r].x + kd * qn;
+                            pn = pr[r] + kd * qn;
                             pn -= cz + x == src ? wsrc : 0.f;
                         } else if (ZF || (iz >= 0 && iz < g.nz)) {
                             if (xband) pn = band_val(0, bf, r);
@@ -1067,14 +1070,18 @@ __device__ __forceinline__ void adj_body(const Arg2D &p)
                             pn = band_get(a.bands, 0, rowprev, band_zstrip(iz, ix, M, g.nz, nx));
                         }
                     }
-                    float2 pmn = make_float2(pn, fmaf(kd, E.y, mu));
-                    if (!ZF && FS && zr <= z0) pmn = make_float2(0.f, 0.f);
-                    if (own) out2[(A_PL / 2) * pT + cz] = pmn;
+                    float ln = lam + E.y;
+                    if (!ZF && FS && zr <= z0) pn = ln = 0.f;
+                    if (own) {
+                        out2[(A_PL / 2) * pT + cz] = make_float2(pn, kd * ln);
+                        outl[cz] = ln;
+                    }
+                    const float kl = __fmul_rn(kd, lam);
                     if (!XF && own && pmlxn)
-                        outf[A_LPVX * pT + cz] = bix * (*reinterpret_cast<const float *>(st1 + L::LVX + r * L::F1R) - mu);
+                        outf[A_LPVX * pT + cz] = bix * (*reinterpret_cast<const float *>(st1 + L::LVX + r * L::F1R) - kl);
                     if (!ZF && own && ((zr <= z0 - 1) || (zr >= z1)))
                         outf[A_LPVZ * pT + cz] =
-                            a.pml.bi[0][zr] * (*reinterpret_cast<const float *>(st1 + L::LVZ + r * L::F1R) - mu);
+                            a.pml.bi[0][zr] * (*reinterpret_cast<const float *>(st1 + L::IM + r * L::F2R) - kl);
                 }
             };
             if (!zf) node_stage(std::false_type{}, std::false_type{});
@@ -1108,13 +1115,16 @@ __device__ __forceinline__ void adj_body(const Arg2D &p)
         const int tile = shot * a.trec.ntiles + blockIdx.y * gridDim.x + blockIdx.x;
         const int b = a.trec.ptr[tile], e = a.trec.ptr[tile + 1];
         float2 *plo = reinterpret_cast<float2 *>(a.out + slot * a.sstride) + (A_PL / 2) * pT;
+        float *lo = a.out + slot * a.sstride + A_L * g.plane;
         for (int i = b + t; i < e; i += NTH) {
             const int2 rc = a.trec.rec[i];
             if (i > b && a.trec.rec[i - 1].x == rc.x) continue;  // run handled by its first entry
             float add = 0.f;
             for (int q = i; q < e && a.trec.rec[q].x == rc.x; ++q)
                 add += a.dstage[(long long)a.trec.rec[q].y * g.nt + (n - 1)];
-            plo[rc.x].y += kdt[rc.x] * add;
+            const float l = lo[rc.x] + add;
+            lo[rc.x] = l;
+            plo[rc.x].y = kdt[rc.x] * l;
         }
     }
 }

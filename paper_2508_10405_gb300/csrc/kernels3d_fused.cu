@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(NTH, kMinBlocks) k3f_born(const __grid_constan
     float2 *out = reinterpret_cast<float2 *>(a.out) + slot * a.out_pairs * plane;
     float2 *psv = reinterpret_cast<float2 *>(a.psiv) + slot * a.psiv_pairs * plane;   // in place: x y z
     const int src = a.src_cell[shot];
-    const float wsrc = a.src_scale * a.wav[(a.wav_per_shot ? (long long)shot * g.nt : 0) + a.n];
+    const float wsrc = a.wav[(a.wav_per_shot ? (long long)shot * g.nt : 0) + a.n];
 
     float *tab = reinterpret_cast<float *>(sm + S::TAB);
     if (t == 0) {
@@ -462,7 +462,7 @@ __global__ void __launch_bounds__(NTH, kMinBlocks) k3f_born(const __grid_constan
                 const float2 kd = tile(S::KD)[t];
                 float2 pn = fma2(-kd.x, Q, P[u]);
                 pn.y = fmaf(-kd.y, Q.x, pn.y);
-                pn.x += c == src ? wsrc : 0.f;
+                pn.x = fmaf(a.src_scale, c == src ? wsrc : 0.f, pn.x);
                 if (!ZF && g.fs && z <= g.z0) pn = make_float2(0.f, 0.f);   // p = 0 on the free surface
                 if (XY || colok) out[F3_P * pl + c] = pn;
             };

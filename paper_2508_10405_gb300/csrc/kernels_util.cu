@@ -76,7 +76,7 @@ __global__ void k_pert_prep(GridDev g, const float *dm, const float *kdt, const 
 }
 
 __global__ void k_inject(GridDev gm, GridDev g, TileRecs tr, int shot0, const float *dstage, int n, const float *kdt,
-                         const int *win_x0, float2 *pl, long long sstride2)
+                         const int *win_x0, float2 *pl, long long sstride2, float *lam)
 {
     int slot = blockIdx.y;
     int t = (shot0 + slot) * tr.ntiles + blockIdx.x;
@@ -90,7 +90,13 @@ __global__ void k_inject(GridDev gm, GridDev g, TileRecs tr, int shot0, const fl
             add += dstage[(long long)tr.rec[k].y * g.nt + n];
         // node of the model grid (windowed shots, 2D: z and the column in the window)
         const long long c = win_x0 ? (long long)(rc.x / g.pitch) * gm.pitch + rc.x % g.pitch + win_x0[shot0 + slot] : rc.x;
-        dst[rc.x].y += kdt[c] * add;
+        if (lam) {   // lambda_p itself is part of the state (2D)
+            float *l = lam + 2 * slot * sstride2 + rc.x;
+            *l += add;
+            dst[rc.x].y = kdt[c] * *l;
+        } else {
+            dst[rc.x].y += kdt[c] * add;
+        }
     }
 }
 
@@ -159,15 +165,16 @@ __global__ void k_band_pack(Bands b, int shot0, int n)
     }
 }
 
-// g_kappa = -sum_n Q (dt kappa lp), g_rho = (dt / 2) / rho * sum_n (products at
+// g_kappa = -dt kappa sum_n Q lp, g_rho = (dt / 2) / rho * sum_n (products at
 // the adjacent half nodes); g_Vp = g_kappa - g_rho, g_Ip = g_kappa + g_rho.
-__global__ void k_image_fin(GridDev g, const double2 *acc, const float *binv, float *gout)
+// kdt null: the sums hold Q (dt kappa lp) (3D).
+__global__ void k_image_fin(GridDev g, const double2 *acc, const float *kdt, const float *binv, float *gout)
 {
     long long nint = (long long)g.nz * g.ny * g.nx;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < nint;
          k += (long long)gridDim.x * blockDim.x) {
         long long c = pad_of(g, k);
-        double gk = -acc[k].x;
+        double gk = kdt ? -(double)kdt[c] * acc[k].x : -acc[k].x;
         double gr = 0.5 * (double)g.dt * (double)binv[c] * acc[k].y;
         gout[k] = (float)(gk - gr);
         gout[nint + k] = (float)(gk + gr);
@@ -533,10 +540,10 @@ cudaError_t launch_pert_prep(const GridDev &g, const float *dm, const float *kdt
 
 cudaError_t launch_inject_residual(const GridDev &gm, const GridDev &g, const TileRecs &tr, int batch, int shot0,
                                    const float *dstage, int n, const float *kdt, const int *win_x0, float2 *pl,
-                                   long long sstride2, cudaStream_t s)
+                                   long long sstride2, float *lam, cudaStream_t s)
 {
     dim3 grid(tr.ntiles, batch);
-    k_inject<<<grid, 64, 0, s>>>(gm, g, tr, shot0, dstage, n, kdt, win_x0, pl, sstride2);
+    k_inject<<<grid, 64, 0, s>>>(gm, g, tr, shot0, dstage, n, kdt, win_x0, pl, sstride2, lam);
     return cudaGetLastError();
 }
 
@@ -554,11 +561,11 @@ cudaError_t launch_band_pack(const Bands &b, int batch, int shot0, int n, cudaSt
     return cudaGetLastError();
 }
 
-cudaError_t launch_image_finalize(const GridDev &g, const double2 *acc, const float *binv, float *gout,
+cudaError_t launch_image_finalize(const GridDev &g, const double2 *acc, const float *kdt, const float *binv, float *gout,
                                   cudaStream_t s)
 {
     long long n = (long long)g.nz * g.ny * g.nx;
-    k_image_fin<<<grid_for(n), NT, 0, s>>>(g, acc, binv, gout);
+    k_image_fin<<<grid_for(n), NT, 0, s>>>(g, acc, kdt, binv, gout);
     return cudaGetLastError();
 }
 

@@ -161,9 +161,11 @@ struct Step2D {
     int *err;             // error word of the TMA-staged kernels (1 = a wait gave up, 2 = misaligned copy refused)
 };
 
-// Planes of a 2D slot when shots have aperture windows: the 10 state planes,
+// Planes of a 2D slot when shots have aperture windows: the 12 state planes,
 // then dt kappa, 1/rho and the two Born pairs of the shot's window.
-constexpr int kWinStatePlanes2D = 16;
+constexpr int kWinStatePlanes2D = 18;
+// The plane of lambda_p in a 2D slot's adjoint state.
+constexpr int kAdjLambda2D = 10;
 
 // Arguments of the 3D background time-step kernels (state updated in place).
 struct Step3D {
@@ -353,14 +355,14 @@ cudaError_t launch_pert_prep(const GridDev &g, const float *dm, const float *kdt
 // s's slot grid g takes the columns from win_x0[s], or all with win_x0 null.
 cudaError_t launch_inject_residual(const GridDev &gm, const GridDev &g, const TileRecs &tr, int batch, int shot0,
                                    const float *dstage, int n, const float *kdt, const int *win_x0, float2 *pl,
-                                   long long sstride2, cudaStream_t s);
+                                   long long sstride2, float *lam, cudaStream_t s);
 // Stacks the batch's per-slot images (grid g) into the FP64 interior image of
 // the model grid gm; with aperture windows (win_x0 non-null) slot b covers the
 // columns [win_x0, win_x0 + win_nx) of shot shot0 + b.
 cudaError_t launch_image_accumulate(const GridDev &gm, const GridDev &g, const float2 *img, int batch, int shot0,
                                     const int *win_x0, const int *win_nx, double2 *acc, cudaStream_t s);
 // acc: (sum Q dt kappa lambda_p, sum of the adjacent half nodes' products).
-cudaError_t launch_image_finalize(const GridDev &g, const double2 *acc, const float *binv, float *gout,
+cudaError_t launch_image_finalize(const GridDev &g, const double2 *acc, const float *kdt, const float *binv, float *gout,
                                   cudaStream_t s);
 cudaError_t launch_hess_accumulate(const GridDev &gm, const GridDev &g, const float *hess, int batch, int shot0,
                                    const int *win_x0, const int *win_nx, double *acc, cudaStream_t s);
