@@ -659,7 +659,7 @@ def deblur_bench(args, rank, world, local):
                        "l2": "image 4.8 MB per input: L2-resident"},
             "roofline": {"bound": "alu", "achieved": flops / t_w / 1e12, "peak": FP32_PEAK_TFLOPS,
                          "unit": "TFLOP/s", "frac": flops / t_w / 1e12 / FP32_PEAK_TFLOPS, "traffic": None,
-                         "kernel": "k_wiener_block + k_wiener_blend", "flops_per_launch": flops,
+                         "kernel": "k_wiener_node + k_wiener_blend", "flops_per_launch": flops,
                          "peak_source": "152 SMs x 128 FP32 lanes x 2 flop x 2070 MHz"},
             "space_domain_filters": {"ms": t_s * 1e3, "kernel": "k_deblur_solve + k_deblur_apply (11 x 11, FP64 "
                                                                "normal equations)"},

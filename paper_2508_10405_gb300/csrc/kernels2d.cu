@@ -192,7 +192,7 @@ __device__ __forceinline__ bool zpml_node(const GridDev &g, int r)
 // a row's was waited for 600 to 1000 cycles); interior rows and warps run
 // straight-line code, and what the strips need in the last stage comes with
 // the copies (their warps took twice the others' time and set the CTA's pace).
-// 96 shots of 424 x 1192 padded cells, order 8: 80.9 G cell-updates/s = 0.77
+// 96 shots of 424 x 1192 padded cells, order 8: 82.0 G cell-updates/s = 0.78
 // of the measured copy rate (a row at a time, one issuing thread: 67.6); the
 // background step with recording, 48 shots: 110.7 G (with per-thread copies:
 // 70.8). Windowed shots: with k_adj2d 1.27x over per-thread copies.
@@ -630,16 +630,17 @@ __global__ void __launch_bounds__(NTH, (BANDS || HESS) ? kBandsMinBlocks : kPlai
 // D+ stencils take, and as lambda_p in a plane of its own, what the images and
 // the update take. Away from the z strips the ring's entry of a row then is
 // the row's own (p, mu): a row needs neither dt kappa of its look-ahead row nor
-// a second copy of the pairs. (With mu alone, 72 B a cell: 55.2 G; but
-// lambda_p then is rounded as mu, and the 64-bit misfits of a CG move by 1e-8.) Which products of the CPML terms are fused into the
-// subtractions, and in the forward step the source's, is written out for the
-// same reason: left to the compiler, it changes with the code around them.
+// a second copy of the pairs. (With mu alone, 72 B a cell: 55.2 G, and
+// lambda_p is rounded as mu, which moves the 64-bit misfits of a CG by 1e-8.)
+// Which products of the CPML terms are fused into the subtractions, and in the
+// forward step the source's, is written out for the same reason: left to the
+// compiler, it changes with the code around them.
 //
-// What bounds it: 80 B a cell, held back like the Born step;
-// 3 tile copies a row where a row at a time took 9. The x strips' band values
+// What bounds it: 80 B a cell, held back like the Born step; 3 tile copies a
+// row where a row at a time took 9. The x strips' band values
 // come one group ahead by asynchronous copies (read where they are used, they
 // doubled the strip warps' time). 96 shots of 424 x 1192, order 8, FP16 bands:
-// 53.7 G cell-updates/s = 0.64 of the measured copy rate (a row at a time with
+// 56.0 G cell-updates/s = 0.67 of the measured copy rate (a row at a time with
 // one issuing thread: 42.4; in groups without the straight-line form: 31.5).
 // ---------------------------------------------------------------------------
 struct AdjLay {
