@@ -185,7 +185,7 @@ __device__ __forceinline__ bool zpml_node(const GridDev &g, int r)
 // background alone as float, with BANDS saving the boundary bands of p^n and
 // v^{n+1/2} and HESS accumulating the pseudo-Hessian diagonal of App. B.
 //
-// What bounds it: the Born step moves 64 B a cell, 57.9 from DRAM (the shots
+// What bounds it: the Born step moves 64 B a cell, 63.1 from DRAM (the shots
 // of a batch share the model), and is held back by latencies between its
 // barriers (54% of the issue slots used). A group of two rows halves the
 // barriers; every warp issues one field's copy (one thread that issued all of
@@ -636,7 +636,7 @@ __global__ void __launch_bounds__(NTH, (BANDS || HESS) ? kBandsMinBlocks : kPlai
 // forward step the source's, is written out for the same reason: left to the
 // compiler, it changes with the code around them.
 //
-// What bounds it: 80 B a cell, held back like the Born step; 3 tile copies a
+// What bounds it: 80 B a cell (81.7 from DRAM), held back like the Born step; 3 tile copies a
 // row where a row at a time took 9. The x strips' band values
 // come one group ahead by asynchronous copies (read where they are used, they
 // doubled the strip warps' time). 96 shots of 424 x 1192, order 8, FP16 bands:
