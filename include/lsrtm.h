@@ -249,7 +249,9 @@ lsrtm_status lsrtm_timing_read(lsrtm_handle *h, lsrtm_timings *out, int reset);
  * call on a device looks up the array's device address and configures the
  * kernels; make it before any stream capture. Inputs are not checked for
  * finiteness (a non-finite model gives non-finite records, not an error).
- * Returns once the work is queued. */
+ * Returns once the work is queued; if a time-step kernel then gives up waiting
+ * for its tile copies (the error lsrtm_synchronize reports for a handle), every
+ * record of the call is NaN. */
 lsrtm_status lsrtm_born_static(const lsrtm_config *cfg, const float *vp, const float *rho,
                                const float *wavelet, const lsrtm_geometry *geom, const float *dm,
                                float *d, void *stream);

@@ -13,7 +13,9 @@
 // afterwards); the call allocates nothing on the device (no cudaMalloc, no
 // cudaFree, no allocating library routine). Inputs are not checked for
 // finiteness: a NaN or Inf in the model gives non-finite records rather than
-// an error status.
+// an error status. The call returns before its kernels run, so a time-step
+// kernel that gives up waiting for its tile copies cannot be reported by the
+// status either: the call's last kernel then makes every record NaN.
 //
 // Shared-state rules:
 //   * the array is shared by every call on a device and keeps the contents of
@@ -152,12 +154,29 @@ __global__ void k_geom_static(GridDev g, int nshot, int txo, int tzc, int ntx, i
         }
 }
 
+// The last kernel of a call: records of a call whose error word is set are
+// incomplete, and none of them is kept.
+__global__ void k_report_static(const int *err, float *d, long long n)
+{
+    if (*err == 0) return;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        d[i] = __int_as_float(0x7fffffff);
+}
+
+// Error word the next call of this host thread starts with (tests only).
+thread_local int t_test_error = 0;
+
 size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
 }  // namespace
 }  // namespace lsrtm
 
 using namespace lsrtm;
+
+// Not in the header; for tests of the error report. The next lsrtm_born_static
+// of this host thread starts with its error word at `code` (0 .. 127), as if
+// a kernel's wait had given up.
+extern "C" void lsrtm_test_static_error(int code) { t_test_error = code; }
 
 extern "C" lsrtm_status lsrtm_born_static(const lsrtm_config *cfg, const float *vp, const float *rho,
                                           const float *wavelet, const lsrtm_geometry *geom, const float *dm,
@@ -360,6 +379,8 @@ extern "C" lsrtm_status lsrtm_born_static(const lsrtm_config *cfg, const float *
     // the kernels' error word takes the first tile cursor's place once the tables are built
     a.err = tcur;
     SCU(cudaMemsetAsync(a.err, 0, sizeof(int), s));
+    if (t_test_error) SCU(cudaMemsetAsync(a.err, t_test_error, 1, s));
+    t_test_error = 0;
     Maps2D maps[2];
     SCU(maps2d(&maps[0], g, g, st0, a.sstride, kdt, binv, kd2, br2, nullptr, psiv, a.vstride, 1));
     SCU(maps2d(&maps[1], g, g, st1, a.sstride, kdt, binv, kd2, br2, nullptr, psiv, a.vstride, 1));
@@ -375,6 +396,8 @@ extern "C" lsrtm_status lsrtm_born_static(const lsrtm_config *cfg, const float *
             SCU(launch_fwd2d(a, maps[n & 1], 1, true, false, false, s));
         }
     }
+    k_report_static<<<152, 256, 0, s>>>(a.err, d, nrec * g.nt);
+    SCU(cudaGetLastError());
 #undef SCU
     return LSRTM_OK;
 }
