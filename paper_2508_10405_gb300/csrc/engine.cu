@@ -2275,37 +2275,40 @@ lsrtm_status lsrtm_autotune(lsrtm_handle *h, int steps, int *tzc_out, double *ms
         if ((st = gather_model(h, 0, bs, true)) != LSRTM_OK) break;
         Step2D a = step_args(h, 0);
         double ms = 0.0;
+        auto step = [&](int i) -> lsrtm_status {
+            if (d3) {
+                Step3F &b = h->f3born[i & 1];
+                b.n = i;
+                b.shot0 = 0;
+                b.trec = h->trv;
+                b.tzc = c;
+                CU(launch_born3f(b, bs, h->work));
+                return adj3f_step(h, i, steps - i, 0, h->bands);
+            }
+            a.n = i;
+            a.in = h->st[i & 1];
+            a.out = h->st[(i + 1) & 1];
+            CU(launch_fwd2d(a, h->m2d[i & 1], bs, true, false, false, h->work));
+            a.n = steps - i;
+            CU(launch_adj2d(a, h->m2d[i & 1], bs, h->work));
+            return LSRTM_OK;
+        };
         for (int rep = 0; rep < 2 && st == LSRTM_OK; ++rep) {   // first pass warms up
             cudaEventRecord(e0, h->work);
-            for (int i = 0; i < steps; ++i) {
-                if (d3) {
-                    Step3F &b = h->f3born[i & 1];
-                    b.n = i;
-                    b.shot0 = 0;
-                    b.trec = h->trv;
-                    b.tzc = c;
-                    launch_born3f(b, bs, h->work);
-                    adj3f_step(h, i, steps - i, 0, h->bands);
-                    continue;
-                }
-                a.n = i;
-                a.in = h->st[i & 1];
-                a.out = h->st[(i + 1) & 1];
-                launch_fwd2d(a, h->m2d[i & 1], bs, true, false, false, h->work);
-                a.n = steps - i;
-                launch_adj2d(a, h->m2d[i & 1], bs, h->work);
-            }
+            for (int i = 0; i < steps && st == LSRTM_OK; ++i) st = step(i);
             cudaEventRecord(e1, h->work);
             cudaError_t e = cudaEventSynchronize(e1);
             if (e == cudaSuccess) e = cudaGetLastError();
-            if (e != cudaSuccess) st = fail(LSRTM_ERR_CUDA, std::string("autotune: ") + cudaGetErrorString(e));
+            if (e != cudaSuccess && st == LSRTM_OK)
+                st = fail(LSRTM_ERR_CUDA, std::string("autotune: ") + cudaGetErrorString(e));
             float f = 0.f;
             cudaEventElapsedTime(&f, e0, e1);
             ms = f / steps;
         }
         h->launches += 4LL * steps;
         times.push_back(ms);
-        if (d3 && st == LSRTM_OK) st = check_kernel_error(h);   // a fused kernel's wait that gave up
+        // steps a kernel gave up or the guard skipped are no timing
+        if (st == LSRTM_OK) st = check_kernel_error(h);
         if (st != LSRTM_OK) break;
         if (ms < best) {
             best = ms;
