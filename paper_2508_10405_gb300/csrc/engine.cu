@@ -47,14 +47,12 @@ lsrtm_status fail(lsrtm_status st, const std::string &msg)
         if (s_ != LSRTM_OK) return s_;         \
     } while (0)
 
-// Planes per wavefield slot: 12 ping-pong planes (Born, 10 of them: (p, dp)
-// (vx, dvx) (vz, dvz) (psi_px, dpsi_px) (psi_pz, dpsi_pz) as float2 pairs;
-// background only: p vx vz psi_px psi_pz; adjoint: (p, dt kappa lambda_p)
-// (vx, lambda_vx) (vz, lambda_vz) pairs, four lambda CPML memories and
-// lambda_p; one unused, pairs go by twos), 4 in-place node CPML planes
-// (forward).
-constexpr int kStatePlanes2D = 12;
-constexpr int kPsivPlanes2D = 4;
+// A 2D wavefield slot has kStatePlanes2D planes in each of two buffers: 10 ping-pong planes
+// (Born: (p, dp) (vx, dvx) (vz, dvz) (psi_px, dpsi_px) (psi_pz, dpsi_pz) as
+// float2 pairs; background only: p vx vz psi_px psi_pz; adjoint: (p, dt kappa
+// lambda_p) (vx, lambda_vx) (vz, lambda_vz) pairs and four lambda CPML
+// memories), then two that hold the in-place node CPML memories of forward
+// passes or the adjoint's lambda_p (kExtra2D).
 constexpr int kStatePlanes3D = 20;
 
 enum GraphKind { G_BORN = 0, G_BG = 1, G_BG_HESS = 2, G_ADJ = 3, G_MODEL = 6 };
@@ -102,7 +100,7 @@ struct lsrtm_handle {
     int batch = 1;
     float *st[2] = {nullptr, nullptr};
     long long sstride = 0;
-    long long sstride1 = 0;      // slot stride of st[1] (3D: the fused kernels' pong buffer)
+    long long sstride1 = 0;      // slot stride of st[1] (3D: the fused kernels' pong buffer; 2D: sstride)
     Step3F f3born[2];            // fused 3D Born step arguments reading st[0] / st[1]
     Adj3F f3adj[2];              // fused 3D adjoint step arguments reading st[0] / st[1]
     Maps2D m2d[2];               // 2D TMA row maps reading st[0] / st[1]
@@ -113,8 +111,6 @@ struct lsrtm_handle {
     std::map<std::pair<int, int>, long long> graph_guards;   // guard launches per captured graph
     int *poll_h = nullptr;       // pinned host copies of the error words, two per CG poll slot
     cudaEvent_t poll_ev[2] = {nullptr, nullptr};
-    float *psiv = nullptr;
-    long long vstride = 0;
     float2 *img = nullptr;
     double2 *img_acc = nullptr;
     float *hess = nullptr;
@@ -316,9 +312,8 @@ Step2D step_args(lsrtm_handle *h, int shot0)
     a.binv = h->binv;
     a.kd2 = h->kd2;
     a.br2 = h->br2;
-    a.psiv = h->psiv;
-    a.sstride = h->sstride;
-    a.vstride = h->vstride;
+    a.psiv = h->st[0] + kExtra2D * h->g.plane;
+    a.sstride = a.vstride = h->sstride;
     a.shot0 = shot0;
     a.wav = h->wav;
     a.wav_per_shot = h->cfg.wavelet_per_shot;
@@ -508,8 +503,7 @@ long long slot_stride(const lsrtm_handle *h, int j) { return j ? h->sstride1 : h
 lsrtm_status zero_slots(lsrtm_handle *h, int bs)
 {
     CU(cudaMemsetAsync(h->st[0], 0, (size_t)bs * h->sstride * sizeof(float), h->work));
-    if (h->st[1]) CU(cudaMemsetAsync(h->st[1], 0, (size_t)bs * h->sstride1 * sizeof(float), h->work));
-    if (h->psiv) CU(cudaMemsetAsync(h->psiv, 0, (size_t)bs * h->vstride * sizeof(float), h->work));
+    if (is3d(h)) CU(cudaMemsetAsync(h->st[1], 0, (size_t)bs * h->sstride1 * sizeof(float), h->work));
     if (h->bands.stage)
         CU(cudaMemsetAsync(h->bands.stage, 0, (size_t)bs * 2 * h->bands.nb * sizeof(float), h->work));
     return LSRTM_OK;
@@ -753,7 +747,7 @@ lsrtm_status ck_forward(lsrtm_handle *h, int s0, int bs, bool hess)
                 a.out = h->st[(n + 1) & 1];
                 if (n % K == 0) {
                     CHECK(ck_copy(h, n / K, h->st[n & 1], h->sstride, 5, 0, bs, true));
-                    CHECK(ck_copy(h, n / K, h->psiv, h->vstride, 2, 5, bs, true));
+                    CHECK(ck_copy(h, n / K, h->st[0] + kExtra2D * plane, h->sstride, 2, 5, bs, true));
                 }
                 CU(launch_fwd2d(a, h->m2d[n & 1], bs, false, false, hess, h->work));
                 CHECK(guard_step(h, GK_BACKGROUND, n, n, a.out, h->sstride, 1, bs));
@@ -895,7 +889,7 @@ lsrtm_status adjoint_core_ckpt(lsrtm_handle *h, float *gout, bool want_hess)
             CU(launch_pack_adjoint(h->g, h->final_state, 0, bs, h->st[0], h->sstride, h->work));
             CU(launch_inject_residual(h->gm, h->g, h->trv, bs, s0, h->dstage, nt - 1, h->kdt,
                                       h->win ? h->win_x0_d : nullptr, reinterpret_cast<float2 *>(h->st[0]),
-                                      h->sstride / 2, h->st[0] + kAdjLambda2D * plane, h->work));
+                                      h->sstride / 2, h->st[0] + kExtra2D * plane, h->work));
             h->launches += 2;
         }
         for (int j = h->ck_nseg - 1; j >= 0; --j) {
@@ -948,7 +942,7 @@ lsrtm_status adjoint_core(lsrtm_handle *h, float *gout, bool want_hess)
             CU(launch_pack_adjoint(h->g, h->final_state, s0, bs, h->st[0], h->sstride, h->work));
             CU(launch_inject_residual(h->gm, h->g, h->trv, bs, s0, h->dstage, nt - 1, h->kdt,
                                       h->win ? h->win_x0_d : nullptr, reinterpret_cast<float2 *>(h->st[0]),
-                                      h->sstride / 2, h->st[0] + kAdjLambda2D * plane, h->work));
+                                      h->sstride / 2, h->st[0] + kExtra2D * plane, h->work));
             h->launches += 2;
             CHECK(run_loop(h, G_ADJ, s0, bs, [&]() -> lsrtm_status {
                 CHECK(gather_model(h, s0, bs, false));
@@ -1481,19 +1475,19 @@ lsrtm_status create_impl(const lsrtm_config *cfg, const float *vp, const float *
     h->fs_planes = d3 ? 4 : 3;
 
     // wavefield slots
-    // 2D: ping-pong state + in-place node CPML planes + image plane; 3D: one in-place state
+    // 2D: two state buffers, one after the other, + image and pseudo-Hessian planes; 3D: one in-place state
     // of 20 planes (pairs, CPML memories, images) + the pseudo-Hessian plane
-    h->sstride = (d3 ? kStatePlanes3D : (h->win ? kWinStatePlanes2D : kStatePlanes2D)) * g.plane;
-    h->vstride = d3 ? 0 : kPsivPlanes2D * g.plane;
+    const long long buf = (d3 ? kStatePlanes3D : (h->win ? kWinStatePlanes2D : kStatePlanes2D)) * g.plane;
+    h->sstride = d3 ? buf : 2 * buf;
     // 3D: st[0] (20 planes; the fused kernels use its first 14 as ping and the
     // last 6 as the in-place node CPML memories), st[1] (14 planes, pong), the
     // float2 image plane and the pseudo-Hessian plane
     h->sstride1 = d3 ? 2LL * kBornPairs3F * g.plane : h->sstride;
-    // the time-step kernels index within a slot with 32-bit offsets (2D: but for the planes of lambda_p)
-    if (h->sstride - (d3 ? 0 : 2 * (long long)g.plane) >= (1LL << 31))
+    // the time-step kernels index within a slot with 32-bit offsets (2D: but for the last two planes)
+    if (buf - (d3 ? 0 : 2 * (long long)g.plane) >= (1LL << 31))
         return fail(LSRTM_ERR_ARG, "grid too large: a wavefield slot exceeds 2^31 floats");
     size_t per_slot = d3 ? ((size_t)h->sstride + h->sstride1 + 3 * g.plane) * sizeof(float)
-                         : (2 * (size_t)h->sstride + h->vstride + 2 * g.plane + g.plane) * sizeof(float);
+                         : ((size_t)h->sstride + 2 * g.plane + g.plane) * sizeof(float);
     if (h->bands.fmt != BAND_F32) per_slot += 2 * (size_t)h->bands.nb * sizeof(float);   // FP32 band stage
     int batch = cfg->plan == LSRTM_PLAN_PLAIN ? 1 : (cfg->shots_per_batch > 0 ? cfg->shots_per_batch : h->nshot);
     batch = std::min(batch, h->nshot);
@@ -1584,8 +1578,8 @@ lsrtm_status create_impl(const lsrtm_config *cfg, const float *vp, const float *
         h->segbands.stage = h->bands.stage;
     }
     CHECK(dalloc_t(h, &h->st[0], (size_t)batch * h->sstride));
-    CHECK(dalloc_t(h, &h->st[1], (size_t)batch * h->sstride1));
-    if (!d3) CHECK(dalloc_t(h, &h->psiv, (size_t)batch * h->vstride));
+    if (d3) CHECK(dalloc_t(h, &h->st[1], (size_t)batch * h->sstride1));
+    else h->st[1] = h->st[0] + buf;
     CHECK(dalloc_t(h, &h->img, (size_t)batch * g.plane));
     CHECK(dalloc_t(h, &h->hess, (size_t)batch * g.plane));
     CHECK(dalloc_t(h, &h->kerr, 4));
@@ -1596,10 +1590,10 @@ lsrtm_status create_impl(const lsrtm_config *cfg, const float *vp, const float *
     if (d3) CHECK(setup_fused3d(h));
     else {
         for (int b = 0; b < 2; ++b) {
-            cudaError_t e = maps2d(&h->m2d[b], h->gm, h->g, h->st[b], h->sstride, h->kdt, h->binv, h->kd2, h->br2, h->img,
-                                   h->psiv, h->vstride, batch);
+            cudaError_t e = maps2d(&h->m2d[b], h->gm, h->g, h->st[b], h->sstride, (int)(buf / g.plane), h->kdt, h->binv,
+                                   h->kd2, h->br2, h->img, h->st[0] + kExtra2D * g.plane, h->sstride, batch);
             if (e == cudaSuccess && ckpt)
-                e = maps2d(&h->m2rec[b], h->gm, h->g, h->rec[b], 5 * g.plane, h->kdt, h->binv, h->kd2, h->br2, nullptr,
+                e = maps2d(&h->m2rec[b], h->gm, h->g, h->rec[b], 5 * g.plane, 5, h->kdt, h->binv, h->kd2, h->br2, nullptr,
                            h->rec_psiv, 2 * g.plane, batch);
             if (e != cudaSuccess) return fail(LSRTM_ERR_CUDA, std::string("tensor maps: ") + cudaGetErrorString(e));
         }

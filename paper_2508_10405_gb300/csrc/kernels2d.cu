@@ -48,17 +48,16 @@ constexpr int kAdjMinBlocks = 3;
 // State layouts, as offsets in float planes within a shot slot.
 // Born: float2 pairs (background, scattered).
 enum { B_P = 0, B_VX = 2, B_VZ = 4, B_PPX = 6, B_PPZ = 8 };
-enum { B_PVX = 0, B_PVZ = 2 };                 // in-place node CPML memories
 // Background only (band saving, pseudo-Hessian): float.
 enum { G_P = 0, G_VX = 1, G_VZ = 2, G_PPX = 3, G_PPZ = 4 };
-enum { G_PVX = 0, G_PVZ = 1 };
 // Adjoint: float2 pairs (p, dt kappa lambda_p), (v, lambda_v), float lambda
-// CPML memories and lambda_p.
+// CPML memories and lambda_p (a plane that holds forward passes' node CPML
+// memories).
 enum { A_PL = 0, A_VX = 2, A_VZ = 4, A_LPPX = 6, A_LPPZ = 7, A_LPVX = 8, A_LPVZ = 9, A_L = 10 };
 // Slots of aperture-windowed shots carry the window's own model after the
 // state: dt kappa and 1/rho (float planes), and the Born pairs (float2).
 enum { W_KDT = 12, W_BINV = 13, W_KD2 = 14, W_BR2 = 16 };
-static_assert(W_BR2 + 2 == kWinStatePlanes2D && A_L == kAdjLambda2D, "slot layout");
+static_assert(W_BR2 + 2 == kWinStatePlanes2D && A_L == kExtra2D, "slot layout");
 
 // ---- packed arithmetic for T = float or float2
 __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
@@ -262,7 +261,7 @@ __device__ __forceinline__ void fwd_issue(const Arg2D &p, int warp, char *st, ch
         if (pz) {
             if (tma::elect_one()) tma::load3(st + L::PZ, ms[1], xs, k, q + (BORN ? B_PPZ / 2 : G_PPZ), b);
         } else if (main && tpn) {   // node CPML memories along x, in the unused place of psi_pz
-            if (tma::elect_one()) tma::load3(st + L::PZ, m.pv[BORN], xs, z, slot * (BORN ? m.pvs / 2 : m.pvs) + (BORN ? B_PVX / 2 : G_PVX), b);
+            if (tma::elect_one()) tma::load3(st + L::PZ, m.pv[BORN], xs, z, slot, b);
         }
     } else {
         if (tma::elect_one())
@@ -307,7 +306,7 @@ __device__ __forceinline__ void fwd_body(const Arg2D &p)
     const int xc = colok ? x : 0;
     const float *in = a.in + slot * a.sstride;
     T *out = reinterpret_cast<T *>(a.out + slot * a.sstride) + xc;
-    T *psiv = reinterpret_cast<T *>(a.psiv + slot * a.vstride) + xc;
+    T *psiv = reinterpret_cast<T *>(a.psiv + slot * a.vstride) + xc;   // along x; along z oPVZ planes further
     const float dt = g.dt;
     const int x0 = g.x0, x1 = g.x0 + nx, z0 = g.z0, z1 = g.z0 + g.nz;
     const int ix = x - x0;
@@ -327,7 +326,7 @@ __device__ __forceinline__ void fwd_body(const Arg2D &p)
     const float wsrc = a.wav[(a.wav_per_shot ? (long long)shot * g.nt : 0) + a.n];
     constexpr int oP = BORN ? B_P / 2 : G_P, oVX = BORN ? B_VX / 2 : G_VX, oVZ = BORN ? B_VZ / 2 : G_VZ;
     constexpr int oPPX = BORN ? B_PPX / 2 : G_PPX, oPPZ = BORN ? B_PPZ / 2 : G_PPZ;
-    constexpr int oPVX = BORN ? B_PVX / 2 : G_PVX, oPVZ = BORN ? B_PVZ / 2 : G_PVZ;
+    constexpr int oPVZ = BORN ? (WIN ? kWinStatePlanes2D : kStatePlanes2D) / 2 : 1;
     const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);   // (known to be uniform)
 
     if (t == 0) {
@@ -394,8 +393,8 @@ __device__ __forceinline__ void fwd_body(const Arg2D &p)
                 // the node CPML memories of this group, read in its last stage
                 const int zn = min(z + 1, zc1 - 1);
                 if (pmlxn) {
-                    prefetch_l1(psiv + oPVX * pT + z * pitch);
-                    prefetch_l1(psiv + oPVX * pT + zn * pitch);
+                    prefetch_l1(psiv + z * pitch);
+                    prefetch_l1(psiv + zn * pitch);
                 }
                 if (z <= z0 - 1 || zn >= z1) {
                     prefetch_l1(psiv + oPVZ * pT + z * pitch);
@@ -519,9 +518,9 @@ __device__ __forceinline__ void fwd_body(const Arg2D &p)
                                          [&](int l) { return VZ[u + r + M - l]; });
                     const bool own = outcol && (ZF || zr < zc1);
                     if (!XF && own && pmlxn) {
-                        const T pv = ZF ? *reinterpret_cast<const T *>(stt + L::PZ + r * L::FR) : psiv[oPVX * pT + cz];
+                        const T pv = ZF ? *reinterpret_cast<const T *>(stt + L::PZ + r * L::FR) : psiv[cz];
                         const T ps = fma_(bix, pv, mul_(aix, qx));
-                        psiv[oPVX * pT + cz] = ps;
+                        psiv[cz] = ps;
                         qx = add_(qx, ps);
                     }
                     if (!ZF && own && ((zr <= z0 - 1) || (zr >= z1))) {
@@ -1359,9 +1358,9 @@ cudaError_t launch_adj2d(const Step2D &a, const Maps2D &maps, int batch, cudaStr
     return launch_adj_M<4>(p, batch, s);
 }
 
-cudaError_t maps2d(Maps2D *m, const GridDev &gm, const GridDev &g, const float *st, long long sstride, const float *kdt,
-                   const float *binv, const float2 *kd2, const float2 *br2, const float2 *img, const float *psiv,
-                   long long vstride, int batch)
+cudaError_t maps2d(Maps2D *m, const GridDev &gm, const GridDev &g, const float *st, long long sstride, int planes,
+                   const float *kdt, const float *binv, const float2 *kd2, const float2 *br2, const float2 *img,
+                   const float *psiv, long long vstride, int batch)
 {
     // the two model arrays of each kind are one map: their planes must be adjacent
     if (binv != kdt + gm.plane || br2 != kd2 + gm.plane) return cudaErrorInvalidValue;
@@ -1369,12 +1368,12 @@ cudaError_t maps2d(Maps2D *m, const GridDev &gm, const GridDev &g, const float *
     // state, is never read)
     m->pps = (int)(sstride / (2 * g.plane));
     m->fps = (int)(sstride / g.plane);
-    m->pvs = (int)(vstride / g.plane);
     const auto u64 = CU_TENSOR_MAP_DATA_TYPE_UINT64, f32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     const cuuint64_t s8[2] = {(cuuint64_t)g.pitch * 8, (cuuint64_t)g.plane * 8};
     const cuuint64_t s4[2] = {(cuuint64_t)g.pitch * 4, (cuuint64_t)g.plane * 4};
     const cuuint64_t nx = (cuuint64_t)g.Nx, nz = (cuuint64_t)g.Nz;
-    const cuuint64_t dpr[3] = {nx, nz, (cuuint64_t)batch * m->pps}, dfl[3] = {nx, nz, (cuuint64_t)batch * m->fps};
+    const cuuint64_t dpr[3] = {nx, nz, (cuuint64_t)((batch - 1LL) * m->pps + planes / 2)};
+    const cuuint64_t dfl[3] = {nx, nz, (cuuint64_t)((batch - 1LL) * m->fps + planes)};
     const cuuint64_t dim[3] = {nx, nz, (cuuint64_t)batch};
     // the model grid (without aperture windows the slots' own grid)
     const cuuint64_t dmd[3] = {(cuuint64_t)gm.Nx, (cuuint64_t)gm.Nz, 2};
@@ -1388,9 +1387,9 @@ cudaError_t maps2d(Maps2D *m, const GridDev &gm, const GridDev &g, const float *
         if ((e = encode_tmap(&m->md[r], f32, 3, kdt, dmd, m4, box)) != cudaSuccess) return e;
         if ((e = encode_tmap(&m->mb[r], u64, 3, kd2, dmd, m8, box)) != cudaSuccess) return e;
         // two-row boxes over its floats and its pairs
-        const cuuint64_t dpv[3] = {nx, nz, (cuuint64_t)batch * (r ? m->pvs / 2 : m->pvs)};
+        const cuuint64_t spv[2] = {(cuuint64_t)g.pitch * (r ? 8 : 4), (cuuint64_t)vstride * 4};
         const cuuint32_t box2[3] = {(cuuint32_t)NTH, 2, 1};
-        if ((e = encode_tmap(&m->pv[r], r ? u64 : f32, 3, psiv, dpv, r ? s8 : s4, box2)) != cudaSuccess) return e;
+        if ((e = encode_tmap(&m->pv[r], r ? u64 : f32, 3, psiv, dim, spv, box2)) != cudaSuccess) return e;
         if (img && (e = encode_tmap(&m->im[r], u64, 3, img, dim, s8, box)) != cudaSuccess) return e;
     }
     return cudaSuccess;

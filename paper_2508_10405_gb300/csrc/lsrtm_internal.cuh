@@ -137,7 +137,8 @@ struct Step2D {
     const float2 *br2;    // (1/rho, dln rho / rho)        [plane] (Born only)
     const float *in;      // ping state, shot slot s at in + s*sstride
     float *out;           // pong state
-    float *psiv;          // in-place node CPML memories, slot stride vstride
+    float *psiv;          // in-place node CPML memories along x, slot stride vstride; those along z a buffer's
+                          // planes further (Born), or one plane (background)
     long long sstride, vstride;
     int n;                // time step
     int tzc;              // rows of the z-chunk each CTA marches through
@@ -161,11 +162,15 @@ struct Step2D {
     int *err;             // error word of the TMA-staged kernels (1 = a wait gave up, 2 = misaligned copy refused)
 };
 
-// Planes of a 2D slot when shots have aperture windows: the 12 state planes,
-// then dt kappa, 1/rho and the two Born pairs of the shot's window.
-constexpr int kWinStatePlanes2D = 18;
-// The plane of lambda_p in a 2D slot's adjoint state.
-constexpr int kAdjLambda2D = 10;
+// Planes of each of a 2D slot's two buffers; with aperture windows the state's,
+// then dt kappa, 1/rho and the two Born pairs of the shot's window. The two
+// buffers of a slot lie one after the other.
+constexpr int kStatePlanes2D = 12, kWinStatePlanes2D = 18;
+// The last two state planes of a 2D slot, in the two ping-pong buffers: the
+// forward passes' in-place node CPML memories (Born: the x pair in buffer 0,
+// the z pair in buffer 1; background: both in buffer 0), migration's lambda_p
+// (the first of them, ping-pong).
+constexpr int kExtra2D = 10;
 
 // Arguments of the 3D background time-step kernels (state updated in place).
 struct Step3D {
@@ -278,24 +283,24 @@ int march2d_txo(int M);
 int march2d_rows(int M, int Nz, long long ctas);
 
 // Launchers (kernels2d.cu). Return the cudaError of the launch.
-// TMA row maps of the 2D kernels reading one state buffer, [0] with boxes of
-// one and [1] of two kThreads2D-wide rows of one field: pr over the float2
-// pair planes of every slot (8-byte elements; coordinates x, z, slot * pps +
-// pair), fl over its float planes (x, z, slot * fps + plane), md over dt kappa
-// and 1/rho (x, z, 0 | 1), mb over the Born model pairs (dt kappa, dt kappa
-// dlnk), (1/rho, rr) (x, z, 0 | 1), im over the image accumulators (x, z,
-// slot). pv: two-row boxes over the in-place node CPML memories (pvs planes a
-// slot) as floats [0] (x, z, slot * pvs + plane) and float2 pairs [1].
+// TMA row maps of the 2D kernels reading one state buffer (`planes` float
+// planes of every slot, sstride floats apart), [0] with boxes of one and [1]
+// of two kThreads2D-wide rows of one field: pr over the float2 pair planes of
+// every slot (8-byte elements; coordinates x, z, slot * pps + pair), fl over
+// its float planes (x, z, slot * fps + plane), md over dt kappa and 1/rho (x,
+// z, 0 | 1), mb over the Born model pairs (dt kappa, dt kappa dlnk), (1/rho, rr) (x, z, 0 | 1), im over the image accumulators (x, z,
+// slot). pv: two-row boxes over the in-place node CPML memories along x (x, z,
+// slot) as floats [0] and float2 pairs [1].
 // Outside the padded grid the copies read zeros. gm is the model's grid,
 // g the slots' (the same without aperture windows); img may be null where no
 // migration step uses the maps.
 struct Maps2D {
     CUtensorMap pr[2], fl[2], md[2], mb[2], im[2], pv[2];
-    int pps, fps, pvs;
+    int pps, fps;
 };
-cudaError_t maps2d(Maps2D *m, const GridDev &gm, const GridDev &g, const float *st, long long sstride, const float *kdt,
-                   const float *binv, const float2 *kd2, const float2 *br2, const float2 *img, const float *psiv,
-                   long long vstride, int batch);
+cudaError_t maps2d(Maps2D *m, const GridDev &gm, const GridDev &g, const float *st, long long sstride, int planes,
+                   const float *kdt, const float *binv, const float2 *kd2, const float2 *br2, const float2 *img,
+                   const float *psiv, long long vstride, int batch);
 cudaError_t launch_fwd2d(const Step2D &a, const Maps2D &maps, int batch, bool born, bool save_bands, bool hess,
                          cudaStream_t s);
 cudaError_t launch_adj2d(const Step2D &a, const Maps2D &maps, int batch, cudaStream_t s);

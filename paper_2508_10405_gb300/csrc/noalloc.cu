@@ -270,9 +270,7 @@ extern "C" lsrtm_status lsrtm_born_static(const lsrtm_config *cfg, const float *
     sz[7] = (size_t)(nrec > 0 ? nrec : 1) * 4;   // rec_idx copy
     sz[8] = (size_t)nshot * 4;              // src_cell
     sz[11] = (size_t)(nrec > 0 ? nrec : 1) * 8;  // tile receivers
-    sz[12] = 10 * P * 4;                    // wavefield ping
-    sz[13] = 10 * P * 4;                    // wavefield pong
-    sz[14] = 4 * P * 4;                     // node CPML memories
+    sz[12] = 2 * kStatePlanes2D * P * 4;    // wavefield ping and pong, node CPML memories
     size_t total = 0;
     for (int fewer = 0; fewer < 2; ++fewer) {
         if (fewer) tzc = (g.Nz + nfew - 1) / nfew;
@@ -280,7 +278,7 @@ extern "C" lsrtm_status lsrtm_born_static(const lsrtm_config *cfg, const float *
         sz[9] = ((size_t)nshot * ntiles + 1) * 4;    // tile receiver offsets
         sz[10] = (size_t)nshot * ntiles * 4;    // tile cursors
         total = 0;
-        for (int i = 0; i < 15; ++i) {
+        for (int i = 0; i < 13; ++i) {
             off[i] = total;
             total += align256(sz[i]);
         }
@@ -319,8 +317,7 @@ extern "C" lsrtm_status lsrtm_born_static(const lsrtm_config *cfg, const float *
     int *tcur = reinterpret_cast<int *>(at(10));
     int2 *trec = reinterpret_cast<int2 *>(at(11));
     float *st0 = reinterpret_cast<float *>(at(12));
-    float *st1 = reinterpret_cast<float *>(at(13));
-    float *psiv = reinterpret_cast<float *>(at(14));
+    float *st1 = st0 + kStatePlanes2D * P;
 
     // model, perturbation and profiles
     SCU(cudaMemsetAsync(kdt, 0, sz[0], s));
@@ -364,9 +361,8 @@ extern "C" lsrtm_status lsrtm_born_static(const lsrtm_config *cfg, const float *
     a.binv = binv;
     a.kd2 = kd2;
     a.br2 = br2;
-    a.psiv = psiv;
-    a.sstride = 10 * g.plane;
-    a.vstride = 4 * g.plane;
+    a.psiv = st0 + kExtra2D * P;
+    a.sstride = a.vstride = 2 * kStatePlanes2D * g.plane;
     a.tzc = tzc;
     a.wav = wavelet;
     a.wav_per_shot = cfg->wavelet_per_shot;
@@ -382,12 +378,10 @@ extern "C" lsrtm_status lsrtm_born_static(const lsrtm_config *cfg, const float *
     if (t_test_error) SCU(cudaMemsetAsync(a.err, t_test_error, 1, s));
     t_test_error = 0;
     Maps2D maps[2];
-    SCU(maps2d(&maps[0], g, g, st0, a.sstride, kdt, binv, kd2, br2, nullptr, psiv, a.vstride, 1));
-    SCU(maps2d(&maps[1], g, g, st1, a.sstride, kdt, binv, kd2, br2, nullptr, psiv, a.vstride, 1));
+    SCU(maps2d(&maps[0], g, g, st0, a.sstride, kStatePlanes2D, kdt, binv, kd2, br2, nullptr, a.psiv, a.vstride, 1));
+    SCU(maps2d(&maps[1], g, g, st1, a.sstride, kStatePlanes2D, kdt, binv, kd2, br2, nullptr, a.psiv, a.vstride, 1));
     for (int shot = 0; shot < nshot; ++shot) {
         SCU(cudaMemsetAsync(st0, 0, sz[12], s));
-        SCU(cudaMemsetAsync(st1, 0, sz[13], s));
-        SCU(cudaMemsetAsync(psiv, 0, sz[14], s));
         a.shot0 = shot;
         for (int n = 0; n < g.nt; ++n) {
             a.n = n;
