@@ -115,6 +115,11 @@ struct Blk<3> {
     using T = Pairs;
 };
 __device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
+// The four blocks unpacked: for y = H x in 3D, but for four rows a thread.
+// There the packed pairs cost more than they save (60 x 60 x 70: s = 10 762 us
+// for 689, s = 8 377 for 345, s = 3 91 for 79; four rows, s = 5, 164 for 173).
+// For y = H^T x they save or cost nothing (s = 8: 302 us for 391).
+using Quad = float4;
 
 template <int BM>
 __device__ __forceinline__ float load_blk(const float4 *pt, int i, float)
@@ -127,6 +132,11 @@ __device__ __forceinline__ Pairs load_blk(const float4 *pt, int i, Pairs)
     const float4 v = __ldg(pt + i);
     return Pairs{make_float2(v.x, v.y), make_float2(v.z, v.w)};
 }
+template <int BM>
+__device__ __forceinline__ Quad load_blk(const float4 *pt, int i, Quad)
+{
+    return __ldg(pt + i);
+}
 // p0 + w (p1 - p0)
 __device__ __forceinline__ float sub_(float a, float b) { return a - b; }
 __device__ __forceinline__ float2 sub_(float2 a, float2 b) { return __ffma2_rn(dup(-1.f), b, a); }
@@ -134,6 +144,11 @@ __device__ __forceinline__ Pairs sub_(Pairs a, Pairs b) { return Pairs{sub_(a.a,
 __device__ __forceinline__ float lerp_(float p0, float p1, float w) { return fmaf(w, p1 - p0, p0); }
 __device__ __forceinline__ float2 lerp_(float2 p0, float2 p1, float w) { return __ffma2_rn(dup(w), sub_(p1, p0), p0); }
 __device__ __forceinline__ Pairs lerp_(Pairs p0, Pairs p1, float w) { return Pairs{lerp_(p0.a, p1.a, w), lerp_(p0.b, p1.b, w)}; }
+__device__ __forceinline__ Quad sub_(Quad a, Quad b) { return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w); }
+__device__ __forceinline__ Quad lerp_(Quad p0, Quad p1, float w)
+{
+    return make_float4(lerp_(p0.x, p1.x, w), lerp_(p0.y, p1.y, w), lerp_(p0.z, p1.z, w), lerp_(p0.w, p1.w, w));
+}
 // q0 + b d1 + c d2 (= (1 - b - c) q0 + b q1 + c q2 with d1 = q1 - q0, d2 = q2 - q0)
 __device__ __forceinline__ float mix3(float q0, float d1, float d2, float b, float c)
 {
@@ -146,6 +161,11 @@ __device__ __forceinline__ float2 mix3(float2 q0, float2 d1, float2 d2, float2 b
 __device__ __forceinline__ Pairs mix3(Pairs q0, Pairs d1, Pairs d2, float2 b, float2 c)
 {
     return Pairs{mix3(q0.a, d1.a, d2.a, b, c), mix3(q0.b, d1.b, d2.b, b, c)};
+}
+__device__ __forceinline__ Quad mix3(Quad q0, Quad d1, Quad d2, float b, float c)
+{
+    return make_float4(mix3(q0.x, d1.x, d2.x, b, c), mix3(q0.y, d1.y, d2.y, b, c), mix3(q0.z, d1.z, d2.z, b, c),
+                       mix3(q0.w, d1.w, d2.w, b, c));
 }
 // q0 + b d1: rows that no node row separates
 __device__ __forceinline__ float mix2(float q0, float d1, float b) { return fmaf(b, d1, q0); }
@@ -175,6 +195,11 @@ __device__ __forceinline__ void accum(float &a0, float &a1, Pairs C, float2 x)
 {
     a0 = fmaf(C.a.x, x.x, fmaf(TR ? C.b.x : C.a.y, x.y, a0));
     a1 = fmaf(TR ? C.a.y : C.b.x, x.x, fmaf(C.b.y, x.y, a1));
+}
+template <bool TR>
+__device__ __forceinline__ void accum(float &a0, float &a1, Quad C, float2 x)
+{
+    accum<TR>(a0, a1, Pairs{make_float2(C.x, C.y), make_float2(C.z, C.w)}, x);
 }
 
 // Weights of R consecutive rows (first corner row kf) on the node rows
@@ -425,7 +450,9 @@ template <int MASK, bool TR, int R>
 __global__ void __launch_bounds__(k3Threads) k_psfh3_rows(const PsfHess3Dev a, const float *__restrict__ in,
                                                            float *__restrict__ out)
 {
-    using V = typename Blk<MASK>::T;
+    constexpr bool QUAD = MASK == 3 && !TR && R != 4;
+    constexpr int PK = QUAD ? 1 : MASK;   // weights as the blocks take them
+    using V = typename std::conditional<QUAD, Quad, typename Blk<MASK>::T>::type;
     constexpr int P0 = MASK == 2 ? 1 : 0;
     constexpr int BM = MASK == 2 ? 3 : 0;
     __shared__ Corner zc[8 + 2 * kPsfHessMaxHalf], yc[k3Y + 2 * kPsfHessMaxHalf], xc[k3X + 2 * kPsfHessMaxHalf];
@@ -447,14 +474,14 @@ __global__ void __launch_bounds__(k3Threads) k_psfh3_rows(const PsfHess3Dev a, c
     const int nky = a.nky, nkx = a.nkx, nkz1 = a.nkz - 1;
     const V zero = V{};
     float acc0[R], acc1[R];
-    typename Wgt<MASK>::T wb[R], wc[R];
+    typename Wgt<PK>::T wb[R], wc[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) acc0[r] = acc1[r] = 0.f;
     if (!TR) {
         for (int dz = -h; dz <= h; ++dz) {
             const int row0 = h - dz;   // zc index of c_z = Z0 - dz
             const int kf = zc[row0].k0;
-            row_weights<MASK, R>(zc + row0, kf, wb, wc);
+            row_weights<PK, R>(zc + row0, kf, wb, wc);
             const int nq[3] = {kf, min(kf + 1, nkz1), min(kf + 2, nkz1)};
             for (int dy = -h; dy <= h; ++dy) {
                 const int cy = y - dy;
@@ -491,7 +518,7 @@ __global__ void __launch_bounds__(k3Threads) k_psfh3_rows(const PsfHess3Dev a, c
         }
     } else {
         const int kf = zc[h].k0;
-        row_weights<MASK, R>(zc + h, kf, wb, wc);
+        row_weights<PK, R>(zc + h, kf, wb, wc);
         const Corner Y = yc[ty + h], X = xc[tx + h];
         int base[3][2][2];
 #pragma unroll
