@@ -50,7 +50,7 @@ namespace lsrtm {
 
 namespace {
 
-constexpr int kSolveThreads = 256, kSolvePanel = 8;
+constexpr int kSolveThreads = 256, kSolveFew = 64, kSolveFewCtas = 12, kSolvePanel = 8;
 
 __device__ __forceinline__ int tri(int i) { return i * (i + 1) / 2; }
 
@@ -63,10 +63,14 @@ __device__ __forceinline__ int tri_row(int e)
     return i;
 }
 
-// ulen: doubles of the region U, at least one lag's row sums, PZ * flen.
-__global__ void __launch_bounds__(kSolveThreads, 3) k_deblur_solve(const float *mref, const float *mrem, int nz,
-                                                                    int nx, int s, int flen, double eps,
-                                                                    float *filt, int *flag, int ulen)
+// ulen: doubles of the region U, at least one lag's row sums, PZ * flen. NT:
+// threads, at least one a tap; few for small windows, whose sums are too short
+// for more and whose serial parts then run under eleven other CTAs' (three or
+// two of kSolveThreads).
+template <int NT>
+__global__ void __launch_bounds__(NT, NT == kSolveThreads ? 3 : kSolveFewCtas)
+    k_deblur_solve(const float *mref, const float *mrem, int nz, int nx, int s, int flen, double eps, float *filt,
+                   int *flag, int ulen)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int n = flen * flen, h = flen / 2, w2 = 2 * h;
@@ -86,7 +90,7 @@ __global__ void __launch_bounds__(kSolveThreads, 3) k_deblur_solve(const float *
     const float *m1 = mref + param * plane;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
 
-    for (int i = t; i < PZ * PX; i += kSolveThreads) {
+    for (int i = t; i < PZ * PX; i += NT) {
         const int pz = i / PX, px = i - pz * PX;
         const int z = z0 - h + pz, x = x0 - h + px;
         P[pz * PS + px] = (z >= 0 && z < nz && x >= 0 && x < nx) ? (double)m2[(long long)z * nx + x] : 0.0;
@@ -103,7 +107,7 @@ __global__ void __launch_bounds__(kSolveThreads, 3) k_deblur_solve(const float *
             const int cnt = min(chunk, w2 + 1 - d0);
             // rs[(dz, r)][ox] = sum_{c = ox}^{ox + WX - 1} P[r][c] P[r + dz][c + dx], the PZ - dz rows of each dz in turn
             const int items = cnt * (PZ - d0) - cnt * (cnt - 1) / 2;
-            for (int e = t; e < items; e += kSolveThreads) {
+            for (int e = t; e < items; e += NT) {
                 int r = e, dz = d0;
                 while (r >= PZ - dz) {
                     r -= PZ - dz;
@@ -123,7 +127,7 @@ __global__ void __launch_bounds__(kSolveThreads, 3) k_deblur_solve(const float *
             }
             __syncthreads();
             // S(oz, ox) = sum_{r = oz}^{oz + WZ - 1} rs[r][ox] -> G[u][v]; d >= 0 in the order of taps: v <= u
-            for (int e = t; e < cnt * nox; e += kSolveThreads) {
+            for (int e = t; e < cnt * nox; e += NT) {
                 const int j = e / nox, ox = ox0 + e - j * nox, dz = d0 + j;
                 const double *rs = U + (j * (PZ - d0) - j * (j - 1) / 2) * nos + (ox - ox0);
                 double acc = 0.0;
@@ -144,7 +148,7 @@ __global__ void __launch_bounds__(kSolveThreads, 3) k_deblur_solve(const float *
         double acc = 0.0;
         for (int q0 = 0; q0 < WZ * WX; q0 += ulen) {
             const int q1 = min(WZ * WX, q0 + ulen);
-            for (int q = q0 + t; q < q1; q += kSolveThreads) {
+            for (int q = q0 + t; q < q1; q += NT) {
                 const int pz = q / WX;
                 U[q - q0] = (double)m1[(long long)(z0 + pz) * nx + x0 + q - pz * WX];
             }
@@ -175,11 +179,10 @@ __global__ void __launch_bounds__(kSolveThreads, 3) k_deblur_solve(const float *
     const double tr = red[0];
     float *out = filt + (((long long)param * nkz + blockIdx.y) * nkx + blockIdx.x) * n;
     if (tr == 0.0) {   // all-zero remigrated window: zero filter
-        for (int u = t; u < n; u += kSolveThreads) out[u] = 0.f;
+        for (int u = t; u < n; u += NT) out[u] = 0.f;
         return;
     }
-    const double reg = eps * tr / n;
-    for (int u = t; u < n; u += kSolveThreads) G[tri(u) + u] += reg;
+    for (int u = t; u < n; u += NT) G[tri(u) + u] += eps * tr / n;   // (the division by warps with taps only)
     __syncthreads();
 
     // Cholesky G = L L^T with 1 / L_kk on the diagonal; row n becomes y of L y = rhs
@@ -212,7 +215,7 @@ __global__ void __launch_bounds__(kSolveThreads, 3) k_deblur_solve(const float *
             if (bad && lane == 0) red[1] = 1.0;
         }
         __syncthreads();
-        for (int i = t; i <= m; i += kSolveThreads) {
+        for (int i = t; i <= m; i += NT) {
             double *row = G + tri(k1 + i) + k0;
             double x[kSolvePanel];
 #pragma unroll
@@ -231,9 +234,9 @@ __global__ void __launch_bounds__(kSolveThreads, 3) k_deblur_solve(const float *
         __syncthreads();
         // the rest, rows k1..n of columns k1..n-1; m > 0 only below a full panel
         const int rest = tri(m + 1) - 1;
-        for (int e = t; e < rest; e += 2 * kSolveThreads) {
-            const bool two = e + kSolveThreads < rest;   // two entries a thread, for two chains
-            const int e1 = two ? e + kSolveThreads : e;
+        for (int e = t; e < rest; e += 2 * NT) {
+            const bool two = e + NT < rest;   // two entries a thread, for two chains
+            const int e1 = two ? e + NT : e;
             const int ia = tri_row(e), ja = e - tri(ia), ib = tri_row(e1), jb = e1 - tri(ib);
             double *ga = G + tri(k1 + ia) + k1 + ja, *gb = G + tri(k1 + ib) + k1 + jb;
             double va = *ga, vb = *gb;
@@ -889,15 +892,16 @@ cudaError_t launch_wiener(const float *mref, const float *mrem, int nz, int nx, 
 // Doubles of k_deblur_solve's region U, and its shared memory in bytes. The
 // patch and the matrix leave two CTAs an SM (three for flen <= 9) at the usual
 // spacings; U, at least one lag's row sums and the panel, takes the rest of
-// the share, up to what all lags of a dx need.
-int deblur_solve_region(int nz, int nx, int s, int flen, size_t *bytes)
+// the share, up to what all lags of a dx need. most_ctas: CTAs an SM that the
+// kernel's registers leave room for.
+int deblur_solve_region(int nz, int nx, int s, int flen, int most_ctas, size_t *bytes)
 {
     const int n = flen * flen, pz = std::min(nz, 2 * s + 1) + flen - 1, px = std::min(nx, 2 * s + 1) + flen - 1;
     const size_t fixed = ((size_t)(n + 1) * (n + 2) / 2 + 2 + (size_t)pz * (px | 1)) * sizeof(double);
     const int least = std::max(pz * flen, kSolvePanel * (n + 1)), most = std::max(least, pz * flen * flen);
     const int wish = std::max(least, 4 * pz * flen);
     int ulen = least;
-    for (int ctas = 3; ctas >= 1; --ctas) {
+    for (int ctas = most_ctas; ctas >= 1; --ctas) {
         const size_t share = std::min<size_t>(228 * 1024 / ctas - 1024, kDeblurSmemLimit);
         if (fixed + (size_t)(ctas > 1 ? wish : least) * sizeof(double) > share) continue;
         ulen = (int)std::min<size_t>(most, (share - fixed) / sizeof(double));
@@ -914,11 +918,15 @@ cudaError_t launch_deblur(const float *mref, const float *mrem, int nz, int nx, 
 {
     const int nkz = deblur_nodes(nz, s), nkx = deblur_nodes(nx, s);
     size_t sm = 0;
-    const int ulen = deblur_solve_region(nz, nx, s, flen, &sm);
+    // windows of at most 13 x 13 pixels and a thread a tap (300 x 2000: s = 2, one tap 1.45 ms for 5.29 of 256
+    // threads, 49 taps 35.7 for 56.7; s = 6 0.55 for 1.45, 6.0 for 8.2; 90 x 130, s = 8, 49 taps 0.21 for 0.19)
+    const bool few = s <= 6 && flen * flen <= kSolveFew;
+    const int ulen = deblur_solve_region(nz, nx, s, flen, few ? kSolveFewCtas : 3, &sm);
     if (sm > kDeblurSmemLimit) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k_deblur_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    auto k = few ? k_deblur_solve<kSolveFew> : k_deblur_solve<kSolveThreads>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    k_deblur_solve<<<dim3(nkx, nkz, 2), kSolveThreads, sm, st>>>(mref, mrem, nz, nx, s, flen, eps, filt, flag, ulen);
+    k<<<dim3(nkx, nkz, 2), few ? kSolveFew : kSolveThreads, sm, st>>>(mref, mrem, nz, nx, s, flen, eps, filt, flag, ulen);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const long long plane = (long long)nz * nx;
     k_deblur_apply<<<dim3((unsigned)((plane + 255) / 256), 2), 256, 0, st>>>(mref, filt, nz, nx, s, flen, nkz, nkx,
