@@ -396,7 +396,10 @@ size_t lsrtm_workspace_bytes(const lsrtm_handle *h);
  * chunks of at least 2M + 8 rows (and the current one), keeps the fastest
  * and rebuilds the receiver tiling; results do not depend on the choice
  * (every cell is computed the same way). Captured graphs and the cached
- * background are dropped. Outputs (each may be NULL):
+ * background are dropped. A candidate whose steps did not run (a kernel that
+ * gave up waiting for its tile copies, or the non-finite guard set by an
+ * earlier call) fails the call with that error, the chunk height unchanged.
+ * Outputs (each may be NULL):
  *   *tzc      chosen rows per chunk
  *   ms        [2*ncand] pairs (tzc, ms per Born + migration step); room for
  *             at least 2*13 doubles

@@ -34,6 +34,8 @@
 // window; 5.3 ms for the two planes' 3000 windows of 300 x 2000, s = 20, flen =
 // 11): 6.8 ms there, 26.7 with P in float, a lag a warp, the whole matrix and a
 // column at a time; the rest are the Cholesky's and the sums' serial chains.
+// Small windows are bound by those chains: they take CTAs of 64 threads, twelve
+// an SM (launch_deblur).
 // k_deblur_apply: one thread per pixel and plane; FP32 taps, at most four
 // covering nodes.
 // The paper's own Fourier form of the filter (per-block Wiener ratio) follows
@@ -341,7 +343,7 @@ __global__ void k_deblur_apply(const float *mref, const float *filt, int nz, int
 // value is read once instead of N1 or N2 times. The inverse is the forward
 // transform with real and imaginary parts exchanged before and after.
 // Bound by issue slots and the shared memory around the twelve passes with a
-// barrier after each (57% of issue, 56% of L1): 300 x 2000, s = 20 (1500 nodes,
+// barrier after each (65% of issue, 65% of L1's data pipe): 300 x 2000, s = 20 (1500 nodes,
 // N = 40) 100 us with the blend, at 64 registers a thread, three CTAs an SM
 // (9% more at 81 registers, two); k_wiener_block took 533 us there.
 // k_wiener_block: the other N; one CTA per (node, plane); the block, its

@@ -186,15 +186,16 @@ __device__ __forceinline__ bool zpml_node(const GridDev &g, int r)
 //
 // What bounds it: the Born step moves 64 B a cell, 63.1 from DRAM (the shots
 // of a batch share the model), and is held back by latencies between its
-// barriers (54% of the issue slots used). A group of two rows halves the
+// barriers (55% of the issue slots used). A group of two rows halves the
 // barriers; every warp issues one field's copy (one thread that issued all of
 // a row's was waited for 600 to 1000 cycles); interior rows and warps run
 // straight-line code, and what the strips need in the last stage comes with
 // the copies (their warps took twice the others' time and set the CTA's pace).
 // 96 shots of 424 x 1192 padded cells, order 8: 82.0 G cell-updates/s = 0.78
 // of the measured copy rate (a row at a time, one issuing thread: 67.6); the
-// background step with recording, 48 shots: 110.7 G (with per-thread copies:
-// 70.8). Windowed shots: with k_adj2d 1.27x over per-thread copies.
+// background step with recording, 48 shots: 115.4 G (with per-thread copies:
+// 70.8), with bands 75.9. Windowed shots: with k_adj2d 1.27x over per-thread
+// copies.
 // ---------------------------------------------------------------------------
 template <int M, bool BORN, bool HESS>
 struct FwdLay {
@@ -620,24 +621,26 @@ __global__ void __launch_bounds__(NTH, (BANDS || HESS) ? kBandsMinBlocks : kPlai
 // (v^{n+1/2}, lambda_v) and the lambda CPML memories. The step applies the
 // transposed Born sub-steps (S4^T, S3^T on the half nodes from mu; S2^T, S1^T
 // on the nodes from lambda_v), accumulates the two zero-lag images (discrete
-// transposed forms of Eqs. gradkappa, gradrho; the kappa image as sum Q mu),
+// transposed forms of Eqs. gradkappa, gradrho; the kappa image as sum Q lambda_p),
 // rebuilds p^{n-1}, v^{n-1/2} in the interior from the saved boundary bands,
 // and pre-adds the residual of step n-1. The D+ stencils of (p^n, u) and the
 // D- stencils of (v^{n+1/2}, w) run as packed pairs.
 //
 // The adjoint pressure is carried twice: as mu in the pairs, the quantity the
-// D+ stencils take, and as lambda_p in a plane of its own, what the images and
-// the update take. Away from the z strips the ring's entry of a row then is
-// the row's own (p, mu): a row needs neither dt kappa of its look-ahead row nor
-// a second copy of the pairs. (With mu alone, 72 B a cell: 55.2 G, and
+// D+ stencils take, and as lambda_p in a plane of its own (the first of the
+// forward passes' node CPML planes), what the images and the update take. Away
+// from the z strips the ring's entry of a row then is the row's own (p, mu): a
+// row needs neither dt kappa of its look-ahead row nor a second copy of the
+// pairs. (With mu alone, 72 B a cell: 55.2 G, and
 // lambda_p is rounded as mu, which moves the 64-bit misfits of a CG by 1e-8.)
 // Which products of the CPML terms are fused into the subtractions, and in the
 // forward step the source's, is written out for the same reason: left to the
 // compiler, it changes with the code around them.
 //
-// What bounds it: 80 B a cell (81.7 from DRAM), held back like the Born step; 3 tile copies a
-// row where a row at a time took 9. The x strips' band values
-// come one group ahead by asynchronous copies (read where they are used, they
+// What bounds it: 80 B a cell (81.6 from DRAM), held back like the Born step; 3
+// tile copies a row where a row at a time took 9; at order 8 three CTAs an SM
+// leave 80 registers and 76 B of spills. The x strips' band values come one
+// group ahead by asynchronous copies (read where they are used, they
 // doubled the strip warps' time). 96 shots of 424 x 1192, order 8, FP16 bands:
 // 56.0 G cell-updates/s = 0.67 of the measured copy rate (a row at a time with
 // one issuing thread: 42.4; in groups without the straight-line form: 31.5).
@@ -998,6 +1001,9 @@ __device__ __forceinline__ void adj_body(const Arg2D &p)
                     float wx = __fmul_rn(dtbu, lv);
                     if (!XF && pmlxh) {
                         const float l1 = *reinterpret_cast<const float *>(st1 + L::LPX + r * L::F1R) - wx;
+                        // Two roundings of one product, each the one that its instances' results on record have (the
+                        // order-8 instance without a free surface was contracted differently): one form for all would
+                        // move that instance's images by 2e-7 and the 64-bit misfits of its CGs by 1e-7
                         wx = M == 4 && !FS ? fmaf(dtbu, lv, -__fmul_rn(ahx, l1)) : fmaf(-ahx, l1, wx);
                         if (own) outf[A_LPPX * pT + cz] = bhx * l1;
                     }

@@ -122,7 +122,7 @@ struct Geo {
 // ---------------------------------------------------------------------------
 // Born modelling step n -> n+1.
 //
-// What bounds it: 80 B a cell in one pass (112 measured: the tiles' halos come
+// What bounds it: 80 B a cell in one pass (105 measured: the tiles' halos come
 // from DRAM again where neighbours run apart in z) and the issue slots of the
 // halo work. So every warp issues one of a row's tile copies (one thread that
 // issued all eleven was waited for by the CTA), the half nodes of a row are
@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(NTH, kMinBlocks) k3f_born(const __grid_constan
 // in the d strips, where u_d is formed once per node).
 //
 // What bounds it: 88 B a cell in one pass, but the kernel is held back by
-// latencies and instructions (51% of the issue slots used): four outputs a half
+// latencies and instructions (56% of the issue slots used): four outputs a half
 // node instead of one. Against the form it replaces: mu in place of lambda_p
 // needs no pass over the wide tile and no dt kappa there; the four values of a
 // half node lie in one float4, read by one load a tap; the image comes by TMA

@@ -288,9 +288,10 @@ int march2d_rows(int M, int Nz, long long ctas);
 // of two kThreads2D-wide rows of one field: pr over the float2 pair planes of
 // every slot (8-byte elements; coordinates x, z, slot * pps + pair), fl over
 // its float planes (x, z, slot * fps + plane), md over dt kappa and 1/rho (x,
-// z, 0 | 1), mb over the Born model pairs (dt kappa, dt kappa dlnk), (1/rho, rr) (x, z, 0 | 1), im over the image accumulators (x, z,
-// slot). pv: two-row boxes over the in-place node CPML memories along x (x, z,
-// slot) as floats [0] and float2 pairs [1].
+// z, 0 | 1), mb over the Born model pairs (dt kappa, dt kappa dlnk), (1/rho,
+// rr) (x, z, 0 | 1), im over the image accumulators (x, z, slot). md[0] and
+// mb[0] are not read. pv: two-row boxes over the in-place node CPML memories
+// along x (x, z, slot) as floats [0] and float2 pairs [1].
 // Outside the padded grid the copies read zeros. gm is the model's grid,
 // g the slots' (the same without aperture windows); img may be null where no
 // migration step uses the maps.
@@ -355,9 +356,11 @@ cudaError_t launch_model_prep(const GridDev &g, const float *vp, const float *rh
                               float *binv, cudaStream_t s);
 cudaError_t launch_pert_prep(const GridDev &g, const float *dm, const float *kdt,
                              const float *binv, float2 *kd2, float2 *br2, cudaStream_t s);
-// Adds dt kappa times the residual of step n to dt kappa lambda_p (the .y of
-// the (p, dt kappa lambda_p) pairs). kdt: of the model grid gm, of which shot
-// s's slot grid g takes the columns from win_x0[s], or all with win_x0 null.
+// Adds the residual of step n to the adjoint pressure: dt kappa times it to dt
+// kappa lambda_p (the .y of the (p, dt kappa lambda_p) pairs) where lam is null
+// (3D), else the residual to lambda_p in lam (2D; slot stride that of pl), of
+// which dt kappa lambda_p is formed anew. kdt: of the model grid gm, of which
+// shot s's slot grid g takes the columns from win_x0[s], or all with win_x0 null.
 cudaError_t launch_inject_residual(const GridDev &gm, const GridDev &g, const TileRecs &tr, int batch, int shot0,
                                    const float *dstage, int n, const float *kdt, const int *win_x0, float2 *pl,
                                    long long sstride2, float *lam, cudaStream_t s);
@@ -366,7 +369,8 @@ cudaError_t launch_inject_residual(const GridDev &gm, const GridDev &g, const Ti
 // columns [win_x0, win_x0 + win_nx) of shot shot0 + b.
 cudaError_t launch_image_accumulate(const GridDev &gm, const GridDev &g, const float2 *img, int batch, int shot0,
                                     const int *win_x0, const int *win_nx, double2 *acc, cudaStream_t s);
-// acc: (sum Q dt kappa lambda_p, sum of the adjacent half nodes' products).
+// acc: (sum Q lambda_p with kdt given (2D), sum Q dt kappa lambda_p with kdt null
+// (3D); sum of the adjacent half nodes' products).
 cudaError_t launch_image_finalize(const GridDev &g, const double2 *acc, const float *kdt, const float *binv, float *gout,
                                   cudaStream_t s);
 cudaError_t launch_hess_accumulate(const GridDev &gm, const GridDev &g, const float *hess, int batch, int shot0,
